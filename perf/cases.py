@@ -162,7 +162,9 @@ def _blobs(g, n, d, k, box, sigma, noise=0.0):
 def _directions(g, n, d, k, spread):
     """Directions spread around k axes-like unit vectors (at least 0.9 rad apart, by
     construction: signed axes), every point with a length of its own."""
-    q, _ = torch.linalg.qr(torch.randn((d, d), generator=g, device=DEV, dtype=torch.float64))
+    q = torch.randn((d, d), generator=g, device=DEV, dtype=torch.float64).cpu().numpy()
+    q = np.linalg.qr(q)[0]
+    q = torch.from_numpy(np.ascontiguousarray(q)).to(DEV)
     dirs = torch.cat([q, -q], 0)[:k]
     lab = torch.randint(dirs.shape[0], (n,), generator=g, device=DEV)
     P = dirs[lab] + spread * torch.randn((n, d), generator=g, device=DEV, dtype=torch.float64)
