@@ -454,8 +454,11 @@ fms_status fms_label_points(const float* points, int64_t n, int32_t d, const flo
  *   dL/dh   += (1/h^3) sum_ij p_ij ||y_i - x_j||^2 a_ij.
  * Weights are recomputed tile by tile (nothing of size m x n is stored); the
  * forward stores the positions every k updates and at the end (Y_T), and each
- * update's W_i and weight shift (one value per seed), in `ckpt`; the backward
- * recomputes the positions between two checkpoints one segment at a time.
+ * update's W_i, weight shift and mean squared distance (one value per seed), in
+ * `ckpt`; the backward recomputes the positions between two checkpoints one
+ * segment at a time.  From B n m of about 4 million on, points and seeds are
+ * sorted into cells and a seed's points farther than its cutoff (weights whose
+ * sum is below 2^-32 of W_i in FP32) are not visited.
  * A seed whose sum of weights underflows (every point farther than ~13 h in
  * FP32) is recomputed with its weights taken relative to its nearest point.
  *
@@ -470,10 +473,7 @@ fms_status fms_label_points(const float* points, int64_t n, int32_t d, const flo
  *           dL/dh of each set.
  * Both calls are asynchronous on `stream`.  Errors: FMS_ERR_INVALID_ARG (null
  * pointer, sizes out of range, h not finite and positive), FMS_ERR_WORKSPACE
- * (buffers too small or misaligned), FMS_ERR_CUDA (a launch failed).  The
- * pair kernels stage rows in shared memory with bulk copies whose waits are
- * bounded; a wait that gives up turns the affected outputs into NaN (the
- * calls do not synchronise, so it is reported through the results).
+ * (buffers too small or misaligned), FMS_ERR_CUDA (a launch failed).
  *
  * The *_f64 entry points are the same computation in FP64 (double pointers,
  * h as double; `ckpt` and `ws` sized by the *_f64 size functions), for

@@ -1,0 +1,269 @@
+// Cells of nearby points, and the walk over the cells that can reach a group
+// of 32 seeds.
+//
+// A Gaussian weight falls below any share of the sum W of a seed's weights at
+// a finite distance: with n points, dropping every point whose weight is below
+// 2^-(32 + log2 n) W changes W and S/W by less than 2^-32 of W, a 256th of one
+// FP32 rounding (guard_bits; more for FP64).  Points are therefore sorted into
+// cells (the nearest of up to P pivots; a stable counting sort, so the order and
+// every sum that follows is the same on each run), each with a bounding ball, and a group of seeds walks only the cells whose ball comes within the
+// cutoff radius of the group's own ball.  The bound is checked against the W that
+// came out: a group whose smallest W asks for a wider cutoff is evaluated again
+// with that one (up to the distance where exp2 itself gives zero), so no
+// assumption about the seeds enters.  A ball test that meets NaN or infinity
+// keeps the cell.
+#pragma once
+
+#include "fms_internal.cuh"
+
+namespace fms {
+namespace cells {
+
+constexpr int kMaxCells = 256;      // cells of one set (ids are bytes)
+constexpr int kChunkRows = 1024;    // rows one block of the sort handles
+constexpr int kTileRows = 32;       // rows of one staged tile
+
+// dropped weight, relative to W: 2^-kGuardBits (FP32: 2^-24 is one rounding)
+template <typename T>
+__host__ __device__ constexpr float guard_bits() {
+  return sizeof(T) == 4 ? 32.0f : 62.0f;
+}
+// exponent from which exp2(-x) is exactly zero (FP32 flushes to zero below 2^-126)
+template <typename T>
+__host__ __device__ constexpr float zero_bits() {
+  return sizeof(T) == 4 ? 128.0f : 1100.0f;
+}
+
+// Cells of B sets of n rows each (row b n + i).
+template <typename T>
+struct View {
+  int P;                 // cells per set; 0: one cell with every row, nothing sorted
+  const int32_t* start;  // [B][P + 1] first row of each cell (within the set)
+  const T* ctr;          // [B][P][DP] cell centres (the pivots)
+  const T* rad;          // [B][P] squared distance of the farthest row
+};
+
+// Groups of at most 32 rows of one cell.
+struct Groups {
+  const int2* table;     // [B][per_set] (first row within the set, rows); null: consecutive rows
+  int per_set;           // groups of a set, some of them empty
+};
+
+template <typename T>
+__device__ __forceinline__ T warp_max(T v) {
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const T u = __shfl_xor_sync(kFull, v, o);
+    v = (u > v || !(u == u)) ? u : v;   // NaN wins
+  }
+  return v;
+}
+template <typename T>
+__device__ __forceinline__ T warp_min(T v) {
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const T u = __shfl_xor_sync(kFull, v, o);
+    v = (u < v || !(u == u)) ? u : v;   // NaN wins
+  }
+  return v;
+}
+
+__device__ __forceinline__ float csqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ double csqrt(double x) { return sqrt(x); }
+
+// Ball around the warp's 32 rows: their mean (same value in every lane) and
+// the distance of the farthest.
+template <typename T, int DP>
+__device__ __forceinline__ T group_ball(const T (&y)[DP], T (&c)[DP]) {
+  T r2 = T(0);
+#pragma unroll
+  for (int k = 0; k < DP; ++k) {
+    T s = y[k];
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    c[k] = s * T(1.0 / 32);
+    const T e = y[k] - c[k];
+    r2 += e * e;
+  }
+  return csqrt(warp_max(r2));
+}
+
+// The exponent below which weights may be dropped for a seed whose weights sum to W.
+template <typename T>
+__device__ __forceinline__ T cut_bits(T W, T log2n) {
+  const T need = T(guard_bits<T>()) + log2n - T(log2f((float)W));
+  return need < T(zero_bits<T>()) ? (need > T(1) ? need : T(1)) : T(zero_bits<T>());
+}
+
+// The warp's list of the cells of one set that a ball (centre c, reach = its
+// radius + the cutoff radius) touches, as (first row, rows); returns its length.
+template <typename T, int DP>
+__device__ __forceinline__ int visible_cells(const View<T>& v, int b, int n, const T (&c)[DP],
+                                             T reach, int2* list, int lane) {
+  if (v.P == 0) {
+    if (lane == 0) list[0] = make_int2(0, n);
+    __syncwarp();
+    return 1;
+  }
+  const int32_t* st = v.start + (int64_t)b * (v.P + 1);
+  int cnt = 0;
+  for (int p0 = 0; p0 < v.P; p0 += 32) {
+    const int p = p0 + lane;
+    const T* q = v.ctr + ((int64_t)b * v.P + p) * DP;
+    T d2 = T(0);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      const T e = q[k] - c[k];
+      d2 += e * e;
+    }
+    // 1e-4 covers the rounding of the distances and of their sum
+    const T lim = (reach + csqrt(v.rad[(int64_t)b * v.P + p])) * T(1.0001);
+    const int a = st[p], e = st[p + 1];
+    const bool see = e > a && !(d2 > lim * lim);
+    const unsigned m = __ballot_sync(kFull, see);
+    if (see) list[cnt + __popc(m & ((1u << lane) - 1u))] = make_int2(a, e - a);
+    cnt += __popc(m);
+  }
+  __syncwarp();
+  return cnt;
+}
+
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Warp w of a team of W walks every W-th tile of the listed row ranges in
+// order: tiles of at most 32 consecutive rows of ROW elements, copied
+// asynchronously one tile ahead into the warp's two-tile ring, tile_fn(rows in
+// shared memory, count) for each.
+template <int ROW, typename T, typename F>
+__device__ __forceinline__ void walk_tiles(const T* __restrict__ rows, const int2* list, int nlist,
+                                           int w, int W, T* ring, int lane, F&& tile_fn) {
+  static_assert((ROW * sizeof(T)) % 16 == 0, "rows are copied 16 bytes at a time");
+  constexpr int PER16 = 16 / (int)sizeof(T);
+  int v = 0, t = w, cnt = 0;
+  int2 cur = nlist > 0 ? list[0] : make_int2(0, 0);
+  auto next = [&](int* row0) -> int {   // rows of the warp's next tile, 0 at the end
+    while (v < nlist) {
+      const int nt = (cur.y + kTileRows - 1) / kTileRows;
+      if (t < nt) {
+        const int r = t * kTileRows;
+        *row0 = cur.x + r;
+        t += W;
+        return min(kTileRows, cur.y - r);
+      }
+      t -= nt;
+      if (++v < nlist) cur = list[v];
+    }
+    return 0;
+  };
+  auto copy = [&](int row0, int c, T* dst) {
+    const T* src = rows + (int64_t)row0 * ROW;
+    const int n16 = c * (ROW / PER16);
+    for (int i = lane; i < n16; i += 32) cp16(dst + i * PER16, src + i * PER16);
+  };
+  int row0 = 0, st = 0;
+  cnt = next(&row0);
+  if (cnt) copy(row0, cnt, ring);
+  cp_commit();
+  while (cnt) {
+    const int c2 = next(&row0);
+    if (c2) copy(row0, c2, ring + (st ^ 1) * kTileRows * ROW);
+    cp_commit();
+    cp_wait<1>();
+    __syncwarp();
+    tile_fn(ring + st * kTileRows * ROW, cnt);
+    __syncwarp();
+    cnt = c2;
+    st ^= 1;
+  }
+  cp_wait<0>();
+}
+
+// Cells for a set of n points and m seeds (a power of two >= 32).  Half of them
+// start from strided points, so a cluster holding a share f of the points is
+// missed by all of those with probability exp(-f P / 2); fewer than 64 rows to a
+// strided cell would leave the groups of 32 mostly padding.
+inline int choose_cells(int64_t n, int64_t m) {
+  const int64_t p = (n < m ? n : m) / 64 * 2;
+  int P = 32;
+  while (P * 2 <= p && P < kMaxCells) P *= 2;
+  return P;
+}
+
+inline int64_t sort_blocks(int64_t rows) { return (rows + kChunkRows - 1) / kChunkRows; }
+inline int group_cap(int64_t rows, int P) { return (int)((rows + 31) / 32) + P; }
+
+// Scratch of one sort of B sets of `rows` rows: cell ids, block counts, farthest rows.
+struct SortScratch {
+  size_t id, counts, far_, total;
+};
+inline SortScratch sort_scratch(int64_t B, int64_t rows, int P) {
+  SortScratch s{};
+  s.counts = align256((size_t)B * rows);
+  s.far_ = s.counts + align256((size_t)B * sort_blocks(rows) * P * 4);
+  s.total = s.far_ + align256((size_t)B * (P / 2) * 8);
+  return s;
+}
+
+// Sorts B sets of nrows rows of DP values (set b at src + b nrows DP) into P
+// cells each.  points: the rows make the pivots, ctr [B][P][DP], npiv [B] and rad
+// [B][P] (squared) are written; else (seeds) ctr and npiv are read.  Writes dst
+// (sorted rows), perm (sorted position -> row of the set), start [B][P + 1] and,
+// where non-null, the table of groups [B][group_cap(nrows, P)].
+template <typename T>
+cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
+                        void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
+                        int32_t* npiv, T* rad, int2* table, cudaStream_t st);
+
+}  // namespace cells
+
+// ---- k_unroll.cu (rows of DP values; seeds and points in sorted order)
+
+// Updates u0 .. u0 + len - 1 of one checkpoint segment: positions before update
+// u (u0 <= u <= u0 + len), and W, the weight shift and the mean squared distance of each update.
+template <typename T>
+struct USegment {
+  const T* ck0;        // positions before update 0 (a checkpoint)
+  const T* ck1;        // positions after the segment's last update (a checkpoint)
+  const T* seg;        // positions before updates 1 .. last
+  int64_t row_values;  // values of one set of positions
+  int seg_len, u0, len;
+  const T* W;          // row 0: update 0
+  const T* Sh;
+  const T* M2;
+  __device__ const T* pos(int u) const {
+    u += u0;
+    return u == 0 ? ck0 : (u == seg_len ? ck1 : seg + (int64_t)(u - 1) * row_values);
+  }
+};
+
+template <typename T>
+cudaError_t unroll_forward_steps(const T* X, const cells::View<T>& cv, const T* Y0,
+                                 const cells::Groups& gr, const UGeom& g, T c, int steps,
+                                 int every, int slot0, T* pos, T* Wout, T* Sh, T* M2, cudaStream_t st);
+// SD: len x [B m] x (2 DP + 4); bctr, breach: len x [B groups] x DP and x 1;
+// dh_part: one per group; first: dX and dh_part are set, not added to.
+template <typename T>
+cudaError_t unroll_backward_segment(const T* X, const cells::View<T>& cv, const USegment<T>& sg,
+                                    const cells::Groups& gx, const cells::Groups& gr,
+                                    const UGeom& g, T c, T inv_h2, double inv_h3, const T* Gin,
+                                    T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX,
+                                    int first, cudaStream_t st);
+cudaError_t unroll_dh_sum(const double* dh_part, int B, int per_set, double* dh, cudaStream_t st);
+template <typename T>
+cudaError_t unroll_pack_rows(const T* src, int64_t rows, int per_set, int d, int DP,
+                             const int32_t* perm, T* dst, cudaStream_t st);
+template <typename T>
+cudaError_t unroll_unpack_rows(const T* src, int64_t rows, int per_set, int d, int DP,
+                               const int32_t* perm, T* dst, cudaStream_t st);
+
+}  // namespace fms

@@ -5,8 +5,7 @@
 #include <string.h>
 
 #include "../../include/fms.h"
-#include "fms_internal.cuh"
-
+#include "fms_cells.cuh"
 
 using namespace fms;
 
@@ -26,18 +25,6 @@ int sm_count() {
   return s;
 }
 
-// Chunks so that (sets x groups of 32 outputs x chunks) ~ 8 tasks per resident warp.
-void chunks(int64_t groups, int64_t len, int sms, int* C, int* L) {
-  const int64_t target = (int64_t)(sms > 0 ? sms : 1) * 16 * 8;
-  int64_t c = (target + groups - 1) / groups;
-  if (c < 1) c = 1;
-  if (c > (len + 63) / 64) c = (len + 63) / 64;
-  if (c < 1) c = 1;
-  int64_t l = (len + c - 1) / c;
-  *C = (int)((len + l - 1) / l);
-  *L = (int)l;
-}
-
 // rows padded to 4, 8, 16 or 32 floats (the kernels know the width at compile time)
 int padded_width(int d) { return d <= 4 ? 4 : (d <= 8 ? 8 : (d <= 16 ? 16 : 32)); }
 
@@ -49,24 +36,55 @@ UGeom geom(int32_t B, int64_t n, int64_t m, int32_t d) {
   g.d = d;
   g.DP = padded_width(d);
   const int sms = sm_count();
-  // seed-major passes: groups of 32 seeds; point-major pass: 64 points (32 at DP = 32)
-  const int ppw = g.DP <= 16 ? 64 : 32;
-  chunks((int64_t)B * ((m + 31) / 32), n, sms, &g.Cp, &g.Lp);
-  chunks((int64_t)B * ((n + ppw - 1) / ppw), m, sms, &g.Cs, &g.Ls);
+  g.sms = sms > 0 ? sms : 1;
   return g;
 }
 
-int grid_blocks() {
-  const int s = sm_count();
-  return (s > 0 ? s : 1) * 8;
+// Cells per set, 0 for none.  Sorting points and seeds takes ~40 us in each
+// direction; below ~4 M pairs an update the whole pass over every pair is cheaper.
+int cells_for(int32_t B, int64_t n, int64_t m) {
+  if (B > 65535 || (double)B * (double)n * (double)m < 4194304.0) return 0;
+  return cells::choose_cells(n, m);
 }
 
 int n_ckpt(int32_t T, int32_t k) { return (T + k - 1) / k; }
 
-struct FwdLayout {
-  size_t Xp, Ya, Yb, part, rlist, status, total;
+int groups_for(int64_t rows, int P) {
+  return P > 0 ? cells::group_cap(rows, P) : (int)((rows + 31) / 32);
+}
+
+// updates of a segment whose seed rows are kept for one point-major pass
+constexpr int kPointBatch = 8;
+
+// Sorted copies of the points (and the scratch of sorting them and the seeds).
+struct SortLayout {
+  size_t Xp, Xs, perm, start, ctr, npiv, rad, table, ystart, scratch;
 };
-FwdLayout fwd_layout(const UGeom& g, size_t es) {
+
+template <typename Take>
+SortLayout sort_layout(const UGeom& g, int P, size_t es, Take&& take) {
+  SortLayout L{};
+  const size_t rows = (size_t)g.B * g.n, pad = (size_t)g.DP * es;
+  L.Xs = take(rows * pad);
+  if (P == 0) return L;
+  L.Xp = take(rows * pad);
+  L.perm = take(rows * 4);
+  L.start = take((size_t)g.B * (P + 1) * 4);
+  L.ctr = take((size_t)g.B * P * pad);
+  L.npiv = take((size_t)g.B * 4);
+  L.rad = take((size_t)g.B * P * es);
+  L.table = take((size_t)g.B * cells::group_cap(g.n, P) * 8);
+  L.ystart = take((size_t)g.B * (P + 1) * 4);
+  const size_t a = cells::sort_scratch(g.B, g.n, P).total, b = cells::sort_scratch(g.B, g.m, P).total;
+  L.scratch = take(a > b ? a : b);
+  return L;
+}
+
+struct FwdLayout {
+  SortLayout s;
+  size_t Yp, total;
+};
+FwdLayout fwd_layout(const UGeom& g, int P, size_t es) {
   FwdLayout L{};
   size_t o = 0;
   auto take = [&](size_t b) {
@@ -74,20 +92,17 @@ FwdLayout fwd_layout(const UGeom& g, size_t es) {
     o += a256(b > 0 ? b : 1);
     return at;
   };
-  L.Xp = take((size_t)g.B * g.n * g.DP * es);
-  L.Ya = take((size_t)g.B * g.m * g.DP * es);
-  L.Yb = take((size_t)g.B * g.m * g.DP * es);
-  L.part = take((size_t)g.B * g.Cp * g.m * (g.DP + 1) * es);
-  L.rlist = take(((size_t)g.B * g.m + 1) * 4);   // rescue list, then its count
-  L.status = take(64);   // kStTimeout if a staged-row wait gave up
+  L.s = sort_layout(g, P, es, take);
+  L.Yp = P > 0 ? take((size_t)g.B * g.m * g.DP * es) : 0;
   L.total = o;
   return L;
 }
 
 struct BwdLayout {
-  size_t Xp, seg, Ga, Gb, part_s, part_p, SD, dh_part, dXp, dh, rlist, status, total;
+  SortLayout s;
+  size_t seg, Ga, Gb, SD, bctr, breach, dh_part, dXp, total;
 };
-BwdLayout bwd_layout(const UGeom& g, int32_t k, size_t es) {
+BwdLayout bwd_layout(const UGeom& g, int P, int32_t k, size_t es) {
   BwdLayout L{};
   size_t o = 0;
   auto take = [&](size_t b) {
@@ -95,37 +110,39 @@ BwdLayout bwd_layout(const UGeom& g, int32_t k, size_t es) {
     o += a256(b > 0 ? b : 1);
     return at;
   };
-  const size_t rowsY = (size_t)g.B * g.m;
-  L.Xp = take((size_t)g.B * g.n * g.DP * es);
+  const size_t rowsY = (size_t)g.B * g.m, NG = (size_t)g.B * groups_for(g.m, P);
+  const size_t pb = (size_t)(k < kPointBatch ? k : kPointBatch);
+  L.s = sort_layout(g, P, es, take);
   L.seg = take((size_t)k * rowsY * g.DP * es);   // recomputed positions inside a segment
   L.Ga = take(rowsY * g.DP * es);
   L.Gb = take(rowsY * g.DP * es);
-  L.part_s = take((size_t)g.B * g.Cp * g.m * (g.DP + 1) * es);
-  L.part_p = take((size_t)g.B * g.Cs * g.n * g.DP * es);
-  L.SD = take(rowsY * (2 * g.DP + 4) * es);
-  L.dh_part = take(rowsY * es);
+  L.SD = take(pb * rowsY * (2 * g.DP + 4) * es);
+  L.bctr = take(pb * NG * g.DP * es);
+  L.breach = take(pb * NG * es);
+  L.dh_part = take(NG * 8);
   L.dXp = take((size_t)g.B * g.n * g.DP * es);
-  L.dh = take((size_t)g.B * 8);
-  L.rlist = take((rowsY + 1) * 4);
-  L.status = take(64);
   L.total = o;
   return L;
 }
 
 // The checkpoint buffer: positions Y_t for t = 0, k, 2k, .. and Y_T (rows of
-// DP values), then W_t and the weight shift of every update t < T (one value
-// per seed each), so the backward recomputes only the positions between
-// checkpoints.
+// DP values, seeds in sorted order), then W_t, the weight shift and the mean
+// squared distance of every update t < T (one value per seed each), so the
+// backward recomputes only the positions between checkpoints; with cells, the
+// seeds' order and groups.
 struct CkptLayout {
-  size_t pos, W, Sh, total;
+  size_t pos, W, Sh, M2, perm, table, total;
 };
-CkptLayout ckpt_layout(int32_t B, int64_t m, int32_t d, int32_t T, int32_t k, size_t es) {
+CkptLayout ckpt_layout(const UGeom& g, int P, int32_t T, int32_t k, size_t es) {
   CkptLayout C{};
-  const size_t rowsY = (size_t)B * m;
+  const size_t rowsY = (size_t)g.B * g.m;
   C.pos = 0;
-  C.W = (size_t)(n_ckpt(T, k) + 1) * rowsY * padded_width(d) * es;
+  C.W = (size_t)(n_ckpt(T, k) + 1) * rowsY * g.DP * es;
   C.Sh = C.W + (size_t)T * rowsY * es;
-  C.total = C.Sh + (size_t)T * rowsY * es;
+  C.M2 = C.Sh + (size_t)T * rowsY * es;
+  C.perm = a256(C.M2 + (size_t)T * rowsY * es);
+  C.table = C.perm + (P > 0 ? a256(rowsY * 4) : 0);
+  C.total = C.table + (P > 0 ? (size_t)g.B * cells::group_cap(g.m, P) * 8 : 0);
   return C;
 }
 
@@ -134,139 +151,155 @@ T* at(void* base, size_t off) {
   return reinterpret_cast<T*>(static_cast<char*>(base) + off);
 }
 
-}  // namespace
-
-namespace {
+// Padded (and, with cells, sorted) copy of the points.
+template <typename E>
+cudaError_t sort_points(const E* points, const UGeom& g, int P, const SortLayout& L, void* ws,
+                        cells::View<E>* cv, cudaStream_t st) {
+  E* Xs = at<E>(ws, L.Xs);
+  const int64_t rows = (int64_t)g.B * g.n;
+  *cv = cells::View<E>{};
+  if (P == 0) return unroll_pack_rows<E>(points, rows, g.n, g.d, g.DP, nullptr, Xs, st);
+  const E* src = points;
+  if (g.d != g.DP || (reinterpret_cast<uintptr_t>(points) & 15u)) {
+    E* Xp = at<E>(ws, L.Xp);
+    const cudaError_t e = unroll_pack_rows<E>(points, rows, g.n, g.d, g.DP, nullptr, Xp, st);
+    if (e != cudaSuccess) return e;
+    src = Xp;
+  }
+  cv->P = P;
+  cv->start = at<int32_t>(ws, L.start);
+  cv->ctr = at<E>(ws, L.ctr);
+  cv->rad = at<E>(ws, L.rad);
+  return cells::launch_sort<E>(src, g.B, g.n, g.DP, true, P, at<void>(ws, L.scratch), Xs,
+                               at<int32_t>(ws, L.perm), at<int32_t>(ws, L.start),
+                               at<E>(ws, L.ctr), at<int32_t>(ws, L.npiv), at<E>(ws, L.rad),
+                               at<int2>(ws, L.table), st);
+}
 
 template <typename E>
-fms_status forward_impl(const E* points, const E* seeds0, int32_t B, int64_t n,
-                                int64_t m, int32_t d, E h, int32_t T, int32_t k,
-                                E* out_seeds, void* ckpt, size_t ckpt_bytes, void* ws,
-                                size_t ws_bytes, void* stream) {
+fms_status forward_impl(const E* points, const E* seeds0, int32_t B, int64_t n, int64_t m,
+                        int32_t d, E h, int32_t T, int32_t k, E* out_seeds, void* ckpt,
+                        size_t ckpt_bytes, void* ws, size_t ws_bytes, void* stream) {
   if (!points || !seeds0 || !out_seeds || !valid(B, n, m, d, T, k) || !(h > 0) || !isfinite(h))
     return FMS_ERR_INVALID_ARG;
   if (!ws || !ckpt) return FMS_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const UGeom g = geom(B, n, m, d);
-  const FwdLayout L = fwd_layout(g, sizeof(E));
-  if (ws_bytes < L.total || ckpt_bytes < ckpt_layout(B, m, d, T, k, sizeof(E)).total ||
-      (reinterpret_cast<uintptr_t>(ws) & 255u) || (reinterpret_cast<uintptr_t>(ckpt) & 15u))
+  const int P = cells_for(B, n, m);
+  const FwdLayout L = fwd_layout(g, P, sizeof(E));
+  const CkptLayout CL = ckpt_layout(g, P, T, k, sizeof(E));
+  if (ws_bytes < L.total || ckpt_bytes < CL.total || (reinterpret_cast<uintptr_t>(ws) & 255u) ||
+      (reinterpret_cast<uintptr_t>(ckpt) & 15u))
     return FMS_ERR_WORKSPACE;
-  E* Xp = at<E>(ws, L.Xp);
-  E* Ya = at<E>(ws, L.Ya);
-  E* Yb = at<E>(ws, L.Yb);
-  E* part = at<E>(ws, L.part);
-  int32_t* rlist = at<int32_t>(ws, L.rlist);
-  int32_t* rcount = rlist + (size_t)B * m;
-  uint32_t* status = at<uint32_t>(ws, L.status);
-  const CkptLayout CL = ckpt_layout(B, m, d, T, k, sizeof(E));
-  E* C = at<E>(ckpt, CL.pos);
-  E* Wh = at<E>(ckpt, CL.W);
-  E* Shh = at<E>(ckpt, CL.Sh);
-  const size_t rowsY = (size_t)B * m;
+  E* pos = at<E>(ckpt, CL.pos);
+  int32_t* yperm = P > 0 ? at<int32_t>(ckpt, CL.perm) : nullptr;
+  const int64_t rowsY = (int64_t)B * m;
   const E c = (E)(1.4426950408889634 / (2.0 * (double)h * (double)h));
-  const int grid = grid_blocks();
-  if (unroll_pack_rows<E>(points, (int64_t)B * n, d, g.DP, Xp, st) != cudaSuccess ||
-      unroll_pack_rows<E>(seeds0, (int64_t)rowsY, d, g.DP, Ya, st) != cudaSuccess ||
-      cudaMemsetAsync(rcount, 0, 4, st) != cudaSuccess ||
-      cudaMemsetAsync(status, 0, 64, st) != cudaSuccess)
+  cells::View<E> cv;
+  if (sort_points<E>(points, g, P, L.s, ws, &cv, st) != cudaSuccess) return FMS_ERR_CUDA;
+  cells::Groups gr{nullptr, groups_for(m, P)};
+  if (P > 0) {
+    const E* src = seeds0;
+    if (d != g.DP || (reinterpret_cast<uintptr_t>(seeds0) & 15u)) {
+      E* Yp = at<E>(ws, L.Yp);
+      if (unroll_pack_rows<E>(seeds0, rowsY, (int)m, d, g.DP, nullptr, Yp, st) != cudaSuccess)
+        return FMS_ERR_CUDA;
+      src = Yp;
+    }
+    int2* table = at<int2>(ckpt, CL.table);
+    gr.table = table;
+    if (cells::launch_sort<E>(src, B, m, g.DP, false, P, at<void>(ws, L.s.scratch), pos, yperm,
+                              at<int32_t>(ws, L.s.ystart), at<E>(ws, L.s.ctr),
+                              at<int32_t>(ws, L.s.npiv), nullptr, table, st) != cudaSuccess)
+      return FMS_ERR_CUDA;
+  } else if (unroll_pack_rows<E>(seeds0, rowsY, (int)m, d, g.DP, nullptr, pos, st) !=
+             cudaSuccess) {
     return FMS_ERR_CUDA;
-  for (int t = 0; t < T; ++t) {
-    if (t % k == 0 &&
-        cudaMemcpyAsync(C + (size_t)(t / k) * rowsY * g.DP, Ya, rowsY * g.DP * sizeof(E),
-                        cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return FMS_ERR_CUDA;
-    if (unroll_fwd_step<E>(Xp, Ya, g, c, part, Yb, Wh + (size_t)t * rowsY, Shh + (size_t)t * rowsY,
-                           rlist, rcount, grid, status, st) != cudaSuccess)
-      return FMS_ERR_CUDA;
-    E* tmp = Ya;
-    Ya = Yb;
-    Yb = tmp;
   }
-  if (cudaMemcpyAsync(C + (size_t)n_ckpt(T, k) * rowsY * g.DP, Ya, rowsY * g.DP * sizeof(E),
-                      cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-      unroll_unpack_rows<E>(Ya, (int64_t)rowsY, d, g.DP, out_seeds, st) != cudaSuccess)
+  if (unroll_forward_steps<E>(at<E>(ws, L.s.Xs), cv, pos, gr, g, c, T, k, 0, pos,
+                              at<E>(ckpt, CL.W), at<E>(ckpt, CL.Sh), at<E>(ckpt, CL.M2), st) != cudaSuccess ||
+      unroll_unpack_rows<E>(pos + (size_t)n_ckpt(T, k) * rowsY * g.DP, rowsY, (int)m, d, g.DP,
+                            yperm, out_seeds, st) != cudaSuccess)
     return FMS_ERR_CUDA;
   return FMS_OK;
 }
 
 template <typename E>
-fms_status backward_impl(const E* points, int32_t B, int64_t n, int64_t m, int32_t d,
-                                 E h, int32_t T, int32_t k, const void* ckpt,
-                                 size_t ckpt_bytes, const E* grad_out, E* grad_points,
-                                 E* grad_seeds0, double* grad_h, void* ws, size_t ws_bytes,
-                                 void* stream) {
+fms_status backward_impl(const E* points, int32_t B, int64_t n, int64_t m, int32_t d, E h,
+                         int32_t T, int32_t k, const void* ckpt, size_t ckpt_bytes,
+                         const E* grad_out, E* grad_points, E* grad_seeds0, double* grad_h,
+                         void* ws, size_t ws_bytes, void* stream) {
   if (!points || !grad_out || !grad_points || !grad_seeds0 || !grad_h ||
       !valid(B, n, m, d, T, k) || !(h > 0) || !isfinite(h))
     return FMS_ERR_INVALID_ARG;
   if (!ws || !ckpt) return FMS_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const UGeom g = geom(B, n, m, d);
-  const BwdLayout L = bwd_layout(g, k, sizeof(E));
-  if (ws_bytes < L.total || ckpt_bytes < ckpt_layout(B, m, d, T, k, sizeof(E)).total ||
-      (reinterpret_cast<uintptr_t>(ws) & 255u) || (reinterpret_cast<uintptr_t>(ckpt) & 15u))
+  const int P = cells_for(B, n, m);
+  const BwdLayout L = bwd_layout(g, P, k, sizeof(E));
+  const CkptLayout CL = ckpt_layout(g, P, T, k, sizeof(E));
+  if (ws_bytes < L.total || ckpt_bytes < CL.total || (reinterpret_cast<uintptr_t>(ws) & 255u) ||
+      (reinterpret_cast<uintptr_t>(ckpt) & 15u))
     return FMS_ERR_WORKSPACE;
-  E* Xp = at<E>(ws, L.Xp);
+  void* ck = const_cast<void*>(ckpt);   // read only
+  const E* Ck = at<E>(ck, CL.pos);
+  const int32_t* yperm = P > 0 ? at<int32_t>(ck, CL.perm) : nullptr;
+  const cells::Groups gr{P > 0 ? at<int2>(ck, CL.table) : nullptr, groups_for(m, P)};
+  const cells::Groups gx{P > 0 ? at<int2>(ws, L.s.table) : nullptr, groups_for(n, P)};
+  E* Xs = at<E>(ws, L.s.Xs);
   E* seg = at<E>(ws, L.seg);
-  int32_t* rlist = at<int32_t>(ws, L.rlist);
-  int32_t* rcount = rlist + (size_t)B * m;
-  E* Ga = at<E>(ws, L.Ga);
-  E* Gb = at<E>(ws, L.Gb);
-  E* part_s = at<E>(ws, L.part_s);
-  E* part_p = at<E>(ws, L.part_p);
-  E* SD = at<E>(ws, L.SD);
-  uint32_t* status = at<uint32_t>(ws, L.status);
-  E* dh_part = at<E>(ws, L.dh_part);
+  E* G = at<E>(ws, L.Ga);
+  E* Gp = at<E>(ws, L.Gb);
   E* dXp = at<E>(ws, L.dXp);
-  double* dh = at<double>(ws, L.dh);
-  const CkptLayout CL = ckpt_layout(B, m, d, T, k, sizeof(E));
-  const E* Ck = static_cast<const E*>(ckpt);
-  const E* Wh = Ck + CL.W / sizeof(E);
-  const E* Shh = Ck + CL.Sh / sizeof(E);
-  const size_t rowsY = (size_t)B * m;
-  const size_t rowY = rowsY * g.DP;
+  double* dh_part = at<double>(ws, L.dh_part);
+  const int64_t rowsY = (int64_t)B * m, rowY = rowsY * g.DP;
   const double hd = (double)h;
   const E c = (E)(1.4426950408889634 / (2.0 * hd * hd));
-  const E inv_h2 = (E)(1.0 / (hd * hd)), inv_h3 = (E)(1.0 / (hd * hd * hd));
-  const int grid = grid_blocks();
-  if (unroll_pack_rows<E>(points, (int64_t)B * n, d, g.DP, Xp, st) != cudaSuccess ||
-      unroll_pack_rows<E>(grad_out, (int64_t)rowsY, d, g.DP, Ga, st) != cudaSuccess ||
-      cudaMemsetAsync(dXp, 0, (size_t)B * n * g.DP * sizeof(E), st) != cudaSuccess ||
-      cudaMemsetAsync(dh, 0, (size_t)B * 8, st) != cudaSuccess ||
-      cudaMemsetAsync(rcount, 0, 4, st) != cudaSuccess ||
-      cudaMemsetAsync(status, 0, 64, st) != cudaSuccess)
+  const E inv_h2 = (E)(1.0 / (hd * hd));
+  const double inv_h3 = 1.0 / (hd * hd * hd);
+  cells::View<E> cv;
+  if (sort_points<E>(points, g, P, L.s, ws, &cv, st) != cudaSuccess ||
+      unroll_pack_rows<E>(grad_out, rowsY, (int)m, d, g.DP, yperm, G, st) != cudaSuccess)
     return FMS_ERR_CUDA;
-  E* G = Ga;
-  E* Gp = Gb;
+  int first = 1;
   for (int s = n_ckpt(T, k) - 1; s >= 0; --s) {
     const int t0 = s * k;
     const int len = (t0 + k <= T) ? k : T - t0;
     // positions of the segment: Y_t0 and Y_{t0+len} are checkpoints (the last
     // is Y_T for the final segment); Y_{t0+1} .. Y_{t0+len-1} are recomputed
     // into seg (W and the shifts of every update were stored by the forward)
-    auto pos = [&](int u) -> const E* {
-      if (u == 0) return Ck + (size_t)s * rowY;
-      if (u == len) return Ck + (size_t)(s + 1) * rowY;
-      return seg + (size_t)(u - 1) * rowY;
-    };
-    for (int u = 0; u + 1 < len; ++u)
-      if (unroll_fwd_step<E>(Xp, pos(u), g, c, part_s, seg + (size_t)u * rowY, nullptr, nullptr,
-                             rlist, rcount, grid, status, st) != cudaSuccess)
-        return FMS_ERR_CUDA;
-    for (int u = len - 1; u >= 0; --u) {
-      const size_t t = (size_t)(t0 + u);
-      if (unroll_bwd_step<E>(Xp, pos(u), pos(u + 1), G, Wh + t * rowsY, Shh + t * rowsY, g, c,
-                             inv_h2, inv_h3, part_s, part_p, SD, dh_part, Gp, dXp, dh, grid,
-                             status, st) != cudaSuccess)
+    if (len > 1 && unroll_forward_steps<E>(Xs, cv, Ck + (size_t)s * rowY, gr, g, c, len - 1, 1, 1,
+                                           seg, nullptr, nullptr, nullptr, st) != cudaSuccess)
+      return FMS_ERR_CUDA;
+    for (int hi = len; hi > 0;) {
+      const int lo = hi > kPointBatch ? hi - kPointBatch : 0;
+      USegment<E> sg{};
+      sg.ck0 = Ck + (size_t)s * rowY;
+      sg.ck1 = Ck + (size_t)(s + 1) * rowY;
+      sg.seg = seg;
+      sg.row_values = rowY;
+      sg.seg_len = len;
+      sg.u0 = lo;
+      sg.len = hi - lo;
+      sg.W = at<E>(ck, CL.W) + (size_t)t0 * rowsY;
+      sg.Sh = at<E>(ck, CL.Sh) + (size_t)t0 * rowsY;
+      sg.M2 = at<E>(ck, CL.M2) + (size_t)t0 * rowsY;
+      if (unroll_backward_segment<E>(Xs, cv, sg, gx, gr, g, c, inv_h2, inv_h3, G, Gp,
+                                     at<E>(ws, L.SD), at<E>(ws, L.bctr), at<E>(ws, L.breach),
+                                     dh_part, dXp, first, st) != cudaSuccess)
         return FMS_ERR_CUDA;
       E* tmp = G;
       G = Gp;
       Gp = tmp;
+      first = 0;
+      hi = lo;
     }
   }
-  if (unroll_unpack_rows<E>(G, (int64_t)rowsY, d, g.DP, grad_seeds0, st) != cudaSuccess ||
-      unroll_unpack_rows<E>(dXp, (int64_t)B * n, d, g.DP, grad_points, st) != cudaSuccess ||
-      cudaMemcpyAsync(grad_h, dh, (size_t)B * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+  if (unroll_unpack_rows<E>(G, rowsY, (int)m, d, g.DP, yperm, grad_seeds0, st) != cudaSuccess ||
+      unroll_unpack_rows<E>(dXp, (int64_t)B * n, (int)n, d, g.DP,
+                            P > 0 ? at<int32_t>(ws, L.s.perm) : nullptr, grad_points,
+                            st) != cudaSuccess ||
+      unroll_dh_sum(dh_part, B, gr.per_set, grad_h, st) != cudaSuccess)
     return FMS_ERR_CUDA;
   return FMS_OK;
 }
@@ -277,14 +310,15 @@ extern "C" {
 
 size_t fms_unrolled_ckpt_size(int32_t B, int64_t n, int64_t m, int32_t d, int32_t T, int32_t k) {
   if (!valid(B, n, m, d, T, k)) return 0;
-  return ckpt_layout(B, m, d, T, k, 4).total;
+  return ckpt_layout(geom(B, n, m, d), cells_for(B, n, m), T, k, 4).total;
 }
 
 size_t fms_unrolled_workspace_size(int32_t B, int64_t n, int64_t m, int32_t d, int32_t T,
                                    int32_t k) {
   if (!valid(B, n, m, d, T, k)) return 0;
   const UGeom g = geom(B, n, m, d);
-  const size_t f = fwd_layout(g, 4).total, b = bwd_layout(g, k, 4).total;
+  const int P = cells_for(B, n, m);
+  const size_t f = fwd_layout(g, P, 4).total, b = bwd_layout(g, P, k, 4).total;
   return f > b ? f : b;
 }
 
@@ -308,14 +342,15 @@ fms_status fms_unrolled_backward(const float* points, int32_t B, int64_t n, int6
 size_t fms_unrolled_ckpt_size_f64(int32_t B, int64_t n, int64_t m, int32_t d, int32_t T,
                                   int32_t k) {
   if (!valid(B, n, m, d, T, k)) return 0;
-  return ckpt_layout(B, m, d, T, k, 8).total;
+  return ckpt_layout(geom(B, n, m, d), cells_for(B, n, m), T, k, 8).total;
 }
 
 size_t fms_unrolled_workspace_size_f64(int32_t B, int64_t n, int64_t m, int32_t d, int32_t T,
                                        int32_t k) {
   if (!valid(B, n, m, d, T, k)) return 0;
   const UGeom g = geom(B, n, m, d);
-  const size_t f = fwd_layout(g, 8).total, b = bwd_layout(g, k, 8).total;
+  const int P = cells_for(B, n, m);
+  const size_t f = fwd_layout(g, P, 8).total, b = bwd_layout(g, P, k, 8).total;
   return f > b ? f : b;
 }
 

@@ -1,0 +1,357 @@
+// Sorting of rows into cells (fms_cells.cuh): nearest pivot, then a stable
+// counting sort over blocks of kChunkRows rows.  Every step gives the same
+// result on each run (maxima, counts and ranks only).
+#include "fms_cells.cuh"
+
+namespace fms {
+namespace cells {
+
+__device__ __forceinline__ void max_bits(float* p, float v) {
+  // squared distances are not negative, so their bits order as integers do
+  // (NaN above infinity)
+  atomicMax(reinterpret_cast<unsigned*>(p), __float_as_uint(v) & 0x7fffffffu);
+}
+__device__ __forceinline__ void max_bits(double* p, double v) {
+  atomicMax(reinterpret_cast<unsigned long long*>(p),
+            (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull);
+}
+
+// Row of pivot p: the middle of the p-th of P equal runs of the set's rows.
+__device__ __forceinline__ int64_t pivot_row(int p, int P, int64_t n) {
+  return ((2 * (int64_t)p + 1) * n) / (2 * (int64_t)P);
+}
+
+// Loads pivot rows p0 .. p1 of a set (strided rows) into shared memory.
+template <typename T, int DP>
+__device__ __forceinline__ void load_pivots(const T* __restrict__ set, int64_t n, int P, T* pv) {
+  for (int e = threadIdx.x; e < P * DP; e += blockDim.x)
+    pv[e] = set[pivot_row(e / DP, P, n) * DP + e % DP];
+}
+
+// Nearest of the pivots [p0, p1) in shared memory for two rows at a time
+// (ties: the lower pivot); b0, b1, i0, i1 carry the best so far.  Bound by FP32
+// issue: 2 DP operations per (row, pivot) pair plus the pivot's broadcast loads.
+template <typename T, int DP>
+__device__ __forceinline__ void nearest(const T (&x0)[DP], const T (&x1)[DP], const T* pv, int p0,
+                                        int p1, T& b0, T& b1, int& i0, int& i1) {
+  for (int p = p0; p < p1; ++p) {
+    T d0 = T(0), d1 = T(0);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      const T q = pv[p * DP + k];
+      const T e0 = x0[k] - q, e1 = x1[k] - q;
+      d0 += e0 * e0;
+      d1 += e1 * e1;
+    }
+    if (p == 0 || d0 < b0) {
+      b0 = d0;
+      i0 = p;
+    }
+    if (p == 0 || d1 < b1) {
+      b1 = d1;
+      i1 = p;
+    }
+  }
+}
+
+template <typename T, int DP>
+__device__ __forceinline__ void row_values(const T* p, T (&x)[DP]) {
+#pragma unroll
+  for (int q = 0; q < DP * (int)sizeof(T) / 16; ++q) {
+    const float4 t = reinterpret_cast<const float4*>(p)[q];
+    const T* u = reinterpret_cast<const T*>(&t);
+#pragma unroll
+    for (int e = 0; e < 16 / (int)sizeof(T); ++e) x[q * (16 / (int)sizeof(T)) + e] = u[e];
+  }
+}
+
+// First pass over the points: the nearest of the P0 strided pivots, and each
+// pivot's farthest row as (squared distance bits, row).
+template <typename T, int DP>
+__global__ void __launch_bounds__(256)
+    pivot_kernel(const T* __restrict__ src, int nrows, int P0, unsigned char* __restrict__ id,
+                 unsigned long long* __restrict__ far_) {
+  extern __shared__ __align__(16) unsigned char cell_smem[];
+  T* pv = reinterpret_cast<T*>(cell_smem);                                        // [P0][DP]
+  unsigned long long* fs = reinterpret_cast<unsigned long long*>(pv + P0 * DP);   // [P0]
+  const int b = blockIdx.y;
+  const T* set = src + (int64_t)b * nrows * DP;
+  load_pivots<T, DP>(set, nrows, P0, pv);
+  for (int p = threadIdx.x; p < P0; p += blockDim.x) fs[p] = 0ull;
+  __syncthreads();
+  const int r_end = min(nrows, ((int)blockIdx.x + 1) * kChunkRows);
+  for (int r0 = blockIdx.x * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
+    const int r1 = r0 + (int)blockDim.x < r_end ? r0 + (int)blockDim.x : r0;
+    T x0[DP], x1[DP], b0 = T(0), b1 = T(0);
+    row_values<T, DP>(set + (int64_t)r0 * DP, x0);
+    row_values<T, DP>(set + (int64_t)r1 * DP, x1);
+    int i0 = 0, i1 = 0;
+    nearest<T, DP>(x0, x1, pv, 0, P0, b0, b1, i0, i1);
+    id[(int64_t)b * nrows + r0] = (unsigned char)i0;
+    id[(int64_t)b * nrows + r1] = (unsigned char)i1;
+    auto key = [](T v, int r) {
+      return ((unsigned long long)(__float_as_uint((float)v) & 0x7fffffffu) << 32) | (unsigned)r;
+    };
+    const unsigned long long k0 = key(b0, r0), k1 = key(b1, r1);
+    if (fs[i0] < k0) atomicMax(&fs[i0], k0);
+    if (fs[i1] < k1) atomicMax(&fs[i1], k1);
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < P0; p += blockDim.x)
+    if (fs[p]) atomicMax(&far_[(int64_t)b * P0 + p], fs[p]);
+}
+
+// The pivots of a set: the P0 strided ones, then the farthest row of every cell
+// whose radius is over twice the median one (a cluster that no strided pivot hit
+// hangs on to a cell of another one and would make its ball span both).  Fills pv,
+// returns their number; sel: P0 ints, red: 64 ints of shared memory.
+template <typename T, int DP>
+__device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
+                          const unsigned long long* __restrict__ far_, T* pv, int* sel, int* red) {
+  __shared__ float median;
+  load_pivots<T, DP>(set, nrows, P0, pv);
+  float* r2s = reinterpret_cast<float*>(sel);
+  const int p = threadIdx.x;
+  unsigned long long k = 0;
+  if (p < P0) {
+    k = far_[p];
+    r2s[p] = __uint_as_float((unsigned)(k >> 32));
+  }
+  if (p == 0) median = INFINITY;
+  __syncthreads();
+  const float r2 = p < P0 ? r2s[p] : 0.0f;
+  if (p < P0) {
+    int rank = 0;
+    for (int q = 0; q < P0; ++q) rank += (r2s[q] < r2 || (r2s[q] == r2 && q < p)) ? 1 : 0;
+    if (rank == P0 / 2) median = r2;
+  }
+  __syncthreads();
+  const int take = p < P0 && r2 > 4.0f * median ? 1 : 0;
+  int K = 0;
+  const int at = block_exclusive_scan(take, &K, red);
+  if (take) sel[at] = (int)(unsigned)k;
+  __syncthreads();
+  for (int e = threadIdx.x; e < K * DP; e += blockDim.x)
+    pv[P0 * DP + e] = set[(int64_t)sel[e / DP] * DP + e % DP];
+  __syncthreads();
+  return P0 + K;
+}
+
+// Second pass (EXTEND: over the points; else over the seeds, against the points'
+// finished pivots): the cell of every row, the rows of every (block, cell) in
+// counts [B][blocks][P], and for the points the cells' centres and squared radii.
+template <typename T, int DP, bool EXTEND>
+__global__ void __launch_bounds__(256)
+    assign_kernel(const T* __restrict__ src, int nrows, int P, unsigned char* __restrict__ id,
+                  const unsigned long long* __restrict__ far_, int32_t* __restrict__ counts,
+                  T* __restrict__ ctr, int32_t* __restrict__ npiv, T* __restrict__ rad) {
+  extern __shared__ __align__(16) unsigned char cell_smem[];
+  __shared__ int red[64];
+  __shared__ int sel[kMaxCells];
+  T* pv = reinterpret_cast<T*>(cell_smem);                 // [P][DP]
+  T* far2 = pv + (size_t)P * DP;                           // [P]
+  int* hist = reinterpret_cast<int*>(far2 + P);            // [P]
+  const int b = blockIdx.y, blk = blockIdx.x, P0 = P / 2;
+  const T* set = src + (int64_t)b * nrows * DP;
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    far2[p] = T(0);
+    hist[p] = 0;
+  }
+  int np;
+  if (EXTEND) {
+    np = all_pivots<T, DP>(set, nrows, P0, far_ + (int64_t)b * P0, pv, sel, red);
+    if (blk == 0) {
+      for (int e = threadIdx.x; e < P * DP; e += blockDim.x)
+        ctr[(int64_t)b * P * DP + e] = e < np * DP ? pv[e] : T(0);   // (the rest: empty cells)
+      if (threadIdx.x == 0) npiv[b] = np;
+    }
+  } else {
+    np = npiv[b];
+    for (int e = threadIdx.x; e < np * DP; e += blockDim.x) pv[e] = ctr[(int64_t)b * P * DP + e];
+    __syncthreads();
+  }
+  const int r_end = min(nrows, (blk + 1) * kChunkRows);
+  for (int r0 = blk * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
+    const int r1 = r0 + (int)blockDim.x < r_end ? r0 + (int)blockDim.x : r0;
+    T x0[DP], x1[DP], b0 = T(0), b1 = T(0);
+    row_values<T, DP>(set + (int64_t)r0 * DP, x0);
+    row_values<T, DP>(set + (int64_t)r1 * DP, x1);
+    int i0 = 0, i1 = 0;
+    if (EXTEND) {
+      i0 = id[(int64_t)b * nrows + r0];
+      i1 = id[(int64_t)b * nrows + r1];
+#pragma unroll
+      for (int k = 0; k < DP; ++k) {
+        const T e0 = x0[k] - pv[i0 * DP + k], e1 = x1[k] - pv[i1 * DP + k];
+        b0 += e0 * e0;
+        b1 += e1 * e1;
+      }
+      nearest<T, DP>(x0, x1, pv, P0, np, b0, b1, i0, i1);
+    } else {
+      nearest<T, DP>(x0, x1, pv, 0, np, b0, b1, i0, i1);
+    }
+    id[(int64_t)b * nrows + r0] = (unsigned char)i0;
+    atomicAdd(&hist[i0], 1);
+    if (rad) max_bits(&far2[i0], b0);
+    if (r1 != r0) {
+      id[(int64_t)b * nrows + r1] = (unsigned char)i1;
+      atomicAdd(&hist[i1], 1);
+      if (rad) max_bits(&far2[i1], b1);
+    }
+  }
+  __syncthreads();
+  int32_t* out = counts + ((int64_t)b * gridDim.x + blk) * P;
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    out[p] = hist[p];
+    if (rad && hist[p] > 0) max_bits(&rad[(int64_t)b * P + p], far2[p]);
+  }
+}
+
+// Each block finds where its rows of every cell go (rows of earlier cells,
+// then of the same cell in earlier blocks), ranks its rows in order warp by
+// warp, and copies them.  Latency bound; blocks x P counters are read by every
+// block from L2.
+template <typename T, int DP>
+__global__ void __launch_bounds__(256)
+    scatter_kernel(const T* __restrict__ src, int nrows, int P,
+                   const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
+                   T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
+                   int2* __restrict__ table, int cap) {
+  constexpr int WARPS = 8, ITER = kChunkRows / (WARPS * 32);
+  __shared__ int wcnt[WARPS][kMaxCells];
+  __shared__ int base[kMaxCells];
+  __shared__ int scan[64];
+  const int b = blockIdx.y, blk = blockIdx.x, nblk = gridDim.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // thread p: rows of cell p in the whole set and in earlier blocks
+  int tot = 0, before = 0;
+  if ((int)threadIdx.x < P) {
+    const int32_t* c = counts + (int64_t)b * nblk * P + threadIdx.x;
+#pragma unroll 8
+    for (int q = 0; q < nblk; ++q) {
+      const int v = c[(int64_t)q * P];
+      tot += v;
+      if (q < blk) before += v;
+    }
+  }
+  int all = 0;
+  const int first = block_exclusive_scan(tot, &all, scan);
+  if ((int)threadIdx.x < P) base[threadIdx.x] = first + before;
+  if (blk == 0) {
+    int32_t* so = start + (int64_t)b * (P + 1);
+    if ((int)threadIdx.x < P) so[threadIdx.x] = first;
+    if (threadIdx.x == 0) so[P] = nrows;
+    if (table) {
+      const int ng = (int)threadIdx.x < P ? (tot + 31) / 32 : 0;
+      int gall = 0;
+      const int g0 = block_exclusive_scan(ng, &gall, scan);
+      int2* to = table + (int64_t)b * cap;
+      for (int g = 0; g < ng; ++g) to[g0 + g] = make_int2(first + 32 * g, min(32, tot - 32 * g));
+      for (int g = gall + threadIdx.x; g < cap; g += blockDim.x) to[g] = make_int2(0, 0);
+    }
+  }
+  for (int e = threadIdx.x; e < WARPS * kMaxCells; e += blockDim.x) (&wcnt[0][0])[e] = 0;
+  __syncthreads();
+  int ids[ITER];
+#pragma unroll
+  for (int i = 0; i < ITER; ++i) {
+    const int r = blk * kChunkRows + (w * ITER + i) * 32 + lane;
+    ids[i] = r < nrows ? (int)id[(int64_t)b * nrows + r] : -1;
+    const unsigned m = __match_any_sync(kFull, ids[i]);
+    if (ids[i] >= 0 && (m & ((1u << lane) - 1u)) == 0) wcnt[w][ids[i]] += __popc(m);
+    __syncwarp();
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < P) {
+    int o = base[threadIdx.x];
+    for (int u = 0; u < WARPS; ++u) {
+      const int v = wcnt[u][threadIdx.x];
+      wcnt[u][threadIdx.x] = o;
+      o += v;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < ITER; ++i) {
+    const int r = blk * kChunkRows + (w * ITER + i) * 32 + lane;
+    const unsigned m = __match_any_sync(kFull, ids[i]);
+    const unsigned lower = m & ((1u << lane) - 1u);
+    int at = 0;
+    if (ids[i] >= 0) at = wcnt[w][ids[i]] + __popc(lower);
+    __syncwarp();
+    if (ids[i] >= 0 && lower == 0) wcnt[w][ids[i]] += __popc(m);
+    __syncwarp();
+    if (ids[i] >= 0) {
+      const int64_t from = (int64_t)b * nrows + r, to = (int64_t)b * nrows + at;
+      perm[to] = r;
+      const float4* s4 = reinterpret_cast<const float4*>(src + from * DP);
+      float4* d4 = reinterpret_cast<float4*>(dst + to * DP);
+#pragma unroll
+      for (int q = 0; q < DP * (int)sizeof(T) / 16; ++q) d4[q] = s4[q];
+    }
+  }
+}
+
+template <typename T, int DP>
+static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P, void* scratch,
+                          T* dst, int32_t* perm, int32_t* start, T* ctr, int32_t* npiv, T* rad,
+                          int2* table, cudaStream_t st) {
+  const SortScratch sc = sort_scratch(B, nrows, P);
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  unsigned char* id = base + sc.id;
+  int32_t* counts = reinterpret_cast<int32_t*>(base + sc.counts);
+  unsigned long long* far_ = reinterpret_cast<unsigned long long*>(base + sc.far_);
+  const dim3 grid((unsigned)sort_blocks(nrows), (unsigned)B);
+  const size_t sm = (size_t)P * (DP + 1) * sizeof(T) + (size_t)P * 4;
+  const size_t sm0 = (size_t)P / 2 * DP * sizeof(T) + (size_t)P / 2 * 8;
+  cudaError_t e = cudaSuccess;
+  if (sm > 40 * 1024) {   // (static arrays count against the default 48 KB)
+    e = cudaFuncSetAttribute(assign_kernel<T, DP, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(assign_kernel<T, DP, false>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  if (points) {
+    e = cudaMemsetAsync(far_, 0, (size_t)B * (P / 2) * 8, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(rad, 0, (size_t)B * P * sizeof(T), st);
+    if (e != cudaSuccess) return e;
+    pivot_kernel<T, DP><<<grid, 256, sm0, st>>>(src, (int)nrows, P / 2, id, far_);
+    assign_kernel<T, DP, true><<<grid, 256, sm, st>>>(src, (int)nrows, P, id, far_, counts, ctr,
+                                                      npiv, rad);
+  } else {
+    assign_kernel<T, DP, false><<<grid, 256, sm, st>>>(src, (int)nrows, P, id, nullptr, counts,
+                                                       ctr, npiv, nullptr);
+  }
+  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, (int)nrows, P, id, counts, dst, perm, start,
+                                             table, group_cap(nrows, P));
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
+                        void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
+                        int32_t* npiv, T* rad, int2* table, cudaStream_t st) {
+  if (P < 32 || P > kMaxCells || (P & 31) || B < 1 || B > 65535) return cudaErrorInvalidValue;
+  switch (DP) {
+    case 4: return sort_t<T, 4>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 8: return sort_t<T, 8>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 16: return sort_t<T, 16>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 32: return sort_t<T, 32>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 64:
+      if constexpr (sizeof(T) == 4)
+        return sort_t<T, 64>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+template cudaError_t launch_sort<float>(const float*, int, int64_t, int, bool, int, void*, float*,
+                                        int32_t*, int32_t*, float*, int32_t*, float*, int2*,
+                                        cudaStream_t);
+template cudaError_t launch_sort<double>(const double*, int, int64_t, int, bool, int, void*,
+                                         double*, int32_t*, int32_t*, double*, int32_t*, double*,
+                                         int2*, cudaStream_t);
+
+}  // namespace cells
+}  // namespace fms

@@ -13,30 +13,44 @@
 // Positions Y_t are checkpointed every k updates; the backward recomputes one
 // segment of k updates from its checkpoint, then walks it in reverse.
 //
-// Kernels (FP32, or FP64 for checking gradients; exact differences,
-// fixed-order reductions; rows padded to DPAD = 4, 8, 16 or 32 values, the
-// padding known at compile time):
-//   fwd_partial   lanes own R seeds, points streamed with warp-uniform loads
-//                 (the next point's row loaded while this one is evaluated),
-//                 partial (W, S = sum w (x - y)) per point chunk
-//   fwd_finish    y' = y + S/W, W_t kept for the backward; a seed whose W
-//                 underflows (every point farther than ~13 h) is listed for
-//   fwd_rescue    which recomputes it with the weights taken relative to its
-//                 nearest point, w = exp2(-c (D2 - D2min)) (the shift cancels
-//                 in w / W), and records the shift c D2min for the backward
-//   seed_data     one row per seed [y | g | 1/W, shift, g . (y - mu)] for
-//                 the adjoint passes (no division or scattered load per pair)
-//   bwd_seed      lanes own seeds: partial sum_j p a (x - y), sum_j p a and
-//                 sum_j p a ||y - x||^2 per point chunk
-//   bwd_point     lanes own R points, seeds streamed: partial
-//                 sum_i p_ij [g_i - a_ij (x_j - y_i) / h^2] per seed chunk
+// Points and seeds are kept sorted into cells (fms_cells.cuh), and a group of 32
+// seeds of one cell walks only the point cells within its cutoff radius.  Seeds
+// do not depend on each other, so one launch takes a group through all T updates
+// (or, in the adjoint, through a whole segment).  Kernels (FP32, or FP64 for
+// checking gradients; exact differences, fixed-order sums; rows padded to DP =
+// 4, 8, 16 or 32 values):
+//   unroll_travel     lanes own the seeds of a group, a team of warps splits
+//                     the tiles of visible points (staged in shared memory,
+//                     read with broadcast loads); T updates in one launch.  A
+//                     seed whose W underflows (every point farther than ~13 h)
+//                     is recomputed with the weights taken relative to its
+//                     nearest point, w = exp2(-c (D2 - D2min)) (the shift
+//                     cancels in w / W), and the shift c D2min kept for the
+//                     backward
+//   unroll_bwd_seed   the same groups backwards through a segment: per update
+//                     the sums of p a (x - y), p a and p a ||y - x||^2, the
+//                     gradient w.r.t. the positions before it, and one row per
+//                     seed [y | g | 1/W, shift, g . (y - mu)] and one ball per
+//                     group for
+//   unroll_bwd_point  lanes own 32 points of a cell, the seed groups of every
+//                     update of the segment whose ball reaches them are
+//                     streamed: sum_i p_ij [g_i - a_ij (x_j - y_i) / h^2]
 // Both adjoint passes take a_ij = g_i . (x_j - y_i) + g_i . (y_i - mu_i): every
 // term is a difference of nearby positions (no cancellation of coordinates).
-//   finish kernels sum the chunk partials in chunk order.
-#include "fms_internal.cuh"
-#include "fms_tc.cuh"
+// Sums go tile by tile (32 rows) into totals, then over the team's warps in order.
+//
+// Bound by FP32 issue (3 DP + 3, 5 DP + 6 and 6 DP + 6 operations per visible pair).
+// 8 sets x 16,384 points and seeds x 16, 32 blobs, T = 20, k = 5: each group sees
+// about 515 of the 16,384 points; forward and backward 390.4 -> 18.3 ms (forward
+// 3.8, recomputed positions 3.1, seed-major 5.2, point-major 6.0) against kernels
+// that took every pair.  3 sets x 1,500 points x 701 seeds x 3, T = 10 (nothing
+// sorted): 0.955 -> 0.561 ms from 94 launches going to 15.
+#include "fms_cells.cuh"
 
 namespace fms {
+
+using cells::Groups;
+using cells::View;
 
 template <int DPAD>
 __device__ __forceinline__ void load_row(const float* __restrict__ p, float (&v)[DPAD]) {
@@ -60,7 +74,7 @@ __device__ __forceinline__ void load_row(const double* __restrict__ p, double (&
   }
 }
 
-// a row already in shared memory (staged by the ring): plain vector loads
+// a row already in shared memory: plain vector loads
 template <int DPAD>
 __device__ __forceinline__ void smem_row(const float* p, float (&v)[DPAD]) {
 #pragma unroll
@@ -82,14 +96,6 @@ __device__ __forceinline__ void smem_row(const double* p, double (&v)[DPAD]) {
   }
 }
 
-// Per-warp staging rings of the three pair kernels (tc::ring_rows): the
-// forward and seed-major passes stream point rows (DPAD values), the
-// point-major pass streams seed rows (2 DPAD + 4 values); 4 warps per CTA.
-template <typename T, int ROW>
-constexpr int unroll_ring_smem() {
-  return 4 * 2 * tc::kRingRows * ROW * (int)sizeof(T);
-}
-
 // the element type's exp2, fma and min (FP32: the MUFU exp2 with flush to zero)
 __device__ __forceinline__ float uex2(float x) { return ex2_ftz(x); }
 __device__ __forceinline__ double uex2(double x) { return exp2(x); }
@@ -105,404 +111,424 @@ __device__ __forceinline__ T unroll_min_w() {
   return sizeof(T) == 4 ? (T)1e-20f : (T)1e-280;
 }
 
-// seeds (forward, seed-major adjoint) or points (point-major adjoint) per lane
-template <typename T, int DPAD>
-constexpr int unroll_fwd_r() {
-  return sizeof(T) != 4 ? 1 : (DPAD <= 4 ? 4 : (DPAD <= 8 ? 2 : 1));
-}
-template <typename T, int DPAD>
-constexpr int unroll_point_r() {
-  return sizeof(T) != 4 ? 1 : (DPAD <= 16 ? 2 : 1);
+// Shared memory of a team of W warps: each warp's tile ring, its list of row
+// ranges, and its share of the sums exchanged at the end of a pass.
+constexpr int kListCap = cells::kMaxCells;
+
+template <typename T, int ROW, int SUMS>
+constexpr int unroll_warp_smem() {
+  return 2 * cells::kTileRows * ROW * (int)sizeof(T) + kListCap * 8 + SUMS * 32 * (int)sizeof(T);
 }
 
-// ---- forward partials: grid-stride over (set, seed group of 32 R, point chunk)
-template <typename T, int DPAD, int R>
-__global__ void __launch_bounds__(128)
-    unroll_fwd_partial(const T* __restrict__ X, const T* __restrict__ Y, UGeom g,
-                       T c, T* __restrict__ part, uint32_t* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char ring_smem[];
-  __shared__ __align__(8) uint64_t ring_bars[4][2];
-  constexpr int SPW = 32 * R;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T* tiles = reinterpret_cast<T*>(ring_smem) + warp * 2 * tc::kRingRows * DPAD;
-  tc::ring_init(ring_bars[warp], lane);
-  uint32_t use0 = 0u, use1 = 0u;
-  const int Gs = (g.m + SPW - 1) / SPW;
-  const int64_t NT = (int64_t)g.B * Gs * g.Cp;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); task < NT;
-       task += nw) {
-    const int ch = (int)(task % g.Cp);
-    const int64_t rest = task / g.Cp;
-    const int gs = (int)(rest % Gs);
-    const int b = (int)(rest / Gs);
-    const T* Xb = X + (int64_t)b * g.n * DPAD;
-    T y[R][DPAD], S[R][DPAD], W[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int i = min(gs * SPW + r * 32 + lane, g.m - 1);
-      load_row<DPAD>(Y + ((int64_t)b * g.m + i) * DPAD, y[r]);
-      W[r] = T(0);
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k) S[r][k] = T(0);
-    }
-    const int j0 = ch * g.Lp, j1 = min(g.n, j0 + g.Lp);
-    const bool ok = tc::ring_rows<DPAD>(Xb, j0, j1, tiles, ring_bars[warp], use0, use1, lane,
-                                        status, [&](const T* row) {
-      T x[DPAD];
-      smem_row<DPAD>(row, x);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        T dx[DPAD], D2 = T(0);
-#pragma unroll
-        for (int k = 0; k < DPAD; ++k) {
-          dx[k] = x[k] - y[r][k];
-          D2 = ufma(dx[k], dx[k], D2);
-        }
-        const T w = uex2(-c * D2);
-        W[r] += w;
-#pragma unroll
-        for (int k = 0; k < DPAD; ++k) S[r][k] = ufma(w, dx[k], S[r][k]);
-      }
-    });
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int i = gs * SPW + r * 32 + lane;
-      if (!ok) W[r] = T(NAN);   // a wait gave up: the seed's update comes out NaN
-      if (i < g.m) {
-        T* o = part + (((int64_t)b * g.Cp + ch) * g.m + i) * (DPAD + 1);
-        o[0] = W[r];
-#pragma unroll
-        for (int k = 0; k < DPAD; ++k)
-          if (k < g.d) o[1 + k] = S[r][k];
-      }
-    }
-    if (!ok) break;
+template <typename T, int ROW, int SUMS>
+struct TeamSmem {
+  T* ring;      // this warp's two tiles
+  int2* list;   // this warp's list
+  T* sums;      // [W][SUMS][32], the whole team's
+  __device__ TeamSmem(unsigned char* base, int w, int W) {
+    constexpr int ring_e = 2 * cells::kTileRows * ROW;
+    ring = reinterpret_cast<T*>(base) + (size_t)w * ring_e;
+    unsigned char* p = base + (size_t)W * ring_e * sizeof(T);
+    sums = reinterpret_cast<T*>(p);
+    list = reinterpret_cast<int2*>(p + (size_t)W * SUMS * 32 * sizeof(T)) + w * kListCap;
   }
-}
+};
 
-// y_next = y + S/W (sums over chunks in chunk order), W kept for the backward.
-// Seeds with W < unroll_min_w<T>() (or not finite) go to the rescue list instead.
-template <typename T>
-__global__ void unroll_fwd_finish(const T* __restrict__ part, const T* __restrict__ Y,
-                                  UGeom g, T* __restrict__ Ynext, T* __restrict__ Wout,
-                                  T* __restrict__ Sh, int32_t* __restrict__ rlist,
-                                  int32_t* __restrict__ rcount) {
-  const int64_t total = (int64_t)g.B * g.m;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / g.m), i = (int)(e % g.m);
-    T W = T(0);
-    for (int ch = 0; ch < g.Cp; ++ch) W += part[(((int64_t)b * g.Cp + ch) * g.m + i) * (g.DP + 1)];
-    if (!(W >= unroll_min_w<T>()) || !isfinite(W)) {
-      rlist[atomicAdd(rcount, 1)] = (int32_t)e;
-      continue;
-    }
-    if (Wout) Wout[e] = W;
-    if (Sh) Sh[e] = T(0);
-    for (int k = 0; k < g.DP; ++k) {
-      T v = T(0);
-      if (k < g.d) {
-        T S = T(0);
-        for (int ch = 0; ch < g.Cp; ++ch)
-          S += part[(((int64_t)b * g.Cp + ch) * g.m + i) * (g.DP + 1) + 1 + k];
-        v = Y[e * g.DP + k] + S / W;
-      }
-      Ynext[e * g.DP + k] = v;
-    }
-  }
-}
-
-// Recomputes the listed seeds (one warp each, points over lanes): pass 1 the
-// nearest squared distance D2min, pass 2 the weights exp2(-c (D2 - D2min)),
-// their sums (fixed xor tree over lanes) and y' = y + S/W; the shift c D2min
-// goes to Sh for the backward.  One block; it clears the list count at the end.
-template <typename T, int DPAD>
-__global__ void __launch_bounds__(1024)
-    unroll_fwd_rescue(const T* __restrict__ X, const T* __restrict__ Y, UGeom g, T c,
-                      const int32_t* __restrict__ rlist, int32_t* rcount,
-                      T* __restrict__ Ynext, T* __restrict__ Wout,
-                      T* __restrict__ Sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cnt = *(volatile int32_t*)rcount;
-  for (int q = warp; q < cnt; q += (int)(blockDim.x >> 5)) {
-    const int64_t e = rlist[q];
-    const int b = (int)(e / g.m);
-    const T* Xb = X + (int64_t)b * g.n * DPAD;
-    T y[DPAD];
-    load_row<DPAD>(Y + e * DPAD, y);
-    T dmin = T(INFINITY);
-    for (int j = lane; j < g.n; j += 32) {
-      T x[DPAD];
-      load_row<DPAD>(Xb + (int64_t)j * DPAD, x);
-      T D2 = T(0);
+// Sums v over the team in warp order; every warp gets the result.
+template <typename T, int N>
+__device__ __forceinline__ void team_sum(T (&v)[N], T* sums, int stride, int w, int W, int lane) {
+  if (W == 1) return;
 #pragma unroll
-      for (int k = 0; k < DPAD; ++k) {
-        const T e = x[k] - y[k];
-        D2 = ufma(e, e, D2);
-      }
-      dmin = umin(dmin, D2);
-    }
+  for (int k = 0; k < N; ++k) sums[(w * stride + k) * 32 + lane] = v[k];
+  __syncthreads();
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) dmin = umin(dmin, __shfl_xor_sync(kFull, dmin, o));
-    const T sh = c * dmin;
-    T W = T(0), S[DPAD];
-#pragma unroll
-    for (int k = 0; k < DPAD; ++k) S[k] = T(0);
-    for (int j = lane; j < g.n; j += 32) {
-      T x[DPAD];
-      load_row<DPAD>(Xb + (int64_t)j * DPAD, x);
-      T dx[DPAD], D2 = T(0);
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k) {
-        dx[k] = x[k] - y[k];
-        D2 = ufma(dx[k], dx[k], D2);
-      }
-      const T w = uex2(ufma(-c, D2, sh));
-      W += w;
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k) S[k] = ufma(w, dx[k], S[k]);
-    }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-      W += __shfl_xor_sync(kFull, W, o);
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k) S[k] += __shfl_xor_sync(kFull, S[k], o);
-    }
-    if (lane == 0) {
-      if (Wout) Wout[e] = W;
-      if (Sh) Sh[e] = sh;
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k)
-        if (k < g.DP) Ynext[e * g.DP + k] = k < g.d ? y[k] + S[k] / W : T(0);
-    }
+  for (int k = 0; k < N; ++k) {
+    T s = sums[k * 32 + lane];
+    for (int u = 1; u < W; ++u) s += sums[(u * stride + k) * 32 + lane];
+    v[k] = s;
   }
   __syncthreads();
-  if (threadIdx.x == 0) *rcount = 0;
 }
 
-// ---- adjoint inputs per seed: SD row = [y | g | 1/W, shift, g . (y - mu), 0]
-template <typename T, int DPAD>
-__global__ void unroll_seed_data(const T* __restrict__ Y, const T* __restrict__ MU,
-                                 const T* __restrict__ G, const T* __restrict__ Wt,
-                                 const T* __restrict__ Sh, UGeom g, T* __restrict__ SD) {
-  constexpr int SDW = 2 * DPAD + 4;
-  const int64_t total = (int64_t)g.B * g.m;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    T* o = SD + e * SDW;
-    T gm = T(0);
+__device__ __forceinline__ bool group_rows(const Groups& g, int b, int gi, int rows, int* row0,
+                                           int* cnt) {
+  if (g.table) {
+    const int2 e = __ldg(g.table + (int64_t)b * g.per_set + gi);
+    *row0 = e.x;
+    *cnt = e.y;
+  } else {
+    *row0 = gi * 32;
+    *cnt = min(32, rows - gi * 32);
+  }
+  return *cnt > 0;
+}
+
+template <typename T, int DP>
+__device__ __forceinline__ void store_row(T* p, const T (&v)[DP]) {
+  constexpr int E = 16 / (int)sizeof(T);
 #pragma unroll
-    for (int k = 0; k < DPAD; ++k) {
-      const T gk = G[e * DPAD + k];
-      o[k] = Y[e * DPAD + k];
-      o[DPAD + k] = gk;
-      gm = ufma(gk, Y[e * DPAD + k] - MU[e * DPAD + k], gm);
-    }
-    o[2 * DPAD] = T(1) / Wt[e];
-    o[2 * DPAD + 1] = Sh[e];
-    o[2 * DPAD + 2] = gm;
-    o[2 * DPAD + 3] = T(0);
+  for (int q = 0; q < DP / E; ++q) {
+    float4 t;
+    T* u = reinterpret_cast<T*>(&t);
+#pragma unroll
+    for (int e = 0; e < E; ++e) u[e] = v[q * E + e];
+    reinterpret_cast<float4*>(p)[q] = t;
   }
 }
 
-// ---- backward, seed-major: partial sums over point chunks of
-//   DY_i = sum_j p_ij a_ij (x_j - mu_i) = sum_j p a (x_j - y_i) + (y_i - mu_i) sum_j p a,
-//   DH_i = sum_j p_ij a_ij ||y_i - x_j||^2 = sum_j p a (||y_i - x_j||^2 - s_i).
-// The last form holds for any s_i because sum_j p_ij a_ij = g_i . sum_j p_ij
-// (x_j - mu_i) = 0; s_i = the seed's weight shift in squared-distance units
-// (0 unless the seed was rescued).  For a seed far from every point (D2 of
-// hundreds) the FP32 rounding of D2 perturbs its weights by ~1e-5, which
-// leaves sum p a at ~1e-5 instead of 0; subtracting s_i keeps that residual
-// from being multiplied by D2.
-template <typename T, int DPAD>
-__global__ void __launch_bounds__(128)
-    unroll_bwd_seed(const T* __restrict__ X, const T* __restrict__ MU,
-                    const T* __restrict__ SD, UGeom g, T c, T* __restrict__ part,
-                    uint32_t* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char ring_smem[];
-  __shared__ __align__(8) uint64_t ring_bars[4][2];
-  constexpr int SDW = 2 * DPAD + 4;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T* tiles = reinterpret_cast<T*>(ring_smem) + warp * 2 * tc::kRingRows * DPAD;
-  tc::ring_init(ring_bars[warp], lane);
-  uint32_t use0 = 0u, use1 = 0u;
-  const int Gs = (g.m + 31) / 32;
-  const int64_t NT = (int64_t)g.B * Gs * g.Cp;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); task < NT;
-       task += nw) {
-    const int ch = (int)(task % g.Cp);
-    const int64_t rest = task / g.Cp;
-    const int gs = (int)(rest % Gs);
-    const int b = (int)(rest / Gs);
-    const int i = min(gs * 32 + lane, g.m - 1);
-    const int64_t row = (int64_t)b * g.m + i;
-    const T* Xb = X + (int64_t)b * g.n * DPAD;
-    const T* sd = SD + row * SDW;
-    T y[DPAD], gg[DPAD], DY[DPAD], DH = T(0), SA = T(0);
-    load_row<DPAD>(sd, y);
-    load_row<DPAD>(sd + DPAD, gg);
-    T tail[4];
-    load_row<4>(sd + 2 * DPAD, tail);
-    const T invW = tail[0], sh = tail[1], gd = tail[2];
-    const T s0 = sh / c;
+// One far seed, recomputed by a warp with the points over its lanes: pass 1 the
+// nearest squared distance D2min, pass 2 the weights exp2(-c (D2 - D2min)) and
+// their sums (fixed xor tree).  acc = (W, S, sum w D2); returns the shift c D2min.
+template <typename T, int DP>
+__device__ T rescue_seed(const T* __restrict__ Xb, int n, T c, const T (&y)[DP], T (&acc)[DP + 2],
+                         int lane) {
+  T dmin = T(INFINITY);
+  for (int j = lane; j < n; j += 32) {
+    T x[DP];
+    load_row<DP>(Xb + (int64_t)j * DP, x);
+    T D2 = T(0);
 #pragma unroll
-    for (int k = 0; k < DPAD; ++k) DY[k] = T(0);
-    const int j0 = ch * g.Lp, j1 = min(g.n, j0 + g.Lp);
-    const bool ok = tc::ring_rows<DPAD>(Xb, j0, j1, tiles, ring_bars[warp], use0, use1, lane,
-                                        status, [&](const T* row) {
-      T x[DPAD];
-      smem_row<DPAD>(row, x);
-      T dx[DPAD], D2 = T(0), a = gd;
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k) {
-        dx[k] = x[k] - y[k];
-        D2 = ufma(dx[k], dx[k], D2);
-        a = ufma(gg[k], dx[k], a);
-      }
-      const T pa = uex2(ufma(-c, D2, sh)) * invW * a;
-      DH = ufma(pa, D2 - s0, DH);
-      SA += pa;
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k) DY[k] = ufma(pa, dx[k], DY[k]);
-    });
-    if (!ok) DH = T(NAN);   // a wait gave up: the gradient comes out NaN
-    if (gs * 32 + lane < g.m) {
-      T mu[DPAD];
-      load_row<DPAD>(MU + row * DPAD, mu);
-      T* o = part + (((int64_t)b * g.Cp + ch) * g.m + i) * (DPAD + 1);
-      o[0] = DH;
-#pragma unroll
-      for (int k = 0; k < DPAD; ++k)
-        if (k < g.d) o[1 + k] = ok ? ufma(y[k] - mu[k], SA, DY[k]) : T(NAN);
+    for (int k = 0; k < DP; ++k) {
+      const T e = x[k] - y[k];
+      D2 = ufma(e, e, D2);
     }
-    if (!ok) break;
+    dmin = umin(dmin, D2);
   }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) dmin = umin(dmin, __shfl_xor_sync(kFull, dmin, o));
+  const T sh = c * dmin;
+#pragma unroll
+  for (int k = 0; k < DP + 2; ++k) acc[k] = T(0);
+  for (int j = lane; j < n; j += 32) {
+    T x[DP];
+    load_row<DP>(Xb + (int64_t)j * DP, x);
+    T dx[DP], D2 = T(0);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      dx[k] = x[k] - y[k];
+      D2 = ufma(dx[k], dx[k], D2);
+    }
+    const T w = uex2(ufma(-c, D2, sh));
+    acc[0] += w;
+    acc[DP + 1] = ufma(w, D2, acc[DP + 1]);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) acc[1 + k] = ufma(w, dx[k], acc[1 + k]);
+  }
+#pragma unroll
+  for (int k = 0; k < DP + 2; ++k)
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) acc[k] += __shfl_xor_sync(kFull, acc[k], o);
+  return sh;
 }
 
-// G_prev = DY / h^2 (the gradient w.r.t. the positions before this update);
-// dh_part[b*m + i] = DH_i / h^3.
-template <typename T>
-__global__ void unroll_bwd_seed_finish(const T* __restrict__ part, UGeom g, T inv_h2,
-                                       T inv_h3, T* __restrict__ Gprev,
-                                       T* __restrict__ dh_part) {
-  const int64_t total = (int64_t)g.B * g.m;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / g.m), i = (int)(e % g.m);
-    T DH = T(0);
-    for (int ch = 0; ch < g.Cp; ++ch) DH += part[(((int64_t)b * g.Cp + ch) * g.m + i) * (g.DP + 1)];
-    dh_part[e] = DH * inv_h3;
-    for (int k = 0; k < g.DP; ++k) {
-      T v = T(0);
-      if (k < g.d) {
-        for (int ch = 0; ch < g.Cp; ++ch)
-          v += part[(((int64_t)b * g.Cp + ch) * g.m + i) * (g.DP + 1) + 1 + k];
-        v *= inv_h2;
-      }
-      Gprev[e * g.DP + k] = v;
-    }
-  }
-}
-
-// ---- backward, point-major: partial over seed chunks of
-//   DX_j = sum_i p_ij g_i - (1/h^2) sum_i p_ij a_ij (x_j - y_i).
-// Lanes own R points; the seed rows (SD) are read with warp-uniform loads.
-template <typename T, int DPAD, int R>
-__global__ void __launch_bounds__(128)
-    unroll_bwd_point(const T* __restrict__ X, const T* __restrict__ SD, UGeom g, T c,
-                     T inv_h2, T* __restrict__ part, uint32_t* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char ring_smem[];
-  __shared__ __align__(8) uint64_t ring_bars[4][2];
-  constexpr int SDW = 2 * DPAD + 4;
-  constexpr int PPW = 32 * R;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T* tiles = reinterpret_cast<T*>(ring_smem) + warp * 2 * tc::kRingRows * SDW;
-  tc::ring_init(ring_bars[warp], lane);
-  uint32_t use0 = 0u, use1 = 0u;
-  const int Gp = (g.n + PPW - 1) / PPW;
-  const int64_t NT = (int64_t)g.B * Gp * g.Cs;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); task < NT;
-       task += nw) {
-    const int ch = (int)(task % g.Cs);
-    const int64_t rest = task / g.Cs;
-    const int gp = (int)(rest % Gp);
-    const int b = (int)(rest / Gp);
-    T x[R][DPAD], DX[R][DPAD];
+// ---- forward: `steps` updates of one group of seeds per block.  After update
+// t the positions go to slot ceil(t / every) - slot0 of pos where t is a
+// multiple of `every` or the last one; W and the shift of update t to row t - 1
+// of Wout and Sh (nullable).
+template <typename T, int DP>
+__global__ void __launch_bounds__(256)
+    unroll_travel(const T* __restrict__ X, View<T> cv, const T* __restrict__ Y0, Groups gr,
+                  UGeom g, T c, int steps, int every, int slot0, T* __restrict__ pos,
+                  T* __restrict__ Wout, T* __restrict__ Sh, T* __restrict__ M2) {
+  extern __shared__ __align__(16) unsigned char unroll_smem[];
+  constexpr int SUMS = DP + 3;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const TeamSmem<T, DP, SUMS> sm(unroll_smem, w, W);
+  const int b = blockIdx.x / gr.per_set;
+  int row0, cnt;
+  if (!group_rows(gr, b, blockIdx.x % gr.per_set, g.m, &row0, &cnt)) return;
+  const T* Xb = X + (int64_t)b * g.n * DP;
+  const int64_t rowsY = (int64_t)g.B * g.m;
+  const int64_t e = (int64_t)b * g.m + row0 + min(lane, cnt - 1);
+  T y[DP];
+  load_row<DP>(Y0 + e * DP, y);
+  const T log2n = T(log2f((float)g.n));
+  T cut = cells::cut_bits(T(0.5), log2n);
+  for (int t = 1; t <= steps; ++t) {
+    T ctr[DP], acc[DP + 2];   // W, S, sum w ||x - y||^2
+    const T rho = cells::group_ball<T, DP>(y, ctr);
+    T need;
+    for (int pass = 0;; ++pass) {
+      const int nl = cells::visible_cells<T, DP>(cv, b, g.n, ctr, rho + cells::csqrt(cut / c),
+                                                 sm.list, lane);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int j = min(gp * PPW + r * 32 + lane, g.n - 1);
-      load_row<DPAD>(X + ((int64_t)b * g.n + j) * DPAD, x[r]);
+      for (int k = 0; k < DP + 2; ++k) acc[k] = T(0);
+      cells::walk_tiles<DP>(Xb, sm.list, nl, w, W, sm.ring, lane, [&](const T* rows, int nr) {
+        T ta[DP + 2];
 #pragma unroll
-      for (int k = 0; k < DPAD; ++k) DX[r][k] = T(0);
-    }
-    const int i0 = ch * g.Ls, i1 = min(g.m, i0 + g.Ls);
-    const T* sdb = SD + (int64_t)b * g.m * SDW;
-    const bool ok = tc::ring_rows<SDW>(sdb, i0, i1, tiles, ring_bars[warp], use0, use1, lane,
-                                       status, [&](const T* sd) {
-      T y[DPAD], gg[DPAD];
-      smem_row<DPAD>(sd, y);
-      smem_row<DPAD>(sd + DPAD, gg);
-      T tail[4];
-      smem_row<4>(sd + 2 * DPAD, tail);
-      const T invW = tail[0], sh = tail[1], gd = tail[2];
+        for (int k = 0; k < DP + 2; ++k) ta[k] = T(0);
+#pragma unroll (DP <= 8 ? 2 : 1)
+        for (int q = 0; q < nr; ++q) {
+          T x[DP];
+          smem_row<DP>(rows + q * DP, x);
+          T D2 = T(0);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        T dx[DPAD], D2 = T(0), a = gd;
+          for (int k = 0; k < DP; ++k) {
+            x[k] -= y[k];
+            D2 = ufma(x[k], x[k], D2);
+          }
+          const T wt = uex2(-c * D2);
+          ta[0] += wt;
+          ta[DP + 1] = ufma(wt, D2, ta[DP + 1]);
 #pragma unroll
-        for (int k = 0; k < DPAD; ++k) {
-          dx[k] = x[r][k] - y[k];
-          D2 = ufma(dx[k], dx[k], D2);
-          a = ufma(gg[k], dx[k], a);
+          for (int k = 0; k < DP; ++k) ta[1 + k] = ufma(wt, x[k], ta[1 + k]);
         }
-        const T p = uex2(ufma(-c, D2, sh)) * invW;
-        const T q = p * a * inv_h2;
 #pragma unroll
-        for (int k = 0; k < DPAD; ++k) DX[r][k] = ufma(p, gg[k], ufma(-q, dx[k], DX[r][k]));
+        for (int k = 0; k < DP + 2; ++k) acc[k] += ta[k];
+      });
+      team_sum(acc, sm.sums, SUMS, w, W, lane);
+      need = cells::cut_bits(cells::warp_min(acc[0]), log2n);
+      if (cv.P == 0 || !(need > cut)) break;
+      cut = pass == 0 ? need : T(cells::zero_bits<T>());
+    }
+    // W does not decrease along a trajectory: one bit covers its rounding
+    cut = umin(need + T(1), T(cells::zero_bits<T>()));
+    T sh = T(0);
+    unsigned bad = __ballot_sync(kFull, !(acc[0] >= unroll_min_w<T>()) || !isfinite(acc[0]));
+    if (bad) {   // the same for every warp of the team
+      for (int u = 0; u < 32; ++u) {
+        if (!((bad >> u) & 1u) || u % W != w) continue;
+        T ys[DP], a2[DP + 2];
+#pragma unroll
+        for (int k = 0; k < DP; ++k) ys[k] = __shfl_sync(kFull, y[k], u);
+        const T s2 = rescue_seed<T, DP>(Xb, g.n, c, ys, a2, lane);
+        if (lane == 0) {
+#pragma unroll
+          for (int k = 0; k < DP + 2; ++k) sm.sums[k * 32 + u] = a2[k];
+          sm.sums[(DP + 2) * 32 + u] = s2;
+        }
       }
-    });
+      __syncthreads();
+      if ((bad >> lane) & 1u) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int j = gp * PPW + r * 32 + lane;
-      if (!ok)
+        for (int k = 0; k < DP + 2; ++k) acc[k] = sm.sums[k * 32 + lane];
+        sh = sm.sums[(DP + 2) * 32 + lane];
+      }
+      __syncthreads();
+    }
 #pragma unroll
-        for (int k = 0; k < DPAD; ++k) DX[r][k] = T(NAN);   // a wait gave up
-      if (j < g.n) {
-        T* o = part + (((int64_t)b * g.Cs + ch) * g.n + j) * DPAD;
+    for (int k = 0; k < DP; ++k)
+      if (k < g.d) y[k] += acc[1 + k] / acc[0];
+    if (w == 0 && lane < cnt) {
+      if (Wout) {
+        Wout[(int64_t)(t - 1) * rowsY + e] = acc[0];
+        Sh[(int64_t)(t - 1) * rowsY + e] = sh;
+        M2[(int64_t)(t - 1) * rowsY + e] = acc[DP + 1] / acc[0];
+      }
+      if (t % every == 0 || t == steps)
+        store_row<T, DP>(pos + ((int64_t)((t + every - 1) / every - slot0) * rowsY + e) * DP, y);
+    }
+  }
+}
+
+// ---- backward, seed-major, updates len-1 .. 0 of one segment: with
+//   DY_i = sum_j p_ij a_ij (x_j - mu_i) = sum_j p a (x_j - y_i) + (y_i - mu_i) sum_j p a,
+//   DH_i = sum_j p_ij a_ij ||y_i - x_j||^2 = sum_j p a (||y_i - x_j||^2 - s_i),
+// g <- DY / h^2 and dh_part += DH / h^3.  The last form of DH holds for any s_i
+// because sum_j p_ij a_ij = g_i . sum_j p_ij (x_j - mu_i) = 0; s_i = the mean of
+// ||y_i - x_j||^2 under p (kept by the forward) makes the terms smallest, and a
+// far seed's residual sum p a (FP32 rounding of a D2 of hundreds leaves ~1e-5
+// instead of 0) is not multiplied by D2.  DH is summed over tiles in FP64.
+template <typename T, int DP>
+__global__ void __launch_bounds__(256)
+    unroll_bwd_seed(const T* __restrict__ X, View<T> cv, USegment<T> sg, Groups gr, UGeom g, T c,
+                    T inv_h2, double inv_h3, const T* __restrict__ Gin, T* __restrict__ Gout,
+                    T* __restrict__ SD, T* __restrict__ bctr, T* __restrict__ breach,
+                    double* __restrict__ dh_part, int first) {
+  extern __shared__ __align__(16) unsigned char unroll_smem[];
+  constexpr int SUMS = DP + 2, SDW = 2 * DP + 4;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  __shared__ double dhs[8];
+  const TeamSmem<T, DP, SUMS> sm(unroll_smem, w, W);
+  const int b = blockIdx.x / gr.per_set, gi = blockIdx.x % gr.per_set;
+  const int64_t NG = (int64_t)g.B * gr.per_set;
+  int row0, cnt;
+  if (!group_rows(gr, b, gi, g.m, &row0, &cnt)) {
+    if (threadIdx.x == 0 && first) dh_part[blockIdx.x] = 0.0;
+    return;
+  }
+  const T* Xb = X + (int64_t)b * g.n * DP;
+  const int64_t rowsY = (int64_t)g.B * g.m;
+  const int64_t e = (int64_t)b * g.m + row0 + min(lane, cnt - 1);
+  const T log2n = T(log2f((float)g.n));
+  T gg[DP];
+  load_row<DP>(Gin + e * DP, gg);
+  double dh = 0.0;
+  for (int u = sg.len - 1; u >= 0; --u) {
+    T y[DP], ym[DP], ctr[DP];
+    load_row<DP>(sg.pos(u) + e * DP, y);
+    load_row<DP>(sg.pos(u + 1) + e * DP, ym);
+    const int64_t ue = (int64_t)(sg.u0 + u) * rowsY + e;
+    const T Wt = sg.W[ue], sh = sg.Sh[ue];
+    const T invW = T(1) / Wt, s0 = sg.M2[ue];
+    T gd = T(0);
 #pragma unroll
-        for (int k = 0; k < DPAD; ++k) o[k] = k < g.d ? DX[r][k] : T(0);
+    for (int k = 0; k < DP; ++k) {
+      ym[k] = y[k] - ym[k];
+      gd = ufma(gg[k], ym[k], gd);
+    }
+    // every weight above the cutoff of its seed (exponent c D2 - sh)
+    const T reach = cells::group_ball<T, DP>(y, ctr) +
+                    cells::warp_max(cells::csqrt((cells::cut_bits(Wt, log2n) + sh) / c));
+    if (w == 0) {
+      if (lane < cnt) {
+        T* o = SD + ((int64_t)u * rowsY + e) * SDW;
+        store_row<T, DP>(o, y);
+        store_row<T, DP>(o + DP, gg);
+        const T tail[4] = {invW, sh, gd, T(0)};
+        store_row<T, 4>(o + 2 * DP, tail);
+      }
+      if (lane == 0) {
+        store_row<T, DP>(bctr + ((int64_t)u * NG + blockIdx.x) * DP, ctr);
+        breach[(int64_t)u * NG + blockIdx.x] = reach;
       }
     }
-    if (!ok) break;
+    const int nl = cells::visible_cells<T, DP>(cv, b, g.n, ctr, reach, sm.list, lane);
+    T acc[DP + 1];   // sum p a, DY
+    double DH = 0.0;
+#pragma unroll
+    for (int k = 0; k <= DP; ++k) acc[k] = T(0);
+    cells::walk_tiles<DP>(Xb, sm.list, nl, w, W, sm.ring, lane, [&](const T* rows, int nr) {
+      T ta[DP + 2];
+#pragma unroll
+      for (int k = 0; k < DP + 2; ++k) ta[k] = T(0);
+#pragma unroll (DP <= 8 ? 2 : 1)
+      for (int q = 0; q < nr; ++q) {
+        T x[DP];
+        smem_row<DP>(rows + q * DP, x);
+        T D2 = T(0), a = gd;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+          x[k] -= y[k];
+          D2 = ufma(x[k], x[k], D2);
+          a = ufma(gg[k], x[k], a);
+        }
+        const T pa = uex2(ufma(-c, D2, sh)) * invW * a;
+        ta[0] = ufma(pa, D2 - s0, ta[0]);
+        ta[1] += pa;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) ta[2 + k] = ufma(pa, x[k], ta[2 + k]);
+      }
+#pragma unroll
+      for (int k = 0; k <= DP; ++k) acc[k] += ta[1 + k];
+      DH += (double)ta[0];
+    });
+    team_sum(acc, sm.sums, SUMS, w, W, lane);
+    dh += DH;   // (this warp's tiles)
+#pragma unroll
+    for (int k = 0; k < DP; ++k) gg[k] = ufma(ym[k], acc[0], acc[1 + k]) * inv_h2;
+  }
+  if (lane >= cnt) dh = 0.0;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) dh += __shfl_xor_sync(kFull, dh, o);
+  if (lane == 0) dhs[w] = dh;
+  __syncthreads();
+  if (w == 0) {
+    if (lane < cnt) store_row<T, DP>(Gout + e * DP, gg);
+    if (lane == 0) {
+      double t = 0.0;
+      for (int u = 0; u < W; ++u) t += dhs[u];
+      t *= inv_h3;
+      dh_part[blockIdx.x] = first ? t : dh_part[blockIdx.x] + t;
+    }
   }
 }
 
-// dX += sum over seed chunks (chunk order).
-template <typename T>
-__global__ void unroll_bwd_point_finish(const T* __restrict__ part, UGeom g,
-                                        T* __restrict__ dX) {
-  const int64_t total = (int64_t)g.B * g.n * g.DP;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t bj = e / g.DP;
-    const int k = (int)(e % g.DP);
-    const int b = (int)(bj / g.n), j = (int)(bj % g.n);
-    T v = T(0);
-    for (int ch = 0; ch < g.Cs; ++ch) v += part[(((int64_t)b * g.Cs + ch) * g.n + j) * g.DP + k];
-    dX[e] += v;
+// ---- backward, point-major, all updates of one segment: one block per group
+// of 32 points adds
+//   DX_j = sum_i p_ij g_i - (1/h^2) sum_i p_ij a_ij (x_j - y_i)
+// to its rows of dX.
+template <typename T, int DP>
+__global__ void __launch_bounds__(256)
+    unroll_bwd_point(const T* __restrict__ X, Groups gx, Groups gr, UGeom g, int len, T c,
+                     T inv_h2, const T* __restrict__ SD, const T* __restrict__ bctr,
+                     const T* __restrict__ breach, T* __restrict__ dX, int first) {
+  extern __shared__ __align__(16) unsigned char unroll_smem[];
+  constexpr int SUMS = DP, SDW = 2 * DP + 4;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const TeamSmem<T, SDW, SUMS> sm(unroll_smem, w, W);
+  const int b = blockIdx.x / gx.per_set;
+  int row0, cnt;
+  if (!group_rows(gx, b, blockIdx.x % gx.per_set, g.n, &row0, &cnt)) return;
+  const int64_t e = (int64_t)b * g.n + row0 + min(lane, cnt - 1);
+  const int64_t rowsY = (int64_t)g.B * g.m, NG = (int64_t)g.B * gr.per_set;
+  T x[DP], ctr[DP], acc[DP];
+  load_row<DP>(X + e * DP, x);
+  const T rho = cells::group_ball<T, DP>(x, ctr);
+#pragma unroll
+  for (int k = 0; k < DP; ++k) acc[k] = T(0);
+  for (int u = 0; u < len; ++u) {
+    const T* sdb = SD + ((int64_t)u * rowsY + (int64_t)b * g.m) * SDW;
+    for (int g0 = 0; g0 < gr.per_set;) {
+      // the next seed groups that reach these points, as many as the list holds
+      int nl = 0;
+      for (; g0 < gr.per_set && nl <= kListCap - 32; g0 += 32) {
+        const int gi = g0 + lane;
+        bool see = false;
+        int r0 = 0, rc = 0;
+        if (gi < gr.per_set && group_rows(gr, b, gi, g.m, &r0, &rc)) {
+          const int64_t at = (int64_t)u * NG + (int64_t)b * gr.per_set + gi;
+          T q[DP];
+          load_row<DP>(bctr + at * DP, q);
+          T d2 = T(0);
+#pragma unroll
+          for (int k = 0; k < DP; ++k) {
+            const T f = q[k] - ctr[k];
+            d2 += f * f;
+          }
+          const T lim = (rho + breach[at]) * T(1.0001);
+          see = !(d2 > lim * lim);
+        }
+        const unsigned m = __ballot_sync(kFull, see);
+        if (see) sm.list[nl + __popc(m & ((1u << lane) - 1u))] = make_int2(r0, rc);
+        nl += __popc(m);
+      }
+      __syncwarp();
+      cells::walk_tiles<SDW>(sdb, sm.list, nl, w, W, sm.ring, lane, [&](const T* rows, int nr) {
+        T ta[DP];
+#pragma unroll
+        for (int k = 0; k < DP; ++k) ta[k] = T(0);
+        for (int q = 0; q < nr; ++q) {
+          const T* sd = rows + q * SDW;
+          T dx[DP], gv[DP], tail[4];
+          smem_row<DP>(sd, dx);
+          smem_row<DP>(sd + DP, gv);
+          smem_row<4>(sd + 2 * DP, tail);
+          T D2 = T(0), a = tail[2];
+#pragma unroll
+          for (int k = 0; k < DP; ++k) {
+            dx[k] = x[k] - dx[k];
+            D2 = ufma(dx[k], dx[k], D2);
+            a = ufma(gv[k], dx[k], a);
+          }
+          const T p = uex2(ufma(-c, D2, tail[1])) * tail[0];
+          const T q2 = p * a * inv_h2;
+#pragma unroll
+          for (int k = 0; k < DP; ++k) ta[k] = ufma(p, gv[k], ufma(-q2, dx[k], ta[k]));
+        }
+#pragma unroll
+        for (int k = 0; k < DP; ++k) acc[k] += ta[k];
+      });
+    }
+  }
+  team_sum(acc, sm.sums, SUMS, w, W, lane);
+  if (w == 0 && lane < cnt) {
+    T* o = dX + e * DP;
+    if (!first) {
+#pragma unroll
+      for (int k = 0; k < DP; ++k) acc[k] += o[k];
+    }
+    store_row<T, DP>(o, acc);
   }
 }
 
-// dh[b] += sum_i dh_part[b, i] in FP64, seeds in order (one block per set).
-template <typename T>
-__global__ void unroll_dh_reduce(const T* __restrict__ dh_part, UGeom g,
+// dh[b] = the sum of set b's group sums in FP64, in a fixed order (one block per set).
+__global__ void unroll_dh_reduce(const double* __restrict__ dh_part, int per_set,
                                  double* __restrict__ dh) {
-  __shared__ double red[32];
-  const int b = blockIdx.x;
+  __shared__ double red[8];
+  const double* p = dh_part + (int64_t)blockIdx.x * per_set;
   double s = 0.0;
-  for (int i = threadIdx.x; i < g.m; i += blockDim.x) s += (double)dh_part[(int64_t)b * g.m + i];
+  for (int i = threadIdx.x; i < per_set; i += blockDim.x) s += p[i];
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -510,30 +536,34 @@ __global__ void unroll_dh_reduce(const T* __restrict__ dh_part, UGeom g,
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    dh[b] += t;
+    dh[blockIdx.x] = t;
   }
 }
 
-// Row repacking between the caller's [rows x d] and the padded [rows x DP].
+// Row repacking between the caller's [rows x d] and the padded [rows x DP]; with
+// perm, padded row i of a set is the caller's row perm[i] of that set.
 template <typename T>
-__global__ void unroll_pack(const T* __restrict__ src, int64_t rows, int d, int DP,
-                            T* __restrict__ dst) {
+__global__ void unroll_pack(const T* __restrict__ src, int64_t rows, int per_set, int d, int DP,
+                            const int32_t* __restrict__ perm, T* __restrict__ dst) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * DP;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = e / DP;
     const int k = (int)(e % DP);
-    dst[e] = k < d ? src[r * d + k] : T(0);
+    const int64_t s = perm ? r / per_set * per_set + perm[r] : r;
+    dst[e] = k < d ? src[s * d + k] : T(0);
   }
 }
 
 template <typename T>
-__global__ void unroll_unpack(const T* __restrict__ src, int64_t rows, int d, int DP,
-                              T* __restrict__ dst) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * d;
+__global__ void unroll_unpack(const T* __restrict__ src, int64_t rows, int per_set, int d, int DP,
+                              const int32_t* __restrict__ perm, T* __restrict__ dst) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * DP;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / d;
-    const int k = (int)(e % d);
-    dst[e] = src[r * DP + k];
+    const int64_t r = e / DP;
+    const int k = (int)(e % DP);
+    if (k >= d) continue;
+    const int64_t s = perm ? r / per_set * per_set + perm[r] : r;
+    dst[s * d + k] = src[e];
   }
 }
 
@@ -544,104 +574,110 @@ static int blocks_for(int64_t work, int per = 256) {
   return (int)b;
 }
 
-// dynamic shared memory above the default 48 KB needs the kernel's attribute
-// (set once per kernel)
+// Warps of a team: enough of them for about 32 warps per SM over all groups, as
+// many as shared memory holds.
+static int team_warps(int64_t groups, int sms, int warp_smem) {
+  int W = 1;
+  while (W < 8 && groups * W < (int64_t)sms * 32 && 2 * W * warp_smem <= 200 * 1024) W *= 2;
+  return W;
+}
+
 template <typename K>
-static cudaError_t ring_attr(K kernel, int bytes, bool& done) {
-  if (done || bytes <= 48 * 1024) return cudaSuccess;
-  const cudaError_t e =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) done = true;
-  return e;
+static cudaError_t team_attr(K kernel, int bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-template <typename T, int DPAD>
-static cudaError_t fwd_step_t(const T* X, const T* Y, const UGeom& g, T c, T* part, T* Ynext,
-                              T* Wout, T* Sh, int32_t* rlist, int32_t* rcount, int grid,
-                              uint32_t* status, cudaStream_t st) {
-  constexpr int sm = unroll_ring_smem<T, DPAD>();
-  static bool attr = false;
-  const cudaError_t ea = ring_attr(unroll_fwd_partial<T, DPAD, unroll_fwd_r<T, DPAD>()>, sm, attr);
-  if (ea != cudaSuccess) return ea;
-  unroll_fwd_partial<T, DPAD, unroll_fwd_r<T, DPAD>()><<<grid, 128, sm, st>>>(X, Y, g, c, part,
-                                                                               status);
-  unroll_fwd_finish<T><<<blocks_for((int64_t)g.B * g.m), 256, 0, st>>>(part, Y, g, Ynext, Wout,
-                                                                       Sh, rlist, rcount);
-  unroll_fwd_rescue<T, DPAD><<<1, 1024, 0, st>>>(X, Y, g, c, rlist, rcount, Ynext, Wout, Sh);
+template <typename T, int DP>
+static cudaError_t travel_t(const T* X, const View<T>& cv, const T* Y0, const Groups& gr,
+                            const UGeom& g, T c, int steps, int every, int slot0, T* pos, T* Wout,
+                            T* Sh, T* M2, cudaStream_t st) {
+  const int64_t NG = (int64_t)g.B * gr.per_set;
+  constexpr int ws = unroll_warp_smem<T, DP, DP + 3>();
+  const int W = team_warps(NG, g.sms, ws);
+  const cudaError_t e = team_attr(unroll_travel<T, DP>, W * ws);
+  if (e != cudaSuccess) return e;
+  unroll_travel<T, DP><<<(unsigned)NG, 32 * W, W * ws, st>>>(X, cv, Y0, gr, g, c, steps, every,
+                                                             slot0, pos, Wout, Sh, M2);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t unroll_fwd_step(const T* X, const T* Y, const UGeom& g, T c, T* part, T* Ynext,
-                            T* Wout, T* Sh, int32_t* rlist, int32_t* rcount, int grid,
-                            uint32_t* status, cudaStream_t st) {
+cudaError_t unroll_forward_steps(const T* X, const View<T>& cv, const T* Y0, const Groups& gr,
+                                 const UGeom& g, T c, int steps, int every, int slot0, T* pos,
+                                 T* Wout, T* Sh, T* M2, cudaStream_t st) {
   switch (g.DP) {
-    case 4: return fwd_step_t<T, 4>(X, Y, g, c, part, Ynext, Wout, Sh, rlist, rcount, grid, status, st);
-    case 8: return fwd_step_t<T, 8>(X, Y, g, c, part, Ynext, Wout, Sh, rlist, rcount, grid, status, st);
-    case 16: return fwd_step_t<T, 16>(X, Y, g, c, part, Ynext, Wout, Sh, rlist, rcount, grid, status, st);
-    case 32: return fwd_step_t<T, 32>(X, Y, g, c, part, Ynext, Wout, Sh, rlist, rcount, grid, status, st);
+    case 4: return travel_t<T, 4>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
+    case 8: return travel_t<T, 8>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
+    case 16: return travel_t<T, 16>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
+    case 32: return travel_t<T, 32>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
   }
   return cudaErrorInvalidValue;
 }
 
-template <typename T, int DPAD>
-static cudaError_t bwd_step_t(const T* X, const T* Y, const T* MU, const T* G, const T* Wt,
-                              const T* Sh, const UGeom& g, T c, T inv_h2, T inv_h3, T* part_s,
-                              T* part_p, T* SD, T* dh_part, T* Gprev, T* dX, double* dh, int grid,
-                              uint32_t* status, cudaStream_t st) {
-  constexpr int sm_p = unroll_ring_smem<T, 2 * DPAD + 4>(), sm_s = unroll_ring_smem<T, DPAD>();
-  static bool attr_p = false, attr_s = false;
-  cudaError_t ea = ring_attr(unroll_bwd_point<T, DPAD, unroll_point_r<T, DPAD>()>, sm_p, attr_p);
-  if (ea == cudaSuccess) ea = ring_attr(unroll_bwd_seed<T, DPAD>, sm_s, attr_s);
-  if (ea != cudaSuccess) return ea;
-  unroll_seed_data<T, DPAD><<<blocks_for((int64_t)g.B * g.m), 256, 0, st>>>(Y, MU, G, Wt, Sh, g,
-                                                                           SD);
-  unroll_bwd_point<T, DPAD, unroll_point_r<T, DPAD>()><<<grid, 128, sm_p, st>>>(
-      X, SD, g, c, inv_h2, part_p, status);
-  unroll_bwd_seed<T, DPAD><<<grid, 128, sm_s, st>>>(X, MU, SD, g, c, part_s, status);
-  unroll_bwd_point_finish<T><<<blocks_for((int64_t)g.B * g.n * g.DP), 256, 0, st>>>(part_p, g, dX);
-  unroll_bwd_seed_finish<T><<<blocks_for((int64_t)g.B * g.m), 256, 0, st>>>(part_s, g, inv_h2,
-                                                                            inv_h3, Gprev,
-                                                                            dh_part);
-  unroll_dh_reduce<T><<<g.B, 256, 0, st>>>(dh_part, g, dh);
+template <typename T, int DP>
+static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, const Groups& gx,
+                         const Groups& gr, const UGeom& g, T c, T inv_h2, double inv_h3, const T* Gin,
+                         T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX, int first,
+                         cudaStream_t st) {
+  const int64_t NG = (int64_t)g.B * gr.per_set, NX = (int64_t)g.B * gx.per_set;
+  constexpr int ws = unroll_warp_smem<T, DP, DP + 2>(), wp = unroll_warp_smem<T, 2 * DP + 4, DP>();
+  const int Ws = team_warps(NG, g.sms, ws), Wp = team_warps(NX, g.sms, wp);
+  cudaError_t e = team_attr(unroll_bwd_seed<T, DP>, Ws * ws);
+  if (e == cudaSuccess) e = team_attr(unroll_bwd_point<T, DP>, Wp * wp);
+  if (e != cudaSuccess) return e;
+  unroll_bwd_seed<T, DP><<<(unsigned)NG, 32 * Ws, Ws * ws, st>>>(
+      X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, first);
+  unroll_bwd_point<T, DP><<<(unsigned)NX, 32 * Wp, Wp * wp, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
+                                                                  SD, bctr, breach, dX, first);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t unroll_bwd_step(const T* X, const T* Y, const T* MU, const T* G, const T* Wt,
-                            const T* Sh, const UGeom& g, T c, T inv_h2, T inv_h3, T* part_s,
-                            T* part_p, T* SD, T* dh_part, T* Gprev, T* dX, double* dh, int grid,
-                            uint32_t* status, cudaStream_t st) {
+cudaError_t unroll_backward_segment(const T* X, const View<T>& cv, const USegment<T>& sg,
+                                    const Groups& gx, const Groups& gr, const UGeom& g, T c,
+                                    T inv_h2, double inv_h3, const T* Gin, T* Gout, T* SD, T* bctr,
+                                    T* breach, double* dh_part, T* dX, int first,
+                                    cudaStream_t st) {
   switch (g.DP) {
-    case 4: return bwd_step_t<T, 4>(X, Y, MU, G, Wt, Sh, g, c, inv_h2, inv_h3, part_s, part_p, SD, dh_part, Gprev, dX, dh, grid, status, st);
-    case 8: return bwd_step_t<T, 8>(X, Y, MU, G, Wt, Sh, g, c, inv_h2, inv_h3, part_s, part_p, SD, dh_part, Gprev, dX, dh, grid, status, st);
-    case 16: return bwd_step_t<T, 16>(X, Y, MU, G, Wt, Sh, g, c, inv_h2, inv_h3, part_s, part_p, SD, dh_part, Gprev, dX, dh, grid, status, st);
-    case 32: return bwd_step_t<T, 32>(X, Y, MU, G, Wt, Sh, g, c, inv_h2, inv_h3, part_s, part_p, SD, dh_part, Gprev, dX, dh, grid, status, st);
+    case 4: return bwd_t<T, 4>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
+    case 8: return bwd_t<T, 8>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
+    case 16: return bwd_t<T, 16>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
+    case 32: return bwd_t<T, 32>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
   }
   return cudaErrorInvalidValue;
 }
 
-template <typename T>
-cudaError_t unroll_pack_rows(const T* src, int64_t rows, int d, int DP, T* dst, cudaStream_t st) {
-  unroll_pack<T><<<blocks_for(rows * DP), 256, 0, st>>>(src, rows, d, DP, dst);
+cudaError_t unroll_dh_sum(const double* dh_part, int B, int per_set, double* dh, cudaStream_t st) {
+  unroll_dh_reduce<<<B, 256, 0, st>>>(dh_part, per_set, dh);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t unroll_unpack_rows(const T* src, int64_t rows, int d, int DP, T* dst,
-                               cudaStream_t st) {
-  unroll_unpack<T><<<blocks_for(rows * d), 256, 0, st>>>(src, rows, d, DP, dst);
+cudaError_t unroll_pack_rows(const T* src, int64_t rows, int per_set, int d, int DP,
+                             const int32_t* perm, T* dst, cudaStream_t st) {
+  unroll_pack<T><<<blocks_for(rows * DP), 256, 0, st>>>(src, rows, per_set, d, DP, perm, dst);
   return cudaGetLastError();
 }
 
-#define FMS_UNROLL_INST(T)                                                                      \
-  template cudaError_t unroll_fwd_step<T>(const T*, const T*, const UGeom&, T, T*, T*, T*, T*,  \
-                                          int32_t*, int32_t*, int, uint32_t*, cudaStream_t);   \
-  template cudaError_t unroll_bwd_step<T>(const T*, const T*, const T*, const T*, const T*,     \
-                                          const T*, const UGeom&, T, T, T, T*, T*, T*, T*, T*, \
-                                          T*, double*, int, uint32_t*, cudaStream_t);          \
-  template cudaError_t unroll_pack_rows<T>(const T*, int64_t, int, int, T*, cudaStream_t);      \
-  template cudaError_t unroll_unpack_rows<T>(const T*, int64_t, int, int, T*, cudaStream_t);
+template <typename T>
+cudaError_t unroll_unpack_rows(const T* src, int64_t rows, int per_set, int d, int DP,
+                               const int32_t* perm, T* dst, cudaStream_t st) {
+  unroll_unpack<T><<<blocks_for(rows * DP), 256, 0, st>>>(src, rows, per_set, d, DP, perm, dst);
+  return cudaGetLastError();
+}
+
+#define FMS_UNROLL_INST(T)                                                                        \
+  template cudaError_t unroll_forward_steps<T>(const T*, const View<T>&, const T*, const Groups&, \
+                                               const UGeom&, T, int, int, int, T*, T*, T*, T*,    \
+                                               cudaStream_t);                                     \
+  template cudaError_t unroll_backward_segment<T>(                                                \
+      const T*, const View<T>&, const USegment<T>&, const Groups&, const Groups&, const UGeom&,   \
+      T, T, double, const T*, T*, T*, T*, T*, double*, T*, int, cudaStream_t);                        \
+  template cudaError_t unroll_pack_rows<T>(const T*, int64_t, int, int, int, const int32_t*, T*,  \
+                                           cudaStream_t);                                         \
+  template cudaError_t unroll_unpack_rows<T>(const T*, int64_t, int, int, int, const int32_t*,    \
+                                             T*, cudaStream_t);
 FMS_UNROLL_INST(float)
 FMS_UNROLL_INST(double)
 #undef FMS_UNROLL_INST

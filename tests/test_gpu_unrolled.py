@@ -160,3 +160,58 @@ def test_gradcheck_fp64_on_gpu():
     h = torch.tensor(1.7, dtype=torch.float64, device="cuda", requires_grad=True)
     fn = lambda X_, Y_, h_: fms.unrolled_mean_shift(X_, Y_, h_, T, k)
     assert torch.autograd.gradcheck(fn, (X, Y0, h), eps=1e-6, atol=1e-7, rtol=1e-5)
+
+
+def _wide_sets(seed, B, n, d, k, box, sigma=1.0):
+    rng = np.random.default_rng(seed)
+    return np.stack([rng.uniform(0, box, (k, d))[rng.integers(0, k, n)]
+                     + sigma * rng.standard_normal((n, d)) for _ in range(B)]).astype(np.float32)
+
+
+# Sorted cells serve B n m >= 4,194,304: the sizes lie just above it, with a last
+# sort block of one row (2049), fewer seeds than points, one large cluster (every
+# cell seen), and clusters of very different sizes.
+@pytest.mark.parametrize("B,n,m,d,k,box,T,kk", [
+    (1, 2049, 2049, 3, 8, 100.0, 5, 2), (1, 4200, 1001, 16, 6, 50.0, 4, 3),
+    (2, 1500, 1500, 2, 1, 5.0, 3, 9), (1, 2050, 2048, 32, 5, 40.0, 3, 1),
+    (1, 2100, 2000, 7, 4, 30.0, 11, 10)])
+def test_sorted_cells_match_oracle(B, n, m, d, k, box, T, kk):
+    h = 2.0
+    X = _wide_sets(d * 7 + n, B, n, d, k, box)
+    rng = np.random.default_rng(5)
+    Y0 = (X[:, :m] + 0.3 * rng.standard_normal((B, m, d))).astype(np.float32)
+    if d == 3:
+        Y0[0, 5] = X[0].max(axis=0) + 60.0       # every weight zero in FP32
+        Y0[0, 6] = X[0].max(axis=0) + 5.0 * h    # W far below 1: the cutoff widens
+    G = rng.standard_normal(Y0.shape).astype(np.float32)
+    Xt, Yt = torch.from_numpy(X).cuda(), torch.from_numpy(Y0).cuda()
+    YT, ck = fms.unrolled_forward(Xt, Yt, h, T, kk)
+    dX, dY, dh = fms.unrolled_backward(Xt, ck, m, h, T, kk, torch.from_numpy(G).cuda())
+    again = fms.unrolled_backward(Xt, ck, m, h, T, kk, torch.from_numpy(G).cuda())
+    torch.cuda.synchronize()
+    for one, two in zip((dX, dY, dh), again):
+        assert torch.equal(one, two)
+    for b in range(B):
+        ref = orc.unrolled_forward(X[b], Y0[b], h, T)[-1]
+        assert np.abs(YT[b].cpu().numpy() - ref).max() <= 2e-4 * (1 + np.abs(ref).max())
+        rdX, rdY, rdh = orc.unrolled_backward(X[b], Y0[b], h, T, G[b])
+        for got, want in ((dX[b], rdX), (dY[b], rdY)):
+            got = got.cpu().numpy().astype(np.float64)
+            assert np.abs(got - want).max() <= 2e-4 * (1 + np.abs(want).max())
+        assert abs(dh[b].item() - rdh) <= 2e-4 * (1 + abs(rdh))
+
+
+def test_sorted_cells_f64_match_oracle():
+    B, n, d, h, T, k = 1, 2100, 3, 2.0, 3, 2
+    X = _wide_sets(3, B, n, d, 6, 60.0).astype(np.float64)
+    G = np.random.default_rng(1).standard_normal(X.shape)
+    Xt = torch.from_numpy(X).cuda()
+    YT, ck = fms.unrolled_forward(Xt, Xt, h, T, k)
+    dX, dY, dh = fms.unrolled_backward(Xt, ck, n, h, T, k, torch.from_numpy(G).cuda())
+    torch.cuda.synchronize()
+    ref = orc.unrolled_forward(X[0], X[0], h, T)[-1]
+    rdX, rdY, rdh = orc.unrolled_backward(X[0], X[0], h, T, G[0])
+    assert np.abs(YT[0].cpu().numpy() - ref).max() <= 1e-9 * (1 + np.abs(ref).max())
+    assert np.abs(dX[0].cpu().numpy() - rdX).max() <= 1e-9 * (1 + np.abs(rdX).max())
+    assert np.abs(dY[0].cpu().numpy() - rdY).max() <= 1e-9 * (1 + np.abs(rdY).max())
+    assert abs(dh[0].item() - rdh) <= 1e-9 * (1 + abs(rdh))
