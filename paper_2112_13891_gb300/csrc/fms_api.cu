@@ -8,7 +8,7 @@
 #include <vector>
 
 #include "../../include/fms.h"
-#include "fms_internal.cuh"
+#include "fms_cells.cuh"
 
 using namespace fms;
 
@@ -44,7 +44,8 @@ struct Layout {
   size_t off_Xs, off_y, off_seed_idx, off_it, off_conv, off_state, off_active, off_kept,
       off_alive, off_acc1, off_acc2, off_score, off_ym, off_mdone, off_mscore, off_modes_full,
       off_part, off_part64, off_ctl, off_mctl, off_status, off_slog, off_yf, off_ract, off_rctl,
-      off_hist, off_S, off_img, off_wlast, off_grid, total;
+      off_hist, off_S, off_img, off_wlast, off_grid, off_sorted, off_perm, off_start, off_ctr,
+      off_npiv, off_rad, off_table, off_ext, off_sort, total;
   int DP, DA, R, grid_ctas;
   int64_t Ncap;
   Tiling tl;
@@ -170,7 +171,45 @@ bool use_tensor_step(int d, int32_t precision) {
   return false;
 }
 
-Layout make_layout(int64_t n, int d, int64_t Ncap, int sms, bool tensor) {
+// How a call's seeds travel.
+enum Travel : int {
+  kTravelSteps = 0,    // grid or cluster rounds (d <= 7), else one launch per update
+  kTravelSeeds = 1,    // travel_seeds: a block takes a seed to convergence
+  kTravelGroups = 2,   // travel_groups: every point a seed, 32 to a group
+};
+struct Route {
+  int travel;
+  int P;         // cells the points are sorted into (0: none)
+  bool tensor;   // updates start on the tensor-core step
+};
+
+// Seeds up to which a block per seed is the better split; more of them reuse a
+// row of points too little (each block reads its own rows from L2), and the
+// tensor-core or wide step takes them.
+constexpr int32_t kTravelMaxSeeds = 4096;
+// Points from which sorting them pays: ~30 us, against the dense passes of
+// 128 seeds, or of every point.
+constexpr int64_t kSortSeedsMin = 8192, kSortGroupsMin = 4096;
+
+Route choose_route(int64_t n, int d, const fms_options& o, int32_t max_iter) {
+  Route r{};
+  const bool plain = o.kernel == FMS_KERNEL_GAUSSIAN && o.metric != FMS_METRIC_COSINE;
+  const int64_t N0 = o.seed_indices ? o.n_seed_indices : o.n_initial;
+  if (max_iter <= kHistCap && n <= INT32_MAX) {
+    if (o.all_seeds) {
+      if (d <= 7) r.travel = kTravelGroups;
+    } else if (d > 7 && N0 <= kTravelMaxSeeds && o.precision != FMS_PRECISION_TENSOR) {
+      r.travel = kTravelSeeds;
+    }
+  }
+  if (r.travel == kTravelSeeds && n >= kSortSeedsMin) r.P = cells::choose_cells(n, n);
+  if (r.travel == kTravelGroups && n >= kSortGroupsMin) r.P = cells::choose_cells(n, n);
+  r.tensor = r.travel == kTravelSteps && plain && use_tensor_step(d, o.precision);
+  return r;
+}
+
+Layout make_layout(int64_t n, int d, int64_t Ncap, int sms, const Route& route) {
+  const bool tensor = route.tensor;
   Layout L{};
   L.DP = padded_dim(d);
   L.DA = step_accumulators(d);
@@ -227,6 +266,17 @@ Layout make_layout(int64_t n, int d, int64_t Ncap, int sms, bool tensor) {
   L.off_img = take(tensor ? tc_image_bytes(n, d) : 0);
   L.off_wlast = take((size_t)Ncap * 4);   // sum w of each seed's latest cluster-round update
   L.off_grid = take(d <= 7 ? grid_scratch_bytes(d) : 0);   // grid rounds: barrier + accumulators
+  if (route.P > 0) {
+    L.off_sorted = take((size_t)n * L.DP * 4);
+    L.off_perm = take((size_t)n * 4);
+    L.off_start = take((size_t)(route.P + 1) * 4);
+    L.off_ctr = take((size_t)route.P * L.DP * 4);
+    L.off_npiv = take(4);
+    L.off_rad = take((size_t)route.P * 4);
+    L.off_table = take((size_t)cells::group_cap(n, route.P) * 8);
+    L.off_ext = take(d > 8 ? (size_t)route.P * route.P * 8 : 0);
+    L.off_sort = take(cells::sort_scratch(1, n, route.P).total);
+  }
   L.total = o;
   return L;
 }
@@ -334,10 +384,10 @@ size_t fms_workspace_size(int64_t n, int32_t d, const fms_options* opt) {
   fill_defaults(opt, &o);
   const int64_t Ncap = seed_capacity(n, o);
   if (Ncap < 1) return 0;
-  return make_layout(n, d, Ncap, device_info().sms,
-                     o.kernel == FMS_KERNEL_GAUSSIAN && o.metric != FMS_METRIC_COSINE &&
-                         use_tensor_step(d, o.precision))
-      .total;
+  // (max_iter only turns trajectories in one launch off, which needs no more)
+  const size_t a = make_layout(n, d, Ncap, device_info().sms, choose_route(n, d, o, 1)).total;
+  const size_t b = make_layout(n, d, Ncap, device_info().sms, choose_route(n, d, o, INT32_MAX)).total;
+  return a > b ? a : b;
 }
 
 // Device-to-host copies of the results that fms_cluster_host queues on the
@@ -403,8 +453,9 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
   const Dev dv = device_info();
   if (dv.sms <= 0) return FMS_ERR_CUDA;
   const int64_t Ncap = seed_capacity(n, o);
-  const bool tensor = kf == kKernelGaussian && !cosine && use_tensor_step(d, o.precision);
-  const Layout Lo = make_layout(n, d, Ncap, dv.sms, tensor);
+  const Route route = choose_route(n, d, o, max_iter);
+  const bool tensor = route.tensor;
+  const Layout Lo = make_layout(n, d, Ncap, dv.sms, route);
   const int DP = Lo.DP, DA = Lo.DA, R = Lo.R;
   bool owns_ws = false;
   void* ws = workspace;
@@ -560,14 +611,53 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       return e;
     };
 
+    // --- the points in cells (trajectories in one launch) ---
+    const int P = route.P;
+    cells::View<float> cv{};
+    float* rows = Xs;   // the rows that the trajectories read
+    int32_t* perm = nullptr;
+    if (P > 0) {
+      rows = at<float>(ws, Lo.off_sorted);
+      perm = at<int32_t>(ws, Lo.off_perm);
+      cv.P = P;
+      cv.start = at<int32_t>(ws, Lo.off_start);
+      cv.ctr = at<float>(ws, Lo.off_ctr);
+      cv.rad = at<float>(ws, Lo.off_rad);
+      if (d > 8) cv.ext = at<float2>(ws, Lo.off_ext);
+    }
+    auto sort_points = [&](cudaStream_t s_) -> cudaError_t {
+      if (P == 0) return cudaSuccess;
+      const cudaError_t e = cells::launch_sort<float>(
+          Xs, 1, n, DP, true, P, at<void>(ws, Lo.off_sort), rows, perm,
+          at<int32_t>(ws, Lo.off_start), at<float>(ws, Lo.off_ctr), at<int32_t>(ws, Lo.off_npiv),
+          at<float>(ws, Lo.off_rad), at<int2>(ws, Lo.off_table), s_);
+      if (e != cudaSuccess || !cv.ext) return e;
+      return cells::launch_extents(rows, DP, P, cv.start, cv.ctr, at<float2>(ws, Lo.off_ext), s_);
+    };
+    auto seeds_launch = [&](const RoundCtl* rcp, int N_, int max_N, int target_,
+                            cudaStream_t s_) -> cudaError_t {
+      return launch_travel_seeds(rows, cv, (int)n, d, DP, y, it, conv, state, wlast, hist,
+                                 hist + kHistCap + 1, rcp, N_, max_N, target_, kf, max_iter,
+                                 tol2_s, sphere_r,
+                                 reinterpret_cast<unsigned long long*>(&ctl->evals), dv.sms, s_);
+    };
+    auto refine_launch = [&](int max_M, double tol2, cudaStream_t s_) -> cudaError_t {
+      return launch_refine_seeds(rows, cv, (int)n, d, DP, y, kept, acc1, &mctl->M, max_M, ym, yf,
+                                 mscore, tol2, kRefineMaxIter, &rctl->steps,
+                                 reinterpret_cast<unsigned long long*>(&rctl->evals), kf,
+                                 sphere_rd, dv.sms, s_);
+    };
+
     // --- Seed Selection (Alg. 2): initial seed count ---
     int32_t N0;
     if (o.all_seeds) N0 = (int32_t)n;
     else if (o.seed_indices) N0 = o.n_seed_indices;
     else N0 = (int32_t)(o.n_initial < n ? o.n_initial : n);
     RoundCtl* rctl_round = at<RoundCtl>(ws, Lo.off_ctl + kCtlRoundOff);
-    const int cap_seeds = gp.ok ? gp.seeds : qmax * kSeedsPerCluster;
-    const int cap_modes = qmax * kModesPerCluster;
+    const bool by_seed = route.travel == kTravelSeeds;
+    const int cap_seeds = gp.ok || by_seed ? (by_seed ? kGridMaxSeeds : gp.seeds)
+                                           : qmax * kSeedsPerCluster;
+    const int cap_modes = by_seed ? 15 * kModesPerCluster : qmax * kModesPerCluster;
     // one grid round over the RUNNING seeds of [0, N) (N and target from rcp
     // when non-null)
     auto grid_launch = [&](const RoundCtl* rcp, int N_, int target_, cudaStream_t s_) {
@@ -598,7 +688,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     // 2 host refinement and labels, 3 the graph did everything
     int resume = 0;
     const bool graph_ok = !graph_cache().disabled && !o.profile && !owns_ws && hbuf &&
-                          qmax > 0 && !tensor &&
+                          (qmax > 0 || by_seed) && !tensor &&
                           !o.all_seeds && !keep_exhausted && !o.seed_indices &&
                           !o.skip_refine && max_iter <= kHistCap && N0 <= cap_seeds;
     if (graph_ok) {
@@ -659,11 +749,12 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
         if (e == cudaSuccess)
           e = launch_pack_points(points, n, d, DP, (float)scale, Xs, status, cs, cosine ? 1 : 0,
                                  pcopy);
+        if (e == cudaSuccess) e = sort_points(cs);
         if (e == cudaSuccess)
           e = launch_seed_init(Xs, n, DP, o.rng_seed, nullptr, 0, 0, N0, seed_idx, y, it, conv,
                                state, status, cs, init_state);
         if (e == cudaSuccess) e = launch_round_begin(rctl_round, N0, o.gamma, cs);
-        slot->kernels_pre = 3;
+        slot->kernels_pre = 3 + (P > 0 ? 4 : 0) + (cv.ext ? 1 : 0);
         // the rounds
         cudaGraph_t body = nullptr;
         if (e == cudaSuccess) e = add_conditional(cs, h_loop, cudaGraphCondTypeWhile, &body);
@@ -672,7 +763,9 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                             cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
           cudaError_t e2 = cudaSuccess;
-          if (gp.ok) {
+          if (by_seed) {
+            e2 = seeds_launch(rctl_round, 0, cap_seeds, 0, cs2);
+          } else if (gp.ok) {
             e2 = grid_launch(rctl_round, 0, 0, cs2);
           } else {
             e2 = launch_round_list(state, 0, active, S_dev, cs2, rctl_round);
@@ -696,7 +789,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           const cudaError_t e3 = cudaStreamEndCapture(cs2, &gb);
           e = e2 != cudaSuccess ? e2 : e3;
         }
-        slot->kernels_round = gp.ok ? 4 : 5;
+        slot->kernels_round = gp.ok || by_seed ? 4 : 5;
         // after the rounds: refinement, second prune, order, labels
         cudaGraph_t post = nullptr;
         if (e == cudaSuccess) e = add_conditional(cs, h_post, cudaGraphCondTypeIf, &post);
@@ -705,7 +798,8 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                             cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
           cudaError_t e2 =
-              gp.ok ? launch_ms_grid_refine(
+              by_seed ? refine_launch(cap_modes, rtol_s * rtol_s, cs2)
+              : gp.ok ? launch_ms_grid_refine(
                           gp, Xs, n, d, y, kept, acc1, &mctl->M, ym, yf, mscore, rtol_s * rtol_s,
                           kRefineMaxIter, &rctl->steps,
                           reinterpret_cast<unsigned long long*>(&rctl->evals), status,
@@ -789,9 +883,15 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       FMS_LAUNCH(launch_pack_points(points, n, d, DP, (float)scale, Xs, status, st,
                                     cosine ? 1 : 0, pcopy));
       if (tensor) FMS_LAUNCH(launch_tc_pack(Xs, n, d, DP, img, st));
+      if (P > 0) {
+        n_launches += cv.ext ? 4 : 3;   // (and the one counted below)
+        FMS_LAUNCH(sort_points(st));
+      }
       N = N0;
-      FMS_LAUNCH(launch_seed_init(Xs, n, DP, o.rng_seed, o.seed_indices, 0, 0, N, seed_idx, y,
-                                  it, conv, state, status, st, init_state));
+      // (travel_groups starts from the points themselves)
+      if (route.travel != kTravelGroups)
+        FMS_LAUNCH(launch_seed_init(Xs, n, DP, o.rng_seed, o.seed_indices, 0, 0, N, seed_idx, y,
+                                    it, conv, state, status, st, init_state));
     }
 
     for (; resume <= 1;) {
@@ -800,14 +900,19 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       if (target < 1) target = 1;
       if (target > N) target = N;
       // --- mean-shift iterations under Early Stopping (Sec. II-C) ---
-      const bool use_grid = gp.ok && N <= gp.seeds;
+      const bool use_travel = route.travel != kTravelSteps;
+      const bool use_grid = !use_travel && gp.ok && N <= gp.seeds;
       const bool use_clusters =
-          use_grid || (qmax > 0 && N <= qmax * kSeedsPerCluster && max_iter <= kHistCap);
+          use_grid || use_travel ||
+          (qmax > 0 && N <= qmax * kSeedsPerCluster && max_iter <= kHistCap);
+      // with gamma = 1 kept seeds need not have converged: their densities come from a
+      // pass at their last positions (travel_groups makes that pass itself)
+      const bool score_pass = keep_exhausted && route.travel != kTravelGroups;
       if (use_clusters) {
         // persistent round (grid of one CTA per SM, or thread-block clusters
         // when the grid plan does not fit): no host round trips
         cudaEvent_t ra = nullptr, rb = nullptr;
-        if (!use_grid) FMS_LAUNCH(launch_round_list(state, N, active, S_dev, st));
+        if (!use_grid && !use_travel) FMS_LAUNCH(launch_round_list(state, N, active, S_dev, st));
         if (o.profile) {
           cudaEventCreate(&ra);
           cudaEventCreate(&rb);
@@ -815,7 +920,16 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           round_evs.push_back(ra);
           round_evs.push_back(rb);
         }
-        if (use_grid) {
+        if (by_seed) {
+          FMS_LAUNCH(seeds_launch(nullptr, N, N, target, st));
+        } else if (use_travel) {
+          const cells::Groups gr{P > 0 ? at<int2>(ws, Lo.off_table) : nullptr,
+                                 P > 0 ? cells::group_cap(n, P) : (int)((n + 31) / 32)};
+          FMS_LAUNCH(launch_travel_groups(
+              rows, cv, (int)n, DP, gr, perm, kf, max_iter, tol2_s, sphere_r, y, it, conv, state,
+              wlast, hist, reinterpret_cast<unsigned long long*>(&ctl->evals),
+              reinterpret_cast<unsigned long long*>(&mctl->evals), dv.sms, st));
+        } else if (use_grid) {
           FMS_LAUNCH(grid_launch(nullptr, N, target, st));
         } else {
           int clusters = (N + 7) / 8;
@@ -831,9 +945,9 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
         // at their positions instead
         FMS_LAUNCH(launch_round_finish(hist, target, max_iter, state, conv, N, keep_exhausted,
                                        kept, mctl, ctl, n, R, Lo.tl, st, nullptr,
-                                       keep_exhausted ? nullptr : wlast, score));
+                                       score_pass ? nullptr : wlast, score));
         mark(1);
-        if (keep_exhausted) {
+        if (score_pass) {
           FMS_LAUNCH(step_launch(y, kept, &mctl->K, &mctl->C, &mctl->Lc));
           FMS_LAUNCH(launch_score_reduce(part, mctl, DA, score, N, st));
         }
@@ -898,7 +1012,15 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     if (resume <= 2) {
     mark(2);
     // --- refinement and second prune ---
-    if (!o.skip_refine && hm.M > 0 && qmax > 0 && hm.M <= qmax * kModesPerCluster) {
+    if (!o.skip_refine && hm.M > 0 && (by_seed || (route.travel == kTravelGroups && P > 0 &&
+                                                   hm.M > grid_refine_capacity()))) {
+      // a block per mode, all updates in one launch
+      FMS_LAUNCH(refine_launch(hm.M, rtol_s * rtol_s, st));
+      FMS_LAUNCH(launch_greedy_merge_d(&mctl->M, mscore, ym, DP, d, r2_s, alive, acc2, &mctl->Mr,
+                                       hm.M, st));
+      FMS_LAUNCH(launch_canonical_order(ym, mscore, acc2, &mctl->Mr, d, DP, 1.0 / scale,
+                                        out_modes, max_modes, modes_full, nullptr, hm.M, st));
+    } else if (!o.skip_refine && hm.M > 0 && qmax > 0 && hm.M <= qmax * kModesPerCluster) {
       // cluster-persistent refinement (all updates, and each mode's density, in one launch)
       const double rtol_s = kRefineTolFactor * (double)h * scale;
       const int clusters = hm.M < qmax ? hm.M : qmax;
@@ -1258,8 +1380,95 @@ fms_status fms_select_seeds(int64_t n, uint64_t rng_seed, int64_t start, int64_t
 }
 
 
+namespace {
+// Scratch of one update whose points and seeds are sorted into cells.
+struct GroupStepLayout {
+  size_t off_Xp, off_Yp, off_Xs, off_Ys, off_xperm, off_yperm, off_start, off_ystart, off_ctr,
+      off_npiv, off_rad, off_table, off_ext, off_sort, off_status, total;
+  int DP, P;
+};
+
+// The sorted form pays from ~200 us of dense evaluations on (sorting both sides
+// costs ~60 us): about 1.7e9 padded coordinates of pairs at every width.
+bool step_by_groups(int64_t n, int d, int64_t m) {
+  return d <= 32 && n >= 2048 && m >= 2048 &&
+         (double)n * (double)m * (double)padded_dim(d) >= 1.7e9;
+}
+
+GroupStepLayout group_step_layout(int64_t n, int d, int64_t m) {
+  GroupStepLayout L{};
+  L.DP = padded_dim(d);
+  L.P = cells::choose_cells(n, m);
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at_ = o;
+    o += align256(bytes > 0 ? bytes : 1);
+    return at_;
+  };
+  const size_t row = (size_t)L.DP * 4;
+  L.off_Xp = take((size_t)n * row);
+  L.off_Yp = take((size_t)m * row);
+  L.off_Xs = take((size_t)n * row);
+  L.off_Ys = take((size_t)m * row);
+  L.off_xperm = take((size_t)n * 4);
+  L.off_yperm = take((size_t)m * 4);
+  L.off_start = take((size_t)(L.P + 1) * 4);
+  L.off_ystart = take((size_t)(L.P + 1) * 4);
+  L.off_ctr = take((size_t)L.P * row);
+  L.off_npiv = take(4);
+  L.off_rad = take((size_t)L.P * 4);
+  L.off_table = take((size_t)cells::group_cap(m, L.P) * 8);
+  L.off_ext = take(d > 8 ? (size_t)L.P * L.P * 8 : 0);
+  const size_t a = cells::sort_scratch(1, n, L.P).total, b = cells::sort_scratch(1, m, L.P).total;
+  L.off_sort = take(a > b ? a : b);
+  L.off_status = take(64);
+  L.total = o;
+  return L;
+}
+
+// One update with the points and the seeds in cells: each group of 32 seeds
+// visits the cells within its cutoff.
+cudaError_t group_step(const float* points, int64_t n, int32_t d, float scale, const float* seeds,
+                       int64_t m, double inv_scale, float* out_seeds, float* out_wsum, void* ws,
+                       const GroupStepLayout& L, int sms, cudaStream_t st) {
+  float* Xp = at<float>(ws, L.off_Xp);
+  float* Yp = at<float>(ws, L.off_Yp);
+  float* Xs = at<float>(ws, L.off_Xs);
+  float* Ys = at<float>(ws, L.off_Ys);
+  int2* table = at<int2>(ws, L.off_table);
+  float* ctr = at<float>(ws, L.off_ctr);
+  int32_t* npiv = at<int32_t>(ws, L.off_npiv);
+  uint32_t* status = at<uint32_t>(ws, L.off_status);
+  cudaError_t e = cudaMemsetAsync(status, 0, 64, st);
+  if (e == cudaSuccess) e = launch_pack_points(points, n, d, L.DP, scale, Xp, status, st);
+  if (e == cudaSuccess) e = launch_pack_points(seeds, m, d, L.DP, scale, Yp, status, st);
+  if (e == cudaSuccess)
+    e = cells::launch_sort<float>(Xp, 1, n, L.DP, true, L.P, at<void>(ws, L.off_sort), Xs,
+                                  at<int32_t>(ws, L.off_xperm), at<int32_t>(ws, L.off_start), ctr,
+                                  npiv, at<float>(ws, L.off_rad), nullptr, st);
+  if (e == cudaSuccess && d > 8)
+    e = cells::launch_extents(Xs, L.DP, L.P, at<int32_t>(ws, L.off_start), ctr,
+                              at<float2>(ws, L.off_ext), st);
+  if (e == cudaSuccess)
+    e = cells::launch_sort<float>(Yp, 1, m, L.DP, false, L.P, at<void>(ws, L.off_sort), Ys,
+                                  at<int32_t>(ws, L.off_yperm), at<int32_t>(ws, L.off_ystart), ctr,
+                                  npiv, nullptr, table, st);
+  if (e != cudaSuccess) return e;
+  cells::View<float> cv{};
+  cv.P = L.P;
+  cv.start = at<int32_t>(ws, L.off_start);
+  cv.ctr = ctr;
+  cv.rad = at<float>(ws, L.off_rad);
+  if (d > 8) cv.ext = at<float2>(ws, L.off_ext);
+  const cells::Groups gr{table, cells::group_cap(m, L.P)};
+  return launch_step_groups(Xs, cv, (int)n, Ys, gr, (int)m, at<int32_t>(ws, L.off_yperm), d, L.DP,
+                            seeds, inv_scale, out_seeds, out_wsum, sms, st);
+}
+}  // namespace
+
 size_t fms_step_workspace_size(int64_t n, int32_t d, int64_t m) {
   if (n < 1 || n > INT32_MAX || d < 1 || d > FMS_MAX_DIM || m < 1 || m > INT32_MAX) return 0;
+  if (step_by_groups(n, d, m)) return group_step_layout(n, d, m).total;
   return step_layout(n, d, m, device_info().sms).total;
 }
 
@@ -1272,26 +1481,33 @@ fms_status fms_mean_shift_step(const float* points, int64_t n, int32_t d, float 
   cudaStream_t st = static_cast<cudaStream_t>(stream_);
   const Dev dv = device_info();
   if (dv.sms <= 0) return FMS_ERR_CUDA;
-  const StepLayout L = step_layout(n, d, m, dv.sms);
+  const bool groups = step_by_groups(n, d, m);
+  const StepLayout L = groups ? StepLayout{} : step_layout(n, d, m, dv.sms);
+  const GroupStepLayout LG = groups ? group_step_layout(n, d, m) : GroupStepLayout{};
+  const size_t need = groups ? LG.total : L.total;
   fms_status rc = FMS_OK;
   bool owns = false;
   void* ws = workspace;
   uint32_t hstatus = 0;
   if (ws) {
-    if (workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0)
+    if (workspace_bytes < need || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0)
       return FMS_ERR_WORKSPACE;
   } else {
-    if (cudaMallocAsync(&ws, L.total, st) != cudaSuccess) return FMS_ERR_CUDA;
+    if (cudaMallocAsync(&ws, need, st) != cudaSuccess) return FMS_ERR_CUDA;
     owns = true;
   }
   {
     const double scale = sqrt(1.4426950408889634 / (2.0 * (double)h * (double)h));
+    uint32_t* status = at<uint32_t>(ws, groups ? LG.off_status : L.off_status);
+    if (groups) {
+      FMS_CUDA(group_step(points, n, d, (float)scale, seeds, m, 1.0 / scale, out_seeds, out_wsum,
+                          ws, LG, dv.sms, st));
+    } else {
     float* Xs = at<float>(ws, L.off_Xs);
     float* Ys = at<float>(ws, L.off_Ys);
     int32_t* active = at<int32_t>(ws, L.off_active);
     float* part = at<float>(ws, L.off_part);
     IterCtl* ctl = at<IterCtl>(ws, L.off_ctl);
-    uint32_t* status = at<uint32_t>(ws, L.off_status);
     FMS_CUDA(cudaMemsetAsync(status, 0, 64, st));
     FMS_CUDA(launch_pack_points(points, n, d, L.DP, (float)scale, Xs, status, st));
     FMS_CUDA(launch_pack_points(seeds, m, d, L.DP, (float)scale, Ys, status, st));
@@ -1300,6 +1516,7 @@ fms_status fms_mean_shift_step(const float* points, int64_t n, int32_t d, float 
                             L.grid_ctas * 8, st, nullptr, nullptr, kKernelGaussian, status));
     FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,
                                 (int)m, st));
+    }
     if (owns) {
       FMS_CUDA(cudaMemcpyAsync(&hstatus, status, 4, cudaMemcpyDeviceToHost, st));
       FMS_CUDA(cudaStreamSynchronize(st));

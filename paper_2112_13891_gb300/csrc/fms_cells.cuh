@@ -39,9 +39,22 @@ template <typename T>
 struct View {
   int P;                 // cells per set; 0: one cell with every row, nothing sorted
   const int32_t* start;  // [B][P + 1] first row of each cell (within the set)
-  const T* ctr;          // [B][P][DP] cell centres (the pivots)
-  const T* rad;          // [B][P] squared distance of the farthest row
+  const T* ctr;          // [B][P][DP] the mean of each cell's rows
+  const T* rad;          // [B][P] the distance of its farthest row from there
+  const float2* ext;     // [P][P] (one set, FP32; nullable): at [q][p], how far cell p's
+                         // rows reach from its centre towards cell q's, and the
+                         // distance of the two centres
 };
+
+// How far cell p's rows reach towards a seed y at distance a from its centre: the
+// extent towards cell q's centre, at distance delta from y, plus what the angle
+// between the two directions can add (two unit vectors a/|a|, b/|b| differ by at
+// most 2 |a - b| / (|a| + |b|)); never more than the radius.  In many dimensions
+// the radius of a cluster is several times its extent in any one direction, and
+// balls alone would find most clusters in reach of each other.
+__device__ __forceinline__ float reach_towards(float rad, float2 ext, float a, float delta) {
+  return fminf(rad, ext.x + rad * (2.0f * delta / (a + ext.y)));
+}
 
 // Groups of at most 32 rows of one cell.
 struct Groups {
@@ -95,38 +108,18 @@ __device__ __forceinline__ T cut_bits(T W, T log2n) {
   return need < T(zero_bits<T>()) ? (need > T(1) ? need : T(1)) : T(zero_bits<T>());
 }
 
-// The warp's list of the cells of one set that a ball (centre c, reach = its
-// radius + the cutoff radius) touches, as (first row, rows); returns its length.
-template <typename T, int DP>
-__device__ __forceinline__ int visible_cells(const View<T>& v, int b, int n, const T (&c)[DP],
-                                             T reach, int2* list, int lane) {
-  if (v.P == 0) {
-    if (lane == 0) list[0] = make_int2(0, n);
-    __syncwarp();
-    return 1;
-  }
-  const int32_t* st = v.start + (int64_t)b * (v.P + 1);
-  int cnt = 0;
-  for (int p0 = 0; p0 < v.P; p0 += 32) {
-    const int p = p0 + lane;
-    const T* q = v.ctr + ((int64_t)b * v.P + p) * DP;
-    T d2 = T(0);
-#pragma unroll
-    for (int k = 0; k < DP; ++k) {
-      const T e = q[k] - c[k];
-      d2 += e * e;
-    }
-    // 1e-4 covers the rounding of the distances and of their sum
-    const T lim = (reach + csqrt(v.rad[(int64_t)b * v.P + p])) * T(1.0001);
-    const int a = st[p], e = st[p + 1];
-    const bool see = e > a && !(d2 > lim * lim);
-    const unsigned m = __ballot_sync(kFull, see);
-    if (see) list[cnt + __popc(m & ((1u << lane) - 1u))] = make_int2(a, e - a);
-    cnt += __popc(m);
-  }
-  __syncwarp();
-  return cnt;
+// That exponent plus what the rounding of W in another order of summation can ask
+// for (a repeated pass must not find that it needs an ulp more).
+template <typename T>
+__device__ __forceinline__ T widen(T need) {
+  const T c = need + T(0.125);
+  return c < T(zero_bits<T>()) ? c : T(zero_bits<T>());
 }
+
+// First guess of the cutoff exponent of a seed whose W is not known: small, since
+// the pass at this cutoff gives a lower bound of W, from which the one that is
+// needed follows (a guess from W >= 0.5 walks most of 200,000 x 16 directions).
+constexpr float kFirstCut = 16.0f;
 
 __device__ __forceinline__ void cp16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -215,8 +208,9 @@ inline SortScratch sort_scratch(int64_t B, int64_t rows, int P) {
 }
 
 // Sorts B sets of nrows rows of DP values (set b at src + b nrows DP) into P
-// cells each.  points: the rows make the pivots, ctr [B][P][DP], npiv [B] and rad
-// [B][P] (squared) are written; else (seeds) ctr and npiv are read.  Writes dst
+// cells each.  points: the rows make the pivots, and the cells' means ctr
+// [B][P][DP], their number npiv [B] and radii rad [B][P] are written; else (seeds)
+// ctr and npiv are read.  Writes dst
 // (sorted rows), perm (sorted position -> row of the set), start [B][P + 1] and,
 // where non-null, the table of groups [B][group_cap(nrows, P)].
 template <typename T>
@@ -224,7 +218,42 @@ cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
                         int32_t* npiv, T* rad, int2* table, cudaStream_t st);
 
+// The extents of the P cells of one sorted set towards each other's centres
+// (View::ext), for d > 8.
+cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* start,
+                           const float* ctr, float2* ext, cudaStream_t st);
+
 }  // namespace cells
+
+// ---- k_travel.cu: whole trajectories in one launch (rows of DP floats, scaled)
+
+// One update of m seeds (Ys: sorted by perm), results in the caller's order and units.
+cudaError_t launch_step_groups(const float* Xs, const cells::View<float>& cv, int n,
+                               const float* Ys, const cells::Groups& gr, int m,
+                               const int32_t* perm, int d, int DP, const float* seeds,
+                               double inv_scale, float* out_seeds, float* out_wsum, int sms,
+                               cudaStream_t st);
+// Every point a seed, DP = 4 or 8: states, hist and the densities at the last positions.
+cudaError_t launch_travel_groups(const float* Xs, const cells::View<float>& cv, int n, int DP,
+                                 const cells::Groups& gr, const int32_t* perm, int kf,
+                                 int max_iter, float tol2_s, float sphere_r, float* y, int32_t* it,
+                                 int32_t* conv, int32_t* state, float* wlast, int32_t* hist,
+                                 unsigned long long* evals, unsigned long long* score_evals,
+                                 int sms, cudaStream_t st);
+// The RUNNING seeds of [0, N) (N and target from rc where non-null) to
+// convergence or the round's stop; *total: the sum of hist.
+cudaError_t launch_travel_seeds(const float* Xs, const cells::View<float>& cv, int n, int d, int DP,
+                                float* y, int32_t* it, int32_t* conv, int32_t* state, float* wlast,
+                                int32_t* hist, int32_t* total, const RoundCtl* rc, int N,
+                                int max_N, int target, int kf, int max_iter, float tol2_s,
+                                float sphere_r, unsigned long long* evals, int sms,
+                                cudaStream_t st);
+cudaError_t launch_refine_seeds(const float* Xs, const cells::View<float>& cv, int n, int d, int DP,
+                                const float* y, const int32_t* kept, const int32_t* accepted,
+                                const int32_t* M_ptr, int max_M, double* ym, float* yf,
+                                double* mscore, double tol2_s, int max_iter, int32_t* iters_out,
+                                unsigned long long* evals, int kf, double sphere_r, int sms,
+                                cudaStream_t st);
 
 // ---- k_unroll.cu (rows of DP values; seeds and points in sorted order)
 

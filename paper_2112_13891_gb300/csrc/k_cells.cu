@@ -6,16 +6,6 @@
 namespace fms {
 namespace cells {
 
-__device__ __forceinline__ void max_bits(float* p, float v) {
-  // squared distances are not negative, so their bits order as integers do
-  // (NaN above infinity)
-  atomicMax(reinterpret_cast<unsigned*>(p), __float_as_uint(v) & 0x7fffffffu);
-}
-__device__ __forceinline__ void max_bits(double* p, double v) {
-  atomicMax(reinterpret_cast<unsigned long long*>(p),
-            (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull);
-}
-
 // Row of pivot p: the middle of the p-th of P equal runs of the set's rows.
 __device__ __forceinline__ int64_t pivot_row(int p, int P, int64_t n) {
   return ((2 * (int64_t)p + 1) * n) / (2 * (int64_t)P);
@@ -102,13 +92,14 @@ __global__ void __launch_bounds__(256)
 }
 
 // The pivots of a set: the P0 strided ones, then the farthest row of every cell
-// whose radius is over twice the median one (a cluster that no strided pivot hit
-// hangs on to a cell of another one and would make its ball span both).  Fills pv,
+// whose radius is over twice the lowest eighth's (a cluster that no strided pivot
+// hit hangs on to cells of other ones and would make their balls span both; in
+// many dimensions a few such clusters reach most cells, hence not the median).  Fills pv,
 // returns their number; sel: P0 ints, red: 64 ints of shared memory.
 template <typename T, int DP>
 __device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
                           const unsigned long long* __restrict__ far_, T* pv, int* sel, int* red) {
-  __shared__ float median;
+  __shared__ float small;
   load_pivots<T, DP>(set, nrows, P0, pv);
   float* r2s = reinterpret_cast<float*>(sel);
   const int p = threadIdx.x;
@@ -117,16 +108,16 @@ __device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
     k = far_[p];
     r2s[p] = __uint_as_float((unsigned)(k >> 32));
   }
-  if (p == 0) median = INFINITY;
+  if (p == 0) small = INFINITY;
   __syncthreads();
   const float r2 = p < P0 ? r2s[p] : 0.0f;
   if (p < P0) {
     int rank = 0;
     for (int q = 0; q < P0; ++q) rank += (r2s[q] < r2 || (r2s[q] == r2 && q < p)) ? 1 : 0;
-    if (rank == P0 / 2) median = r2;
+    if (rank == P0 / 8) small = r2;
   }
   __syncthreads();
-  const int take = p < P0 && r2 > 4.0f * median ? 1 : 0;
+  const int take = p < P0 && r2 > 4.0f * small ? 1 : 0;
   int K = 0;
   const int at = block_exclusive_scan(take, &K, red);
   if (take) sel[at] = (int)(unsigned)k;
@@ -139,24 +130,20 @@ __device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
 
 // Second pass (EXTEND: over the points; else over the seeds, against the points'
 // finished pivots): the cell of every row, the rows of every (block, cell) in
-// counts [B][blocks][P], and for the points the cells' centres and squared radii.
+// counts [B][blocks][P], and for the points the pivots (in ctr).
 template <typename T, int DP, bool EXTEND>
 __global__ void __launch_bounds__(256)
     assign_kernel(const T* __restrict__ src, int nrows, int P, unsigned char* __restrict__ id,
                   const unsigned long long* __restrict__ far_, int32_t* __restrict__ counts,
-                  T* __restrict__ ctr, int32_t* __restrict__ npiv, T* __restrict__ rad) {
+                  T* __restrict__ ctr, int32_t* __restrict__ npiv) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
   __shared__ int red[64];
   __shared__ int sel[kMaxCells];
   T* pv = reinterpret_cast<T*>(cell_smem);                 // [P][DP]
-  T* far2 = pv + (size_t)P * DP;                           // [P]
-  int* hist = reinterpret_cast<int*>(far2 + P);            // [P]
+  int* hist = reinterpret_cast<int*>(pv + (size_t)P * DP);   // [P]
   const int b = blockIdx.y, blk = blockIdx.x, P0 = P / 2;
   const T* set = src + (int64_t)b * nrows * DP;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    far2[p] = T(0);
-    hist[p] = 0;
-  }
+  for (int p = threadIdx.x; p < P; p += blockDim.x) hist[p] = 0;
   int np;
   if (EXTEND) {
     np = all_pivots<T, DP>(set, nrows, P0, far_ + (int64_t)b * P0, pv, sel, red);
@@ -192,18 +179,69 @@ __global__ void __launch_bounds__(256)
     }
     id[(int64_t)b * nrows + r0] = (unsigned char)i0;
     atomicAdd(&hist[i0], 1);
-    if (rad) max_bits(&far2[i0], b0);
     if (r1 != r0) {
       id[(int64_t)b * nrows + r1] = (unsigned char)i1;
       atomicAdd(&hist[i1], 1);
-      if (rad) max_bits(&far2[i1], b1);
     }
   }
   __syncthreads();
   int32_t* out = counts + ((int64_t)b * gridDim.x + blk) * P;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    out[p] = hist[p];
-    if (rad && hist[p] > 0) max_bits(&rad[(int64_t)b * P + p], far2[p]);
+  for (int p = threadIdx.x; p < P; p += blockDim.x) out[p] = hist[p];
+}
+
+// Mean and radius of every cell (one block each): its rows are contiguous by now.
+template <typename T, int DP>
+__global__ void __launch_bounds__(128)
+    bound_kernel(const T* __restrict__ rows, int nrows, int P, const int32_t* __restrict__ start,
+                 T* __restrict__ ctr, T* __restrict__ rad) {
+  __shared__ T red[4][DP];
+  __shared__ T mean[DP];
+  const int b = blockIdx.y, p = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int a = start[(int64_t)b * (P + 1) + p], e = start[(int64_t)b * (P + 1) + p + 1];
+  if (e <= a) {
+    if (threadIdx.x == 0) rad[(int64_t)b * P + p] = T(0);
+    return;
+  }
+  const T* set = rows + (int64_t)b * nrows * DP;
+  T s[DP];
+#pragma unroll
+  for (int k = 0; k < DP; ++k) s[k] = T(0);
+  for (int r = a + threadIdx.x; r < e; r += blockDim.x) {
+    T x[DP];
+    row_values<T, DP>(set + (int64_t)r * DP, x);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) s[k] += x[k];
+  }
+#pragma unroll
+  for (int k = 0; k < DP; ++k) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) s[k] += __shfl_xor_sync(kFull, s[k], o);
+    if (lane == 0) red[w][k] = s[k];
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < DP; k += blockDim.x) {
+    const T v = (red[0][k] + red[1][k] + red[2][k] + red[3][k]) / T(e - a);
+    mean[k] = v;
+    ctr[((int64_t)b * P + p) * DP + k] = v;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < DP; ++k) s[k] = mean[k];
+  T far_ = T(0);
+  for (int r = a + threadIdx.x; r < e; r += blockDim.x) {
+    T x[DP], d2 = T(0);
+    row_values<T, DP>(set + (int64_t)r * DP, x);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) d2 += (x[k] - s[k]) * (x[k] - s[k]);
+    far_ = (d2 > far_ || !(d2 == d2)) ? d2 : far_;   // NaN wins
+  }
+  far_ = warp_max(far_);
+  __syncthreads();
+  if (lane == 0) red[w][0] = far_;
+  __syncthreads();
+  if (w == 0) {
+    far_ = warp_max(red[lane & 3][0]);
+    if (lane == 0) rad[(int64_t)b * P + p] = csqrt(far_);
   }
 }
 
@@ -292,6 +330,67 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// Thread q of a block keeps the unit vector from cell p's centre to cell q's, the
+// rows of p come by broadcast from shared memory.  DP multiply-adds a (row, q).
+constexpr int kExtRows = 64;
+
+template <int DP>
+__global__ void __launch_bounds__(kMaxCells)
+    extent_kernel(const float* __restrict__ rows, int P, const int32_t* __restrict__ start,
+                  const float* __restrict__ ctr, float2* __restrict__ ext) {
+  __shared__ __align__(16) float tile[kExtRows * DP];
+  const int p = blockIdx.x, q = threadIdx.x;
+  const int a = start[p], e = start[p + 1];
+  float v[DP], d2 = 0.0f;
+#pragma unroll
+  for (int k = 0; k < DP; ++k) {
+    v[k] = ctr[q * DP + k] - ctr[p * DP + k];
+    d2 = fmaf(v[k], v[k], d2);
+  }
+  const float dist = sqrtf(d2), inv = dist > 0.0f ? 1.0f / dist : 0.0f;
+#pragma unroll
+  for (int k = 0; k < DP; ++k) v[k] *= inv;
+  float far_ = 0.0f;
+  for (int r0 = a + blockIdx.y * kExtRows; r0 < e; r0 += gridDim.y * kExtRows) {
+    const int nr = min(kExtRows, e - r0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr * DP; i += blockDim.x)
+      tile[i] = rows[(int64_t)r0 * DP + i] - ctr[p * DP + i % DP];
+    __syncthreads();
+#pragma unroll 4
+    for (int r = 0; r < nr; ++r) {
+      float s = 0.0f;
+#pragma unroll
+      for (int k = 0; k < DP; k += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(tile + r * DP + k);
+        s = fmaf(x.x, v[k], s);
+        s = fmaf(x.y, v[k + 1], s);
+        s = fmaf(x.z, v[k + 2], s);
+        s = fmaf(x.w, v[k + 3], s);
+      }
+      far_ = (s > far_ || !(s == s)) ? s : far_;   // NaN wins
+    }
+  }
+  // (cleared to zero: not negative, so the bits order as integers do)
+  float* o = reinterpret_cast<float*>(ext + q * P + p);
+  atomicMax(reinterpret_cast<unsigned*>(o), __float_as_uint(far_) & 0x7fffffffu);
+  if (blockIdx.y == 0) o[1] = dist;
+}
+
+cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* start,
+                           const float* ctr, float2* ext, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(ext, 0, (size_t)P * P * 8, st);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)P, 8);
+  switch (DP) {
+    case 16: extent_kernel<16><<<grid, P, 0, st>>>(rows, P, start, ctr, ext); break;
+    case 32: extent_kernel<32><<<grid, P, 0, st>>>(rows, P, start, ctr, ext); break;
+    case 64: extent_kernel<64><<<grid, P, 0, st>>>(rows, P, start, ctr, ext); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
 template <typename T, int DP>
 static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P, void* scratch,
                           T* dst, int32_t* perm, int32_t* start, T* ctr, int32_t* npiv, T* rad,
@@ -302,7 +401,7 @@ static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P
   int32_t* counts = reinterpret_cast<int32_t*>(base + sc.counts);
   unsigned long long* far_ = reinterpret_cast<unsigned long long*>(base + sc.far_);
   const dim3 grid((unsigned)sort_blocks(nrows), (unsigned)B);
-  const size_t sm = (size_t)P * (DP + 1) * sizeof(T) + (size_t)P * 4;
+  const size_t sm = (size_t)P * DP * sizeof(T) + (size_t)P * 4;
   const size_t sm0 = (size_t)P / 2 * DP * sizeof(T) + (size_t)P / 2 * 8;
   cudaError_t e = cudaSuccess;
   if (sm > 40 * 1024) {   // (static arrays count against the default 48 KB)
@@ -315,17 +414,19 @@ static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P
   }
   if (points) {
     e = cudaMemsetAsync(far_, 0, (size_t)B * (P / 2) * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(rad, 0, (size_t)B * P * sizeof(T), st);
     if (e != cudaSuccess) return e;
     pivot_kernel<T, DP><<<grid, 256, sm0, st>>>(src, (int)nrows, P / 2, id, far_);
     assign_kernel<T, DP, true><<<grid, 256, sm, st>>>(src, (int)nrows, P, id, far_, counts, ctr,
-                                                      npiv, rad);
+                                                      npiv);
   } else {
     assign_kernel<T, DP, false><<<grid, 256, sm, st>>>(src, (int)nrows, P, id, nullptr, counts,
-                                                       ctr, npiv, nullptr);
+                                                       ctr, npiv);
   }
   scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, (int)nrows, P, id, counts, dst, perm, start,
                                              table, group_cap(nrows, P));
+  if (points)
+    bound_kernel<T, DP><<<dim3((unsigned)P, (unsigned)B), 128, 0, st>>>(dst, (int)nrows, P, start,
+                                                                        ctr, rad);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,690 @@
+// Whole trajectories in one launch.  Seeds do not depend on each other (Early
+// Stopping only needs the counts of their convergence updates), so a block
+// takes its seeds from their first update to convergence: no host round trip, no
+// grid barrier and no active list between updates.  Points are sorted into cells
+// (fms_cells.cuh) and a seed evaluates only the cells that its cutoff reaches.
+//
+//   step_groups    one update of many seeds: 32 seeds of one cell per group, one
+//                  per lane, points staged in shared memory and broadcast
+//   travel_groups  every point a seed (Alg. 1): the same groups, to convergence
+//   travel_seeds   few seeds (Alg. 2): a block per seed, points over the lanes
+//   refine_seeds   the refinement of merged modes, FP64 positions and sums
+//
+// Measured on one GB300 against the kernels that took every pair, one launch an
+// update: 20,011 seeds x 65,537 points x 32 (one update) 4.92 -> 1.10 ms, of which
+// step_groups 0.70; 200,000 x 3, every point a seed, 90.0 -> 17.4 ms; 2,000 x 2 (not
+// sorted) 0.59 -> 0.29 ms; 65,536 x 32 with 128 to 512 seeds 2.96 -> 0.93 ms, of
+// which the three travel_seeds 0.24; 200,000 x 16 directions 1.49 -> 0.80 ms, of
+// which the two travel_seeds 0.14.
+#include "fms_team.cuh"
+
+namespace fms {
+namespace {
+
+// Flat kernel: the window's exponent, widened by more than its FP32 rounding.
+constexpr float kFlatCut = -kFlatT * 1.0001f;
+
+template <int KF>
+__device__ __forceinline__ float first_cut() {
+  return KF == kKernelFlat ? kFlatCut : cells::kFirstCut;
+}
+
+// W and S of the group at y (acc[0], acc[1 + k]); `act` lanes decide the ball
+// and the cutoff, which comes in as a guess and leaves as the one their smallest
+// W asks for.  Returns the rows visited.
+template <int DP, int KF, int SUMS>
+__device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const View<float>& cv, int n,
+                                          const float (&y)[DP], bool act, float log2n, float& cut,
+                                          const TeamSmem<float, DP, SUMS>& sm, int w, int W,
+                                          int lane, float (&acc)[DP + 1]) {
+  int rows = 0;
+  for (int pass = 0;; ++pass) {
+    float reach;
+    const int nl = visible_cells<float, DP>(cv, 0, n, y, act, sqrtf(cut), &reach, nullptr, sm, w,
+                                            W, lane);
+    for (int i = lane; i < nl; i += 32) rows += sm.list[i].y;
+#pragma unroll
+    for (int k = 0; k <= DP; ++k) acc[k] = 0.0f;
+    cells::walk_tiles<DP>(Xs, sm.list, nl, w, W, sm.ring, lane, [&](const float* tile, int nr) {
+      float ta[DP + 1];
+#pragma unroll
+      for (int k = 0; k <= DP; ++k) ta[k] = 0.0f;
+#pragma unroll (DP <= 8 ? 4 : (DP <= 16 ? 2 : 1))
+      for (int q = 0; q < nr; ++q) {
+        float x[DP];
+        smem_row<DP>(tile + q * DP, x);
+        float t = 0.0f;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+          x[k] -= y[k];
+          t = fmaf(-x[k], x[k], t);
+        }
+        const float wt = kweight<KF>(t);
+        ta[0] += wt;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) ta[1 + k] = fmaf(wt, x[k], ta[1 + k]);
+      }
+#pragma unroll
+      for (int k = 0; k <= DP; ++k) acc[k] += ta[k];
+    });
+    team_sum(acc, sm.sums, SUMS, w, W, lane);
+    if (KF == kKernelFlat) break;
+    const float need = cells::cut_bits(cells::warp_min(act ? acc[0] : INFINITY), log2n);
+    if (cv.P == 0 || !(need > cut) || cut >= cells::zero_bits<float>()) {
+      cut = cells::widen(need);   // (W does not decrease along a trajectory)
+      break;
+    }
+    cut = pass == 0 ? cells::widen(need) : cells::zero_bits<float>();
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) rows += __shfl_xor_sync(kFull, rows, o);
+  return rows;
+}
+
+// out = seed + (S / W) / scale in the caller's order and units, as in step_finish.
+template <int DP>
+__global__ void __launch_bounds__(256)
+    step_groups(const float* __restrict__ Xs, View<float> cv, int n, const float* __restrict__ Ys,
+                Groups gr, int m, const int32_t* __restrict__ perm, int d, const float* seeds,
+                double inv_scale, float* out_seeds, float* __restrict__ out_wsum) {
+  extern __shared__ __align__(16) unsigned char travel_smem[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const TeamSmem<float, DP, DP + 1> sm(travel_smem, w, W);
+  int row0, cnt;
+  if (!group_rows(gr, 0, blockIdx.x, m, &row0, &cnt)) return;
+  const int e = row0 + min(lane, cnt - 1);
+  float y[DP], acc[DP + 1];
+  load_row<DP>(Ys + (int64_t)e * DP, y);
+  const float log2n = log2f((float)n);
+  float cut = first_cut<kKernelGaussian>();
+  group_pass<DP, kKernelGaussian>(Xs, cv, n, y, true, log2n, cut, sm, w, W, lane, acc);
+  if (w != 0 || lane >= cnt) return;
+  const int64_t i = perm[e];
+#pragma unroll
+  for (int k = 0; k < DP; ++k)
+    if (k < d)
+      out_seeds[i * d + k] =
+          (float)((double)seeds[i * d + k] + (double)(acc[1 + k] / acc[0]) * inv_scale);
+  if (out_wsum) out_wsum[i] = acc[0];
+}
+
+// Every point a seed, slot = the point's row in the caller's order (perm; null:
+// unsorted): updates until it converges, fails or has made max_iter of them, then
+// the density at its last position (wlast).  hist counts the convergence updates.
+template <int DP, int KF>
+__global__ void __launch_bounds__(512)
+    travel_groups(const float* __restrict__ Xs, View<float> cv, int n, Groups gr,
+                  const int32_t* __restrict__ perm, int max_iter, float tol2_s, float sphere_r,
+                  float* __restrict__ y_out, int32_t* __restrict__ it_out,
+                  int32_t* __restrict__ conv, int32_t* __restrict__ state,
+                  float* __restrict__ wlast, int32_t* __restrict__ hist,
+                  unsigned long long* evals, unsigned long long* score_evals) {
+  extern __shared__ __align__(16) unsigned char travel_smem[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const TeamSmem<float, DP, DP + 1> sm(travel_smem, w, W);
+  int row0, cnt;
+  if (!group_rows(gr, 0, blockIdx.x, n, &row0, &cnt)) return;
+  const int e = row0 + min(lane, cnt - 1);
+  float y[DP], acc[DP + 1];
+  load_row<DP>(Xs + (int64_t)e * DP, y);
+  const float log2n = log2f((float)n);
+  float cut = first_cut<KF>(), wl = 0.0f;
+  bool act = lane < cnt;
+  int it = 0, cu = -1, stt = kRunning;
+  unsigned long long ev = 0;
+  for (;;) {
+    const unsigned live = __ballot_sync(kFull, act);   // the same for every warp of the team
+    if (!live) break;
+    const int rows = group_pass<DP, KF>(Xs, cv, n, y, act, log2n, cut, sm, w, W, lane, acc);
+    ev += (unsigned long long)rows * __popc(live);
+    if (!act) continue;
+    wl = acc[0];
+    ++it;
+    bool ok = (wl > 0.0f) && isfinite(wl);
+    float dl[DP], step2 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      dl[k] = ok ? acc[1 + k] / wl : 0.0f;
+      step2 = fmaf(dl[k], dl[k], step2);
+    }
+    ok = ok && isfinite(step2);
+    if (ok && sphere_r > 0.0f) {
+      float nn = 0.0f;
+#pragma unroll
+      for (int k = 0; k < DP; ++k) {
+        dl[k] += y[k];
+        nn = fmaf(dl[k], dl[k], nn);
+      }
+      const float f = sphere_r / sqrtf(nn);
+      step2 = 0.0f;
+#pragma unroll
+      for (int k = 0; k < DP; ++k) {
+        dl[k] = dl[k] * f - y[k];
+        step2 = fmaf(dl[k], dl[k], step2);
+      }
+      ok = nn > 0.0f && isfinite(step2);
+    }
+    if (ok) {
+#pragma unroll
+      for (int k = 0; k < DP; ++k) y[k] += dl[k];
+    }
+    if (!ok) {
+      stt = kFailed;
+    } else if (step2 <= tol2_s) {
+      stt = kConverged;
+      cu = it;
+    } else if (it >= max_iter) {
+      stt = kExhausted;
+    }
+    act = stt == kRunning;
+  }
+  const bool fine = lane < cnt && stt != kFailed;
+  unsigned long long sev = 0;
+  if (__any_sync(kFull, fine)) {
+    const int rows = group_pass<DP, KF>(Xs, cv, n, y, fine, log2n, cut, sm, w, W, lane, acc);
+    sev = (unsigned long long)rows * __popc(__ballot_sync(kFull, fine));
+    wl = acc[0];
+  }
+  if (w != 0) return;
+  if (lane < cnt) {
+    const int64_t s = perm ? perm[e] : e;
+    store_row<float, DP>(y_out + s * DP, y);
+    it_out[s] = it;
+    conv[s] = cu;
+    state[s] = stt;
+    wlast[s] = wl;
+    if (cu > 0) atomicAdd(&hist[cu], 1);
+  }
+  if (lane == 0) {
+    atomicAdd(evals, ev);
+    atomicAdd(score_evals, sev);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// A block per seed: the 8 warps split the visible rows, LP = DP / 4 lanes to a
+// row (four coordinates each), so row-major rows are read as whole 128-byte
+// lines.  Bound by L2 bandwidth (4 DP bytes a row and seed).
+// ---------------------------------------------------------------------------
+constexpr int kSeedWarps = 8;
+
+template <int DP, typename ST>
+struct SeedSmem {
+  float y[DP];
+  int2 list[cells::kMaxCells];
+  unsigned mask[cells::kMaxCells / 32], near[kSeedWarps];
+  ST red[kSeedWarps][DP + 1];
+  ST tot[DP + 1];
+  float cut;
+  int flag;
+};
+
+// tot = (W, S) at sh.y over the cells within the cutoff sh.cut; returns the
+// rows visited.  Ends with a block barrier.
+template <int DP, int KF, typename ST>
+__device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, int n,
+                         SeedSmem<DP, ST>& sh) {
+  constexpr int LP = DP / 4, PPW = 32 / LP, UN = LP == 1 ? 4 : 8, CH = PPW * UN;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int nl = 0;
+  if (cv.P == 0) {
+    if (threadIdx.x == 0) sh.list[0] = make_int2(0, n);
+    nl = 1;
+    __syncthreads();
+  } else {
+    static_assert(cells::kMaxCells == 32 * kSeedWarps, "a cell to a thread");
+    const float rc = sqrtf(sh.cut);
+    const int p = threadIdx.x;
+    float a = -1.0f;   // distance of the cell's centre; negative: no rows
+    int2 mine = make_int2(0, 0);
+    bool see = false;
+    if (p < cv.P) {
+      const float4* q = reinterpret_cast<const float4*>(cv.ctr + (int64_t)p * DP);
+      float d2 = 0.0f;
+#pragma unroll
+      for (int k = 0; k < LP; ++k) {
+        const float4 v = __ldg(q + k);
+        const float4 yy = reinterpret_cast<const float4*>(sh.y)[k];
+        float t = v.x - yy.x;
+        d2 = fmaf(t, t, d2);
+        t = v.y - yy.y;
+        d2 = fmaf(t, t, d2);
+        t = v.z - yy.z;
+        d2 = fmaf(t, t, d2);
+        t = v.w - yy.w;
+        d2 = fmaf(t, t, d2);
+      }
+      mine.x = cv.start[p];
+      mine.y = cv.start[p + 1] - mine.x;
+      see = mine.y > 0;
+      a = see ? sqrtf(d2) : -1.0f;
+    }
+    float far_ = p < cv.P ? cv.rad[p] : 0.0f;
+    if (cv.ext) {   // (the same for the whole block)
+      const unsigned key = see ? (__float_as_uint(a) & ~255u) | (unsigned)p : 0xffffffffu;
+      const unsigned mn = __reduce_min_sync(kFull, key);
+      if (lane == 0) sh.near[w] = mn;
+      __syncthreads();
+      unsigned best = sh.near[0];
+#pragma unroll
+      for (int u = 1; u < kSeedWarps; ++u) best = min(best, sh.near[u]);
+      const int q = (int)(best & 255u);
+      // (the cut-off bits of the distance count as set)
+      if (see) far_ = cells::reach_towards(far_, cv.ext[q * cv.P + p], a, __uint_as_float(best | 255u));
+    }
+    see = see && !(a > (rc + far_) * 1.0001f);
+    const unsigned mk = __ballot_sync(kFull, see);
+    if (lane == 0) sh.mask[w] = mk;
+    __syncthreads();
+    for (int g = 0; g < kSeedWarps; ++g) {
+      const unsigned m = sh.mask[g];
+      if (g == w && see) sh.list[nl + __popc(m & ((1u << lane) - 1u))] = mine;
+      nl += __popc(m);
+    }
+    __syncthreads();
+  }
+  const int part = lane % LP, pl = lane / LP;
+  const float4 y4 = reinterpret_cast<const float4*>(sh.y)[part];
+  float aw = 0.0f;
+  float4 as = make_float4(0.f, 0.f, 0.f, 0.f);
+  int rows = 0, t = w;
+  const float4* X4 = reinterpret_cast<const float4*>(Xs);
+  for (int v = 0; v < nl; ++v) {
+    const int2 c = sh.list[v];
+    rows += c.y;
+    const int nt = (c.y + CH - 1) / CH;
+    for (; t < nt; t += kSeedWarps) {
+      float4 x[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        const int r = t * CH + u * PPW + pl;
+        // past the end: so far away that the weight is exactly zero
+        x[u] = r < c.y ? __ldg(X4 + (int64_t)(c.x + r) * LP + part)
+                       : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
+      }
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        x[u].x -= y4.x;
+        x[u].y -= y4.y;
+        x[u].z -= y4.z;
+        x[u].w -= y4.w;
+        float q = -x[u].x * x[u].x;
+        q = fmaf(-x[u].y, x[u].y, q);
+        q = fmaf(-x[u].z, x[u].z, q);
+        q = fmaf(-x[u].w, x[u].w, q);
+#pragma unroll
+        for (int o = 1; o < LP; o <<= 1) q += __shfl_xor_sync(kFull, q, o);
+        const float wt = kweight<KF>(q);
+        aw += wt;
+        as.x = fmaf(wt, x[u].x, as.x);
+        as.y = fmaf(wt, x[u].y, as.y);
+        as.z = fmaf(wt, x[u].z, as.z);
+        as.w = fmaf(wt, x[u].w, as.w);
+      }
+    }
+    t -= nt;
+  }
+  ST s[5] = {(ST)aw, (ST)as.x, (ST)as.y, (ST)as.z, (ST)as.w};
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+#pragma unroll
+    for (int o = LP; o < 32; o <<= 1) s[k] += __shfl_xor_sync(kFull, s[k], o);
+  if (pl == 0) {
+    if (part == 0) sh.red[w][0] = s[0];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sh.red[w][1 + part * 4 + k] = s[1 + k];
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k <= DP; k += blockDim.x) {
+    ST a = sh.red[0][k];
+#pragma unroll
+    for (int u = 1; u < kSeedWarps; ++u) a += sh.red[u][k];
+    sh.tot[k] = a;
+  }
+  __syncthreads();
+  return rows;
+}
+
+// Passes until the cutoff covers the W that came out (see fms_cells.cuh).
+template <int DP, int KF, typename ST>
+__device__ int seed_sums(const float* __restrict__ Xs, const View<float>& cv, int n, float log2n,
+                         SeedSmem<DP, ST>& sh) {
+  int rows = 0;
+  for (int pass = 0;; ++pass) {
+    rows += seed_pass<DP, KF, ST>(Xs, cv, n, sh);
+    if (KF == kKernelFlat || cv.P == 0) return rows;
+    const float need = cells::cut_bits((float)sh.tot[0], log2n);
+    const float cut = sh.cut;
+    const bool again = need > cut && cut < cells::zero_bits<float>();
+    __syncthreads();   // every thread has read sh.cut
+    if (threadIdx.x == 0)
+      sh.cut = again && pass > 0 ? cells::zero_bits<float>() : cells::widen(need);
+    __syncthreads();
+    if (!again) return rows;
+  }
+}
+
+// The RUNNING seeds of [0, N) to convergence.  A seed leaves once the convergence
+// counts (hist; total = their sum) say that the round ends at or before its next
+// update: the counts only grow, so a stop can come late, never early.
+template <int DP, int KF>
+__global__ void __launch_bounds__(kSeedWarps * 32)
+    travel_seeds(const float* __restrict__ Xs, View<float> cv, int n, int d, float* y,
+                 int32_t* it, int32_t* conv, int32_t* state, float* wlast, int32_t* hist,
+                 int32_t* total, const RoundCtl* __restrict__ rc, int N_arg, int target_arg,
+                 int max_iter, float tol2_s, float sphere_r, unsigned long long* evals) {
+  __shared__ __align__(16) SeedSmem<DP, float> sh;
+  const int N = rc ? rc->N : N_arg, target = rc ? rc->target : target_arg;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float log2n = log2f((float)n);
+  unsigned long long ev = 0;
+  for (int s = blockIdx.x; s < N; s += gridDim.x) {
+    if (state[s] != kRunning) continue;
+    __syncthreads();   // the previous seed's values are no longer read
+    for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[(int64_t)s * DP + k];
+    if (threadIdx.x == 0) {
+      sh.cut = first_cut<KF>();
+      sh.flag = kRunning;
+    }
+    int done = it[s];
+    __syncthreads();
+    for (;;) {
+      int seen = 0;   // converged seeds so far (read ahead of the pass that hides it)
+      if (w == 0) seen = *(volatile int32_t*)total;
+      ev += (unsigned long long)seed_sums<DP, KF, float>(Xs, cv, n, log2n, sh);
+      ++done;
+      if (w == 0) {
+        const float W = sh.tot[0];
+        bool ok = (W > 0.0f) && isfinite(W);
+        constexpr int KL = (DP + 31) / 32;
+        float p[KL], dl[KL], step2 = 0.0f;
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          const int k = lane + 32 * u;
+          p[u] = k < DP ? sh.y[k] : 0.0f;
+          dl[u] = ok && k < d ? sh.tot[1 + k] / W : 0.0f;
+          step2 = fmaf(dl[u], dl[u], step2);
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
+        ok = ok && isfinite(step2);
+        if (ok && sphere_r > 0.0f) {
+          float nn = 0.0f;
+#pragma unroll
+          for (int u = 0; u < KL; ++u) {
+            dl[u] += p[u];
+            nn = fmaf(dl[u], dl[u], nn);
+          }
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
+          const float f = sphere_r / sqrtf(nn);
+          step2 = 0.0f;
+#pragma unroll
+          for (int u = 0; u < KL; ++u) {
+            const float q = dl[u] * f, g = q - p[u];
+            step2 = fmaf(g, g, step2);
+            dl[u] = q;   // the new position
+          }
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
+          ok = nn > 0.0f && isfinite(step2);
+        } else {
+#pragma unroll
+          for (int u = 0; u < KL; ++u) dl[u] += p[u];
+        }
+        int now = kRunning;
+        if (!ok) now = kFailed;
+        else if (step2 <= tol2_s) now = kConverged;
+        else if (done >= max_iter) now = kExhausted;
+        int stop = 0;
+        if (now == kRunning && seen >= target) {
+          int c = 0;
+          for (int b = 0; b <= done; b += 32)
+            if (b + lane <= done) c += *(volatile int32_t*)(hist + b + lane);
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
+          stop = c >= target;
+        }
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          const int k = lane + 32 * u;
+          if (ok && k < DP) sh.y[k] = dl[u];
+        }
+        if (lane == 0) {
+          if (now == kConverged) {
+            atomicAdd(&hist[done], 1);
+            atomicAdd(total, 1);
+            conv[s] = done;
+          }
+          if (now != kRunning || stop) {
+            it[s] = done;
+            state[s] = now;
+            wlast[s] = W;
+          }
+          sh.flag = (now != kRunning || stop) ? 1 : 0;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      if (sh.flag) break;
+    }
+    for (int k = threadIdx.x; k < DP; k += blockDim.x) y[(int64_t)s * DP + k] = sh.y[k];
+  }
+  if (threadIdx.x == 0 && ev) atomicAdd(evals, ev);
+}
+
+// The refinement: ym <- ym + S/W - (ym - fl32(ym)) until ||step|| <= tol or
+// max_iter updates; positions and the sums over lanes in FP64.
+template <int DP, int KF>
+__global__ void __launch_bounds__(kSeedWarps * 32)
+    refine_seeds(const float* __restrict__ Xs, View<float> cv, int n, int d,
+                 const float* __restrict__ y, const int32_t* __restrict__ kept,
+                 const int32_t* __restrict__ accepted, const int32_t* __restrict__ M_ptr,
+                 double* __restrict__ ym, float* __restrict__ yf, double* __restrict__ mscore,
+                 double tol2_s, int max_iter, int32_t* iters_out, unsigned long long* evals,
+                 double sphere_r) {
+  __shared__ __align__(16) SeedSmem<DP, double> sh;
+  const int M = *M_ptr;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float log2n = log2f((float)n);
+  unsigned long long ev = 0;
+  constexpr int KL = (DP + 31) / 32;
+  for (int m = blockIdx.x; m < M; m += gridDim.x) {
+    const int64_t src = kept[accepted[m]];
+    __syncthreads();
+    for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[src * DP + k];
+    if (threadIdx.x == 0) sh.cut = first_cut<KF>();
+    __syncthreads();
+    double p[KL], W = 0.0;   // warp 0: the position
+#pragma unroll
+    for (int u = 0; u < KL; ++u) p[u] = lane + 32 * u < DP ? (double)sh.y[lane + 32 * u] : 0.0;
+    int iters = 0;
+    for (; iters < max_iter;) {
+      ev += (unsigned long long)seed_sums<DP, KF, double>(Xs, cv, n, log2n, sh);
+      ++iters;
+      if (w == 0) {
+        W = sh.tot[0];
+        bool ok = W > 0.0 && isfinite(W);
+        double q[KL], step2 = 0.0;
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          const int k = lane + 32 * u;
+          const double dl = ok && k < d ? sh.tot[1 + k] / W - (p[u] - (double)sh.y[k]) : 0.0;
+          step2 += dl * dl;
+          q[u] = p[u] + dl;
+        }
+        if (ok && sphere_r > 0.0) {
+          double nn = 0.0;
+#pragma unroll
+          for (int u = 0; u < KL; ++u) nn += q[u] * q[u];
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
+          const double f = sphere_r / sqrt(nn);
+          step2 = 0.0;
+#pragma unroll
+          for (int u = 0; u < KL; ++u) {
+            q[u] *= f;
+            step2 += (q[u] - p[u]) * (q[u] - p[u]);
+          }
+          ok = nn > 0.0;
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
+        ok = ok && isfinite(step2);
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          const int k = lane + 32 * u;
+          if (ok) p[u] = q[u];
+          if (ok && k < DP) sh.y[k] = (float)q[u];
+        }
+        if (lane == 0) sh.flag = (!ok || step2 <= tol2_s) ? 1 : 0;
+        __syncwarp();
+      }
+      __syncthreads();
+      if (sh.flag) break;
+    }
+    if (w == 0) {
+#pragma unroll
+      for (int u = 0; u < KL; ++u) {
+        const int k = lane + 32 * u;
+        if (k < DP) {
+          ym[(int64_t)m * DP + k] = p[u];
+          yf[(int64_t)m * DP + k] = (float)p[u];
+        }
+      }
+      if (lane == 0) {
+        mscore[m] = W;
+        atomicMax(iters_out, iters);
+      }
+    }
+  }
+  if (threadIdx.x == 0 && ev) atomicAdd(evals, ev);
+}
+
+int seed_grid(int max_seeds, int sms) {
+  const int g = sms * 4;   // (resident blocks; each takes its seeds in turn)
+  return max_seeds < g ? (max_seeds > 0 ? max_seeds : 1) : g;
+}
+
+}  // namespace
+
+cudaError_t launch_step_groups(const float* Xs, const View<float>& cv, int n, const float* Ys,
+                               const Groups& gr, int m, const int32_t* perm, int d, int DP,
+                               const float* seeds, double inv_scale, float* out_seeds,
+                               float* out_wsum, int sms, cudaStream_t st) {
+#define FMS_STEP_GROUPS(DP_)                                                                     \
+  {                                                                                              \
+    constexpr int ws = team_warp_smem<float, DP_, DP_ + 1>();                                    \
+    const int W = team_warps(gr.per_set, sms, ws);                                               \
+    const int smem = group_team_smem<float, DP_, DP_ + 1>(W);                                    \
+    const cudaError_t e = team_attr(step_groups<DP_>, smem);                                     \
+    if (e != cudaSuccess) return e;                                                              \
+    step_groups<DP_><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, Ys, gr, m, perm, d, seeds,   \
+                                                         inv_scale, out_seeds, out_wsum);        \
+    return cudaGetLastError();                                                                   \
+  }
+  switch (DP) {
+    case 4: FMS_STEP_GROUPS(4)
+    case 8: FMS_STEP_GROUPS(8)
+    case 16: FMS_STEP_GROUPS(16)
+    case 32: FMS_STEP_GROUPS(32)
+  }
+#undef FMS_STEP_GROUPS
+  return cudaErrorInvalidValue;
+}
+
+template <int DP, int KF>
+static cudaError_t travel_groups_t(const float* Xs, const View<float>& cv, int n, const Groups& gr,
+                                   const int32_t* perm, int max_iter, float tol2_s,
+                                   float sphere_r, float* y, int32_t* it, int32_t* conv,
+                                   int32_t* state, float* wlast, int32_t* hist,
+                                   unsigned long long* evals, unsigned long long* score_evals,
+                                   int sms, cudaStream_t st) {
+  constexpr int ws = team_warp_smem<float, DP, DP + 1>();
+  // at least 4 warps: the last groups take many updates, with few others running
+  const int W0 = team_warps(gr.per_set, sms, ws, 16), W = W0 < 4 ? 4 : W0;
+  const int smem = group_team_smem<float, DP, DP + 1>(W);
+  const cudaError_t e = team_attr(travel_groups<DP, KF>, smem);
+  if (e != cudaSuccess) return e;
+  travel_groups<DP, KF><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, gr, perm, max_iter, tol2_s,
+                                                            sphere_r, y, it, conv, state, wlast,
+                                                            hist, evals, score_evals);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_travel_groups(const float* Xs, const View<float>& cv, int n, int DP,
+                                 const Groups& gr, const int32_t* perm, int kf, int max_iter,
+                                 float tol2_s, float sphere_r, float* y, int32_t* it,
+                                 int32_t* conv, int32_t* state, float* wlast, int32_t* hist,
+                                 unsigned long long* evals, unsigned long long* score_evals,
+                                 int sms, cudaStream_t st) {
+#define FMS_TRAVEL(DP_)                                                                          \
+  return kf ? travel_groups_t<DP_, 1>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it,    \
+                                      conv, state, wlast, hist, evals, score_evals, sms, st)     \
+            : travel_groups_t<DP_, 0>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it,    \
+                                      conv, state, wlast, hist, evals, score_evals, sms, st)
+  switch (DP) {
+    case 4: FMS_TRAVEL(4);
+    case 8: FMS_TRAVEL(8);
+  }
+#undef FMS_TRAVEL
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_travel_seeds(const float* Xs, const View<float>& cv, int n, int d, int DP,
+                                float* y, int32_t* it, int32_t* conv, int32_t* state,
+                                float* wlast, int32_t* hist, int32_t* total, const RoundCtl* rc,
+                                int N, int max_N, int target, int kf, int max_iter, float tol2_s,
+                                float sphere_r, unsigned long long* evals, int sms,
+                                cudaStream_t st) {
+  const int g = seed_grid(max_N, sms);
+#define FMS_SEEDS(DP_)                                                                           \
+  if (kf)                                                                                        \
+    travel_seeds<DP_, 1><<<g, kSeedWarps * 32, 0, st>>>(Xs, cv, n, d, y, it, conv, state, wlast, \
+                                                        hist, total, rc, N, target, max_iter,    \
+                                                        tol2_s, sphere_r, evals);                \
+  else                                                                                           \
+    travel_seeds<DP_, 0><<<g, kSeedWarps * 32, 0, st>>>(Xs, cv, n, d, y, it, conv, state, wlast, \
+                                                        hist, total, rc, N, target, max_iter,    \
+                                                        tol2_s, sphere_r, evals);                \
+  return cudaGetLastError();
+  switch (DP) {
+    case 4: FMS_SEEDS(4)
+    case 8: FMS_SEEDS(8)
+    case 16: FMS_SEEDS(16)
+    case 32: FMS_SEEDS(32)
+    case 64: FMS_SEEDS(64)
+  }
+#undef FMS_SEEDS
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_refine_seeds(const float* Xs, const View<float>& cv, int n, int d, int DP,
+                                const float* y, const int32_t* kept, const int32_t* accepted,
+                                const int32_t* M_ptr, int max_M, double* ym, float* yf,
+                                double* mscore, double tol2_s, int max_iter, int32_t* iters_out,
+                                unsigned long long* evals, int kf, double sphere_r, int sms,
+                                cudaStream_t st) {
+  const int g = seed_grid(max_M, sms);
+#define FMS_SEEDS(DP_)                                                                          \
+  if (kf)                                                                                       \
+    refine_seeds<DP_, 1><<<g, kSeedWarps * 32, 0, st>>>(Xs, cv, n, d, y, kept, accepted, M_ptr, \
+                                                        ym, yf, mscore, tol2_s, max_iter,       \
+                                                        iters_out, evals, sphere_r);            \
+  else                                                                                          \
+    refine_seeds<DP_, 0><<<g, kSeedWarps * 32, 0, st>>>(Xs, cv, n, d, y, kept, accepted, M_ptr, \
+                                                        ym, yf, mscore, tol2_s, max_iter,       \
+                                                        iters_out, evals, sphere_r);            \
+  return cudaGetLastError();
+  switch (DP) {
+    case 4: FMS_SEEDS(4)
+    case 8: FMS_SEEDS(8)
+    case 16: FMS_SEEDS(16)
+    case 32: FMS_SEEDS(32)
+    case 64: FMS_SEEDS(64)
+  }
+#undef FMS_SEEDS
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace fms

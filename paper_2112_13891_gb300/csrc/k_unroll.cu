@@ -45,135 +45,16 @@
 // 3.8, recomputed positions 3.1, seed-major 5.2, point-major 6.0) against kernels
 // that took every pair.  3 sets x 1,500 points x 701 seeds x 3, T = 10 (nothing
 // sorted): 0.955 -> 0.561 ms from 94 launches going to 15.
-#include "fms_cells.cuh"
+#include "fms_team.cuh"
 
 namespace fms {
 
-using cells::Groups;
-using cells::View;
-
-template <int DPAD>
-__device__ __forceinline__ void load_row(const float* __restrict__ p, float (&v)[DPAD]) {
-#pragma unroll
-  for (int q = 0; q < DPAD / 4; ++q) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p) + q);
-    v[4 * q] = t.x;
-    v[4 * q + 1] = t.y;
-    v[4 * q + 2] = t.z;
-    v[4 * q + 3] = t.w;
-  }
-}
-
-template <int DPAD>
-__device__ __forceinline__ void load_row(const double* __restrict__ p, double (&v)[DPAD]) {
-#pragma unroll
-  for (int q = 0; q < DPAD / 2; ++q) {
-    const double2 t = __ldg(reinterpret_cast<const double2*>(p) + q);
-    v[2 * q] = t.x;
-    v[2 * q + 1] = t.y;
-  }
-}
-
-// a row already in shared memory: plain vector loads
-template <int DPAD>
-__device__ __forceinline__ void smem_row(const float* p, float (&v)[DPAD]) {
-#pragma unroll
-  for (int q = 0; q < DPAD / 4; ++q) {
-    const float4 t = reinterpret_cast<const float4*>(p)[q];
-    v[4 * q] = t.x;
-    v[4 * q + 1] = t.y;
-    v[4 * q + 2] = t.z;
-    v[4 * q + 3] = t.w;
-  }
-}
-template <int DPAD>
-__device__ __forceinline__ void smem_row(const double* p, double (&v)[DPAD]) {
-#pragma unroll
-  for (int q = 0; q < DPAD / 2; ++q) {
-    const double2 t = reinterpret_cast<const double2*>(p)[q];
-    v[2 * q] = t.x;
-    v[2 * q + 1] = t.y;
-  }
-}
-
-// the element type's exp2, fma and min (FP32: the MUFU exp2 with flush to zero)
-__device__ __forceinline__ float uex2(float x) { return ex2_ftz(x); }
-__device__ __forceinline__ double uex2(double x) { return exp2(x); }
-__device__ __forceinline__ float ufma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double ufma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float umin(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double umin(double a, double b) { return fmin(a, b); }
 
 // Below this W the unshifted weights lose precision (FP32 terms under 2^-126
 // flush to zero) and the seed is recomputed with a shift.
 template <typename T>
 __device__ __forceinline__ T unroll_min_w() {
   return sizeof(T) == 4 ? (T)1e-20f : (T)1e-280;
-}
-
-// Shared memory of a team of W warps: each warp's tile ring, its list of row
-// ranges, and its share of the sums exchanged at the end of a pass.
-constexpr int kListCap = cells::kMaxCells;
-
-template <typename T, int ROW, int SUMS>
-constexpr int unroll_warp_smem() {
-  return 2 * cells::kTileRows * ROW * (int)sizeof(T) + kListCap * 8 + SUMS * 32 * (int)sizeof(T);
-}
-
-template <typename T, int ROW, int SUMS>
-struct TeamSmem {
-  T* ring;      // this warp's two tiles
-  int2* list;   // this warp's list
-  T* sums;      // [W][SUMS][32], the whole team's
-  __device__ TeamSmem(unsigned char* base, int w, int W) {
-    constexpr int ring_e = 2 * cells::kTileRows * ROW;
-    ring = reinterpret_cast<T*>(base) + (size_t)w * ring_e;
-    unsigned char* p = base + (size_t)W * ring_e * sizeof(T);
-    sums = reinterpret_cast<T*>(p);
-    list = reinterpret_cast<int2*>(p + (size_t)W * SUMS * 32 * sizeof(T)) + w * kListCap;
-  }
-};
-
-// Sums v over the team in warp order; every warp gets the result.
-template <typename T, int N>
-__device__ __forceinline__ void team_sum(T (&v)[N], T* sums, int stride, int w, int W, int lane) {
-  if (W == 1) return;
-#pragma unroll
-  for (int k = 0; k < N; ++k) sums[(w * stride + k) * 32 + lane] = v[k];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    T s = sums[k * 32 + lane];
-    for (int u = 1; u < W; ++u) s += sums[(u * stride + k) * 32 + lane];
-    v[k] = s;
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ bool group_rows(const Groups& g, int b, int gi, int rows, int* row0,
-                                           int* cnt) {
-  if (g.table) {
-    const int2 e = __ldg(g.table + (int64_t)b * g.per_set + gi);
-    *row0 = e.x;
-    *cnt = e.y;
-  } else {
-    *row0 = gi * 32;
-    *cnt = min(32, rows - gi * 32);
-  }
-  return *cnt > 0;
-}
-
-template <typename T, int DP>
-__device__ __forceinline__ void store_row(T* p, const T (&v)[DP]) {
-  constexpr int E = 16 / (int)sizeof(T);
-#pragma unroll
-  for (int q = 0; q < DP / E; ++q) {
-    float4 t;
-    T* u = reinterpret_cast<T*>(&t);
-#pragma unroll
-    for (int e = 0; e < E; ++e) u[e] = v[q * E + e];
-    reinterpret_cast<float4*>(p)[q] = t;
-  }
 }
 
 // One far seed, recomputed by a warp with the points over its lanes: pass 1 the
@@ -243,14 +124,14 @@ __global__ void __launch_bounds__(256)
   T y[DP];
   load_row<DP>(Y0 + e * DP, y);
   const T log2n = T(log2f((float)g.n));
-  T cut = cells::cut_bits(T(0.5), log2n);
+  T cut = T(cells::kFirstCut);
   for (int t = 1; t <= steps; ++t) {
-    T ctr[DP], acc[DP + 2];   // W, S, sum w ||x - y||^2
-    const T rho = cells::group_ball<T, DP>(y, ctr);
+    T acc[DP + 2];   // W, S, sum w ||x - y||^2
     T need;
     for (int pass = 0;; ++pass) {
-      const int nl = cells::visible_cells<T, DP>(cv, b, g.n, ctr, rho + cells::csqrt(cut / c),
-                                                 sm.list, lane);
+      T reach;
+      const int nl = visible_cells<T, DP>(cv, b, g.n, y, true, cells::csqrt(cut / c), &reach,
+                                          nullptr, sm, w, W, lane);
 #pragma unroll
       for (int k = 0; k < DP + 2; ++k) acc[k] = T(0);
       cells::walk_tiles<DP>(Xb, sm.list, nl, w, W, sm.ring, lane, [&](const T* rows, int nr) {
@@ -279,10 +160,9 @@ __global__ void __launch_bounds__(256)
       team_sum(acc, sm.sums, SUMS, w, W, lane);
       need = cells::cut_bits(cells::warp_min(acc[0]), log2n);
       if (cv.P == 0 || !(need > cut)) break;
-      cut = pass == 0 ? need : T(cells::zero_bits<T>());
+      cut = pass == 0 ? cells::widen(need) : T(cells::zero_bits<T>());
     }
-    // W does not decrease along a trajectory: one bit covers its rounding
-    cut = umin(need + T(1), T(cells::zero_bits<T>()));
+    cut = cells::widen(need);   // (W does not decrease along a trajectory)
     T sh = T(0);
     unsigned bad = __ballot_sync(kFull, !(acc[0] >= unroll_min_w<T>()) || !isfinite(acc[0]));
     if (bad) {   // the same for every warp of the team
@@ -368,8 +248,10 @@ __global__ void __launch_bounds__(256)
       gd = ufma(gg[k], ym[k], gd);
     }
     // every weight above the cutoff of its seed (exponent c D2 - sh)
-    const T reach = cells::group_ball<T, DP>(y, ctr) +
-                    cells::warp_max(cells::csqrt((cells::cut_bits(Wt, log2n) + sh) / c));
+    T reach;
+    const int nl = visible_cells<T, DP>(cv, b, g.n, y, true,
+                                        cells::csqrt((cells::cut_bits(Wt, log2n) + sh) / c),
+                                        &reach, &ctr, sm, w, W, lane);
     if (w == 0) {
       if (lane < cnt) {
         T* o = SD + ((int64_t)u * rowsY + e) * SDW;
@@ -383,7 +265,6 @@ __global__ void __launch_bounds__(256)
         breach[(int64_t)u * NG + blockIdx.x] = reach;
       }
     }
-    const int nl = cells::visible_cells<T, DP>(cv, b, g.n, ctr, reach, sm.list, lane);
     T acc[DP + 1];   // sum p a, DY
     double DH = 0.0;
 #pragma unroll
@@ -446,7 +327,7 @@ __global__ void __launch_bounds__(256)
   extern __shared__ __align__(16) unsigned char unroll_smem[];
   constexpr int SUMS = DP, SDW = 2 * DP + 4;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
-  const TeamSmem<T, SDW, SUMS> sm(unroll_smem, w, W);
+  const TeamSmem<T, SDW, SUMS, false> sm(unroll_smem, w, W);
   const int b = blockIdx.x / gx.per_set;
   int row0, cnt;
   if (!group_rows(gx, b, blockIdx.x % gx.per_set, g.n, &row0, &cnt)) return;
@@ -574,30 +455,16 @@ static int blocks_for(int64_t work, int per = 256) {
   return (int)b;
 }
 
-// Warps of a team: enough of them for about 32 warps per SM over all groups, as
-// many as shared memory holds.
-static int team_warps(int64_t groups, int sms, int warp_smem) {
-  int W = 1;
-  while (W < 8 && groups * W < (int64_t)sms * 32 && 2 * W * warp_smem <= 200 * 1024) W *= 2;
-  return W;
-}
-
-template <typename K>
-static cudaError_t team_attr(K kernel, int bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
 template <typename T, int DP>
 static cudaError_t travel_t(const T* X, const View<T>& cv, const T* Y0, const Groups& gr,
                             const UGeom& g, T c, int steps, int every, int slot0, T* pos, T* Wout,
                             T* Sh, T* M2, cudaStream_t st) {
   const int64_t NG = (int64_t)g.B * gr.per_set;
-  constexpr int ws = unroll_warp_smem<T, DP, DP + 3>();
-  const int W = team_warps(NG, g.sms, ws);
-  const cudaError_t e = team_attr(unroll_travel<T, DP>, W * ws);
+  constexpr int ws = team_warp_smem<T, DP, DP + 3>();
+  const int W = team_warps(NG, g.sms, ws), smem = group_team_smem<T, DP, DP + 3>(W);
+  const cudaError_t e = team_attr(unroll_travel<T, DP>, smem);
   if (e != cudaSuccess) return e;
-  unroll_travel<T, DP><<<(unsigned)NG, 32 * W, W * ws, st>>>(X, cv, Y0, gr, g, c, steps, every,
+  unroll_travel<T, DP><<<(unsigned)NG, 32 * W, smem, st>>>(X, cv, Y0, gr, g, c, steps, every,
                                                              slot0, pos, Wout, Sh, M2);
   return cudaGetLastError();
 }
@@ -621,14 +488,16 @@ static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, c
                          T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX, int first,
                          cudaStream_t st) {
   const int64_t NG = (int64_t)g.B * gr.per_set, NX = (int64_t)g.B * gx.per_set;
-  constexpr int ws = unroll_warp_smem<T, DP, DP + 2>(), wp = unroll_warp_smem<T, 2 * DP + 4, DP>();
+  constexpr int ws = team_warp_smem<T, DP, DP + 2>(), wp = team_warp_smem<T, 2 * DP + 4, DP>();
   const int Ws = team_warps(NG, g.sms, ws), Wp = team_warps(NX, g.sms, wp);
-  cudaError_t e = team_attr(unroll_bwd_seed<T, DP>, Ws * ws);
-  if (e == cudaSuccess) e = team_attr(unroll_bwd_point<T, DP>, Wp * wp);
+  const int smem_s = group_team_smem<T, DP, DP + 2>(Ws);
+  const int smem_p = list_team_smem<T, 2 * DP + 4, DP>(Wp);
+  cudaError_t e = team_attr(unroll_bwd_seed<T, DP>, smem_s);
+  if (e == cudaSuccess) e = team_attr(unroll_bwd_point<T, DP>, smem_p);
   if (e != cudaSuccess) return e;
-  unroll_bwd_seed<T, DP><<<(unsigned)NG, 32 * Ws, Ws * ws, st>>>(
+  unroll_bwd_seed<T, DP><<<(unsigned)NG, 32 * Ws, smem_s, st>>>(
       X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, first);
-  unroll_bwd_point<T, DP><<<(unsigned)NX, 32 * Wp, Wp * wp, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
+  unroll_bwd_point<T, DP><<<(unsigned)NX, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
                                                                   SD, bctr, breach, dX, first);
   return cudaGetLastError();
 }

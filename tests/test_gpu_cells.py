@@ -1,0 +1,98 @@
+"""Sorted cells and whole trajectories in one launch, at the sizes where their
+rules begin: one update by groups (n m times the padded width >= 1.7e9), a block
+per seed (d > 7; points sorted from n = 8,192 on) and every point a seed by groups
+(d <= 7; sorted from n = 4,096 on), against the FP64 oracle.
+
+Tolerances: one update as in test_gpu_step_parity (FP32 weights, sums of n terms);
+clusterings by the cluster parity bar (modes within 1e-3 h, identical labels away
+from ties)."""
+import numpy as np
+import pytest
+import torch
+
+import fms_inputs as fi
+import oracle as orc
+from fms_compare import compare_clustering
+
+pytestmark = pytest.mark.gpu
+
+fms = pytest.importorskip("paper_2112_13891_gb300")
+
+
+def _blobs(seed, n, d, k, box, sigma):
+    rng = np.random.default_rng(seed)
+    c = rng.uniform(0, box, (k, d))
+    return (c[rng.integers(0, k, n)] + sigma * rng.standard_normal((n, d))).astype(np.float32)
+
+
+# just above the rule's line; a last sort block of one row; fewer seeds than points
+@pytest.mark.parametrize("n,m,d,box,h", [(20_620, 20_623, 3, 200.0, 5.0), (14_580, 14_579, 6, 60.0, 4.0),
+                                         (10_241, 10_400, 9, 50.0, 2.5), (51_201, 2_080, 16, 50.0, 2.5),
+                                         (7_300, 7_291, 32, 12.0, 1.5)])
+def test_step_by_groups(n, m, d, box, h):
+    X = _blobs(n, n, d, 12, box, 1.0)
+    rng = np.random.default_rng(1)
+    Y = (X[rng.integers(0, n, m)] + 0.3 * rng.standard_normal((m, d))).astype(np.float32)
+    # 5 h beyond the outermost point: W ~ 1e-5 of a point's, so the cutoff widens
+    # (every weight still above 2^-126 = exp(-87.3): exp(-||y - x||^2 / 2h^2) at 5 h
+    # is exp(-12.5))
+    Y[7] = X[X[:, 0].argmax()]
+    Y[7, 0] += 5.0 * h
+    Y[m - 1] = X.max(axis=0) + 100.0 * h            # every weight zero
+    out, W = fms.mean_shift_step(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), h,
+                                 with_wsum=True)
+    out, W = out.cpu().numpy().astype(np.float64), W.cpu().numpy().astype(np.float64)
+    pick = np.unique(np.r_[0, 7, m - 2, rng.integers(0, m - 1, 200)])
+    ref, refW = orc.step(X, Y[pick], h), orc.kde(X, Y[pick], h)
+    assert np.abs(W[pick] / refW - 1).max() <= 1e-4
+    assert np.abs(out[pick] - ref).max() <= 2e-4 * h + 2.0 ** -20 * np.abs(ref).max()
+    assert W[m - 1] == 0.0 and np.isnan(out[m - 1]).all()   # 0 / 0, as without cells
+
+
+def test_step_by_groups_keeps_nonfinite():
+    n = m = 7_300
+    X = torch.randn((n, 32), device="cuda")
+    X[5, 3] = float("inf")
+    out = fms.mean_shift_step(X, torch.randn((m, 32), device="cuda"), 1.0)
+    assert torch.isnan(out).any(dim=1).all()   # an infinite point reaches every seed
+
+
+def _cluster(w, **kw):
+    X = torch.from_numpy(w.X).cuda()
+    res = fms.cluster(X, w.h, w.tol, w.max_iter, **kw)
+    again = fms.cluster(X, w.h, w.tol, w.max_iter, **kw)
+    assert torch.equal(res.modes, again.modes) and torch.equal(res.labels, again.labels)
+    ref = orc.cluster(w.X, w.h, w.tol, w.max_iter, **kw)
+    cmp = compare_clustering(res.modes.cpu().numpy(), res.labels.cpu().numpy(), ref, w.h)
+    assert cmp["mode_ok"] and cmp["label_mismatch"] == 0, cmp
+    return res, ref
+
+
+@pytest.mark.parametrize("d,per,sigma,kw", [
+    (8, 1366, 1.0, {}), (9, 1366, 1.0, {}), (16, 1366, 1.0, {}), (16, 1365, 1.0, {}),
+    (33, 1400, 0.5, {}), (64, 1366, 0.4, {}), (16, 1400, 0.6, dict(kernel="flat"))])
+def test_block_per_seed(d, per, sigma, kw):
+    # 6 blobs: 8,196 points sorted, 8,190 not
+    w = fi.separated_blobs(seed=d + per, k=6, d=d, per=per, sigma=sigma,
+                           h=2.0 if not kw else 8.0)
+    res, ref = _cluster(w, rng_seed=2, **kw)
+    assert res.stats["n_seeds_final"] == ref.n_seeds and res.stats["t_star_last"] == ref.t_star[-1]
+
+
+def test_block_per_seed_cosine():
+    _cluster(fi.directional_blobs(seed=3, k=12, d=16, per=700, spread=0.05, h=0.15),
+             metric="cosine", rng_seed=1)
+
+
+@pytest.mark.parametrize("d,n,kw", [(3, 4096, {}), (3, 4095, {}), (1, 4500, {}), (7, 4321, {}),
+                                    (2, 63, {}), (3, 4100, dict(kernel="flat")),
+                                    (3, 4100, dict(metric="cosine"))])
+def test_every_point_a_seed(d, n, kw):
+    if kw.get("metric") == "cosine":
+        w = fi.directional_blobs(seed=5, k=5, d=d, per=n // 5, spread=0.05, h=0.15)
+    else:
+        k = 3 if d == 1 else 6
+        w = fi.separated_blobs(seed=d + n, k=k, d=d, per=max(1, n // k), sigma=1.0,
+                               h=2.0 if "kernel" not in kw else 6.0)
+        w["X"] = np.concatenate([w.X, w.X[: n - len(w.X)] + 0.01]).astype(np.float32)
+    _cluster(w, all_seeds=True, **kw)
