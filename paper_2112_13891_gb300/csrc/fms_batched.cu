@@ -12,7 +12,7 @@
 #include <vector>
 
 #include "../../include/fms.h"
-#include "fms_internal.cuh"
+#include "fms_cells.cuh"
 
 namespace fms {
 cudaError_t launch_batched_seed_init(SetCtl* sc, int B, const float* Xs, int DP, uint64_t seed,
@@ -27,7 +27,16 @@ cudaError_t launch_batched_step(const float* Xs, int d, int DP, const float* y,
                                 const int32_t* list, const SetCtl* sc, int B, int kind,
                                 const int64_t* task_off, const int64_t* part_off,
                                 const int64_t* totals, float* part, int target_warps,
-                                uint32_t* status, cudaStream_t st);
+                                cudaStream_t st);
+cudaError_t launch_queue_seeds(SetCtl* sc, int B, const int32_t* state, int32_t* list,
+                               int64_t* list_off, int64_t* totals, int32_t* counters,
+                               const uint32_t* status, cudaStream_t st);
+cudaError_t launch_queue_kept(SetCtl* sc, int B, const int32_t* state, const int32_t* conv,
+                              const float* wlast, int keep_exhausted, int max_iter, int32_t* kept,
+                              float* score, int64_t* list_off, int64_t* totals, int32_t* counters,
+                              cudaStream_t st);
+cudaError_t launch_queue_modes(const SetCtl* sc, int B, int64_t* list_off, int64_t* totals,
+                               cudaStream_t st);
 cudaError_t launch_batched_update(const float* part, const int32_t* active, const SetCtl* sc,
                                   int B, const int64_t* list_off, const int64_t* part_off,
                                   const int64_t* totals, float* y, int32_t* it, int32_t* conv,
@@ -99,18 +108,34 @@ int sms_now() {
 struct BLayout {
   size_t Xs, y, it, conv, state, active, kept, acc1, acc2, plist, score, ym, yf, ract, mdone,
       mscore, modes_full, part, sc, task_off, part_off, list_off, totals, counters, pt_off, status,
-      total;
-  int DP, DA, R, TW;
+      sorted, start, ctr, npiv, rad, sort, wlast, total;
+  int DP, DA, R, TW, P;
   Tiling tl;
 };
 
-// Partial-sum capacity: per set C_b * cnt_b * DA with C_b from choose_chunks
+// d > 7: every seed is taken to convergence by one block (k_travel.cu).  For
+// d <= 7 a low-d warp task shares each point it loads among up to 8 seeds and an
+// update of all sets is one launch.
+bool by_queue(int d) { return d > 7; }
+
+// Cells of every set (0: sets too small to gain from them): as for one set of the
+// mean size, half as many at most (4 to 40 clusters a set; the cost of finding the
+// nearest pivot grows with them).
+int batch_cells(int64_t total, int B) {
+  if (total / B < 512) return 0;
+  const int P = cells::choose_cells(total / B, total / B);
+  return P < 128 ? P : 128;
+}
+
+// Partial-sum capacity (d <= 7): per set C_b * cnt_b * DA with C_b from choose_chunks
 // (<= 4 * tl.target_warps / G_b + 1), so sum_b <= (4 * TWb * B + total_groups) * R * DA.
-BLayout make_blayout(int64_t total, int B, int d, int sms, int tw_mult, int min_chunk) {
+BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw_mult,
+                     int min_chunk) {
   BLayout L{};
   L.DP = padded(d);
   L.DA = step_accumulators(d);
-  L.R = batched_seeds_per_warp(d);
+  L.R = step_seeds_per_warp(d);
+  L.P = by_queue(d) ? batch_cells(total, B) : 0;
   L.TW = (sms > 0 ? sms : 1) * step_resident_warps_per_sm(d);
   // every set gets a share of the GPU's warps for its chunking (all sets run
   // in the same launches)
@@ -147,7 +172,7 @@ BLayout make_blayout(int64_t total, int B, int d, int sms, int tw_mult, int min_
   L.mdone = take((size_t)total * 4);
   L.mscore = take((size_t)total * 8);
   L.modes_full = take((size_t)total * d * 4);
-  L.part = take(part_floats * 4);
+  L.part = take(by_queue(d) ? 0 : part_floats * 4);
   L.sc = take((size_t)B * sizeof(SetCtl));
   L.task_off = take((size_t)(B + 1) * 8);
   L.part_off = take((size_t)(B + 1) * 8);
@@ -156,8 +181,24 @@ BLayout make_blayout(int64_t total, int B, int d, int sms, int tw_mult, int min_
   L.counters = take(64);
   L.pt_off = take((size_t)(B + 1) * 8);
   L.status = take(64);
+  if (by_queue(d)) L.wlast = take((size_t)total * 4);
+  if (L.P > 0) {
+    L.sorted = take((size_t)total * L.DP * 4);
+    L.start = take((size_t)B * (L.P + 1) * 4);
+    L.ctr = take((size_t)B * L.P * L.DP * 4);
+    L.npiv = take((size_t)B * 4);
+    L.rad = take((size_t)B * L.P * 4);
+    L.sort = take(cells::sort_scratch(B, max_n, L.P, total).total);
+  }
   L.total = o;
   return L;
+}
+
+int64_t largest_set(const int64_t* offsets, int32_t B) {
+  int64_t m = 1;
+  for (int b = 0; b < B; ++b)
+    if (offsets[b + 1] - offsets[b] > m) m = offsets[b + 1] - offsets[b];
+  return m;
 }
 
 // Autotuner state: best (tw_mult, min_chunk) per (device, d, log2 total, B bucket).
@@ -269,7 +310,7 @@ size_t fms_batched_workspace_size(const int64_t* offsets, int32_t B, int32_t d,
   if (!offsets || B < 1 || d < 1 || d > FMS_MAX_DIM) return 0;
   const int64_t total = offsets[B] - offsets[0];
   if (total < 1 || total > INT32_MAX) return 0;
-  return make_blayout(total, B, d, sms_now(), kTwMults[0], 32).total;
+  return make_blayout(total, largest_set(offsets, B), B, d, sms_now(), kTwMults[0], 32).total;
 }
 
 fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int32_t B, int32_t d,
@@ -314,9 +355,9 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
   int dev = 0;
   cudaGetDevice(&dev);
   const auto key = std::make_tuple(dev, (int)d, ilog2(total), ilog2(B));
-  bool tuned = false;
+  bool tuned = by_queue(d);   // (the queue has no tiling)
   std::pair<int, int> cfg{kTwMults[0], d <= 7 ? kMinChunksLow[1] : kMinChunksWide[1]};
-  {
+  if (!tuned) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto itc = g_tuned.find(key);
     if (itc != g_tuned.end()) {
@@ -324,7 +365,8 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       tuned = true;
     }
   }
-  BLayout Lo = make_blayout(total, B, d, sms, cfg.first, cfg.second);
+  const int max_n = (int)largest_set(offsets, B);
+  BLayout Lo = make_blayout(total, max_n, B, d, sms, cfg.first, cfg.second);
   const size_t need = Lo.total;  // identical for every candidate tiling
   bool owns = false;
   void* ws = workspace;
@@ -373,6 +415,20 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
     int32_t* counters = at<int32_t>(ws, Lo.counters);
     int64_t* pt_off = at<int64_t>(ws, Lo.pt_off);
     uint32_t* status = at<uint32_t>(ws, Lo.status);
+    const bool queued = by_queue(d);
+    float* wlast = at<float>(ws, Lo.wlast);
+    float* rows = Lo.P > 0 ? at<float>(ws, Lo.sorted) : Xs;
+    cells::View<float> cv{};
+    if (Lo.P > 0) {
+      cv.P = Lo.P;
+      cv.start = at<int32_t>(ws, Lo.start);
+      cv.ctr = at<float>(ws, Lo.ctr);
+      cv.rad = at<float>(ws, Lo.rad);
+    }
+    auto queue = [&](const int32_t* l) {
+      return SeedQueue{l, list_off, totals, reinterpret_cast<unsigned long long*>(totals + 1), sc,
+                       B};
+    };
     const double scale = sqrt(1.4426950408889634 / (2.0 * (double)h * (double)h));
     const double tol_s = (double)tol * scale;
     const float tol2_s = (float)(tol_s * tol_s);
@@ -380,7 +436,6 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
     const double r2_s = (r_merge * scale) * (r_merge * scale);
     const int grid_upd = sms * 8;
     const BatchCond no_cond{0, 0};
-    int max_n = 1;
 
     for (int b = 0; b < B; ++b) {
       SetCtl& c = hsc[b];
@@ -391,7 +446,6 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       c.prevN = 0;
       const int t = (int)ceil((double)o.gamma * (double)c.N);
       c.target = t < 1 ? 1 : (t > c.N ? c.N : t);
-      if (c.n > max_n) max_n = c.n;
     }
     BC(cudaMemcpyAsync(sc, hsc.data(), (size_t)B * sizeof(SetCtl), cudaMemcpyHostToDevice, st));
     BC(cudaMemcpyAsync(pt_off, offsets, (size_t)(B + 1) * 8, cudaMemcpyHostToDevice, st));
@@ -411,13 +465,13 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       for (int tm : kTwMults)
         for (int ci = 0; ci < 3; ++ci) {
           const int mc = cands[ci];
-          const BLayout Lc = make_blayout(total, B, d, sms, tm, mc);
+          const BLayout Lc = make_blayout(total, max_n, B, d, sms, tm, mc);
           BC(launch_batched_compact(sc, B, state, it, conv, active, 1, max_iter, R, DA, Lc.tl,
                                     task_off, part_off, list_off, totals, counters, no_cond,
                                     status, st));
           BC(cudaEventRecord(e0, st));
           BC(launch_batched_step(Xs, d, DP, y, active, sc, B, kPlanActive, task_off, part_off,
-                                 totals, part, Lc.TW, status, st));
+                                 totals, part, Lc.TW, st));
           BC(cudaEventRecord(e1, st));
           BC(cudaEventSynchronize(e1));
           float ms = 0.f;
@@ -432,7 +486,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       // the trial compactions counted evaluations: the real run starts afresh
       BC(cudaMemcpyAsync(sc, hsc.data(), (size_t)B * sizeof(SetCtl), cudaMemcpyHostToDevice, st));
       cfg = best;
-      Lo = make_blayout(total, B, d, sms, cfg.first, cfg.second);
+      Lo = make_blayout(total, max_n, B, d, sms, cfg.first, cfg.second);
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tuned[key] = cfg;
     }
@@ -472,7 +526,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       bool capturing = false;
       if (e == cudaSuccess)
         e = cudaGraphConditionalHandleCreate(&h_round, g, 1, cudaGraphCondAssignDefault);
-      if (e == cudaSuccess)
+      if (e == cudaSuccess && !queued)
         e = cudaGraphConditionalHandleCreate(&h_ref, g, 0, cudaGraphCondAssignDefault);
       if (e == cudaSuccess)
         e = cudaStreamBeginCaptureToGraph(cs0, g, nullptr, nullptr, 0,
@@ -485,12 +539,32 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         e = launch_pack_points(points, total, d, DP, (float)scale, Xs, status, cs0);
       if (e == cudaSuccess)
         e = launch_batched_seed_init(sc, B, Xs, DP, o.rng_seed, y, it, conv, state, cs0);
+      if (e == cudaSuccess && cv.P > 0)
+        e = cells::launch_sort<float>(Xs, B, max_n, DP, true, Lo.P, at<void>(ws, Lo.sort), rows,
+                                      nullptr, at<int32_t>(ws, Lo.start), at<float>(ws, Lo.ctr),
+                                      at<int32_t>(ws, Lo.npiv), at<float>(ws, Lo.rad), nullptr,
+                                      cs0, pt_off, total);
       // seed rounds: WHILE any set doubles its seed count
       cudaGraph_t round_body = nullptr;
       if (e == cudaSuccess) e = begin_while(cs0, h_round, cs1, &round_body);
       if (e == cudaSuccess) {
-        cudaError_t e2 =
-            cudaGraphConditionalHandleCreate(&h_upd, round_body, 0, cudaGraphCondAssignDefault);
+        const int keep_exhausted = o.gamma >= 1.f ? 1 : 0;
+        cudaError_t e2 = cudaSuccess;
+        if (queued) {
+          // every seed of the round to its stop; kept seeds with their densities (sum w
+          // of the last update, or with gamma = 1, when kept seeds need not have
+          // converged, a pass at their positions)
+          e2 = launch_queue_seeds(sc, B, state, active, list_off, totals, counters, status, cs1);
+          if (e2 == cudaSuccess)
+            e2 = launch_travel_queue(rows, cv, d, DP, queue(active), y, it, conv, state, wlast,
+                                     max_iter, tol2_s, sms, cs1);
+          if (e2 == cudaSuccess)
+            e2 = launch_queue_kept(sc, B, state, conv, wlast, keep_exhausted, max_iter, kept,
+                                   score, list_off, totals, counters, cs1);
+          if (e2 == cudaSuccess && keep_exhausted)
+            e2 = launch_density_queue(rows, cv, DP, queue(kept), y, score, nullptr, sms, cs1);
+        } else {
+        e2 = cudaGraphConditionalHandleCreate(&h_upd, round_body, 0, cudaGraphCondAssignDefault);
         if (e2 == cudaSuccess)
           e2 = launch_batched_compact(sc, B, state, it, conv, active, 1, max_iter, R, DA, tl,
                                       task_off, part_off, list_off, totals, counters,
@@ -500,7 +574,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         if (e2 == cudaSuccess) e2 = begin_while(cs1, h_upd, cs2, &upd_body);
         if (e2 == cudaSuccess) {
           cudaError_t e3 = launch_batched_step(Xs, d, DP, y, active, sc, B, kPlanActive, task_off,
-                                               part_off, totals, part, Lo.TW, status, cs2);
+                                               part_off, totals, part, Lo.TW, cs2);
           if (e3 == cudaSuccess)
             e3 = launch_batched_update(part, active, sc, B, list_off, part_off, totals, y, it,
                                        conv, state, d, DP, DA, tol2_s, max_iter, grid_upd, cs2);
@@ -512,14 +586,15 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         }
         // prune: kept seeds, their densities, the per-set prune, seed-count decision
         if (e2 == cudaSuccess)
-          e2 = launch_batched_kept(sc, B, state, conv, o.gamma >= 1.f ? 1 : 0, kept, R, DA, tl,
+          e2 = launch_batched_kept(sc, B, state, conv, keep_exhausted, kept, R, DA, tl,
                                    task_off, part_off, list_off, totals, counters, cs1);
         if (e2 == cudaSuccess)
           e2 = launch_batched_step(Xs, d, DP, y, kept, sc, B, kPlanKept, task_off, part_off,
-                                   totals, part, Lo.TW, status, cs1);
+                                   totals, part, Lo.TW, cs1);
         if (e2 == cudaSuccess)
           e2 = launch_batched_score(part, sc, B, list_off, part_off, totals, DA, score, grid_upd,
                                     cs1);
+        }
         if (e2 == cudaSuccess)
           e2 = launch_batched_prune_f(sc, B, kept, score, y, DP, d, (float)r2_s, acc1, plist,
                                       max_n, cs1);
@@ -534,8 +609,17 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       if (e == cudaSuccess)
         e = launch_batched_refine_setup(sc, B, y, kept, acc1, DP, ym, yf, ract, mdone, 1, R, tl,
                                         cs0);
+      const double rtol_s = 1e-5 * (double)h * scale;
+      if (queued) {
+        if (e == cudaSuccess) e = launch_queue_modes(sc, B, list_off, totals, cs0);
+        if (e == cudaSuccess)
+          e = o.skip_refine
+                  ? launch_density_queue(rows, cv, DP, queue(ract), yf, nullptr, mscore, sms, cs0)
+                  : launch_refine_queue(rows, cv, d, DP, queue(ract), ym, yf, mscore,
+                                        rtol_s * rtol_s, kRefineMax, counters + kCtrRefine, sms,
+                                        cs0);
+      } else {
       if (!o.skip_refine) {
-        const double rtol_s = 1e-5 * (double)h * scale;
         if (e == cudaSuccess)
           e = launch_plan(sc, B, kPlanModes, R, DA, task_off, part_off, list_off, totals,
                           BatchCond{h_ref, 1}, status, cs0);
@@ -543,7 +627,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         if (e == cudaSuccess) e = begin_while(cs0, h_ref, cs1, &ref_body);
         if (e == cudaSuccess) {
           cudaError_t e2 = launch_batched_step(Xs, d, DP, yf, ract, sc, B, kPlanModes, task_off,
-                                               part_off, totals, part, Lo.TW, status, cs1);
+                                               part_off, totals, part, Lo.TW, cs1);
           if (e2 == cudaSuccess)
             e2 = launch_batched_refine_update(part, ract, sc, B, list_off, part_off, totals, ym,
                                               yf, mdone, mscore, d, DP, DA, rtol_s * rtol_s, 0,
@@ -564,10 +648,11 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
                         status, cs0);
       if (e == cudaSuccess)
         e = launch_batched_step(Xs, d, DP, yf, ract, sc, B, kPlanModes, task_off, part_off,
-                                totals, part, Lo.TW, status, cs0);
+                                totals, part, Lo.TW, cs0);
       if (e == cudaSuccess)
         e = launch_batched_refine_update(part, ract, sc, B, list_off, part_off, totals, ym, yf,
                                          mdone, mscore, d, DP, DA, 0.0, 1, grid_upd, cs0);
+      }
       // second prune, canonical order, labels
       if (e == cudaSuccess)
         e = launch_batched_prune_d(sc, B, mscore, ym, DP, d, r2_s, acc2, plist, max_n, cs0);
@@ -632,8 +717,11 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       stats->n_discarded = seeds - kept_n;
       stats->n_modes = modes;
       stats->refine_iterations = refines;
-      stats->kernel_launches = 2 + 7 * rounds + 3 * updates +
-                               (o.skip_refine ? 0 : 2 + 3 * refines) + 4 + 3;
+      // (d > 7: pack, the sort's four, seed init; per round seeds, travel, kept,
+      // (density,) prune, advance, seed init; setup, queue, refinement or density)
+      stats->kernel_launches =
+          queued ? 2 + (cv.P > 0 ? 4 : 0) + (o.gamma >= 1.f ? 7 : 6) * rounds + 3 + 3
+                 : 2 + 7 * rounds + 3 * updates + (o.skip_refine ? 0 : 2 + 3 * refines) + 4 + 3;
       stats->evals = ev;
       stats->workspace_bytes = need;
       stats->graph = 1;

@@ -199,10 +199,12 @@ inline int group_cap(int64_t rows, int P) { return (int)((rows + 31) / 32) + P; 
 struct SortScratch {
   size_t id, counts, far_, total;
 };
-inline SortScratch sort_scratch(int64_t B, int64_t rows, int P) {
+// (rows: of the largest set; total: of all sets, 0: B rows)
+inline SortScratch sort_scratch(int64_t B, int64_t rows, int P, int64_t total = 0) {
   SortScratch s{};
-  s.counts = align256((size_t)B * rows);
-  s.far_ = s.counts + align256((size_t)B * sort_blocks(rows) * P * 4);
+  s.counts = align256((size_t)(total > 0 ? total : B * rows));
+  const size_t chunks = total > 0 ? (size_t)(total / kChunkRows + B) + 1 : (size_t)(B * sort_blocks(rows));
+  s.far_ = s.counts + align256(chunks * P * 4);
   s.total = s.far_ + align256((size_t)B * (P / 2) * 8);
   return s;
 }
@@ -211,12 +213,15 @@ inline SortScratch sort_scratch(int64_t B, int64_t rows, int P) {
 // cells each.  points: the rows make the pivots, and the cells' means ctr
 // [B][P][DP], their number npiv [B] and radii rad [B][P] are written; else (seeds)
 // ctr and npiv are read.  Writes dst
-// (sorted rows), perm (sorted position -> row of the set), start [B][P + 1] and,
-// where non-null, the table of groups [B][group_cap(nrows, P)].
+// (sorted rows), start [B][P + 1] and, where non-null, perm (sorted position -> row
+// of the set) and the table of groups [B][group_cap(nrows, P)].  Sets of different
+// sizes: set b has the rows [offs[b], offs[b + 1]) of `total` (offs on the device),
+// nrows is the largest, and there is no table.
 template <typename T>
 cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
-                        int32_t* npiv, T* rad, int2* table, cudaStream_t st);
+                        int32_t* npiv, T* rad, int2* table, cudaStream_t st,
+                        const int64_t* offs = nullptr, int64_t total = 0);
 
 // The extents of the P cells of one sorted set towards each other's centres
 // (View::ext), for d > 8.
@@ -253,6 +258,30 @@ cudaError_t launch_refine_seeds(const float* Xs, const cells::View<float>& cv, i
                                 const int32_t* M_ptr, int max_M, double* ym, float* yf,
                                 double* mscore, double tol2_s, int max_iter, int32_t* iters_out,
                                 unsigned long long* evals, int kf, double sphere_r, int sms,
+                                cudaStream_t st);
+
+// The batched call (k_batched.cu): queue entries [0, *n_entries) of a list of (set,
+// seed) pairs, taken in turn from *queue (zero on entry); set b's cells are at
+// [b] of cv and its rows at p0_b.
+struct SeedQueue {
+  const int32_t* list;       // set b's entries from p0_b on: seed or mode slots
+  const int64_t* list_off;   // [B + 1] entries before set b's
+  const int64_t* n_entries;
+  unsigned long long* queue;
+  SetCtl* sc;
+  int B;
+};
+cudaError_t launch_travel_queue(const float* Xs, const cells::View<float>& cv, int d, int DP,
+                                const SeedQueue& q, float* y, int32_t* it, int32_t* conv,
+                                int32_t* state, float* wlast, int max_iter, float tol2_s, int sms,
+                                cudaStream_t st);
+// W at every listed slot's position, to score[p0 + entry] or mscore[slot].
+cudaError_t launch_density_queue(const float* Xs, const cells::View<float>& cv, int DP,
+                                 const SeedQueue& q, const float* y, float* score, double* mscore,
+                                 int sms, cudaStream_t st);
+cudaError_t launch_refine_queue(const float* Xs, const cells::View<float>& cv, int d, int DP,
+                                const SeedQueue& q, double* ym, float* yf, double* mscore,
+                                double tol2_s, int max_iter, int32_t* iters_out, int sms,
                                 cudaStream_t st);
 
 // ---- k_unroll.cu (rows of DP values; seeds and points in sorted order)

@@ -133,7 +133,7 @@ struct SetCtl {
   int32_t rr;      // refinement clock
   int32_t rdone;
   int32_t Mr;      // modes after refinement and the second prune
-  int32_t pad0;
+  int32_t total;   // (d > 7) seeds converged so far, in all rounds
   int64_t evals;
 };
 
@@ -148,7 +148,7 @@ enum BatchCounter : int {
   kCtrBlocksDone = 0,   // atomic ticket of the per-set kernels
   kCtrRounds = 1,       // seed rounds run
   kCtrUpdates = 2,      // seed updates run (all rounds)
-  kCtrRefine = 3,       // refinement updates run
+  kCtrRefine = 3,       // refinement updates run (of the slowest mode)
 };
 
 // Tiling of a (seed-group x point-chunk) warp-task grid.
@@ -456,7 +456,6 @@ cudaError_t launch_ms_step(const float* Xs, int64_t n, int d, int DP, const floa
                            const int32_t* p_lo_ptr = nullptr, int kf = kKernelGaussian,
                            uint32_t* status = nullptr);
 int step_seeds_per_warp(int d);
-int batched_seeds_per_warp(int d);   // the batched step's wide tasks (32 lanes x RG seeds)
 int step_resident_warps_per_sm(int d);
 // smallest chunk (points) of a warp task: the low-d kernel splits a chunk over
 // 32 lanes, the quad kernel (d = 8) over 4 point lanes, the wide kernel

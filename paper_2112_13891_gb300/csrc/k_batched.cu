@@ -7,13 +7,15 @@
 // control blocks (SetCtl) hold each set's clock, counts and chunking; a plan
 // (prefix sums over sets of warp tasks, partial-sum blocks and list entries)
 // lets one launch of the step / update kernels map a global task or list
-// index to (set, local index) by binary search.  One CTA per set runs the
+// index to (set, local index) by binary search.  For d > 7 one queue of all sets'
+// seeds takes each of them to convergence in one launch instead (k_travel.cu).  One CTA per set runs the
 // per-set bookkeeping (compaction under the Early Stopping clock rule, kept
 // list, prune, ordering); the last CTA to finish (atomic ticket, no waiting)
 // rebuilds the plan for the next launch.  The whole call runs as one CUDA
 // graph: the compaction, advance and refinement kernels decide on the device,
 // through conditional-node handles, whether another update, another seed round
 // or another refinement update follows.
+#include "fms_cells.cuh"
 #include "fms_prune_body.cuh"
 #include "fms_seedperm.cuh"
 #include "fms_step_body.cuh"
@@ -298,60 +300,12 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-template <int DPAD, int RG>
-__global__ void __launch_bounds__(128)
-    batched_step_wide(const float* __restrict__ Xs, const float* __restrict__ y,
-                      const int32_t* __restrict__ list, const SetCtl* __restrict__ sc, int B,
-                      int kind, const int64_t* __restrict__ task_off,
-                      const int64_t* __restrict__ part_off, const int64_t* __restrict__ totals,
-                      float* __restrict__ part, uint32_t* __restrict__ status) {
-  extern __shared__ __align__(16) float wide_tiles[];
-  __shared__ __align__(8) uint64_t wide_bars[4][2];
-  constexpr int SPW = 32 * RG;
-  const int64_t T = totals[0];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint64_t* bars = wide_bars[warp];
-  float* tiles = wide_tiles + warp * 2 * kWideTile * DPAD;
-  tc::ring_init(bars, lane);
-  uint32_t use0 = 0u, use1 = 0u;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; t < T; t += nw) {
-    const int b = find_set(task_off, B, t);
-    const SetCtl& c = sc[b];
-    int cnt, C, Lc;
-    plan_counts(c, kind, &cnt, &C, &Lc);
-    const int64_t local = t - task_off[b];
-    const int G = (cnt + SPW - 1) / SPW;
-    const int g = (int)(local % G), ch = (int)(local / G);
-    const int j0 = ch * Lc, j1 = min(c.n, j0 + Lc);
-    if (!wide_task<DPAD, RG>(Xs + (int64_t)c.p0 * DPAD, j0, j1, y, list + c.p0, cnt, g, ch,
-                             part + part_off[b], lane, 0, tiles, bars, use0, use1, status))
-      break;
-  }
-}
-
-template <int DPAD, int RG>
-static void launch_bwide(int grid, const float* Xs, const float* y, const int32_t* list,
-                         const SetCtl* sc, int B, int kind, const int64_t* task_off,
-                         const int64_t* part_off, const int64_t* totals, float* part,
-                         uint32_t* status, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr && wide_smem_bytes<DPAD>() > 48 * 1024) {
-    cudaFuncSetAttribute(batched_step_wide<DPAD, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         wide_smem_bytes<DPAD>());
-    attr = true;
-  }
-  batched_step_wide<DPAD, RG><<<grid, 128, wide_smem_bytes<DPAD>(), st>>>(
-      Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status);
-}
-
 cudaError_t launch_batched_step(const float* Xs, int d, int DP, const float* y,
                                 const int32_t* list, const SetCtl* sc, int B, int kind,
                                 const int64_t* task_off, const int64_t* part_off,
                                 const int64_t* totals, float* part, int target_warps,
-                                uint32_t* status, cudaStream_t st) {
+                                cudaStream_t st) {
   const int g = (target_warps + 7) / 8;
-  if (d > 7 && DP != padded_dim(d)) return cudaErrorInvalidValue;   // rows of the compiled width
   switch (d) {
     case 1: batched_step_lowd<1, 4, 2><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
     case 2: batched_step_lowd<2, 4, 4><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
@@ -360,12 +314,7 @@ cudaError_t launch_batched_step(const float* Xs, int d, int DP, const float* y,
     case 5: batched_step_lowd<5, 8, 8><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
     case 6: batched_step_lowd<6, 8, 8><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
     case 7: batched_step_lowd<7, 8, 8><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
-    default:
-      if (d <= 8) launch_bwide<8, 4>(2 * g, Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status, st);
-      else if (d <= 16) launch_bwide<16, 2>(2 * g, Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status, st);
-      else if (d <= 32) launch_bwide<32, 1>(2 * g, Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status, st);
-      else launch_bwide<64, 1>(2 * g, Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status, st);
-      break;
+    default: return cudaErrorInvalidValue;   // (d > 7: the queue of k_travel.cu)
   }
   return cudaGetLastError();
 }
@@ -526,6 +475,137 @@ __global__ void batched_score(const float* __restrict__ part, const SetCtl* __re
     for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
     if (lane == 0) score[c.p0 + p] = s;
   }
+}
+
+// ---------------------------------------------------------------------------
+// d > 7: the queues of k_travel.cu
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int queue_count(const SetCtl& c, int kind) {
+  if (kind == kPlanActive) return __ldcg(&c.s);
+  if (kind == kPlanKept) return __ldcg(&c.final_) ? 0 : __ldcg(&c.K);
+  return __ldcg(&c.M);
+}
+
+// Prefix sums over sets of list entries (list_off [B + 1]); totals[0] = all of
+// them, totals[1] = the queue's next entry (0).  One block.
+__device__ void build_queue(const SetCtl* __restrict__ sc, int B, int kind,
+                           int64_t* __restrict__ list_off, int64_t* __restrict__ totals) {
+  // serial over blocks of sets with a block scan (B is at most a few thousand; a
+  // block's sets have less than 2^31 seeds, as all points have)
+  __shared__ int scratch[64];
+  int64_t carry = 0;
+  for (int b0 = 0; b0 < B; b0 += blockDim.x) {
+    const int b = b0 + threadIdx.x;
+    const int v = b < B ? queue_count(sc[b], kind) : 0;
+    int tot;
+    const int before = block_exclusive_scan(v, &tot, scratch);
+    if (b < B) list_off[b] = carry + before;
+    carry += tot;
+  }
+  if (threadIdx.x == 0) {
+    list_off[B] = carry;
+    totals[0] = carry;
+    totals[1] = 0;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The seeds of a round: every RUNNING seed of a set that has no final result (new
+// seeds, and those that an earlier round's stop left unconverged).  One CTA per
+// set; the last CTA builds the queue.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool last_block(int32_t* counters, int B) {
+  __shared__ int sh_last;
+  int32_t* blocks_done = counters + kCtrBlocksDone;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sh_last = (atomicAdd(blocks_done, 1) == B - 1);
+    if (sh_last) *blocks_done = 0;
+  }
+  __syncthreads();
+  if (sh_last) __threadfence();
+  return sh_last;
+}
+
+__global__ void __launch_bounds__(1024)
+    queue_seeds(SetCtl* sc, int B, const int32_t* __restrict__ state, int32_t* __restrict__ list,
+                  int64_t* list_off, int64_t* totals, int32_t* counters,
+                  const uint32_t* status) {
+  __shared__ int scratch[64];
+  SetCtl* c = sc + blockIdx.x;
+  const bool bad = (__ldcg(status) & kStNonFinite) != 0;   // (bad input: nothing travels)
+  const int N = c->final_ || bad ? 0 : c->N, p0 = c->p0;
+  int base = 0;
+  for (int b0 = 0; b0 < N; b0 += blockDim.x) {
+    const int i = b0 + threadIdx.x;
+    const int take = i < N && state[p0 + i] == kRunning ? 1 : 0;
+    int tot;
+    const int off = block_exclusive_scan(take, &tot, scratch);
+    if (take) list[p0 + base + off] = p0 + i;
+    base += tot;
+  }
+  if (threadIdx.x == 0) c->s = base;
+  if (last_block(counters, B)) build_queue(sc, B, kPlanActive, list_off, totals);
+}
+
+// ---------------------------------------------------------------------------
+// The round's stop t* (the first update by which the target of Early Stopping has
+// converged, max_iter if it never does) and the kept seeds of each set with the
+// densities of their last updates (keep_exhausted: a density pass over the queue of them follows).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(1024)
+    queue_kept(SetCtl* sc, int B, const int32_t* __restrict__ state,
+                 const int32_t* __restrict__ conv, const float* __restrict__ wlast,
+                 int keep_exhausted, int max_iter, int32_t* __restrict__ kept,
+                 float* __restrict__ score, int64_t* list_off, int64_t* totals,
+                 int32_t* counters) {
+  __shared__ int scratch[64];
+  SetCtl* c = sc + blockIdx.x;
+  const int N = c->final_ ? 0 : c->N, p0 = c->p0;
+  // the smallest t with at least `target` seeds converged by update t
+  int lo = 0, hi = max_iter;   // the count at lo is below the target
+  auto by = [&](int t) {
+    int k = 0;
+    for (int i = threadIdx.x; i < N; i += blockDim.x)
+      k += state[p0 + i] == kConverged && conv[p0 + i] <= t ? 1 : 0;
+    return block_sum(k, scratch);
+  };
+  while (hi - lo > 1) {
+    const int mid = lo + (hi - lo) / 2;
+    if (by(mid) >= c->target) hi = mid;
+    else lo = mid;
+  }
+  const int t_star = hi, convd = by(t_star);
+  int base = 0;
+  for (int b0 = 0; b0 < N; b0 += blockDim.x) {
+    const int i = b0 + threadIdx.x;
+    int take = 0;
+    if (i < N) {
+      const int st = state[p0 + i];
+      take = keep_exhausted ? (st == kConverged || st == kExhausted)
+                            : (st == kConverged && conv[p0 + i] <= t_star);
+    }
+    int tot;
+    const int off = block_exclusive_scan(take, &tot, scratch);
+    if (take) {
+      kept[p0 + base + off] = p0 + i;
+      score[p0 + base + off] = wlast[p0 + i];
+    }
+    base += tot;
+  }
+  if (threadIdx.x == 0 && !c->final_) {
+    c->K = base;
+    c->t_star = t_star;
+    c->n_conv = convd;
+    c->steps += t_star;
+  }
+  if (last_block(counters, B)) build_queue(sc, B, kPlanKept, list_off, totals);
+}
+
+__global__ void __launch_bounds__(1024)
+    queue_modes(const SetCtl* sc, int B, int64_t* list_off, int64_t* totals) {
+  build_queue(sc, B, kPlanModes, list_off, totals);
 }
 
 // Prune of each set (one CTA per set): the sorted visit while its sort keys
@@ -863,6 +943,28 @@ cudaError_t launch_batched_score(const float* part, const SetCtl* sc, int B,
                                  const int64_t* totals, int DA, float* score, int grid,
                                  cudaStream_t st) {
   batched_score<<<grid, 256, 0, st>>>(part, sc, B, list_off, part_off, totals, DA, score);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_queue_seeds(SetCtl* sc, int B, const int32_t* state, int32_t* list,
+                               int64_t* list_off, int64_t* totals, int32_t* counters,
+                               const uint32_t* status, cudaStream_t st) {
+  queue_seeds<<<B, 1024, 0, st>>>(sc, B, state, list, list_off, totals, counters, status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_queue_kept(SetCtl* sc, int B, const int32_t* state, const int32_t* conv,
+                              const float* wlast, int keep_exhausted, int max_iter, int32_t* kept,
+                              float* score, int64_t* list_off, int64_t* totals, int32_t* counters,
+                              cudaStream_t st) {
+  queue_kept<<<B, 1024, 0, st>>>(sc, B, state, conv, wlast, keep_exhausted, max_iter, kept, score,
+                                 list_off, totals, counters);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_queue_modes(const SetCtl* sc, int B, int64_t* list_off, int64_t* totals,
+                               cudaStream_t st) {
+  queue_modes<<<1, 1024, 0, st>>>(sc, B, list_off, totals);
   return cudaGetLastError();
 }
 

@@ -6,6 +6,24 @@
 namespace fms {
 namespace cells {
 
+// First row and rows of set b: offs [B + 1] or, null, sets of `each` rows.
+__device__ __forceinline__ int64_t set_rows(const int64_t* __restrict__ offs, int b, int64_t each,
+                                            int* n) {
+  if (!offs) {
+    *n = (int)each;
+    return (int64_t)b * each;
+  }
+  const int64_t o = offs[b];
+  *n = (int)(offs[b + 1] - o);
+  return o;
+}
+
+// Blocks run over (set, chunk of kChunkRows rows), `per` chunks to a set; the
+// counters of set b's first chunk are row chunk0 of counts [chunks][P].
+__device__ __forceinline__ int64_t chunk0(const int64_t* __restrict__ offs, int b, int per) {
+  return offs ? offs[b] / kChunkRows + b : (int64_t)b * per;
+}
+
 // Row of pivot p: the middle of the p-th of P equal runs of the set's rows.
 __device__ __forceinline__ int64_t pivot_row(int p, int P, int64_t n) {
   return ((2 * (int64_t)p + 1) * n) / (2 * (int64_t)P);
@@ -59,26 +77,29 @@ __device__ __forceinline__ void row_values(const T* p, T (&x)[DP]) {
 // pivot's farthest row as (squared distance bits, row).
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
-    pivot_kernel(const T* __restrict__ src, int nrows, int P0, unsigned char* __restrict__ id,
-                 unsigned long long* __restrict__ far_) {
+    pivot_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int P0,
+                 int per, unsigned char* __restrict__ id, unsigned long long* __restrict__ far_) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
   T* pv = reinterpret_cast<T*>(cell_smem);                                        // [P0][DP]
   unsigned long long* fs = reinterpret_cast<unsigned long long*>(pv + P0 * DP);   // [P0]
-  const int b = blockIdx.y;
-  const T* set = src + (int64_t)b * nrows * DP;
+  const int b = blockIdx.x / per, blk = blockIdx.x % per;
+  int nrows;
+  const int64_t row0 = set_rows(offs, b, each, &nrows);
+  if ((int64_t)blk * kChunkRows >= nrows) return;
+  const T* set = src + row0 * DP;
   load_pivots<T, DP>(set, nrows, P0, pv);
   for (int p = threadIdx.x; p < P0; p += blockDim.x) fs[p] = 0ull;
   __syncthreads();
-  const int r_end = min(nrows, ((int)blockIdx.x + 1) * kChunkRows);
-  for (int r0 = blockIdx.x * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
+  const int r_end = min((int64_t)nrows, ((int64_t)blk + 1) * kChunkRows);
+  for (int r0 = blk * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
     const int r1 = r0 + (int)blockDim.x < r_end ? r0 + (int)blockDim.x : r0;
     T x0[DP], x1[DP], b0 = T(0), b1 = T(0);
     row_values<T, DP>(set + (int64_t)r0 * DP, x0);
     row_values<T, DP>(set + (int64_t)r1 * DP, x1);
     int i0 = 0, i1 = 0;
     nearest<T, DP>(x0, x1, pv, 0, P0, b0, b1, i0, i1);
-    id[(int64_t)b * nrows + r0] = (unsigned char)i0;
-    id[(int64_t)b * nrows + r1] = (unsigned char)i1;
+    id[row0 + r0] = (unsigned char)i0;
+    id[row0 + r1] = (unsigned char)i1;
     auto key = [](T v, int r) {
       return ((unsigned long long)(__float_as_uint((float)v) & 0x7fffffffu) << 32) | (unsigned)r;
     };
@@ -133,7 +154,8 @@ __device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
 // counts [B][blocks][P], and for the points the pivots (in ctr).
 template <typename T, int DP, bool EXTEND>
 __global__ void __launch_bounds__(256)
-    assign_kernel(const T* __restrict__ src, int nrows, int P, unsigned char* __restrict__ id,
+    assign_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int per,
+                  int P, unsigned char* __restrict__ id,
                   const unsigned long long* __restrict__ far_, int32_t* __restrict__ counts,
                   T* __restrict__ ctr, int32_t* __restrict__ npiv) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
@@ -141,8 +163,11 @@ __global__ void __launch_bounds__(256)
   __shared__ int sel[kMaxCells];
   T* pv = reinterpret_cast<T*>(cell_smem);                 // [P][DP]
   int* hist = reinterpret_cast<int*>(pv + (size_t)P * DP);   // [P]
-  const int b = blockIdx.y, blk = blockIdx.x, P0 = P / 2;
-  const T* set = src + (int64_t)b * nrows * DP;
+  const int b = blockIdx.x / per, blk = blockIdx.x % per, P0 = P / 2;
+  int nrows;
+  const int64_t row0 = set_rows(offs, b, each, &nrows);
+  if ((int64_t)blk * kChunkRows >= nrows) return;
+  const T* set = src + row0 * DP;
   for (int p = threadIdx.x; p < P; p += blockDim.x) hist[p] = 0;
   int np;
   if (EXTEND) {
@@ -157,7 +182,7 @@ __global__ void __launch_bounds__(256)
     for (int e = threadIdx.x; e < np * DP; e += blockDim.x) pv[e] = ctr[(int64_t)b * P * DP + e];
     __syncthreads();
   }
-  const int r_end = min(nrows, (blk + 1) * kChunkRows);
+  const int r_end = min((int64_t)nrows, ((int64_t)blk + 1) * kChunkRows);
   for (int r0 = blk * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
     const int r1 = r0 + (int)blockDim.x < r_end ? r0 + (int)blockDim.x : r0;
     T x0[DP], x1[DP], b0 = T(0), b1 = T(0);
@@ -165,8 +190,8 @@ __global__ void __launch_bounds__(256)
     row_values<T, DP>(set + (int64_t)r1 * DP, x1);
     int i0 = 0, i1 = 0;
     if (EXTEND) {
-      i0 = id[(int64_t)b * nrows + r0];
-      i1 = id[(int64_t)b * nrows + r1];
+      i0 = id[row0 + r0];
+      i1 = id[row0 + r1];
 #pragma unroll
       for (int k = 0; k < DP; ++k) {
         const T e0 = x0[k] - pv[i0 * DP + k], e1 = x1[k] - pv[i1 * DP + k];
@@ -177,32 +202,34 @@ __global__ void __launch_bounds__(256)
     } else {
       nearest<T, DP>(x0, x1, pv, 0, np, b0, b1, i0, i1);
     }
-    id[(int64_t)b * nrows + r0] = (unsigned char)i0;
+    id[row0 + r0] = (unsigned char)i0;
     atomicAdd(&hist[i0], 1);
     if (r1 != r0) {
-      id[(int64_t)b * nrows + r1] = (unsigned char)i1;
+      id[row0 + r1] = (unsigned char)i1;
       atomicAdd(&hist[i1], 1);
     }
   }
   __syncthreads();
-  int32_t* out = counts + ((int64_t)b * gridDim.x + blk) * P;
+  int32_t* out = counts + (chunk0(offs, b, per) + blk) * P;
   for (int p = threadIdx.x; p < P; p += blockDim.x) out[p] = hist[p];
 }
 
 // Mean and radius of every cell (one block each): its rows are contiguous by now.
 template <typename T, int DP>
 __global__ void __launch_bounds__(128)
-    bound_kernel(const T* __restrict__ rows, int nrows, int P, const int32_t* __restrict__ start,
+    bound_kernel(const T* __restrict__ rows, const int64_t* __restrict__ offs, int each, int P,
+                 const int32_t* __restrict__ start,
                  T* __restrict__ ctr, T* __restrict__ rad) {
   __shared__ T red[4][DP];
   __shared__ T mean[DP];
-  const int b = blockIdx.y, p = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int b = blockIdx.x / P, p = blockIdx.x % P, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int a = start[(int64_t)b * (P + 1) + p], e = start[(int64_t)b * (P + 1) + p + 1];
   if (e <= a) {
     if (threadIdx.x == 0) rad[(int64_t)b * P + p] = T(0);
     return;
   }
-  const T* set = rows + (int64_t)b * nrows * DP;
+  int nrows;
+  const T* set = rows + set_rows(offs, b, each, &nrows) * DP;
   T s[DP];
 #pragma unroll
   for (int k = 0; k < DP; ++k) s[k] = T(0);
@@ -251,7 +278,8 @@ __global__ void __launch_bounds__(128)
 // block from L2.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
-    scatter_kernel(const T* __restrict__ src, int nrows, int P,
+    scatter_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int per,
+                   int P,
                    const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
                    T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
                    int2* __restrict__ table, int cap) {
@@ -259,12 +287,16 @@ __global__ void __launch_bounds__(256)
   __shared__ int wcnt[WARPS][kMaxCells];
   __shared__ int base[kMaxCells];
   __shared__ int scan[64];
-  const int b = blockIdx.y, blk = blockIdx.x, nblk = gridDim.x;
+  const int b = blockIdx.x / per, blk = blockIdx.x % per;
+  int nrows;
+  const int64_t row0 = set_rows(offs, b, each, &nrows);
+  const int nblk = (int)(((int64_t)nrows + kChunkRows - 1) / kChunkRows);
+  if (blk >= nblk) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // thread p: rows of cell p in the whole set and in earlier blocks
   int tot = 0, before = 0;
   if ((int)threadIdx.x < P) {
-    const int32_t* c = counts + (int64_t)b * nblk * P + threadIdx.x;
+    const int32_t* c = counts + chunk0(offs, b, per) * P + threadIdx.x;
 #pragma unroll 8
     for (int q = 0; q < nblk; ++q) {
       const int v = c[(int64_t)q * P];
@@ -294,7 +326,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int i = 0; i < ITER; ++i) {
     const int r = blk * kChunkRows + (w * ITER + i) * 32 + lane;
-    ids[i] = r < nrows ? (int)id[(int64_t)b * nrows + r] : -1;
+    ids[i] = r < nrows ? (int)id[row0 + r] : -1;
     const unsigned m = __match_any_sync(kFull, ids[i]);
     if (ids[i] >= 0 && (m & ((1u << lane) - 1u)) == 0) wcnt[w][ids[i]] += __popc(m);
     __syncwarp();
@@ -320,8 +352,8 @@ __global__ void __launch_bounds__(256)
     if (ids[i] >= 0 && lower == 0) wcnt[w][ids[i]] += __popc(m);
     __syncwarp();
     if (ids[i] >= 0) {
-      const int64_t from = (int64_t)b * nrows + r, to = (int64_t)b * nrows + at;
-      perm[to] = r;
+      const int64_t from = row0 + r, to = row0 + at;
+      if (perm) perm[to] = r;
       const float4* s4 = reinterpret_cast<const float4*>(src + from * DP);
       float4* d4 = reinterpret_cast<float4*>(dst + to * DP);
 #pragma unroll
@@ -392,15 +424,18 @@ cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* star
 }
 
 template <typename T, int DP>
-static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P, void* scratch,
-                          T* dst, int32_t* perm, int32_t* start, T* ctr, int32_t* npiv, T* rad,
+static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrows, bool points, int P,
+                          int64_t total, void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr, int32_t* npiv, T* rad,
                           int2* table, cudaStream_t st) {
-  const SortScratch sc = sort_scratch(B, nrows, P);
+  const SortScratch sc = sort_scratch(B, nrows, P, total);
   unsigned char* base = static_cast<unsigned char*>(scratch);
   unsigned char* id = base + sc.id;
   int32_t* counts = reinterpret_cast<int32_t*>(base + sc.counts);
   unsigned long long* far_ = reinterpret_cast<unsigned long long*>(base + sc.far_);
-  const dim3 grid((unsigned)sort_blocks(nrows), (unsigned)B);
+  const int64_t per64 = sort_blocks(nrows);
+  if (per64 * B > INT32_MAX || (int64_t)P * B > INT32_MAX) return cudaErrorInvalidValue;
+  const int per = (int)per64;
+  const unsigned grid = (unsigned)(per64 * B);
   const size_t sm = (size_t)P * DP * sizeof(T) + (size_t)P * 4;
   const size_t sm0 = (size_t)P / 2 * DP * sizeof(T) + (size_t)P / 2 * 8;
   cudaError_t e = cudaSuccess;
@@ -415,17 +450,17 @@ static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P
   if (points) {
     e = cudaMemsetAsync(far_, 0, (size_t)B * (P / 2) * 8, st);
     if (e != cudaSuccess) return e;
-    pivot_kernel<T, DP><<<grid, 256, sm0, st>>>(src, (int)nrows, P / 2, id, far_);
-    assign_kernel<T, DP, true><<<grid, 256, sm, st>>>(src, (int)nrows, P, id, far_, counts, ctr,
+    pivot_kernel<T, DP><<<grid, 256, sm0, st>>>(src, offs, (int)nrows, P / 2, per, id, far_);
+    assign_kernel<T, DP, true><<<grid, 256, sm, st>>>(src, offs, (int)nrows, per, P, id, far_, counts, ctr,
                                                       npiv);
   } else {
-    assign_kernel<T, DP, false><<<grid, 256, sm, st>>>(src, (int)nrows, P, id, nullptr, counts,
+    assign_kernel<T, DP, false><<<grid, 256, sm, st>>>(src, offs, (int)nrows, per, P, id, nullptr, counts,
                                                        ctr, npiv);
   }
-  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, (int)nrows, P, id, counts, dst, perm, start,
+  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, (int)nrows, per, P, id, counts, dst, perm, start,
                                              table, group_cap(nrows, P));
   if (points)
-    bound_kernel<T, DP><<<dim3((unsigned)P, (unsigned)B), 128, 0, st>>>(dst, (int)nrows, P, start,
+    bound_kernel<T, DP><<<(unsigned)(P * B), 128, 0, st>>>(dst, offs, (int)nrows, P, start,
                                                                         ctr, rad);
   return cudaGetLastError();
 }
@@ -433,26 +468,28 @@ static cudaError_t sort_t(const T* src, int B, int64_t nrows, bool points, int P
 template <typename T>
 cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
-                        int32_t* npiv, T* rad, int2* table, cudaStream_t st) {
-  if (P < 32 || P > kMaxCells || (P & 31) || B < 1 || B > 65535) return cudaErrorInvalidValue;
+                        int32_t* npiv, T* rad, int2* table, cudaStream_t st, const int64_t* offs,
+                        int64_t total) {
+  if (total == 0) total = (int64_t)B * nrows;
+  if (P < 32 || P > kMaxCells || (P & 31) || B < 1) return cudaErrorInvalidValue;
   switch (DP) {
-    case 4: return sort_t<T, 4>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
-    case 8: return sort_t<T, 8>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
-    case 16: return sort_t<T, 16>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
-    case 32: return sort_t<T, 32>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 4: return sort_t<T, 4>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 8: return sort_t<T, 8>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 16: return sort_t<T, 16>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 32: return sort_t<T, 32>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
     case 64:
       if constexpr (sizeof(T) == 4)
-        return sort_t<T, 64>(src, B, nrows, points, P, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+        return sort_t<T, 64>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
   }
   return cudaErrorInvalidValue;
 }
 
 template cudaError_t launch_sort<float>(const float*, int, int64_t, int, bool, int, void*, float*,
                                         int32_t*, int32_t*, float*, int32_t*, float*, int2*,
-                                        cudaStream_t);
+                                        cudaStream_t, const int64_t*, int64_t);
 template cudaError_t launch_sort<double>(const double*, int, int64_t, int, bool, int, void*,
                                          double*, int32_t*, int32_t*, double*, int32_t*, double*,
-                                         int2*, cudaStream_t);
+                                         int2*, cudaStream_t, const int64_t*, int64_t);
 
 }  // namespace cells
 }  // namespace fms

@@ -9,13 +9,16 @@
 //   travel_groups  every point a seed (Alg. 1): the same groups, to convergence
 //   travel_seeds   few seeds (Alg. 2): a block per seed, points over the lanes
 //   refine_seeds   the refinement of merged modes, FP64 positions and sums
+//   *_queue        the same for many sets (and the density at given positions): blocks
+//                  take the next (set, seed) from a queue
 //
 // Measured on one GB300 against the kernels that took every pair, one launch an
 // update: 20,011 seeds x 65,537 points x 32 (one update) 4.92 -> 1.10 ms, of which
 // step_groups 0.70; 200,000 x 3, every point a seed, 90.0 -> 17.4 ms; 2,000 x 2 (not
 // sorted) 0.59 -> 0.29 ms; 65,536 x 32 with 128 to 512 seeds 2.96 -> 0.93 ms, of
 // which the three travel_seeds 0.24; 200,000 x 16 directions 1.49 -> 0.80 ms, of
-// which the two travel_seeds 0.14.
+// which the two travel_seeds 0.14; 256 sets of 1,000 to 50,000 x 16 in one call
+// (travel_queue, 4 warps a seed) 29.0 -> 7.3 ms.
 #include "fms_team.cuh"
 
 namespace fms {
@@ -202,18 +205,19 @@ __global__ void __launch_bounds__(512)
 }
 
 // ---------------------------------------------------------------------------
-// A block per seed: the 8 warps split the visible rows, LP = DP / 4 lanes to a
+// A block per seed: its NW warps split the visible rows, LP = DP / 4 lanes to a
 // row (four coordinates each), so row-major rows are read as whole 128-byte
 // lines.  Bound by L2 bandwidth (4 DP bytes a row and seed).
 // ---------------------------------------------------------------------------
-constexpr int kSeedWarps = 8;
+constexpr int kSeedWarps = 8;    // one set: as many warps as the seeds leave idle
+constexpr int kQueueWarps = 4;   // many sets: more seeds in flight instead
 
-template <int DP, typename ST>
+template <int DP, typename ST, int NW>
 struct SeedSmem {
   float y[DP];
   int2 list[cells::kMaxCells];
-  unsigned mask[cells::kMaxCells / 32], near[kSeedWarps];
-  ST red[kSeedWarps][DP + 1];
+  unsigned mask[cells::kMaxCells / 32], near[NW];
+  ST red[NW][DP + 1];
   ST tot[DP + 1];
   float cut;
   int flag;
@@ -221,9 +225,9 @@ struct SeedSmem {
 
 // tot = (W, S) at sh.y over the cells within the cutoff sh.cut; returns the
 // rows visited.  Ends with a block barrier.
-template <int DP, int KF, typename ST>
+template <int DP, int KF, typename ST, int NW>
 __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, int n,
-                         SeedSmem<DP, ST>& sh) {
+                         SeedSmem<DP, ST, NW>& sh) {
   constexpr int LP = DP / 4, PPW = 32 / LP, UN = LP == 1 ? 4 : 8, CH = PPW * UN;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int nl = 0;
@@ -232,13 +236,17 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
     nl = 1;
     __syncthreads();
   } else {
-    static_assert(cells::kMaxCells == 32 * kSeedWarps, "a cell to a thread");
+    constexpr int U = cells::kMaxCells / 32 / NW;   // cells of a thread
     const float rc = sqrtf(sh.cut);
-    const int p = threadIdx.x;
-    float a = -1.0f;   // distance of the cell's centre; negative: no rows
-    int2 mine = make_int2(0, 0);
-    bool see = false;
-    if (p < cv.P) {
+    float a[U], far_[U];   // distance of the cell's centre, reach of its rows from there
+    int2 mine[U];
+    unsigned best = 0xffffffffu;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int p = (u * NW + w) * 32 + lane;
+      mine[u] = make_int2(0, 0);
+      a[u] = far_[u] = 0.0f;
+      if (p >= cv.P) continue;
       const float4* q = reinterpret_cast<const float4*>(cv.ctr + (int64_t)p * DP);
       float d2 = 0.0f;
 #pragma unroll
@@ -254,31 +262,39 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
         t = v.w - yy.w;
         d2 = fmaf(t, t, d2);
       }
-      mine.x = cv.start[p];
-      mine.y = cv.start[p + 1] - mine.x;
-      see = mine.y > 0;
-      a = see ? sqrtf(d2) : -1.0f;
+      mine[u].x = cv.start[p];
+      mine[u].y = cv.start[p + 1] - mine[u].x;
+      a[u] = sqrtf(d2);
+      far_[u] = cv.rad[p];
+      if (mine[u].y > 0) best = min(best, (__float_as_uint(a[u]) & ~255u) | (unsigned)p);
     }
-    float far_ = p < cv.P ? cv.rad[p] : 0.0f;
     if (cv.ext) {   // (the same for the whole block)
-      const unsigned key = see ? (__float_as_uint(a) & ~255u) | (unsigned)p : 0xffffffffu;
-      const unsigned mn = __reduce_min_sync(kFull, key);
-      if (lane == 0) sh.near[w] = mn;
+      best = __reduce_min_sync(kFull, best);
+      if (lane == 0) sh.near[w] = best;
       __syncthreads();
-      unsigned best = sh.near[0];
 #pragma unroll
-      for (int u = 1; u < kSeedWarps; ++u) best = min(best, sh.near[u]);
+      for (int u = 0; u < NW; ++u) best = min(best, sh.near[u]);
       const int q = (int)(best & 255u);
       // (the cut-off bits of the distance count as set)
-      if (see) far_ = cells::reach_towards(far_, cv.ext[q * cv.P + p], a, __uint_as_float(best | 255u));
+      const float delta = __uint_as_float(best | 255u);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (mine[u].y > 0)
+          far_[u] = cells::reach_towards(far_[u], cv.ext[q * cv.P + (u * NW + w) * 32 + lane],
+                                         a[u], delta);
     }
-    see = see && !(a > (rc + far_) * 1.0001f);
-    const unsigned mk = __ballot_sync(kFull, see);
-    if (lane == 0) sh.mask[w] = mk;
+    bool see[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      see[u] = mine[u].y > 0 && !(a[u] > (rc + far_[u]) * 1.0001f);
+      const unsigned mk = __ballot_sync(kFull, see[u]);
+      if (lane == 0) sh.mask[u * NW + w] = mk;
+    }
     __syncthreads();
-    for (int g = 0; g < kSeedWarps; ++g) {
+#pragma unroll
+    for (int g = 0; g < cells::kMaxCells / 32; ++g) {
       const unsigned m = sh.mask[g];
-      if (g == w && see) sh.list[nl + __popc(m & ((1u << lane) - 1u))] = mine;
+      if (g % NW == w && see[g / NW]) sh.list[nl + __popc(m & ((1u << lane) - 1u))] = mine[g / NW];
       nl += __popc(m);
     }
     __syncthreads();
@@ -293,7 +309,7 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
     const int2 c = sh.list[v];
     rows += c.y;
     const int nt = (c.y + CH - 1) / CH;
-    for (; t < nt; t += kSeedWarps) {
+    for (; t < nt; t += NW) {
       float4 x[UN];
 #pragma unroll
       for (int u = 0; u < UN; ++u) {
@@ -338,7 +354,7 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
   for (int k = threadIdx.x; k <= DP; k += blockDim.x) {
     ST a = sh.red[0][k];
 #pragma unroll
-    for (int u = 1; u < kSeedWarps; ++u) a += sh.red[u][k];
+    for (int u = 1; u < NW; ++u) a += sh.red[u][k];
     sh.tot[k] = a;
   }
   __syncthreads();
@@ -346,12 +362,12 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
 }
 
 // Passes until the cutoff covers the W that came out (see fms_cells.cuh).
-template <int DP, int KF, typename ST>
+template <int DP, int KF, typename ST, int NW>
 __device__ int seed_sums(const float* __restrict__ Xs, const View<float>& cv, int n, float log2n,
-                         SeedSmem<DP, ST>& sh) {
+                         SeedSmem<DP, ST, NW>& sh) {
   int rows = 0;
   for (int pass = 0;; ++pass) {
-    rows += seed_pass<DP, KF, ST>(Xs, cv, n, sh);
+    rows += seed_pass<DP, KF, ST, NW>(Xs, cv, n, sh);
     if (KF == kKernelFlat || cv.P == 0) return rows;
     const float need = cells::cut_bits((float)sh.tot[0], log2n);
     const float cut = sh.cut;
@@ -364,117 +380,293 @@ __device__ int seed_sums(const float* __restrict__ Xs, const View<float>& cv, in
   }
 }
 
-// The RUNNING seeds of [0, N) to convergence.  A seed leaves once the convergence
-// counts (hist; total = their sum) say that the round ends at or before its next
-// update: the counts only grow, so a stop can come late, never early.
+// One RUNNING seed to convergence, failure, max_iter updates or the round's stop.
+// seen(): seeds converged so far; stop(t): whether the convergence counts say that
+// the round ends at or before update t (warp 0 calls; the counts only grow, so a
+// stop can come late, never early); converged(t): counts this one.
+template <int DP, int KF, int NW, typename Seen, typename Stop, typename Conv>
+__device__ int travel_seed(const float* __restrict__ Xs, const View<float>& cv, int n, int d,
+                           int64_t s, float* y, int32_t* it, int32_t* conv, int32_t* state,
+                           float* wlast, int target, int max_iter, float tol2_s, float sphere_r,
+                           SeedSmem<DP, float, NW>& sh, Seen&& seen_, Stop&& stop_, Conv&& conv_) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float log2n = log2f((float)n);
+  __syncthreads();   // the previous seed's values are no longer read
+  for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[s * DP + k];
+  if (threadIdx.x == 0) sh.cut = first_cut<KF>();
+  int done = it[s], rows = 0;
+  __syncthreads();
+  for (;;) {
+    int seen = 0;   // (read ahead of the pass that hides it)
+    if (w == 0) seen = __shfl_sync(kFull, seen_(), 0);
+    rows += seed_sums<DP, KF, float, NW>(Xs, cv, n, log2n, sh);
+    ++done;
+    if (w == 0) {
+      const float W = sh.tot[0];
+      bool ok = (W > 0.0f) && isfinite(W);
+      constexpr int KL = (DP + 31) / 32;
+      float p[KL], dl[KL], step2 = 0.0f;
+#pragma unroll
+      for (int u = 0; u < KL; ++u) {
+        const int k = lane + 32 * u;
+        p[u] = k < DP ? sh.y[k] : 0.0f;
+        dl[u] = ok && k < d ? sh.tot[1 + k] / W : 0.0f;
+        step2 = fmaf(dl[u], dl[u], step2);
+      }
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
+      ok = ok && isfinite(step2);
+      if (ok && sphere_r > 0.0f) {
+        float nn = 0.0f;
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          dl[u] += p[u];
+          nn = fmaf(dl[u], dl[u], nn);
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
+        const float f = sphere_r / sqrtf(nn);
+        step2 = 0.0f;
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          const float q = dl[u] * f, g = q - p[u];
+          step2 = fmaf(g, g, step2);
+          dl[u] = q;   // the new position
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
+        ok = nn > 0.0f && isfinite(step2);
+      } else {
+#pragma unroll
+        for (int u = 0; u < KL; ++u) dl[u] += p[u];
+      }
+      int now = kRunning;
+      if (!ok) now = kFailed;
+      else if (step2 <= tol2_s) now = kConverged;
+      else if (done >= max_iter) now = kExhausted;
+      const bool stop = now == kRunning && seen >= target && stop_(done);
+#pragma unroll
+      for (int u = 0; u < KL; ++u) {
+        const int k = lane + 32 * u;
+        if (ok && k < DP) sh.y[k] = dl[u];
+      }
+      if (lane == 0) {
+        if (now == kConverged) {
+          conv[s] = done;
+          conv_(done);
+        }
+        if (now != kRunning || stop) {
+          it[s] = done;
+          state[s] = now;
+          wlast[s] = W;
+        }
+        sh.flag = (now != kRunning || stop) ? 1 : 0;
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    if (sh.flag) break;
+  }
+  for (int k = threadIdx.x; k < DP; k += blockDim.x) y[s * DP + k] = sh.y[k];
+  return rows;
+}
+
+// The RUNNING seeds of [0, N); hist counts convergence updates, *total sums it.
 template <int DP, int KF>
 __global__ void __launch_bounds__(kSeedWarps * 32)
     travel_seeds(const float* __restrict__ Xs, View<float> cv, int n, int d, float* y,
                  int32_t* it, int32_t* conv, int32_t* state, float* wlast, int32_t* hist,
                  int32_t* total, const RoundCtl* __restrict__ rc, int N_arg, int target_arg,
                  int max_iter, float tol2_s, float sphere_r, unsigned long long* evals) {
-  __shared__ __align__(16) SeedSmem<DP, float> sh;
+  __shared__ __align__(16) SeedSmem<DP, float, kSeedWarps> sh;
   const int N = rc ? rc->N : N_arg, target = rc ? rc->target : target_arg;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const float log2n = log2f((float)n);
+  const int lane = threadIdx.x & 31;
   unsigned long long ev = 0;
   for (int s = blockIdx.x; s < N; s += gridDim.x) {
     if (state[s] != kRunning) continue;
-    __syncthreads();   // the previous seed's values are no longer read
-    for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[(int64_t)s * DP + k];
-    if (threadIdx.x == 0) {
-      sh.cut = first_cut<KF>();
-      sh.flag = kRunning;
-    }
-    int done = it[s];
-    __syncthreads();
-    for (;;) {
-      int seen = 0;   // converged seeds so far (read ahead of the pass that hides it)
-      if (w == 0) seen = *(volatile int32_t*)total;
-      ev += (unsigned long long)seed_sums<DP, KF, float>(Xs, cv, n, log2n, sh);
-      ++done;
-      if (w == 0) {
-        const float W = sh.tot[0];
-        bool ok = (W > 0.0f) && isfinite(W);
-        constexpr int KL = (DP + 31) / 32;
-        float p[KL], dl[KL], step2 = 0.0f;
-#pragma unroll
-        for (int u = 0; u < KL; ++u) {
-          const int k = lane + 32 * u;
-          p[u] = k < DP ? sh.y[k] : 0.0f;
-          dl[u] = ok && k < d ? sh.tot[1 + k] / W : 0.0f;
-          step2 = fmaf(dl[u], dl[u], step2);
-        }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
-        ok = ok && isfinite(step2);
-        if (ok && sphere_r > 0.0f) {
-          float nn = 0.0f;
-#pragma unroll
-          for (int u = 0; u < KL; ++u) {
-            dl[u] += p[u];
-            nn = fmaf(dl[u], dl[u], nn);
-          }
-#pragma unroll
-          for (int o = 16; o >= 1; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
-          const float f = sphere_r / sqrtf(nn);
-          step2 = 0.0f;
-#pragma unroll
-          for (int u = 0; u < KL; ++u) {
-            const float q = dl[u] * f, g = q - p[u];
-            step2 = fmaf(g, g, step2);
-            dl[u] = q;   // the new position
-          }
-#pragma unroll
-          for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
-          ok = nn > 0.0f && isfinite(step2);
-        } else {
-#pragma unroll
-          for (int u = 0; u < KL; ++u) dl[u] += p[u];
-        }
-        int now = kRunning;
-        if (!ok) now = kFailed;
-        else if (step2 <= tol2_s) now = kConverged;
-        else if (done >= max_iter) now = kExhausted;
-        int stop = 0;
-        if (now == kRunning && seen >= target) {
+    ev += (unsigned long long)travel_seed<DP, KF, kSeedWarps>(
+        Xs, cv, n, d, s, y, it, conv, state, wlast, target, max_iter, tol2_s, sphere_r, sh,
+        [&] { return *(volatile int32_t*)total; },
+        [&](int t) {
           int c = 0;
-          for (int b = 0; b <= done; b += 32)
-            if (b + lane <= done) c += *(volatile int32_t*)(hist + b + lane);
+          for (int b = 0; b <= t; b += 32)
+            if (b + lane <= t) c += *(volatile int32_t*)(hist + b + lane);
 #pragma unroll
           for (int o = 16; o >= 1; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-          stop = c >= target;
-        }
-#pragma unroll
-        for (int u = 0; u < KL; ++u) {
-          const int k = lane + 32 * u;
-          if (ok && k < DP) sh.y[k] = dl[u];
-        }
-        if (lane == 0) {
-          if (now == kConverged) {
-            atomicAdd(&hist[done], 1);
-            atomicAdd(total, 1);
-            conv[s] = done;
-          }
-          if (now != kRunning || stop) {
-            it[s] = done;
-            state[s] = now;
-            wlast[s] = W;
-          }
-          sh.flag = (now != kRunning || stop) ? 1 : 0;
-        }
-        __syncwarp();
-      }
-      __syncthreads();
-      if (sh.flag) break;
-    }
-    for (int k = threadIdx.x; k < DP; k += blockDim.x) y[(int64_t)s * DP + k] = sh.y[k];
+          return c >= target;
+        },
+        [&](int t) {
+          atomicAdd(&hist[t], 1);
+          atomicAdd(total, 1);
+        });
   }
   if (threadIdx.x == 0 && ev) atomicAdd(evals, ev);
 }
 
-// The refinement: ym <- ym + S/W - (ym - fl32(ym)) until ||step|| <= tol or
-// max_iter updates; positions and the sums over lanes in FP64.
+// ---- many sets: a queue of (set, seed) entries
+
+__device__ __forceinline__ int queue_set(const int64_t* __restrict__ off, int B, int64_t x) {
+  int lo = 0, hi = B - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(off + mid) <= x) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+template <int DP>
+__device__ __forceinline__ View<float> set_view(const View<float>& cv, int b) {
+  View<float> v = cv;
+  if (cv.P == 0) return v;
+  v.start += (int64_t)b * (cv.P + 1);
+  v.ctr += (int64_t)b * cv.P * DP;
+  v.rad += (int64_t)b * cv.P;
+  return v;
+}
+
+// The block's next entry: its set and place in the set's list; false at the end.
+__device__ __forceinline__ bool next_entry(const SeedQueue& q, int* set, int* at) {
+  __shared__ long long sh_e;
+  __syncthreads();
+  if (threadIdx.x == 0) sh_e = (long long)atomicAdd(q.queue, 1ull);
+  __syncthreads();
+  const int64_t e = sh_e;
+  if (e >= *q.n_entries) return false;
+  *set = queue_set(q.list_off, q.B, e);
+  *at = (int)(e - q.list_off[*set]);
+  return true;
+}
+
+template <int DP>
+__global__ void __launch_bounds__(kQueueWarps * 32)
+    travel_queue(const float* __restrict__ Xs, View<float> cv, int d, SeedQueue q, float* y,
+                 int32_t* it, int32_t* conv, int32_t* state, float* wlast, int max_iter,
+                 float tol2_s) {
+  __shared__ __align__(16) SeedSmem<DP, float, kQueueWarps> sh;
+  const int lane = threadIdx.x & 31;
+  int b, at;
+  while (next_entry(q, &b, &at)) {
+    SetCtl* c = q.sc + b;
+    const int p0 = c->p0, N = c->N, target = c->target;
+    const int rows = travel_seed<DP, kKernelGaussian, kQueueWarps>(
+        Xs + (int64_t)p0 * DP, set_view<DP>(cv, b), c->n, d, q.list[p0 + at], y, it, conv, state,
+        wlast, target, max_iter, tol2_s, 0.0f, sh,
+        [&] { return *(volatile int32_t*)&c->total; },
+        [&](int t) {
+          int k = 0;
+          for (int i = lane; i < N; i += 32) {
+            const int v = *(volatile int32_t*)(conv + p0 + i);
+            k += v > 0 && v <= t ? 1 : 0;
+          }
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) k += __shfl_xor_sync(kFull, k, o);
+          return k >= target;
+        },
+        [&](int) { atomicAdd(&c->total, 1); });
+    if (threadIdx.x == 0)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&c->evals), (unsigned long long)rows);
+  }
+}
+
+template <int DP>
+__global__ void __launch_bounds__(kQueueWarps * 32)
+    density_queue(const float* __restrict__ Xs, View<float> cv, SeedQueue q,
+                  const float* __restrict__ y, float* __restrict__ score,
+                  double* __restrict__ mscore) {
+  __shared__ __align__(16) SeedSmem<DP, double, kQueueWarps> sh;
+  int b, at;
+  while (next_entry(q, &b, &at)) {
+    SetCtl* c = q.sc + b;
+    const int64_t s = q.list[c->p0 + at];
+    __syncthreads();
+    for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[s * DP + k];
+    if (threadIdx.x == 0) sh.cut = first_cut<kKernelGaussian>();
+    __syncthreads();
+    const int rows = seed_sums<DP, kKernelGaussian, double, kQueueWarps>(
+        Xs + (int64_t)c->p0 * DP, set_view<DP>(cv, b), c->n, log2f((float)c->n), sh);
+    if (threadIdx.x == 0) {
+      if (score) score[c->p0 + at] = (float)sh.tot[0];
+      if (mscore) mscore[s] = sh.tot[0];
+      atomicAdd(reinterpret_cast<unsigned long long*>(&c->evals), (unsigned long long)rows);
+    }
+  }
+}
+
+// The refinement of one mode from sh.y: ym <- ym + S/W - (ym - fl32(ym)) until
+// ||step|| <= tol or max_iter updates; the position (and the sums over lanes) in
+// FP64, the density is W of the last update.  Returns the updates made.
+template <int DP, int KF, int NW>
+__device__ int refine_seed(const float* __restrict__ Xs, const View<float>& cv, int n, int d,
+                           double* ym, float* yf, double* mscore, double tol2_s, int max_iter,
+                           double sphere_r, SeedSmem<DP, double, NW>& sh, unsigned long long& ev) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float log2n = log2f((float)n);
+  constexpr int KL = (DP + 31) / 32;
+  if (threadIdx.x == 0) sh.cut = first_cut<KF>();
+  __syncthreads();
+  double p[KL], W = 0.0;   // warp 0: the position
+#pragma unroll
+  for (int u = 0; u < KL; ++u) p[u] = lane + 32 * u < DP ? (double)sh.y[lane + 32 * u] : 0.0;
+  int iters = 0;
+  for (; iters < max_iter;) {
+    ev += (unsigned long long)seed_sums<DP, KF, double, NW>(Xs, cv, n, log2n, sh);
+    ++iters;
+    if (w == 0) {
+      W = sh.tot[0];
+      bool ok = W > 0.0 && isfinite(W);
+      double q[KL], step2 = 0.0;
+#pragma unroll
+      for (int u = 0; u < KL; ++u) {
+        const int k = lane + 32 * u;
+        const double dl = ok && k < d ? sh.tot[1 + k] / W - (p[u] - (double)sh.y[k]) : 0.0;
+        step2 += dl * dl;
+        q[u] = p[u] + dl;
+      }
+      if (ok && sphere_r > 0.0) {
+        double nn = 0.0;
+#pragma unroll
+        for (int u = 0; u < KL; ++u) nn += q[u] * q[u];
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
+        const double f = sphere_r / sqrt(nn);
+        step2 = 0.0;
+#pragma unroll
+        for (int u = 0; u < KL; ++u) {
+          q[u] *= f;
+          step2 += (q[u] - p[u]) * (q[u] - p[u]);
+        }
+        ok = nn > 0.0;
+      }
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
+      ok = ok && isfinite(step2);
+#pragma unroll
+      for (int u = 0; u < KL; ++u) {
+        const int k = lane + 32 * u;
+        if (ok) p[u] = q[u];
+        if (ok && k < DP) sh.y[k] = (float)q[u];
+      }
+      if (lane == 0) sh.flag = (!ok || step2 <= tol2_s) ? 1 : 0;
+      __syncwarp();
+    }
+    __syncthreads();
+    if (sh.flag) break;
+  }
+  if (w == 0) {
+#pragma unroll
+    for (int u = 0; u < KL; ++u) {
+      const int k = lane + 32 * u;
+      if (k < DP) {
+        ym[k] = p[u];
+        yf[k] = (float)p[u];
+      }
+    }
+    if (lane == 0) *mscore = W;
+  }
+  return iters;
+}
+
 template <int DP, int KF>
 __global__ void __launch_bounds__(kSeedWarps * 32)
     refine_seeds(const float* __restrict__ Xs, View<float> cv, int n, int d,
@@ -483,82 +675,42 @@ __global__ void __launch_bounds__(kSeedWarps * 32)
                  double* __restrict__ ym, float* __restrict__ yf, double* __restrict__ mscore,
                  double tol2_s, int max_iter, int32_t* iters_out, unsigned long long* evals,
                  double sphere_r) {
-  __shared__ __align__(16) SeedSmem<DP, double> sh;
+  __shared__ __align__(16) SeedSmem<DP, double, kSeedWarps> sh;
   const int M = *M_ptr;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const float log2n = log2f((float)n);
   unsigned long long ev = 0;
-  constexpr int KL = (DP + 31) / 32;
   for (int m = blockIdx.x; m < M; m += gridDim.x) {
     const int64_t src = kept[accepted[m]];
     __syncthreads();
     for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[src * DP + k];
-    if (threadIdx.x == 0) sh.cut = first_cut<KF>();
-    __syncthreads();
-    double p[KL], W = 0.0;   // warp 0: the position
-#pragma unroll
-    for (int u = 0; u < KL; ++u) p[u] = lane + 32 * u < DP ? (double)sh.y[lane + 32 * u] : 0.0;
-    int iters = 0;
-    for (; iters < max_iter;) {
-      ev += (unsigned long long)seed_sums<DP, KF, double>(Xs, cv, n, log2n, sh);
-      ++iters;
-      if (w == 0) {
-        W = sh.tot[0];
-        bool ok = W > 0.0 && isfinite(W);
-        double q[KL], step2 = 0.0;
-#pragma unroll
-        for (int u = 0; u < KL; ++u) {
-          const int k = lane + 32 * u;
-          const double dl = ok && k < d ? sh.tot[1 + k] / W - (p[u] - (double)sh.y[k]) : 0.0;
-          step2 += dl * dl;
-          q[u] = p[u] + dl;
-        }
-        if (ok && sphere_r > 0.0) {
-          double nn = 0.0;
-#pragma unroll
-          for (int u = 0; u < KL; ++u) nn += q[u] * q[u];
-#pragma unroll
-          for (int o = 16; o >= 1; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
-          const double f = sphere_r / sqrt(nn);
-          step2 = 0.0;
-#pragma unroll
-          for (int u = 0; u < KL; ++u) {
-            q[u] *= f;
-            step2 += (q[u] - p[u]) * (q[u] - p[u]);
-          }
-          ok = nn > 0.0;
-        }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) step2 += __shfl_xor_sync(kFull, step2, o);
-        ok = ok && isfinite(step2);
-#pragma unroll
-        for (int u = 0; u < KL; ++u) {
-          const int k = lane + 32 * u;
-          if (ok) p[u] = q[u];
-          if (ok && k < DP) sh.y[k] = (float)q[u];
-        }
-        if (lane == 0) sh.flag = (!ok || step2 <= tol2_s) ? 1 : 0;
-        __syncwarp();
-      }
-      __syncthreads();
-      if (sh.flag) break;
-    }
-    if (w == 0) {
-#pragma unroll
-      for (int u = 0; u < KL; ++u) {
-        const int k = lane + 32 * u;
-        if (k < DP) {
-          ym[(int64_t)m * DP + k] = p[u];
-          yf[(int64_t)m * DP + k] = (float)p[u];
-        }
-      }
-      if (lane == 0) {
-        mscore[m] = W;
-        atomicMax(iters_out, iters);
-      }
-    }
+    const int iters = refine_seed<DP, KF, kSeedWarps>(Xs, cv, n, d, ym + (int64_t)m * DP,
+                                                      yf + (int64_t)m * DP, mscore + m, tol2_s,
+                                                      max_iter, sphere_r, sh, ev);
+    if (threadIdx.x == 0) atomicMax(iters_out, iters);
   }
   if (threadIdx.x == 0 && ev) atomicAdd(evals, ev);
+}
+
+// The modes at the slots of the queue's list, from yf.
+template <int DP>
+__global__ void __launch_bounds__(kQueueWarps * 32)
+    refine_queue(const float* __restrict__ Xs, View<float> cv, int d, SeedQueue q, double* ym,
+                 float* yf, double* mscore, double tol2_s, int max_iter, int32_t* iters_out) {
+  __shared__ __align__(16) SeedSmem<DP, double, kQueueWarps> sh;
+  int b, at;
+  while (next_entry(q, &b, &at)) {
+    SetCtl* c = q.sc + b;
+    const int64_t s = q.list[c->p0 + at];
+    __syncthreads();
+    for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = yf[s * DP + k];
+    unsigned long long ev = 0;
+    const int iters = refine_seed<DP, kKernelGaussian, kQueueWarps>(
+        Xs + (int64_t)c->p0 * DP, set_view<DP>(cv, b), c->n, d, ym + s * DP, yf + s * DP,
+        mscore + s, tol2_s, max_iter, 0.0, sh, ev);
+    if (threadIdx.x == 0) {
+      atomicMax(iters_out, iters);
+      atomicAdd(reinterpret_cast<unsigned long long*>(&c->evals), ev);
+    }
+  }
 }
 
 int seed_grid(int max_seeds, int sms) {
@@ -685,6 +837,48 @@ cudaError_t launch_refine_seeds(const float* Xs, const View<float>& cv, int n, i
   }
 #undef FMS_SEEDS
   return cudaErrorInvalidValue;
+}
+
+#define FMS_BY_WIDTH(RUN)             \
+  switch (DP) {                       \
+    case 4: RUN(4); break;            \
+    case 8: RUN(8); break;            \
+    case 16: RUN(16); break;          \
+    case 32: RUN(32); break;          \
+    case 64: RUN(64); break;          \
+    default: return cudaErrorInvalidValue; \
+  }                                   \
+  return cudaGetLastError()
+
+cudaError_t launch_travel_queue(const float* Xs, const View<float>& cv, int d, int DP,
+                                const SeedQueue& q, float* y, int32_t* it, int32_t* conv,
+                                int32_t* state, float* wlast, int max_iter, float tol2_s, int sms,
+                                cudaStream_t st) {
+#define FMS_RUN(DP_)                                                                            \
+  travel_queue<DP_><<<sms * 8, kQueueWarps * 32, 0, st>>>(Xs, cv, d, q, y, it, conv, state, wlast, \
+                                                          max_iter, tol2_s)
+  FMS_BY_WIDTH(FMS_RUN);
+#undef FMS_RUN
+}
+
+cudaError_t launch_density_queue(const float* Xs, const View<float>& cv, int DP, const SeedQueue& q,
+                                 const float* y, float* score, double* mscore, int sms,
+                                 cudaStream_t st) {
+#define FMS_RUN(DP_) \
+  density_queue<DP_><<<sms * 8, kQueueWarps * 32, 0, st>>>(Xs, cv, q, y, score, mscore)
+  FMS_BY_WIDTH(FMS_RUN);
+#undef FMS_RUN
+}
+
+cudaError_t launch_refine_queue(const float* Xs, const View<float>& cv, int d, int DP,
+                                const SeedQueue& q, double* ym, float* yf, double* mscore,
+                                double tol2_s, int max_iter, int32_t* iters_out, int sms,
+                                cudaStream_t st) {
+#define FMS_RUN(DP_)                                                                           \
+  refine_queue<DP_><<<sms * 8, kQueueWarps * 32, 0, st>>>(Xs, cv, d, q, ym, yf, mscore, tol2_s, \
+                                                          max_iter, iters_out)
+  FMS_BY_WIDTH(FMS_RUN);
+#undef FMS_RUN
 }
 
 }  // namespace fms

@@ -96,3 +96,22 @@ def test_every_point_a_seed(d, n, kw):
                                h=2.0 if "kernel" not in kw else 6.0)
         w["X"] = np.concatenate([w.X, w.X[: n - len(w.X)] + 0.01]).astype(np.float32)
     _cluster(w, all_seeds=True, **kw)
+
+
+# d > 7: sets below and above the mean size from which they are sorted (512), sets of
+# one chunk, one row more and several chunks of the sort (1,024 rows), unconverged
+# seeds kept (gamma = 1)
+@pytest.mark.parametrize("d,per,kw", [(8, (100, 60, 128), {}), (16, (256, 205, 700), {}),
+                                      (33, (256, 341, 200), {}), (9, (300, 120, 205), dict(gamma=1.0))])
+def test_batched_queue(d, per, kw):
+    h = 2.5
+    sets = [fi.separated_blobs(seed=7 * d + i, k=4 + (i > 0), d=d, per=p, sigma=0.8, h=h)
+            for i, p in enumerate(per)]
+    X = [torch.from_numpy(w.X).cuda() for w in sets]
+    res = fms.cluster_batched(X, h, 1e-3 * h, 300, rng_seed=3, max_modes=64, **kw)
+    off = np.concatenate([[0], np.cumsum([w.X.shape[0] for w in sets])])
+    for b, w in enumerate(sets):
+        ref = orc.cluster(w.X, h, 1e-3 * h, 300, rng_seed=3, **kw)
+        cmp = compare_clustering(res.modes[b].cpu().numpy(),
+                                 res.labels[off[b]:off[b + 1]].cpu().numpy(), ref, h)
+        assert cmp["mode_ok"] and cmp["label_mismatch"] == 0, (b, cmp)
