@@ -1533,29 +1533,120 @@ namespace {
 struct CoarseLayout {
   size_t off_Xs, off_img, off_Ys, off_active, off_part, off_ctl, off_status, total;
   int DP, DA, C, Lc, grid;
+  // P > 0: points and seeds in cells, tiles of up to 128 rows of one cell
+  int P, tiles, seed_tiles;
+  size_t off_Xc, off_Yc, off_xperm, off_yperm, off_start, off_ystart, off_ctr, off_npiv, off_rad,
+      off_xtable, off_xcell, off_ytable, off_list, off_count, off_outrow, off_sort;
 };
+
+// Sorting takes ~120 us; the dense step takes that from about 3e8 pairs on.
+// (The list of visible tiles takes 4 bytes a pair of tiles: up to 1 GB.)
+bool coarse_by_cells(int64_t n, int64_t m) {
+  const double pairs = (double)n * (double)m;
+  return n >= 4096 && m >= 512 && pairs >= 6e8 && pairs <= 4e12;
+}
 
 CoarseLayout coarse_layout(int64_t n, int d, int64_t m) {
   CoarseLayout L{};
   L.DP = padded_dim(d);
   L.DA = L.DP + 4;
   L.grid = tc_grid(d);
-  tc_choose_chunks(n, (int32_t)m, L.grid, &L.C, &L.Lc);
+  L.P = coarse_by_cells(n, m) ? cells::choose_cells(n, m) : 0;
   size_t o = 0;
   auto take = [&](size_t bytes) {
     const size_t at_ = o;
     o += align256(bytes > 0 ? bytes : 1);
     return at_;
   };
+  int64_t places = m;
+  if (L.P > 0) {
+    L.tiles = cells::group_cap(n, L.P, kTcTile);
+    L.seed_tiles = cells::group_cap(m, L.P, kTcTile);
+    places = (int64_t)L.seed_tiles * kTcTile;
+    // about 4 tasks to a CTA
+    L.C = (4 * L.grid + L.seed_tiles - 1) / L.seed_tiles;
+    L.Lc = kTcTile;
+  } else {
+    tc_choose_chunks(n, (int32_t)m, L.grid, &L.C, &L.Lc);
+  }
   L.off_Xs = take((size_t)n * L.DP * 4);
-  L.off_img = take(tc_image_bytes(n, d));
+  L.off_img = take(L.P > 0 ? tc_tile_images(L.tiles, d) : tc_image_bytes(n, d));
   L.off_Ys = take((size_t)m * L.DP * 4);
-  L.off_active = take((size_t)m * 4);
-  L.off_part = take((size_t)L.C * (size_t)m * L.DA * 4);
+  L.off_active = take((size_t)places * 4);
+  L.off_part = take((size_t)L.C * (size_t)places * L.DA * 4);
   L.off_ctl = take(sizeof(IterCtl));
   L.off_status = take(64);
+  if (L.P > 0) {
+    L.off_Xc = take((size_t)n * L.DP * 4);
+    L.off_Yc = take((size_t)m * L.DP * 4);
+    L.off_xperm = take((size_t)n * 4);
+    L.off_yperm = take((size_t)m * 4);
+    L.off_start = take((size_t)(L.P + 1) * 4);
+    L.off_ystart = take((size_t)(L.P + 1) * 4);
+    L.off_ctr = take((size_t)L.P * L.DP * 4);
+    L.off_npiv = take(4);
+    L.off_rad = take((size_t)L.P * 4);
+    L.off_xtable = take((size_t)L.tiles * 8);
+    L.off_xcell = take((size_t)L.tiles * 4);
+    L.off_ytable = take((size_t)L.seed_tiles * 8);
+    L.off_list = take((size_t)L.seed_tiles * L.tiles * 4);
+    L.off_count = take((size_t)L.seed_tiles * 4);
+    L.off_outrow = take((size_t)places * 4);
+    const size_t a = cells::sort_scratch(1, n, L.P).total, b = cells::sort_scratch(1, m, L.P).total;
+    L.off_sort = take(a > b ? a : b);
+  }
   L.total = o;
   return L;
+}
+
+// The coarse step over cells: only the tile pairs that can have a nonzero weight.
+cudaError_t coarse_cells(const CoarseLayout& L, void* ws, int64_t n, int d, int64_t m,
+                         const float* seeds, double inv_scale, float* out_seeds, float* out_wsum,
+                         cudaStream_t st) {
+  float* Xc = at<float>(ws, L.off_Xc);
+  float* Yc = at<float>(ws, L.off_Yc);
+  unsigned char* img = at<unsigned char>(ws, L.off_img);
+  int32_t* active = at<int32_t>(ws, L.off_active);
+  int32_t* list = at<int32_t>(ws, L.off_list);
+  int32_t* count = at<int32_t>(ws, L.off_count);
+  int32_t* out_row = at<int32_t>(ws, L.off_outrow);
+  int32_t* yperm = at<int32_t>(ws, L.off_yperm);
+  int2* xtable = at<int2>(ws, L.off_xtable);
+  int2* ytable = at<int2>(ws, L.off_ytable);
+  int32_t* xcell = at<int32_t>(ws, L.off_xcell);
+  float* ctr = at<float>(ws, L.off_ctr);
+  int32_t* npiv = at<int32_t>(ws, L.off_npiv);
+  float* part = at<float>(ws, L.off_part);
+  IterCtl* ctl = at<IterCtl>(ws, L.off_ctl);
+  uint32_t* status = at<uint32_t>(ws, L.off_status);
+  void* scratch = at<void>(ws, L.off_sort);
+  const int places = L.seed_tiles * kTcTile;
+  cells::View<float> cv{};
+  cv.P = L.P;
+  cv.start = at<int32_t>(ws, L.off_start);
+  cv.ctr = ctr;
+  cv.rad = at<float>(ws, L.off_rad);
+  cudaError_t e = cells::launch_sort<float>(
+      at<float>(ws, L.off_Xs), 1, n, L.DP, true, L.P, scratch, Xc, at<int32_t>(ws, L.off_xperm),
+      at<int32_t>(ws, L.off_start), ctr, npiv, at<float>(ws, L.off_rad), xtable, st, nullptr, 0,
+      kTcTile, xcell);
+  if (e == cudaSuccess)
+    e = cells::launch_sort<float>(at<float>(ws, L.off_Ys), 1, m, L.DP, false, L.P, scratch, Yc,
+                                  yperm, at<int32_t>(ws, L.off_ystart), ctr, npiv, nullptr, ytable,
+                                  st, nullptr, 0, kTcTile);
+  if (e == cudaSuccess)
+    e = launch_tc_pack_table(Xc, n, d, L.DP, xtable, L.tiles, img, st);
+  if (e == cudaSuccess) e = launch_step_setup(active, places, ctl, L.C, L.Lc, st);
+  if (e == cudaSuccess)
+    e = launch_tc_visible(Yc, L.DP, ytable, L.seed_tiles, yperm, cv, xtable, xcell, L.tiles, list,
+                          count, active, out_row, st);
+  if (e == cudaSuccess)
+    e = launch_ms_step_tc(img, n, d, L.DP, L.DA, Yc, active, &ctl->s, &ctl->s, &ctl->C, &ctl->Lc,
+                          part, status, st, nullptr, TcTiles{list, count, L.tiles});
+  if (e == cudaSuccess)
+    e = launch_step_finish(part, ctl, seeds, d, L.DA, inv_scale, out_seeds, out_wsum, places, st,
+                           out_row);
+  return e;
 }
 }  // namespace
 
@@ -1597,13 +1688,17 @@ fms_status fms_mean_shift_step_coarse(const float* points, int64_t n, int32_t d,
     uint32_t* status = at<uint32_t>(ws, L.off_status);
     FMS_CUDA(cudaMemsetAsync(status, 0, 64, st));
     FMS_CUDA(launch_pack_points(points, n, d, L.DP, (float)scale, Xs, status, st));
-    FMS_CUDA(launch_tc_pack(Xs, n, d, L.DP, img, st));
     FMS_CUDA(launch_pack_points(seeds, m, d, L.DP, (float)scale, Ys, status, st));
-    FMS_CUDA(launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, st));
-    FMS_CUDA(launch_ms_step_tc(img, n, d, L.DP, L.DA, Ys, active, &ctl->s, &ctl->s, &ctl->C,
-                               &ctl->Lc, part, status, st));
-    FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,
-                                (int)m, st));
+    if (L.P > 0) {
+      FMS_CUDA(coarse_cells(L, ws, n, d, m, seeds, 1.0 / scale, out_seeds, out_wsum, st));
+    } else {
+      FMS_CUDA(launch_tc_pack(Xs, n, d, L.DP, img, st));
+      FMS_CUDA(launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, st));
+      FMS_CUDA(launch_ms_step_tc(img, n, d, L.DP, L.DA, Ys, active, &ctl->s, &ctl->s, &ctl->C,
+                                 &ctl->Lc, part, status, st));
+      FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,
+                                  (int)m, st));
+    }
     if (owns) {
       FMS_CUDA(cudaMemcpyAsync(&hstatus, status, 4, cudaMemcpyDeviceToHost, st));
       FMS_CUDA(cudaStreamSynchronize(st));

@@ -193,7 +193,9 @@ inline int choose_cells(int64_t n, int64_t m) {
 }
 
 inline int64_t sort_blocks(int64_t rows) { return (rows + kChunkRows - 1) / kChunkRows; }
-inline int group_cap(int64_t rows, int P) { return (int)((rows + 31) / 32) + P; }
+inline int group_cap(int64_t rows, int P, int size = 32) {
+  return (int)((rows + size - 1) / size) + P;
+}
 
 // Scratch of one sort of B sets of `rows` rows: cell ids, block counts, farthest rows.
 struct SortScratch {
@@ -216,12 +218,14 @@ inline SortScratch sort_scratch(int64_t B, int64_t rows, int P, int64_t total = 
 // (sorted rows), start [B][P + 1] and, where non-null, perm (sorted position -> row
 // of the set) and the table of groups [B][group_cap(nrows, P)].  Sets of different
 // sizes: set b has the rows [offs[b], offs[b + 1]) of `total` (offs on the device),
-// nrows is the largest, and there is no table.
+// nrows is the largest, and there is no table.  The groups of the table hold up to
+// `group` rows, group_cell (nullable) is the cell of each.
 template <typename T>
 cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
                         int32_t* npiv, T* rad, int2* table, cudaStream_t st,
-                        const int64_t* offs = nullptr, int64_t total = 0);
+                        const int64_t* offs = nullptr, int64_t total = 0, int group = 32,
+                        int32_t* group_cell = nullptr);
 
 // The extents of the P cells of one sorted set towards each other's centres
 // (View::ext), for d > 8.
@@ -229,6 +233,16 @@ cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* star
                            const float* ctr, float2* ext, cudaStream_t st);
 
 }  // namespace cells
+
+// ---- k_step_tc.cu: tiles of one cell each (up to 128 rows)
+size_t tc_tile_images(int64_t tiles, int d);
+cudaError_t launch_tc_pack_table(const float* Xs, int64_t n, int d, int DP, const int2* table,
+                                 int tiles, unsigned char* img, cudaStream_t st);
+cudaError_t launch_tc_visible(const float* Ys, int DP, const int2* seed_table, int seed_tiles,
+                              const int32_t* yperm, const cells::View<float>& cv,
+                              const int2* tile_table, const int32_t* tile_cell, int tiles,
+                              int32_t* list, int32_t* count, int32_t* active, int32_t* out_row,
+                              cudaStream_t st);
 
 // ---- k_travel.cu: whole trajectories in one launch (rows of DP floats, scaled)
 

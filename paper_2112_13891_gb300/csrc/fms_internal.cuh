@@ -351,9 +351,10 @@ cudaError_t launch_update(const float* part, int32_t* active, IterCtl* ctl, floa
                           float* wlast = nullptr);  // sum w of each seed's last update
 cudaError_t launch_step_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t C, int32_t Lc,
                               cudaStream_t st);
+// out_row (nullable): the caller's row of each active position, -1 for none
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,
-                               int m, cudaStream_t st);
+                               int m, cudaStream_t st, const int32_t* out_row = nullptr);
 
 // k_round.cu
 cudaError_t launch_ms_round(const float* Xs, int64_t n, int d, float* y, int32_t* it,
@@ -514,6 +515,13 @@ inline StepLayout step_layout(int64_t n, int d, int64_t m, int sms) {
 // handles active positions [0, *count_ptr) of a list whose partials have the
 // stride *s_total_ptr, with chunks of *Lc_ptr (a multiple of 128) points.
 constexpr int kTcMaxDim = 32;
+// Point tiles that each tile of 128 active positions visits (count null: all of
+// them, in order): count[s] of list[s stride ..].
+struct TcTiles {
+  const int32_t* list;
+  const int32_t* count;
+  int stride;
+};
 size_t tc_image_bytes(int64_t n, int d);
 cudaError_t launch_tc_pack(const float* Xs, int64_t n, int d, int DP, unsigned char* img,
                            cudaStream_t st);
@@ -522,7 +530,7 @@ cudaError_t launch_ms_step_tc(const unsigned char* img, int64_t n, int d, int DP
                               const float* y, const int32_t* active, const int32_t* s_total_ptr,
                               const int32_t* count_ptr, const int32_t* C_ptr,
                               const int32_t* Lc_ptr, float* part, uint32_t* status,
-                              cudaStream_t st, int32_t* s_log = nullptr);
+                              cudaStream_t st, int32_t* s_log = nullptr, TcTiles tl = TcTiles{});
 
 // k_merge.cu
 cudaError_t launch_kept_list(const IterCtl* ctl, const int32_t* state, const int32_t* conv,

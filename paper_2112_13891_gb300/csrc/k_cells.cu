@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256)
                    int P,
                    const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
                    T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
-                   int2* __restrict__ table, int cap) {
+                   int2* __restrict__ table, int cap, int gsz, int32_t* __restrict__ gcell) {
   constexpr int WARPS = 8, ITER = kChunkRows / (WARPS * 32);
   __shared__ int wcnt[WARPS][kMaxCells];
   __shared__ int base[kMaxCells];
@@ -312,11 +312,14 @@ __global__ void __launch_bounds__(256)
     if ((int)threadIdx.x < P) so[threadIdx.x] = first;
     if (threadIdx.x == 0) so[P] = nrows;
     if (table) {
-      const int ng = (int)threadIdx.x < P ? (tot + 31) / 32 : 0;
+      const int ng = (int)threadIdx.x < P ? (tot + gsz - 1) / gsz : 0;
       int gall = 0;
       const int g0 = block_exclusive_scan(ng, &gall, scan);
       int2* to = table + (int64_t)b * cap;
-      for (int g = 0; g < ng; ++g) to[g0 + g] = make_int2(first + 32 * g, min(32, tot - 32 * g));
+      for (int g = 0; g < ng; ++g) {
+        to[g0 + g] = make_int2(first + gsz * g, min(gsz, tot - gsz * g));
+        if (gcell) gcell[(int64_t)b * cap + g0 + g] = threadIdx.x;
+      }
       for (int g = gall + threadIdx.x; g < cap; g += blockDim.x) to[g] = make_int2(0, 0);
     }
   }
@@ -426,7 +429,7 @@ cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* star
 template <typename T, int DP>
 static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrows, bool points, int P,
                           int64_t total, void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr, int32_t* npiv, T* rad,
-                          int2* table, cudaStream_t st) {
+                          int2* table, int group, int32_t* gcell, cudaStream_t st) {
   const SortScratch sc = sort_scratch(B, nrows, P, total);
   unsigned char* base = static_cast<unsigned char*>(scratch);
   unsigned char* id = base + sc.id;
@@ -458,7 +461,7 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
                                                        ctr, npiv);
   }
   scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, (int)nrows, per, P, id, counts, dst, perm, start,
-                                             table, group_cap(nrows, P));
+                                             table, group_cap(nrows, P, group), group, gcell);
   if (points)
     bound_kernel<T, DP><<<(unsigned)(P * B), 128, 0, st>>>(dst, offs, (int)nrows, P, start,
                                                                         ctr, rad);
@@ -469,27 +472,27 @@ template <typename T>
 cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
                         int32_t* npiv, T* rad, int2* table, cudaStream_t st, const int64_t* offs,
-                        int64_t total) {
+                        int64_t total, int group, int32_t* gcell) {
   if (total == 0) total = (int64_t)B * nrows;
   if (P < 32 || P > kMaxCells || (P & 31) || B < 1) return cudaErrorInvalidValue;
   switch (DP) {
-    case 4: return sort_t<T, 4>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
-    case 8: return sort_t<T, 8>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
-    case 16: return sort_t<T, 16>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
-    case 32: return sort_t<T, 32>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+    case 4: return sort_t<T, 4>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
+    case 8: return sort_t<T, 8>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
+    case 16: return sort_t<T, 16>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
+    case 32: return sort_t<T, 32>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
     case 64:
       if constexpr (sizeof(T) == 4)
-        return sort_t<T, 64>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, st);
+        return sort_t<T, 64>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
   }
   return cudaErrorInvalidValue;
 }
 
 template cudaError_t launch_sort<float>(const float*, int, int64_t, int, bool, int, void*, float*,
                                         int32_t*, int32_t*, float*, int32_t*, float*, int2*,
-                                        cudaStream_t, const int64_t*, int64_t);
+                                        cudaStream_t, const int64_t*, int64_t, int, int32_t*);
 template cudaError_t launch_sort<double>(const double*, int, int64_t, int, bool, int, void*,
                                          double*, int32_t*, int32_t*, double*, int32_t*, double*,
-                                         int2*, cudaStream_t, const int64_t*, int64_t);
+                                         int2*, cudaStream_t, const int64_t*, int64_t, int, int32_t*);
 
 }  // namespace cells
 }  // namespace fms

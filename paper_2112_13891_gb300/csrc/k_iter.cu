@@ -613,11 +613,14 @@ cudaError_t launch_step_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t 
 // out_seeds[i] = seeds[i] + (S_i / W_i) / scale (original units), out_wsum[i] = W_i.
 __global__ void step_finish_kernel(const float* __restrict__ part, const IterCtl* __restrict__ ctl,
                                    const float* __restrict__ seeds, int d, int DA, double inv_scale,
-                                   float* __restrict__ out_seeds, float* __restrict__ out_wsum) {
+                                   float* __restrict__ out_seeds, float* __restrict__ out_wsum,
+                                   const int32_t* __restrict__ out_row) {
   const int s = ctl->s, C = ctl->C;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
   for (int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < s; p += nw) {
+    const int64_t i = out_row ? out_row[p] : p;
+    if (i < 0) continue;   // (the same for the whole warp)
     float a[3] = {0.f, 0.f, 0.f};
     reduce_chunks(part, s, p, C, DA, d, lane, a);
     const float W = __shfl_sync(kFull, a[0], 0);
@@ -626,27 +629,27 @@ __global__ void step_finish_kernel(const float* __restrict__ part, const IterCtl
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
       const int k = lane + 32 * u;
-      v[u] = (k >= 1 && k <= d) ? seeds[(int64_t)p * d + (k - 1)] : 0.0f;
+      v[u] = (k >= 1 && k <= d) ? seeds[i * d + (k - 1)] : 0.0f;
     }
     __syncwarp();
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
       const int k = lane + 32 * u;
       if (k >= 1 && k <= d)
-        out_seeds[(int64_t)p * d + (k - 1)] = (float)((double)v[u] + (double)(a[u] / W) * inv_scale);
+        out_seeds[i * d + (k - 1)] = (float)((double)v[u] + (double)(a[u] / W) * inv_scale);
     }
-    if (lane == 0 && out_wsum) out_wsum[p] = W;
+    if (lane == 0 && out_wsum) out_wsum[i] = W;
   }
 }
 
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,
-                               int m, cudaStream_t st) {
+                               int m, cudaStream_t st, const int32_t* out_row) {
   int blocks = (m + 7) / 8;
   if (blocks < 1) blocks = 1;
   if (blocks > 4096) blocks = 4096;
   step_finish_kernel<<<blocks, 256, 0, st>>>(part, ctl, seeds, d, DA, inv_scale, out_seeds,
-                                             out_wsum);
+                                             out_wsum, out_row);
   return cudaGetLastError();
 }
 

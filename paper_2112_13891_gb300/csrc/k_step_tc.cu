@@ -33,7 +33,7 @@
 // an error bit instead of hanging.
 #include <cuda_bf16.h>
 
-#include "fms_internal.cuh"
+#include "fms_cells.cuh"
 #include "fms_tc.cuh"
 
 namespace fms {
@@ -64,28 +64,32 @@ struct Geo {
 };
 }  // namespace tc
 
-// Tile images of the scaled points Xs [n][DP] (DP >= d, zero padded).
+// Tile images of the scaled points Xs [n][DP] (DP >= d, zero padded); with a
+// table, tile t holds the rows table[t] = (first, count <= 128).
 template <int DPAD>
 __global__ void tc_pack_tiles(const float* __restrict__ Xs, int n, int DP,
-                              unsigned char* __restrict__ img) {
+                              unsigned char* __restrict__ img, const int2* __restrict__ table) {
   using G = tc::Geo<DPAD>;
   const int t = blockIdx.x;
+  const int first = table ? table[t].x : t * tc::kP;
+  const int rows = table ? table[t].y : min(tc::kP, n - first);
+  if (rows <= 0) return;
   unsigned char* base = img + (size_t)t * G::kTileBytes;
   __nv_bfloat16* x2 = reinterpret_cast<__nv_bfloat16*>(base);
   for (int e = threadIdx.x; e < tc::kP * DPAD; e += blockDim.x) {
     const int p = e / DPAD, k = e % DPAD;
-    const int j = t * tc::kP + p;
-    const float v = (j < n && k < DP) ? Xs[(size_t)j * DP + k] : 0.f;
+    const int j = first + p;
+    const float v = (p < rows && k < DP) ? Xs[(size_t)j * DP + k] : 0.f;
     const __nv_bfloat16 hi = __float2bfloat16_rn(v);
     const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
     x2[tc::core_index(p, k, G::N2)] = hi;
     x2[tc::core_index(p, DPAD + k, G::N2)] = lo;
   }
   for (int e = threadIdx.x; e < tc::kP; e += blockDim.x) {
-    const int j = t * tc::kP + e;
+    const int j = first + e;
     // e0 + e1 + e2 = -||x||^2 / 2 (FP32 norm, split into three BF16 pieces)
     float e0 = -INFINITY, e1 = 0.f, e2 = 0.f;
-    if (j < n) {
+    if (e < rows) {
       float s = 0.f;
       for (int k = 0; k < DP; ++k) {
         const float v = Xs[(size_t)j * DP + k];
@@ -138,7 +142,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
                int DA, const int32_t* __restrict__ active, const int32_t* __restrict__ s_total_ptr,
                const int32_t* __restrict__ count_ptr, const int32_t* __restrict__ C_ptr,
                const int32_t* __restrict__ Lc_ptr, float* __restrict__ part, uint32_t* status,
-               int32_t* __restrict__ s_log) {
+               int32_t* __restrict__ s_log, TcTiles tl) {
   using G = tc::Geo<DPAD>;
   constexpr int S = G::kStages;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -201,6 +205,18 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
   const uint32_t tD2 = tmem + G::kD2;                  // D1[i] = tmem + 128 i, i < 3
   const int tiles_per_chunk = Lc / tc::kP;
   const int ntiles_total = (n + tc::kP - 1) / tc::kP;
+  // tiles of (seed tile, chunk): first place and count, in the order of the points
+  // or of the seed tile's list
+  auto span = [&](long task, int* t0) -> int {
+    const int c = (int)(task / ntile_seed);
+    int per = tiles_per_chunk, all = ntiles_total;
+    if (tl.count) {
+      all = tl.count[task % ntile_seed];
+      per = (all + C - 1) / C;
+    }
+    *t0 = c * per;
+    return max(0, min(all, *t0 + per) - *t0);
+  };
   bool bad = false;
   const bool issuer = warp >= kCtl;
   auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
@@ -261,15 +277,16 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
       };
       uint32_t g0 = 0;                                 // global number of the task's tile 0
       for (long task = blockIdx.x; task < T && !s_abort; task += gridDim.x) {
-        const int c = (int)(task / ntile_seed);
-        const int t0 = c * tiles_per_chunk;
-        const int nt = max(0, min(ntiles_total, t0 + tiles_per_chunk) - t0);
+        int t0;
+        const int nt = span(task, &t0);
         if (nt == 0) continue;                         // (no handshake for an empty task)
+        const int32_t* list = tl.count ? tl.list + (task % ntile_seed) * (long)tl.stride : nullptr;
+        auto tile = [&](int i) { return list ? __ldg(list + i) : i; };
         if (!wait(&bar_y, n_task & 1u)) break;         // Y tile written, last D2 read
         ++n_task;
         tc::fence_after();
         const uint32_t base = n_load;                  // load number of tile 0 (== g0)
-        for (int i = 0; i < nt && i < S; ++i) issue_load(t0 + i);
+        for (int i = 0; i < nt && i < S; ++i) issue_load(tile(t0 + i));
         if (!wait_load(base)) break;
         issue_s(base % S);
         if (nt > 1) {
@@ -280,7 +297,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
           const uint32_t g = g0 + (uint32_t)j;
           if (j >= 1 && j - 1 + S < nt) {              // refill the buffer of tile j-1
             if (!wait(&bar_o[(g - 1) % 3u], ((g - 1) / 3u) & 1u)) break;  // P(j-1) read it
-            issue_load(t0 + j - 1 + S);
+            issue_load(tile(t0 + j - 1 + S));
           }
           if (j + 2 < nt) {                            // S(j+2) into the accumulator
             if (j >= 1 && !wait(&bar_p[(g - 1) % 3u], ((g - 1) / 3u) & 1u)) break;
@@ -307,9 +324,8 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
       const uint32_t a_sbo = (tc::kP / 8) * 128;
       uint32_t n_o = 0;
       for (long task = blockIdx.x; task < T && !s_abort; task += gridDim.x) {
-        const int c = (int)(task / ntile_seed);
-        const int t0 = c * tiles_per_chunk;
-        const int nt = max(0, min(ntiles_total, t0 + tiles_per_chunk) - t0);
+        int t0;
+        const int nt = span(task, &t0);
         for (int j = 0; j < nt; ++j) {
           if (!wait(&bar_p[n_o % 3u], (n_o / 3u) & 1u)) break;  // epilogue of tile j done
           tc::fence_after();
@@ -341,8 +357,8 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
     for (long task = blockIdx.x; task < T && !s_abort; task += gridDim.x) {
       const int st = (int)(task % ntile_seed);
       const int c = (int)(task / ntile_seed);
-      const int t0 = c * tiles_per_chunk;
-      const int nt = max(0, min(ntiles_total, t0 + tiles_per_chunk) - t0);
+      int t0;
+      const int nt = span(task, &t0);
       const int prow = st * tc::kM + r_row;
       const bool valid = prow < count;
       if (nt == 0) {                                   // (no handshake for an empty task)
@@ -478,8 +494,123 @@ size_t tc_image_bytes(int64_t n, int d) {
 cudaError_t launch_tc_pack(const float* Xs, int64_t n, int d, int DP, unsigned char* img,
                            cudaStream_t st) {
   const int tiles = (int)((n + tc::kP - 1) / tc::kP);
-  if (d <= 16) tc_pack_tiles<16><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img);
-  else tc_pack_tiles<32><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img);
+  if (d <= 16) tc_pack_tiles<16><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, nullptr);
+  else tc_pack_tiles<32><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, nullptr);
+  return cudaGetLastError();
+}
+
+// Bytes of `tiles` tile images.
+size_t tc_tile_images(int64_t tiles, int d) {
+  return (size_t)tiles * (d <= 16 ? tc::Geo<16>::kTileBytes : tc::Geo<32>::kTileBytes);
+}
+
+cudaError_t launch_tc_pack_table(const float* Xs, int64_t n, int d, int DP, const int2* table,
+                                 int tiles, unsigned char* img, cudaStream_t st) {
+  if (d <= 16) tc_pack_tiles<16><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, table);
+  else tc_pack_tiles<32><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, table);
+  return cudaGetLastError();
+}
+
+// The point tiles that a tile of up to 128 seeds (one block) can see: those of
+// cells whose ball comes within the distance from which every weight is exactly
+// zero in FP32 of the ball around the seeds.  Also the tile's places in the list of
+// seeds (a place past its rows repeats the last seed, out_row -1).
+template <int DP>
+__global__ void __launch_bounds__(128)
+    tc_visible(const float* __restrict__ Ys, const int2* __restrict__ seed_table,
+               const int32_t* __restrict__ yperm, cells::View<float> cv,
+               const int2* __restrict__ tile_table, const int32_t* __restrict__ tile_cell,
+               int tiles, int32_t* __restrict__ list, int32_t* __restrict__ count,
+               int32_t* __restrict__ active, int32_t* __restrict__ out_row) {
+  __shared__ float red[4][DP + 1];
+  __shared__ float ball[DP + 1];
+  __shared__ unsigned char sees[cells::kMaxCells];
+  __shared__ int scan[64];
+  const int st = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int2 g = seed_table[st];
+  const int place = st * 128 + threadIdx.x;
+  if (g.y <= 0) {
+    active[place] = 0;
+    out_row[place] = -1;
+    if (threadIdx.x == 0) count[st] = 0;
+    return;
+  }
+  const int row = g.x + min((int)threadIdx.x, g.y - 1);
+  active[place] = row;
+  out_row[place] = (int)threadIdx.x < g.y ? yperm[row] : -1;
+  float y[DP], r2 = 0.0f, far2 = 0.0f;
+#pragma unroll
+  for (int k = 0; k < DP; ++k) y[k] = Ys[(int64_t)row * DP + k];
+#pragma unroll
+  for (int k = 0; k < DP; ++k) {
+    float v = y[k];
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    if (lane == 0) red[w][k] = v;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < DP; k += blockDim.x)
+    ball[k] = (red[0][k] + red[1][k] + red[2][k] + red[3][k]) * (1.0f / 128);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < DP; ++k) {
+    r2 += (y[k] - ball[k]) * (y[k] - ball[k]);
+    far2 += y[k] * y[k];
+  }
+  r2 = cells::warp_max(r2);
+  far2 = cells::warp_max(far2);
+  __syncthreads();
+  if (lane == 0) {
+    red[w][0] = r2;
+    red[w][1] = far2;
+  }
+  __syncthreads();
+  const float rho = sqrtf(cells::warp_max(red[lane & 3][0]));
+  const float ny = cells::warp_max(red[lane & 3][1]);
+  for (int p = threadIdx.x; p < cv.P; p += blockDim.x) {
+    float d2 = 0.0f, nc = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      const float c = cv.ctr[(int64_t)p * DP + k];
+      d2 += (c - ball[k]) * (c - ball[k]);
+      nc += c * c;
+    }
+    // the split cross term and FP32 norms are off by under 2^-13 (|x|^2 + |y|^2) in the
+    // exponent
+    const float nx = sqrtf(nc) + cv.rad[p];
+    const float bits = cells::zero_bits<float>() + (ny + nx * nx) * (1.0f / 8192);
+    const float lim = (rho + cv.rad[p] + sqrtf(bits)) * 1.0001f;
+    sees[p] = cv.start[p + 1] > cv.start[p] && !(d2 > lim * lim) ? 1 : 0;
+  }
+  __syncthreads();
+  int n = 0;
+  for (int t0 = 0; t0 < tiles; t0 += blockDim.x) {
+    const int t = t0 + threadIdx.x;
+    const int take = t < tiles && tile_table[t].y > 0 && sees[tile_cell[t]] ? 1 : 0;
+    int tot;
+    const int at = block_exclusive_scan(take, &tot, scan);
+    if (take) list[(int64_t)st * tiles + n + at] = t;
+    n += tot;
+  }
+  if (threadIdx.x == 0) count[st] = n;
+}
+
+cudaError_t launch_tc_visible(const float* Ys, int DP, const int2* seed_table, int seed_tiles,
+                              const int32_t* yperm, const cells::View<float>& cv,
+                              const int2* tile_table, const int32_t* tile_cell, int tiles,
+                              int32_t* list, int32_t* count, int32_t* active, int32_t* out_row,
+                              cudaStream_t st) {
+#define FMS_VIS(DP_)                                                                             \
+  tc_visible<DP_><<<seed_tiles, 128, 0, st>>>(Ys, seed_table, yperm, cv, tile_table, tile_cell, \
+                                              tiles, list, count, active, out_row)
+  switch (DP) {
+    case 4: FMS_VIS(4); break;
+    case 8: FMS_VIS(8); break;
+    case 16: FMS_VIS(16); break;
+    case 32: FMS_VIS(32); break;
+    default: return cudaErrorInvalidValue;
+  }
+#undef FMS_VIS
   return cudaGetLastError();
 }
 
@@ -508,17 +639,17 @@ cudaError_t launch_ms_step_tc(const unsigned char* img, int64_t n, int d, int DP
                               const float* y, const int32_t* active, const int32_t* s_total_ptr,
                               const int32_t* count_ptr, const int32_t* C_ptr,
                               const int32_t* Lc_ptr, float* part, uint32_t* status,
-                              cudaStream_t st, int32_t* s_log) {
+                              cudaStream_t st, int32_t* s_log, TcTiles tl) {
   if (d < 1 || d > kTcMaxDim || DP < d || DA < DP + 1) return cudaErrorInvalidValue;
   const int grid = tc_grid(d);
   if (d <= 16)
     ms_step_tc<16><<<grid, tc::kThreads, tc::Geo<16>::kSmem, st>>>(
         img, (int)n, y, DP, DA, active, s_total_ptr, count_ptr, C_ptr, Lc_ptr, part, status,
-        s_log);
+        s_log, tl);
   else
     ms_step_tc<32><<<grid, tc::kThreads, tc::Geo<32>::kSmem, st>>>(
         img, (int)n, y, DP, DA, active, s_total_ptr, count_ptr, C_ptr, Lc_ptr, part, status,
-        s_log);
+        s_log, tl);
   return cudaGetLastError();
 }
 

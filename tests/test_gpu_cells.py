@@ -115,3 +115,24 @@ def test_batched_queue(d, per, kw):
         cmp = compare_clustering(res.modes[b].cpu().numpy(),
                                  res.labels[off[b]:off[b + 1]].cpu().numpy(), ref, h)
         assert cmp["mode_ok"] and cmp["label_mismatch"] == 0, (b, cmp)
+
+
+# the tensor-core step from 6e8 pairs on: tiles of one cell, tile pairs out of reach
+# skipped.  The bound is the BF16 one of test_gpu_coarse_step.
+@pytest.mark.parametrize("n,m,d,box,h", [(24_577, 24_500, 9, 60.0, 2.5), (49_000, 12_300, 16, 50.0, 2.5),
+                                         (600_001, 1_001, 3, 100.0, 3.0), (24_600, 24_601, 32, 3.0, 2.0)])
+def test_coarse_step_by_cells(n, m, d, box, h):
+    from test_gpu_coarse_step import _bound
+    X = _blobs(n + d, n, d, 12, box, 1.0)
+    rng = np.random.default_rng(2)
+    Y = (X[rng.integers(0, n, m)] + 0.3 * rng.standard_normal((m, d))).astype(np.float32)
+    Y[3] = X.max(axis=0) + 100.0 * h                # every weight zero
+    out, W = fms.mean_shift_step_coarse(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), h,
+                                        with_wsum=True)
+    out, W = out.cpu().numpy().astype(np.float64), W.cpu().numpy().astype(np.float64)
+    pick = np.unique(np.r_[0, m - 1, rng.integers(4, m, 24)])
+    ref, refW = orc.step(X, Y[pick], h), orc.kde(X, Y[pick], h)
+    bnd, eps = _bound(X, Y[pick], h, ref)
+    assert np.all(np.abs(out[pick] - ref).max(axis=1) <= bnd)
+    assert np.all(np.abs(W[pick] - refW) <= 1.5 * eps * refW)
+    assert W[3] == 0.0 and np.isnan(out[3]).all()
