@@ -1395,6 +1395,14 @@ bool step_by_groups(int64_t n, int d, int64_t m) {
          (double)n * (double)m * (double)padded_dim(d) >= 1.7e9;
 }
 
+// One launch where it takes no longer than the five of the general path: a thread
+// walks n / 256 points (2^18 coordinates to a seed: ~8 us), and a block per seed
+// reads every point, which pays up to ~2^27 coordinates of pairs (~12 us).
+bool step_small(int64_t n, int d, int64_t m) {
+  const double coords = (double)n * padded_dim(d);
+  return d <= 32 && coords <= 262144.0 && coords * (double)m <= 134217728.0;
+}
+
 GroupStepLayout group_step_layout(int64_t n, int d, int64_t m) {
   GroupStepLayout L{};
   L.DP = padded_dim(d);
@@ -1499,7 +1507,11 @@ fms_status fms_mean_shift_step(const float* points, int64_t n, int32_t d, float 
   {
     const double scale = sqrt(1.4426950408889634 / (2.0 * (double)h * (double)h));
     uint32_t* status = at<uint32_t>(ws, groups ? LG.off_status : L.off_status);
-    if (groups) {
+    if (step_small(n, d, m)) {
+      if (owns) FMS_CUDA(cudaMemsetAsync(status, 0, 64, st));   // (read below)
+      FMS_CUDA(launch_step_small(points, n, d, (float)scale, seeds, m, 1.0 / scale, out_seeds,
+                                 out_wsum, status, st));
+    } else if (groups) {
       FMS_CUDA(group_step(points, n, d, (float)scale, seeds, m, 1.0 / scale, out_seeds, out_wsum,
                           ws, LG, dv.sms, st));
     } else {

@@ -351,6 +351,11 @@ cudaError_t launch_update(const float* part, int32_t* active, IterCtl* ctl, floa
                           float* wlast = nullptr);  // sum w of each seed's last update
 cudaError_t launch_step_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t C, int32_t Lc,
                               cudaStream_t st);
+// One update of m seeds in one launch, for small problems (d <= 32); non-finite
+// inputs set kStNonFinite in *status.
+cudaError_t launch_step_small(const float* X, int64_t n, int d, float scale, const float* seeds,
+                              int64_t m, double inv_scale, float* out_seeds, float* out_wsum,
+                              uint32_t* status, cudaStream_t st);
 // out_row (nullable): the caller's row of each active position, -1 for none
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,

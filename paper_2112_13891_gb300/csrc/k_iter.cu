@@ -588,6 +588,92 @@ cudaError_t launch_update(const float* part, int32_t* active, IterCtl* ctl, floa
 namespace fms {
 
 // ---------------------------------------------------------------------------
+// A small stand-alone update in one launch (fms_mean_shift_step): a block per
+// seed, threads over the points as the caller has them (scaled and rounded on the
+// way in as the packing kernels do), block-wide sums in a fixed tree.  Bound by
+// launch latency: five launches (two packings, set-up, step, finish) of 2-3 us each
+// did little else.  D: the dimension up to 8, else its padded width.
+// ---------------------------------------------------------------------------
+template <int D>
+__global__ void __launch_bounds__(256)
+    step_small_kernel(const float* __restrict__ X, int n, int d_arg, float scale,
+                      const float* seeds, double inv_scale, float* out_seeds,
+                      float* __restrict__ out_wsum, uint32_t* status) {
+  __shared__ float red[8][D + 1];
+  const int d = D <= 8 ? D : d_arg;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t s = blockIdx.x;
+  float y[D], acc[D + 1];
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const float v = k < d ? seeds[s * d + k] : 0.0f;
+    bad = bad || !isfinite(v);
+    y[k] = v * scale;
+  }
+#pragma unroll
+  for (int k = 0; k <= D; ++k) acc[k] = 0.0f;
+#pragma unroll (D <= 8 ? 4 : 1)
+  for (int j = threadIdx.x; j < n; j += 256) {
+    float x[D], t = 0.0f;
+#pragma unroll
+    for (int k = 0; k < D; ++k) x[k] = k < d ? __ldg(X + (int64_t)j * d + k) : 0.0f;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      bad = bad || !isfinite(x[k]);
+      x[k] = x[k] * scale - y[k];
+    }
+#pragma unroll
+    for (int k = 0; k < D; ++k) t = fmaf(-x[k], x[k], t);
+    const float w = ex2_ftz(t);
+    acc[0] += w;
+#pragma unroll
+    for (int k = 0; k < D; ++k) acc[1 + k] = fmaf(w, x[k], acc[1 + k]);
+  }
+#pragma unroll
+  for (int k = 0; k <= D; ++k) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) acc[k] += __shfl_xor_sync(kFull, acc[k], o);
+    if (lane == 0) red[wid][k] = acc[k];
+  }
+  if (__any_sync(kFull, bad) && lane == 0) atomicOr(status, kStNonFinite);
+  __syncthreads();
+  if (wid == 0) {
+    float W = red[0][0];
+    for (int w = 1; w < 8; ++w) W += red[w][0];
+    for (int k = lane; k < d; k += 32) {
+      float v = red[0][1 + k];
+      for (int w = 1; w < 8; ++w) v += red[w][1 + k];
+      out_seeds[s * d + k] = (float)((double)seeds[s * d + k] + (double)(v / W) * inv_scale);
+    }
+    if (lane == 0 && out_wsum) out_wsum[s] = W;
+  }
+}
+
+cudaError_t launch_step_small(const float* X, int64_t n, int d, float scale, const float* seeds,
+                              int64_t m, double inv_scale, float* out_seeds, float* out_wsum,
+                              uint32_t* status, cudaStream_t st) {
+#define FMS_SMALL(D_)                                                                        \
+  step_small_kernel<D_><<<(unsigned)m, 256, 0, st>>>(X, (int)n, d, scale, seeds, inv_scale, \
+                                                     out_seeds, out_wsum, status);          \
+  return cudaGetLastError()
+  switch (d) {
+    case 1: FMS_SMALL(1);
+    case 2: FMS_SMALL(2);
+    case 3: FMS_SMALL(3);
+    case 4: FMS_SMALL(4);
+    case 5: FMS_SMALL(5);
+    case 6: FMS_SMALL(6);
+    case 7: FMS_SMALL(7);
+    case 8: FMS_SMALL(8);
+  }
+  if (d <= 16) { FMS_SMALL(16); }
+  if (d <= 32) { FMS_SMALL(32); }
+  return cudaErrorInvalidValue;
+#undef FMS_SMALL
+}
+
+// ---------------------------------------------------------------------------
 // Stand-alone single update (fms_mean_shift_step): every seed is active.
 // ---------------------------------------------------------------------------
 __global__ void step_setup_kernel(int32_t* __restrict__ active, int32_t m, IterCtl* ctl, int32_t C,
