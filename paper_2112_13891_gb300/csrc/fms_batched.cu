@@ -81,9 +81,9 @@ cudaError_t launch_batched_canonical(const SetCtl* sc, int B, const double* ym,
                                      const double* mscore, const int32_t* acc2, int d, int DP,
                                      double inv_scale, float* out_modes, int max_modes,
                                      float* modes_full, int32_t* out_n, cudaStream_t st);
-cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int d,
+cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int max_n, int d,
                                  const SetCtl* sc, const float* modes_full, int32_t* labels,
-                                 float* margins, int64_t total, cudaStream_t st);
+                                 float* margins, cudaStream_t st);
 }  // namespace fms
 
 using namespace fms;
@@ -660,8 +660,8 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         e = launch_batched_canonical(sc, B, ym, mscore, acc2, d, DP, 1.0 / scale, out_modes,
                                      max_modes, modes_full, out_n_modes, cs0);
       if (e == cudaSuccess)
-        e = launch_batched_label(points, pt_off, B, d, sc, modes_full, out_labels, out_margins,
-                                 total, cs0);
+        e = launch_batched_label(points, pt_off, B, max_n, d, sc, modes_full, out_labels,
+                                 out_margins, cs0);
       if (capturing) {
         cudaGraph_t gout = g;
         const cudaError_t e3 = cudaStreamEndCapture(cs0, &gout);

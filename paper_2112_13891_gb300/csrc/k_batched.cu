@@ -16,6 +16,7 @@
 // through conditional-node handles, whether another update, another seed round
 // or another refinement update follows.
 #include "fms_cells.cuh"
+#include "fms_label.cuh"
 #include "fms_prune_body.cuh"
 #include "fms_seedperm.cuh"
 #include "fms_step_body.cuh"
@@ -860,34 +861,20 @@ __global__ void batched_canonical(const SetCtl* __restrict__ sc, const double* _
   }
 }
 
+// Blocks run over (set, run of kLabelRun points), `per` runs to a set.
+constexpr int kLabelRun = 1024;
+
+template <int DP>
 __global__ void __launch_bounds__(256)
-    batched_label(const float* __restrict__ X, const int64_t* __restrict__ pt_off, int B, int d,
+    batched_label(const float* __restrict__ X, const int64_t* __restrict__ pt_off, int per, int d,
                   const SetCtl* __restrict__ sc, const float* __restrict__ modes_full,
-                  int32_t* __restrict__ labels, float* __restrict__ margins, int64_t total) {
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < total;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int b = find_set(pt_off, B, j);
-    const SetCtl& c = sc[b];
-    const float* mb = modes_full + (int64_t)c.p0 * d;
-    float b1 = INFINITY, b2 = INFINITY;
-    int arg = -1;
-    for (int m = 0; m < c.Mr; ++m) {
-      float d2 = 0.f;
-      for (int k = 0; k < d; ++k) {
-        const float e = X[j * d + k] - mb[(int64_t)m * d + k];
-        d2 = fmaf(e, e, d2);
-      }
-      if (d2 < b1) {
-        b2 = b1;
-        b1 = d2;
-        arg = m;
-      } else if (d2 < b2) {
-        b2 = d2;
-      }
-    }
-    labels[j] = arg;
-    if (margins) margins[j] = c.Mr > 1 ? sqrtf(b2) - sqrtf(b1) : INFINITY;
-  }
+                  int32_t* __restrict__ labels, float* __restrict__ margins) {
+  __shared__ __align__(16) float sm[kLabelFloats];
+  const int b = blockIdx.x / per;
+  const int64_t p0 = pt_off[b], p1 = pt_off[b + 1];
+  const int64_t j0 = p0 + (int64_t)(blockIdx.x % per) * kLabelRun, j1 = min(p1, j0 + kLabelRun);
+  if (j0 < j1)
+    label_block<DP, false>(X, j0, j1, d, modes_full + p0 * d, sc[b].Mr, labels, margins, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1067,14 +1054,23 @@ cudaError_t launch_batched_canonical(const SetCtl* sc, int B, const double* ym,
   return cudaGetLastError();
 }
 
-cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int d,
+cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int max_n, int d,
                                  const SetCtl* sc, const float* modes_full, int32_t* labels,
-                                 float* margins, int64_t total, cudaStream_t st) {
-  int64_t blocks = (total + 255) / 256;
-  if (blocks > 8192) blocks = 8192;
-  if (blocks < 1) blocks = 1;
-  batched_label<<<(int)blocks, 256, 0, st>>>(X, pt_off, B, d, sc, modes_full, labels, margins,
-                                             total);
+                                 float* margins, cudaStream_t st) {
+  const int64_t per = ((int64_t)max_n + kLabelRun - 1) / kLabelRun;
+  if (per * B > INT32_MAX) return cudaErrorInvalidValue;
+  const unsigned g = (unsigned)(per * B);
+#define FMS_LABEL(DP_)                                                                        \
+  batched_label<DP_><<<g, 256, 0, st>>>(X, pt_off, (int)per, d, sc, modes_full, labels, margins); \
+  break
+  switch (padded_dim(d)) {
+    case 4: FMS_LABEL(4);
+    case 8: FMS_LABEL(8);
+    case 16: FMS_LABEL(16);
+    case 32: FMS_LABEL(32);
+    default: FMS_LABEL(64);
+  }
+#undef FMS_LABEL
   return cudaGetLastError();
 }
 
