@@ -119,11 +119,12 @@ def _check(code: int, where: str):
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream's handle (an int: ctypes converts it faster than an object)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
 def _points(x: torch.Tensor) -> torch.Tensor:
@@ -131,6 +132,8 @@ def _points(x: torch.Tensor) -> torch.Tensor:
         raise ValueError("points must be a CUDA tensor")
     if x.dim() != 2:
         raise ValueError("points must be [n, d]")
+    if x.dtype == torch.float32 and x.is_contiguous():
+        return x
     return x.to(torch.float32).contiguous()
 
 
@@ -165,6 +168,18 @@ def _workspace_need(n: int, d: int, o: FmsOptions) -> int:
     need = _NEED_CACHE.get(key)
     if need is None:
         need = int(_lib.fms_workspace_size(n, d, ctypes.byref(o)))
+        if len(_NEED_CACHE) > 256:
+            _NEED_CACHE.clear()
+        _NEED_CACHE[key] = need
+    return need
+
+
+def _step_need(n: int, d: int, m: int) -> int:
+    """fms_step_workspace_size, remembered per (device, n, d, m)."""
+    key = (torch._C._cuda_getDevice(), n, d, m)
+    need = _NEED_CACHE.get(key)
+    if need is None:
+        need = int(_lib.fms_step_workspace_size(n, d, m))
         if len(_NEED_CACHE) > 256:
             _NEED_CACHE.clear()
         _NEED_CACHE[key] = need
@@ -360,7 +375,7 @@ def mean_shift_step(points: torch.Tensor, seeds: torch.Tensor, h: float, with_ws
     m = Y.shape[0]
     out = torch.empty_like(Y)
     wsum = torch.empty(m, dtype=torch.float32, device=X.device) if with_wsum else None
-    need = int(_lib.fms_step_workspace_size(n, d, m))
+    need = _step_need(n, d, m)
     if workspace is None or workspace.nbytes < need:
         workspace = Workspace(need, X.device)
     _check(_lib.fms_mean_shift_step(_ptr(X), n, d, float(h), _ptr(Y), m, _ptr(out), _ptr(wsum),
