@@ -181,6 +181,13 @@ __device__ __forceinline__ void walk_tiles(const T* __restrict__ rows, const int
   cp_wait<0>();
 }
 
+// The same for n unsorted rows that all lie in shared memory.
+template <int ROW, typename T, typename F>
+__device__ __forceinline__ void walk_resident(const T* rows, int n, int w, int W, F&& tile_fn) {
+  for (int r = w * kTileRows; r < n; r += W * kTileRows)
+    tile_fn(rows + r * ROW, min(kTileRows, n - r));
+}
+
 // Cells for a set of n points and m seeds (a power of two >= 32).  Half of them
 // start from strided points, so a cluster holding a share f of the points is
 // missed by all of those with probability exp(-f P / 2); fewer than 64 rows to a
@@ -330,6 +337,9 @@ cudaError_t unroll_backward_segment(const T* X, const cells::View<T>& cv, const 
                                     const UGeom& g, T c, T inv_h2, double inv_h3, const T* Gin,
                                     T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX,
                                     int first, cudaStream_t st);
+// Entries of dh_part per set (groups of the seed-major pass; per_set: of 32 seeds).
+template <typename T>
+int unroll_seed_groups(int P, const UGeom& g, int per_set);
 cudaError_t unroll_dh_sum(const double* dh_part, int B, int per_set, double* dh, cudaStream_t st);
 template <typename T>
 cudaError_t unroll_pack_rows(const T* src, int64_t rows, int per_set, int d, int DP,

@@ -92,41 +92,88 @@ constexpr int team_warp_smem() {
 }
 template <typename T, int DP, int SUMS>   // a team that walks cells
 constexpr int group_team_smem(int W) {
-  return W * team_warp_smem<T, DP, SUMS>() + kListCap * 8 + (int)sizeof(GroupSmem<T, DP>);
+  return W * team_warp_smem<T, DP, SUMS>() + SUMS * 32 * (int)sizeof(T) + kListCap * 8 + (int)sizeof(GroupSmem<T, DP>);
+}
+// Few unsorted points are kept in shared memory by every team for all its updates,
+// in the place of the rings: an update of 1,500 points by 16 warps is three tiles a
+// warp, whose copies from L2 it would wait for.
+constexpr int kResidentBytes = 48 * 1024;
+template <typename T, int DP>
+inline bool team_resident(int P, int64_t n) {
+  return P == 0 && n * DP * (int64_t)sizeof(T) <= kResidentBytes;
+}
+template <typename T, int DP, int SUMS>
+inline int resident_team_smem(int W, int64_t n) {
+  return (int)(n * DP * sizeof(T)) + (W + 1) * SUMS * 32 * (int)sizeof(T) + kListCap * 8 +
+         (int)sizeof(GroupSmem<T, DP>);
 }
 template <typename T, int ROW, int SUMS>   // a team with a list per warp
 constexpr int list_team_smem(int W) {
-  return W * (team_warp_smem<T, ROW, SUMS>() + kListCap * 8);
+  return W * (team_warp_smem<T, ROW, SUMS>() + kListCap * 8) + SUMS * 32 * (int)sizeof(T);
 }
 
 template <typename T, int ROW, int SUMS, bool GROUP = true>
 struct TeamSmem {
   T* ring;      // this warp's two tiles
   int2* list;   // the team's list (GROUP), or this warp's
-  T* sums;      // [W][SUMS][32], the whole team's
+  T* sums;      // [W + 1][SUMS][32], the whole team's (the last: totals)
   GroupSmem<T, ROW>* group;
-  __device__ TeamSmem(unsigned char* base, int w, int W) {
+  T* all;       // every point (few unsorted ones), else null
+  // n_all > 0: the points at `rows` are resident (copied here; ends with a barrier)
+  __device__ TeamSmem(unsigned char* base, int w, int W, const T* rows = nullptr, int n_all = 0) {
     constexpr int ring_e = 2 * cells::kTileRows * ROW;
-    ring = reinterpret_cast<T*>(base) + (size_t)w * ring_e;
-    unsigned char* p = base + (size_t)W * ring_e * sizeof(T);
+    ring = reinterpret_cast<T*>(base) + (n_all > 0 ? 0 : (size_t)w * ring_e);
+    all = n_all > 0 ? ring : nullptr;
+    unsigned char* p = base + (n_all > 0 ? (size_t)n_all * ROW : (size_t)W * ring_e) * sizeof(T);
     sums = reinterpret_cast<T*>(p);
-    p += (size_t)W * SUMS * 32 * sizeof(T);
+    p += (size_t)(W + 1) * SUMS * 32 * sizeof(T);
     list = reinterpret_cast<int2*>(p) + (GROUP ? 0 : w * kListCap);
     group = reinterpret_cast<GroupSmem<T, ROW>*>(p + kListCap * 8);
+    if (n_all > 0) {
+      const int n16 = n_all * (ROW * (int)sizeof(T) / 16);
+      for (int i = threadIdx.x; i < n16; i += blockDim.x)
+        reinterpret_cast<float4*>(all)[i] = __ldg(reinterpret_cast<const float4*>(rows) + i);
+      __syncthreads();
+    }
+  }
+  // the team's tiles: of the listed cells of X, or of the resident points
+  template <typename F>
+  __device__ __forceinline__ void walk(const T* X, int n, int nl, int w, int W, int lane,
+                                       F&& tile_fn) const {
+    if (all) cells::walk_resident<ROW>(all, n, w, W, tile_fn);
+    else cells::walk_tiles<ROW>(X, list, nl, w, W, ring, lane, tile_fn);
   }
 };
+
+// warps a block may have: 16 where the registers allow
+template <typename T, int DP>
+constexpr int most_warps() {
+  return sizeof(T) == 4 && DP <= 8 ? 16 : 8;
+}
+// rows evaluated together (independent chains)
+template <typename T, int DP>
+constexpr int row_unroll() {
+  return DP <= 4 ? 8 : (DP <= 8 ? 4 : 1);
+}
 
 // The team's list of the cells of set b that can hold a point within the distance
 // rc of an active lane's seed y, as (first row, rows); returns its length.  First
 // the ball around the active seeds against each cell's ball, then the cells left,
 // one per lane, against every active seed: in many dimensions the ball around the
 // seeds is as wide as their cluster, and only the second test keeps its neighbours
-// out.  At least one lane is active; every thread of the team calls.
+// out.  At least one lane is active; every thread of the team calls.  Without cells
+// (P = 0) the list is every row, and *reach and *ball are not set.
 template <typename T, int DP, int SUMS>
 __device__ __forceinline__ int visible_cells(const View<T>& v, int b, int n, const T (&y)[DP],
                                              bool act, T rc, T* reach,
                                              T (*ball)[DP], const TeamSmem<T, DP, SUMS>& sm,
                                              int w, int W, int lane) {
+  if (v.P == 0) {
+    if (sm.all) return 0;   // (walk takes the resident points)
+    if (threadIdx.x == 0) sm.list[0] = make_int2(0, n);
+    __syncthreads();
+    return 1;
+  }
   const unsigned live = __ballot_sync(kFull, act);
   const int src = __ffs(live) - 1, nact = __popc(live);
   T c[DP];
@@ -144,11 +191,6 @@ __device__ __forceinline__ int visible_cells(const View<T>& v, int b, int n, con
   if (ball) {
 #pragma unroll
     for (int k = 0; k < DP; ++k) (*ball)[k] = c[k];
-  }
-  if (v.P == 0) {
-    if (threadIdx.x == 0) sm.list[0] = make_int2(0, n);
-    __syncthreads();
-    return 1;
   }
   GroupSmem<T, DP>& g = *sm.group;
   const int32_t* st = v.start + (int64_t)b * (v.P + 1);
@@ -241,31 +283,74 @@ __device__ __forceinline__ int visible_cells(const View<T>& v, int b, int n, con
   return nl;
 }
 
-// Sums v over the team in warp order; every warp gets the result.
-template <typename T, int N>
+// PH > 1 (few seeds, nothing sorted): a group is 32 / PH seeds, lane l holds seed
+// l % (32 / PH) and takes rows l / (32 / PH), + PH, ... of a tile, so PH times as many
+// blocks share the work.  row_fn(row, inside) for each of the lane's rows; a row
+// outside the tile repeats its last one and must count nothing.
+template <int ROW, int PH, int UNROLL, typename T, typename F>
+__device__ __forceinline__ void tile_rows(const T* rows, int nr, int lane, F&& row_fn) {
+  if constexpr (PH == 1) {
+#pragma unroll UNROLL
+    for (int q = 0; q < nr; ++q) row_fn(rows + q * ROW, true);
+  } else {
+    const int ph = lane / (32 / PH);
+    if (nr == cells::kTileRows) {
+#pragma unroll UNROLL
+      for (int q = 0; q < cells::kTileRows / PH; ++q) row_fn(rows + (q * PH + ph) * ROW, true);
+    } else {
+      for (int q = 0; q < nr; q += PH)
+        row_fn(rows + min(q + ph, nr - 1) * ROW, q + ph < nr);
+    }
+  }
+}
+// ... and their sums over the PH lanes of a seed.
+template <int PH, typename T, int N>
+__device__ __forceinline__ void phase_sum(T (&v)[N]) {
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+#pragma unroll
+    for (int o = 16; o >= 32 / PH && PH > 1; o >>= 1) v[k] += __shfl_xor_sync(kFull, v[k], o);
+}
+// PH for `seeds` seeds of all sets: enough groups for the GPU's SMs.
+template <typename T, int DP>
+inline int team_phases(int P, int64_t seeds, int sms) {
+  if (P > 0 || sizeof(T) != 4 || DP > 16) return 1;
+  return (seeds + 31) / 32 >= sms ? 1 : 4;
+}
+
+// Sums v over the team in warp order; every warp gets the result.  Lanes l and
+// l + GS hold the same values; a thread adds one value's W parts (every warp adding
+// all of them would read W^2 rows of shared memory).
+template <int GS, typename T, int N>
 __device__ __forceinline__ void team_sum(T (&v)[N], T* sums, int stride, int w, int W, int lane) {
   if (W == 1) return;
+  T* total = sums + W * stride * 32;
+  if (lane < GS) {
 #pragma unroll
-  for (int k = 0; k < N; ++k) sums[(w * stride + k) * 32 + lane] = v[k];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    T s = sums[k * 32 + lane];
-    for (int u = 1; u < W; ++u) s += sums[(u * stride + k) * 32 + lane];
-    v[k] = s;
+    for (int k = 0; k < N; ++k) sums[(w * stride + k) * 32 + lane] = v[k];
   }
   __syncthreads();
+  for (int i = threadIdx.x; i < N * GS; i += 32 * W) {
+    const int at = i / GS * 32 + i % GS;
+    T s = sums[at];
+    for (int u = 1; u < W; ++u) s += sums[u * stride * 32 + at];
+    total[at] = s;
+  }
+  __syncthreads();
+  // (rewritten only after the next call's first barrier)
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k] = total[k * 32 + lane % GS];
 }
 
 __device__ __forceinline__ bool group_rows(const Groups& g, int b, int gi, int rows, int* row0,
-                                           int* cnt) {
+                                           int* cnt, int size = 32) {
   if (g.table) {
     const int2 e = __ldg(g.table + (int64_t)b * g.per_set + gi);
     *row0 = e.x;
     *cnt = e.y;
   } else {
-    *row0 = gi * 32;
-    *cnt = min(32, rows - gi * 32);
+    *row0 = gi * size;
+    *cnt = min(size, rows - gi * size);
   }
   return *cnt > 0;
 }

@@ -112,6 +112,9 @@ BwdLayout bwd_layout(const UGeom& g, int P, int32_t k, size_t es) {
   };
   const size_t rowsY = (size_t)g.B * g.m, NG = (size_t)g.B * groups_for(g.m, P);
   const size_t pb = (size_t)(k < kPointBatch ? k : kPointBatch);
+  const size_t seed_groups =
+      es == 4 ? unroll_seed_groups<float>(P, g, groups_for(g.m, P))
+              : unroll_seed_groups<double>(P, g, groups_for(g.m, P));
   L.s = sort_layout(g, P, es, take);
   L.seg = take((size_t)k * rowsY * g.DP * es);   // recomputed positions inside a segment
   L.Ga = take(rowsY * g.DP * es);
@@ -119,7 +122,7 @@ BwdLayout bwd_layout(const UGeom& g, int P, int32_t k, size_t es) {
   L.SD = take(pb * rowsY * (2 * g.DP + 4) * es);
   L.bctr = take(pb * NG * g.DP * es);
   L.breach = take(pb * NG * es);
-  L.dh_part = take(NG * 8);
+  L.dh_part = take((size_t)g.B * seed_groups * 8);
   L.dXp = take((size_t)g.B * g.n * g.DP * es);
   L.total = o;
   return L;
@@ -299,7 +302,7 @@ fms_status backward_impl(const E* points, int32_t B, int64_t n, int64_t m, int32
       unroll_unpack_rows<E>(dXp, (int64_t)B * n, (int)n, d, g.DP,
                             P > 0 ? at<int32_t>(ws, L.s.perm) : nullptr, grad_points,
                             st) != cudaSuccess ||
-      unroll_dh_sum(dh_part, B, gr.per_set, grad_h, st) != cudaSuccess)
+      unroll_dh_sum(dh_part, B, unroll_seed_groups<E>(P, g, gr.per_set), grad_h, st) != cudaSuccess)
     return FMS_ERR_CUDA;
   return FMS_OK;
 }

@@ -35,7 +35,7 @@ __device__ __forceinline__ float first_cut() {
 // W and S of the group at y (acc[0], acc[1 + k]); `act` lanes decide the ball
 // and the cutoff, which comes in as a guess and leaves as the one their smallest
 // W asks for.  Returns the rows visited.
-template <int DP, int KF, int SUMS>
+template <int DP, int KF, int PH, int SUMS>
 __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const View<float>& cv, int n,
                                           const float (&y)[DP], bool act, float log2n, float& cut,
                                           const TeamSmem<float, DP, SUMS>& sm, int w, int W,
@@ -45,35 +45,38 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
     float reach;
     const int nl = visible_cells<float, DP>(cv, 0, n, y, act, sqrtf(cut), &reach, nullptr, sm, w,
                                             W, lane);
-    for (int i = lane; i < nl; i += 32) rows += sm.list[i].y;
+    if (cv.P == 0) rows = lane == 0 ? n : 0;
+    else
+      for (int i = lane; i < nl; i += 32) rows += sm.list[i].y;
 #pragma unroll
     for (int k = 0; k <= DP; ++k) acc[k] = 0.0f;
-    cells::walk_tiles<DP>(Xs, sm.list, nl, w, W, sm.ring, lane, [&](const float* tile, int nr) {
+    sm.walk(Xs, n, nl, w, W, lane, [&](const float* tile, int nr) {
       float ta[DP + 1];
 #pragma unroll
       for (int k = 0; k <= DP; ++k) ta[k] = 0.0f;
-#pragma unroll (DP <= 8 ? 4 : (DP <= 16 ? 2 : 1))
-      for (int q = 0; q < nr; ++q) {
+      constexpr int UNROLL = DP <= 4 ? 8 : (DP <= 8 ? 4 : (DP <= 16 ? 2 : 1));
+      tile_rows<DP, PH, UNROLL>(tile, nr, lane, [&](const float* row, bool in) {
         float x[DP];
-        smem_row<DP>(tile + q * DP, x);
+        smem_row<DP>(row, x);
         float t = 0.0f;
 #pragma unroll
         for (int k = 0; k < DP; ++k) {
           x[k] -= y[k];
           t = fmaf(-x[k], x[k], t);
         }
-        const float wt = kweight<KF>(t);
+        const float wt = in ? kweight<KF>(t) : 0.0f;
         ta[0] += wt;
 #pragma unroll
         for (int k = 0; k < DP; ++k) ta[1 + k] = fmaf(wt, x[k], ta[1 + k]);
-      }
+      });
 #pragma unroll
       for (int k = 0; k <= DP; ++k) acc[k] += ta[k];
     });
-    team_sum(acc, sm.sums, SUMS, w, W, lane);
-    if (KF == kKernelFlat) break;
+    phase_sum<PH>(acc);
+    team_sum<32 / PH>(acc, sm.sums, SUMS, w, W, lane);
+    if (KF == kKernelFlat || cv.P == 0) break;
     const float need = cells::cut_bits(cells::warp_min(act ? acc[0] : INFINITY), log2n);
-    if (cv.P == 0 || !(need > cut) || cut >= cells::zero_bits<float>()) {
+    if (!(need > cut) || cut >= cells::zero_bits<float>()) {
       cut = cells::widen(need);   // (W does not decrease along a trajectory)
       break;
     }
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(256)
   load_row<DP>(Ys + (int64_t)e * DP, y);
   const float log2n = log2f((float)n);
   float cut = first_cut<kKernelGaussian>();
-  group_pass<DP, kKernelGaussian>(Xs, cv, n, y, true, log2n, cut, sm, w, W, lane, acc);
+  group_pass<DP, kKernelGaussian, 1>(Xs, cv, n, y, true, log2n, cut, sm, w, W, lane, acc);
   if (w != 0 || lane >= cnt) return;
   const int64_t i = perm[e];
 #pragma unroll
@@ -114,32 +117,33 @@ __global__ void __launch_bounds__(256)
 // Every point a seed, slot = the point's row in the caller's order (perm; null:
 // unsorted): updates until it converges, fails or has made max_iter of them, then
 // the density at its last position (wlast).  hist counts the convergence updates.
-template <int DP, int KF>
+template <int DP, int KF, int PH>
 __global__ void __launch_bounds__(512)
     travel_groups(const float* __restrict__ Xs, View<float> cv, int n, Groups gr,
                   const int32_t* __restrict__ perm, int max_iter, float tol2_s, float sphere_r,
                   float* __restrict__ y_out, int32_t* __restrict__ it_out,
                   int32_t* __restrict__ conv, int32_t* __restrict__ state,
                   float* __restrict__ wlast, int32_t* __restrict__ hist,
-                  unsigned long long* evals, unsigned long long* score_evals) {
+                  unsigned long long* evals, unsigned long long* score_evals, int resident) {
   extern __shared__ __align__(16) unsigned char travel_smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
-  const TeamSmem<float, DP, DP + 1> sm(travel_smem, w, W);
+  constexpr int GS = 32 / PH;   // seeds of a group
   int row0, cnt;
-  if (!group_rows(gr, 0, blockIdx.x, n, &row0, &cnt)) return;
-  const int e = row0 + min(lane, cnt - 1);
+  if (!group_rows(gr, 0, blockIdx.x, n, &row0, &cnt, GS)) return;
+  const TeamSmem<float, DP, DP + 1> sm(travel_smem, w, W, Xs, resident ? n : 0);
+  const int e = row0 + min(lane % GS, cnt - 1);
   float y[DP], acc[DP + 1];
   load_row<DP>(Xs + (int64_t)e * DP, y);
   const float log2n = log2f((float)n);
   float cut = first_cut<KF>(), wl = 0.0f;
-  bool act = lane < cnt;
+  bool act = lane % GS < cnt;
   int it = 0, cu = -1, stt = kRunning;
   unsigned long long ev = 0;
   for (;;) {
     const unsigned live = __ballot_sync(kFull, act);   // the same for every warp of the team
     if (!live) break;
-    const int rows = group_pass<DP, KF>(Xs, cv, n, y, act, log2n, cut, sm, w, W, lane, acc);
-    ev += (unsigned long long)rows * __popc(live);
+    const int rows = group_pass<DP, KF, PH>(Xs, cv, n, y, act, log2n, cut, sm, w, W, lane, acc);
+    ev += (unsigned long long)rows * (__popc(live) / PH);
     if (!act) continue;
     wl = acc[0];
     ++it;
@@ -181,11 +185,11 @@ __global__ void __launch_bounds__(512)
     }
     act = stt == kRunning;
   }
-  const bool fine = lane < cnt && stt != kFailed;
+  const bool fine = lane % GS < cnt && stt != kFailed;
   unsigned long long sev = 0;
   if (__any_sync(kFull, fine)) {
-    const int rows = group_pass<DP, KF>(Xs, cv, n, y, fine, log2n, cut, sm, w, W, lane, acc);
-    sev = (unsigned long long)rows * __popc(__ballot_sync(kFull, fine));
+    const int rows = group_pass<DP, KF, PH>(Xs, cv, n, y, fine, log2n, cut, sm, w, W, lane, acc);
+    sev = (unsigned long long)rows * (__popc(__ballot_sync(kFull, fine)) / PH);
     wl = acc[0];
   }
   if (w != 0) return;
@@ -745,22 +749,26 @@ cudaError_t launch_step_groups(const float* Xs, const View<float>& cv, int n, co
   return cudaErrorInvalidValue;
 }
 
-template <int DP, int KF>
-static cudaError_t travel_groups_t(const float* Xs, const View<float>& cv, int n, const Groups& gr,
+template <int DP, int KF, int PH>
+static cudaError_t travel_groups_t(const float* Xs, const View<float>& cv, int n, Groups gr,
                                    const int32_t* perm, int max_iter, float tol2_s,
                                    float sphere_r, float* y, int32_t* it, int32_t* conv,
                                    int32_t* state, float* wlast, int32_t* hist,
                                    unsigned long long* evals, unsigned long long* score_evals,
                                    int sms, cudaStream_t st) {
+  if (PH > 1) gr.per_set = (n + 32 / PH - 1) / (32 / PH);
   constexpr int ws = team_warp_smem<float, DP, DP + 1>();
   // at least 4 warps: the last groups take many updates, with few others running
   const int W0 = team_warps(gr.per_set, sms, ws, 16), W = W0 < 4 ? 4 : W0;
-  const int smem = group_team_smem<float, DP, DP + 1>(W);
-  const cudaError_t e = team_attr(travel_groups<DP, KF>, smem);
+  const bool res = team_resident<float, DP>(cv.P, n);
+  const int smem =
+      res ? resident_team_smem<float, DP, DP + 1>(W, n) : group_team_smem<float, DP, DP + 1>(W);
+  const cudaError_t e = team_attr(travel_groups<DP, KF, PH>, smem);
   if (e != cudaSuccess) return e;
-  travel_groups<DP, KF><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, gr, perm, max_iter, tol2_s,
+  travel_groups<DP, KF, PH><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, gr, perm, max_iter, tol2_s,
                                                             sphere_r, y, it, conv, state, wlast,
-                                                            hist, evals, score_evals);
+                                                            hist, evals, score_evals,
+                                                            res ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -770,16 +778,19 @@ cudaError_t launch_travel_groups(const float* Xs, const View<float>& cv, int n, 
                                  int32_t* conv, int32_t* state, float* wlast, int32_t* hist,
                                  unsigned long long* evals, unsigned long long* score_evals,
                                  int sms, cudaStream_t st) {
-#define FMS_TRAVEL(DP_)                                                                          \
-  return kf ? travel_groups_t<DP_, 1>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it,    \
-                                      conv, state, wlast, hist, evals, score_evals, sms, st)     \
-            : travel_groups_t<DP_, 0>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it,    \
-                                      conv, state, wlast, hist, evals, score_evals, sms, st)
+#define FMS_TRAVEL_PH(DP_, KF_, PH_)                                                            \
+  travel_groups_t<DP_, KF_, PH_>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it, conv,  \
+                                 state, wlast, hist, evals, score_evals, sms, st)
+#define FMS_TRAVEL(DP_)                                                                        \
+  if (team_phases<float, DP_>(cv.P, n, sms) == 4)                                              \
+    return kf ? FMS_TRAVEL_PH(DP_, 1, 4) : FMS_TRAVEL_PH(DP_, 0, 4);                           \
+  return kf ? FMS_TRAVEL_PH(DP_, 1, 1) : FMS_TRAVEL_PH(DP_, 0, 1)
   switch (DP) {
     case 4: FMS_TRAVEL(4);
     case 8: FMS_TRAVEL(8);
   }
 #undef FMS_TRAVEL
+#undef FMS_TRAVEL_PH
   return cudaErrorInvalidValue;
 }
 

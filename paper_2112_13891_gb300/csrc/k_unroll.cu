@@ -106,67 +106,68 @@ __device__ T rescue_seed(const T* __restrict__ Xb, int n, T c, const T (&y)[DP],
 // t the positions go to slot ceil(t / every) - slot0 of pos where t is a
 // multiple of `every` or the last one; W and the shift of update t to row t - 1
 // of Wout and Sh (nullable).
-template <typename T, int DP>
-__global__ void __launch_bounds__(256)
+template <typename T, int DP, int PH>
+__global__ void __launch_bounds__(32 * most_warps<T, DP>())
     unroll_travel(const T* __restrict__ X, View<T> cv, const T* __restrict__ Y0, Groups gr,
                   UGeom g, T c, int steps, int every, int slot0, T* __restrict__ pos,
-                  T* __restrict__ Wout, T* __restrict__ Sh, T* __restrict__ M2) {
+                  T* __restrict__ Wout, T* __restrict__ Sh, T* __restrict__ M2, int resident) {
   extern __shared__ __align__(16) unsigned char unroll_smem[];
-  constexpr int SUMS = DP + 3;
+  constexpr int SUMS = DP + 3, GS = 32 / PH;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
-  const TeamSmem<T, DP, SUMS> sm(unroll_smem, w, W);
   const int b = blockIdx.x / gr.per_set;
   int row0, cnt;
-  if (!group_rows(gr, b, blockIdx.x % gr.per_set, g.m, &row0, &cnt)) return;
+  if (!group_rows(gr, b, blockIdx.x % gr.per_set, g.m, &row0, &cnt, GS)) return;
   const T* Xb = X + (int64_t)b * g.n * DP;
+  const TeamSmem<T, DP, SUMS> sm(unroll_smem, w, W, Xb, resident ? g.n : 0);
   const int64_t rowsY = (int64_t)g.B * g.m;
-  const int64_t e = (int64_t)b * g.m + row0 + min(lane, cnt - 1);
+  const int64_t e = (int64_t)b * g.m + row0 + min(lane % GS, cnt - 1);
   T y[DP];
   load_row<DP>(Y0 + e * DP, y);
   const T log2n = T(log2f((float)g.n));
   T cut = T(cells::kFirstCut);
   for (int t = 1; t <= steps; ++t) {
     T acc[DP + 2];   // W, S, sum w ||x - y||^2
-    T need;
+    T need = T(0);
     for (int pass = 0;; ++pass) {
       T reach;
       const int nl = visible_cells<T, DP>(cv, b, g.n, y, true, cells::csqrt(cut / c), &reach,
                                           nullptr, sm, w, W, lane);
 #pragma unroll
       for (int k = 0; k < DP + 2; ++k) acc[k] = T(0);
-      cells::walk_tiles<DP>(Xb, sm.list, nl, w, W, sm.ring, lane, [&](const T* rows, int nr) {
+      sm.walk(Xb, g.n, nl, w, W, lane, [&](const T* rows, int nr) {
         T ta[DP + 2];
 #pragma unroll
         for (int k = 0; k < DP + 2; ++k) ta[k] = T(0);
-#pragma unroll (DP <= 8 ? 2 : 1)
-        for (int q = 0; q < nr; ++q) {
+        tile_rows<DP, PH, row_unroll<T, DP>()>(rows, nr, lane, [&](const T* row, bool in) {
           T x[DP];
-          smem_row<DP>(rows + q * DP, x);
+          smem_row<DP>(row, x);
           T D2 = T(0);
 #pragma unroll
           for (int k = 0; k < DP; ++k) {
             x[k] -= y[k];
             D2 = ufma(x[k], x[k], D2);
           }
-          const T wt = uex2(-c * D2);
+          const T wt = in ? uex2(-c * D2) : T(0);
           ta[0] += wt;
           ta[DP + 1] = ufma(wt, D2, ta[DP + 1]);
 #pragma unroll
           for (int k = 0; k < DP; ++k) ta[1 + k] = ufma(wt, x[k], ta[1 + k]);
-        }
+        });
 #pragma unroll
         for (int k = 0; k < DP + 2; ++k) acc[k] += ta[k];
       });
-      team_sum(acc, sm.sums, SUMS, w, W, lane);
+      phase_sum<PH>(acc);
+      team_sum<GS>(acc, sm.sums, SUMS, w, W, lane);
+      if (cv.P == 0) break;
       need = cells::cut_bits(cells::warp_min(acc[0]), log2n);
-      if (cv.P == 0 || !(need > cut)) break;
+      if (!(need > cut)) break;
       cut = pass == 0 ? cells::widen(need) : T(cells::zero_bits<T>());
     }
     cut = cells::widen(need);   // (W does not decrease along a trajectory)
     T sh = T(0);
     unsigned bad = __ballot_sync(kFull, !(acc[0] >= unroll_min_w<T>()) || !isfinite(acc[0]));
     if (bad) {   // the same for every warp of the team
-      for (int u = 0; u < 32; ++u) {
+      for (int u = 0; u < GS; ++u) {
         if (!((bad >> u) & 1u) || u % W != w) continue;
         T ys[DP], a2[DP + 2];
 #pragma unroll
@@ -181,8 +182,8 @@ __global__ void __launch_bounds__(256)
       __syncthreads();
       if ((bad >> lane) & 1u) {
 #pragma unroll
-        for (int k = 0; k < DP + 2; ++k) acc[k] = sm.sums[k * 32 + lane];
-        sh = sm.sums[(DP + 2) * 32 + lane];
+        for (int k = 0; k < DP + 2; ++k) acc[k] = sm.sums[k * 32 + lane % GS];
+        sh = sm.sums[(DP + 2) * 32 + lane % GS];
       }
       __syncthreads();
     }
@@ -209,38 +210,60 @@ __global__ void __launch_bounds__(256)
 // ||y_i - x_j||^2 under p (kept by the forward) makes the terms smallest, and a
 // far seed's residual sum p a (FP32 rounding of a D2 of hundreds leaves ~1e-5
 // instead of 0) is not multiplied by D2.  DH is summed over tiles in FP64.
-template <typename T, int DP>
-__global__ void __launch_bounds__(256)
+template <typename T, int DP, int PH>
+__global__ void __launch_bounds__(32 * most_warps<T, DP>())
     unroll_bwd_seed(const T* __restrict__ X, View<T> cv, USegment<T> sg, Groups gr, UGeom g, T c,
                     T inv_h2, double inv_h3, const T* __restrict__ Gin, T* __restrict__ Gout,
                     T* __restrict__ SD, T* __restrict__ bctr, T* __restrict__ breach,
-                    double* __restrict__ dh_part, int first) {
+                    double* __restrict__ dh_part, int first, int resident) {
   extern __shared__ __align__(16) unsigned char unroll_smem[];
-  constexpr int SUMS = DP + 2, SDW = 2 * DP + 4;
+  constexpr int SUMS = DP + 2, SDW = 2 * DP + 4, GS = 32 / PH;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
-  __shared__ double dhs[8];
-  const TeamSmem<T, DP, SUMS> sm(unroll_smem, w, W);
+  __shared__ double dhs[16];
   const int b = blockIdx.x / gr.per_set, gi = blockIdx.x % gr.per_set;
   const int64_t NG = (int64_t)g.B * gr.per_set;
   int row0, cnt;
-  if (!group_rows(gr, b, gi, g.m, &row0, &cnt)) {
+  if (!group_rows(gr, b, gi, g.m, &row0, &cnt, GS)) {
     if (threadIdx.x == 0 && first) dh_part[blockIdx.x] = 0.0;
     return;
   }
   const T* Xb = X + (int64_t)b * g.n * DP;
+  const TeamSmem<T, DP, SUMS> sm(unroll_smem, w, W, Xb, resident ? g.n : 0);
   const int64_t rowsY = (int64_t)g.B * g.m;
-  const int64_t e = (int64_t)b * g.m + row0 + min(lane, cnt - 1);
+  const int64_t e = (int64_t)b * g.m + row0 + min(lane % GS, cnt - 1);
   const T log2n = T(log2f((float)g.n));
   T gg[DP];
   load_row<DP>(Gin + e * DP, gg);
   double dh = 0.0;
+  // the next update's row and values are loaded a pass ahead where registers allow
+  constexpr bool kAhead = DP <= 8;
+  T yn[DP], ya[DP], Wn, shn, m2n;
+  auto fetch = [&](int u) {
+    const int64_t ue = (int64_t)(sg.u0 + u) * rowsY + e;
+    load_row<DP>(sg.pos(u) + e * DP, yn);
+    Wn = sg.W[ue];
+    shn = sg.Sh[ue];
+    m2n = sg.M2[ue];
+  };
+  if (kAhead) {
+    load_row<DP>(sg.pos(sg.len) + e * DP, ya);
+    fetch(sg.len - 1);
+  }
   for (int u = sg.len - 1; u >= 0; --u) {
     T y[DP], ym[DP], ctr[DP];
-    load_row<DP>(sg.pos(u) + e * DP, y);
-    load_row<DP>(sg.pos(u + 1) + e * DP, ym);
-    const int64_t ue = (int64_t)(sg.u0 + u) * rowsY + e;
-    const T Wt = sg.W[ue], sh = sg.Sh[ue];
-    const T invW = T(1) / Wt, s0 = sg.M2[ue];
+    if (!kAhead) {
+      load_row<DP>(sg.pos(u + 1) + e * DP, ya);
+      fetch(u);
+    }
+    const T Wt = Wn, sh = shn, s0 = m2n;
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      y[k] = yn[k];
+      ym[k] = ya[k];
+      if (kAhead) ya[k] = y[k];
+    }
+    if (kAhead && u > 0) fetch(u - 1);
+    const T invW = T(1) / Wt;
     T gd = T(0);
 #pragma unroll
     for (int k = 0; k < DP; ++k) {
@@ -260,7 +283,7 @@ __global__ void __launch_bounds__(256)
         const T tail[4] = {invW, sh, gd, T(0)};
         store_row<T, 4>(o + 2 * DP, tail);
       }
-      if (lane == 0) {
+      if (lane == 0 && cv.P > 0) {
         store_row<T, DP>(bctr + ((int64_t)u * NG + blockIdx.x) * DP, ctr);
         breach[(int64_t)u * NG + blockIdx.x] = reach;
       }
@@ -269,14 +292,13 @@ __global__ void __launch_bounds__(256)
     double DH = 0.0;
 #pragma unroll
     for (int k = 0; k <= DP; ++k) acc[k] = T(0);
-    cells::walk_tiles<DP>(Xb, sm.list, nl, w, W, sm.ring, lane, [&](const T* rows, int nr) {
+    sm.walk(Xb, g.n, nl, w, W, lane, [&](const T* rows, int nr) {
       T ta[DP + 2];
 #pragma unroll
       for (int k = 0; k < DP + 2; ++k) ta[k] = T(0);
-#pragma unroll (DP <= 8 ? 2 : 1)
-      for (int q = 0; q < nr; ++q) {
+      tile_rows<DP, PH, row_unroll<T, DP>()>(rows, nr, lane, [&](const T* row, bool in) {
         T x[DP];
-        smem_row<DP>(rows + q * DP, x);
+        smem_row<DP>(row, x);
         T D2 = T(0), a = gd;
 #pragma unroll
         for (int k = 0; k < DP; ++k) {
@@ -284,22 +306,23 @@ __global__ void __launch_bounds__(256)
           D2 = ufma(x[k], x[k], D2);
           a = ufma(gg[k], x[k], a);
         }
-        const T pa = uex2(ufma(-c, D2, sh)) * invW * a;
+        const T pa = in ? uex2(ufma(-c, D2, sh)) * invW * a : T(0);
         ta[0] = ufma(pa, D2 - s0, ta[0]);
         ta[1] += pa;
 #pragma unroll
         for (int k = 0; k < DP; ++k) ta[2 + k] = ufma(pa, x[k], ta[2 + k]);
-      }
+      });
 #pragma unroll
       for (int k = 0; k <= DP; ++k) acc[k] += ta[1 + k];
       DH += (double)ta[0];
     });
-    team_sum(acc, sm.sums, SUMS, w, W, lane);
+    phase_sum<PH>(acc);
+    team_sum<GS>(acc, sm.sums, SUMS, w, W, lane);
     dh += DH;   // (this warp's tiles)
 #pragma unroll
     for (int k = 0; k < DP; ++k) gg[k] = ufma(ym[k], acc[0], acc[1 + k]) * inv_h2;
   }
-  if (lane >= cnt) dh = 0.0;
+  if (lane % GS >= cnt) dh = 0.0;
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) dh += __shfl_xor_sync(kFull, dh, o);
   if (lane == 0) dhs[w] = dh;
@@ -320,7 +343,7 @@ __global__ void __launch_bounds__(256)
 //   DX_j = sum_i p_ij g_i - (1/h^2) sum_i p_ij a_ij (x_j - y_i)
 // to its rows of dX.
 template <typename T, int DP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(32 * most_warps<T, DP>())
     unroll_bwd_point(const T* __restrict__ X, Groups gx, Groups gr, UGeom g, int len, T c,
                      T inv_h2, const T* __restrict__ SD, const T* __restrict__ bctr,
                      const T* __restrict__ breach, T* __restrict__ dX, int first) {
@@ -340,10 +363,15 @@ __global__ void __launch_bounds__(256)
   for (int k = 0; k < DP; ++k) acc[k] = T(0);
   for (int u = 0; u < len; ++u) {
     const T* sdb = SD + ((int64_t)u * rowsY + (int64_t)b * g.m) * SDW;
-    for (int g0 = 0; g0 < gr.per_set;) {
+    if (!gr.table) {   // nothing sorted: every seed
+      if (lane == 0) sm.list[0] = make_int2(0, g.m);
+      __syncwarp();
+    }
+    for (int g0 = 0; gr.table ? g0 < gr.per_set : g0 == 0;) {
       // the next seed groups that reach these points, as many as the list holds
-      int nl = 0;
-      for (; g0 < gr.per_set && nl <= kListCap - 32; g0 += 32) {
+      int nl = gr.table ? 0 : 1;
+      if (!gr.table) g0 = 1;
+      for (; gr.table && g0 < gr.per_set && nl <= kListCap - 32; g0 += 32) {
         const int gi = g0 + lane;
         bool see = false;
         int r0 = 0, rc = 0;
@@ -369,6 +397,7 @@ __global__ void __launch_bounds__(256)
         T ta[DP];
 #pragma unroll
         for (int k = 0; k < DP; ++k) ta[k] = T(0);
+#pragma unroll (DP <= 4 ? 4 : 1)
         for (int q = 0; q < nr; ++q) {
           const T* sd = rows + q * SDW;
           T dx[DP], gv[DP], tail[4];
@@ -392,7 +421,7 @@ __global__ void __launch_bounds__(256)
       });
     }
   }
-  team_sum(acc, sm.sums, SUMS, w, W, lane);
+  team_sum<32>(acc, sm.sums, SUMS, w, W, lane);
   if (w == 0 && lane < cnt) {
     T* o = dX + e * DP;
     if (!first) {
@@ -455,18 +484,31 @@ static int blocks_for(int64_t work, int per = 256) {
   return (int)b;
 }
 
+template <typename T, int DP, int PH>
+static cudaError_t travel_p(const T* X, const View<T>& cv, const T* Y0, Groups gr, const UGeom& g,
+                            T c, int steps, int every, int slot0, T* pos, T* Wout, T* Sh, T* M2,
+                            cudaStream_t st) {
+  if (PH > 1) gr.per_set = (g.m + 32 / PH - 1) / (32 / PH);
+  const int64_t NG = (int64_t)g.B * gr.per_set;
+  constexpr int ws = team_warp_smem<T, DP, DP + 3>();
+  const int W = team_warps(NG, g.sms, ws, most_warps<T, DP>());
+  const bool res = team_resident<T, DP>(cv.P, g.n);
+  const int smem = res ? resident_team_smem<T, DP, DP + 3>(W, g.n) : group_team_smem<T, DP, DP + 3>(W);
+  const cudaError_t e = team_attr(unroll_travel<T, DP, PH>, smem);
+  if (e != cudaSuccess) return e;
+  unroll_travel<T, DP, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
+      X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, res ? 1 : 0);
+  return cudaGetLastError();
+}
+
 template <typename T, int DP>
 static cudaError_t travel_t(const T* X, const View<T>& cv, const T* Y0, const Groups& gr,
                             const UGeom& g, T c, int steps, int every, int slot0, T* pos, T* Wout,
                             T* Sh, T* M2, cudaStream_t st) {
-  const int64_t NG = (int64_t)g.B * gr.per_set;
-  constexpr int ws = team_warp_smem<T, DP, DP + 3>();
-  const int W = team_warps(NG, g.sms, ws), smem = group_team_smem<T, DP, DP + 3>(W);
-  const cudaError_t e = team_attr(unroll_travel<T, DP>, smem);
-  if (e != cudaSuccess) return e;
-  unroll_travel<T, DP><<<(unsigned)NG, 32 * W, smem, st>>>(X, cv, Y0, gr, g, c, steps, every,
-                                                             slot0, pos, Wout, Sh, M2);
-  return cudaGetLastError();
+  if constexpr (sizeof(T) == 4 && DP <= 16)
+    if (team_phases<T, DP>(cv.P, (int64_t)g.B * g.m, g.sms) == 4)
+      return travel_p<T, DP, 4>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
+  return travel_p<T, DP, 1>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
 }
 
 template <typename T>
@@ -482,25 +524,65 @@ cudaError_t unroll_forward_steps(const T* X, const View<T>& cv, const T* Y0, con
   return cudaErrorInvalidValue;
 }
 
-template <typename T, int DP>
-static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, const Groups& gx,
-                         const Groups& gr, const UGeom& g, T c, T inv_h2, double inv_h3, const T* Gin,
-                         T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX, int first,
-                         cudaStream_t st) {
-  const int64_t NG = (int64_t)g.B * gr.per_set, NX = (int64_t)g.B * gx.per_set;
-  constexpr int ws = team_warp_smem<T, DP, DP + 2>(), wp = team_warp_smem<T, 2 * DP + 4, DP>();
-  const int Ws = team_warps(NG, g.sms, ws), Wp = team_warps(NX, g.sms, wp);
-  const int smem_s = group_team_smem<T, DP, DP + 2>(Ws);
-  const int smem_p = list_team_smem<T, 2 * DP + 4, DP>(Wp);
-  cudaError_t e = team_attr(unroll_bwd_seed<T, DP>, smem_s);
-  if (e == cudaSuccess) e = team_attr(unroll_bwd_point<T, DP>, smem_p);
+// the seed-major pass; *groups: its groups in all (the entries of dh_part)
+template <typename T, int DP, int PH>
+static cudaError_t bwd_seed_p(const T* X, const View<T>& cv, const USegment<T>& sg, Groups gr,
+                              const UGeom& g, T c, T inv_h2, double inv_h3, const T* Gin, T* Gout,
+                              T* SD, T* bctr, T* breach, double* dh_part, int first,
+                              cudaStream_t st) {
+  if (PH > 1) gr.per_set = (g.m + 32 / PH - 1) / (32 / PH);
+  const int64_t NG = (int64_t)g.B * gr.per_set;
+  constexpr int ws = team_warp_smem<T, DP, DP + 2>();
+  const int W = team_warps(NG, g.sms, ws, most_warps<T, DP>());
+  const bool res = team_resident<T, DP>(cv.P, g.n);
+  const int smem = res ? resident_team_smem<T, DP, DP + 2>(W, g.n) : group_team_smem<T, DP, DP + 2>(W);
+  const cudaError_t e = team_attr(unroll_bwd_seed<T, DP, PH>, smem);
   if (e != cudaSuccess) return e;
-  unroll_bwd_seed<T, DP><<<(unsigned)NG, 32 * Ws, smem_s, st>>>(
-      X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, first);
-  unroll_bwd_point<T, DP><<<(unsigned)NX, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
-                                                                  SD, bctr, breach, dX, first);
+  unroll_bwd_seed<T, DP, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
+      X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, first, res ? 1 : 0);
   return cudaGetLastError();
 }
+
+template <typename T, int DP>
+static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, const Groups& gx,
+                         const Groups& gr, const UGeom& g, T c, T inv_h2, double inv_h3,
+                         const T* Gin, T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX,
+                         int first, cudaStream_t st) {
+  cudaError_t e = cudaErrorInvalidValue;
+  bool done = false;
+  if constexpr (sizeof(T) == 4 && DP <= 16)
+    if (team_phases<T, DP>(cv.P, (int64_t)g.B * g.m, g.sms) == 4) {
+      e = bwd_seed_p<T, DP, 4>(X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach,
+                               dh_part, first, st);
+      done = true;
+    }
+  if (!done)
+    e = bwd_seed_p<T, DP, 1>(X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach,
+                             dh_part, first, st);
+  if (e != cudaSuccess) return e;
+  const int64_t NX = (int64_t)g.B * gx.per_set;
+  constexpr int wp = team_warp_smem<T, 2 * DP + 4, DP>();
+  const int Wp = team_warps(NX, g.sms, wp, most_warps<T, DP>());
+  const int smem_p = list_team_smem<T, 2 * DP + 4, DP>(Wp);
+  e = team_attr(unroll_bwd_point<T, DP>, smem_p);
+  if (e != cudaSuccess) return e;
+  unroll_bwd_point<T, DP><<<(unsigned)NX, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
+                                                                 SD, bctr, breach, dX, first);
+  return cudaGetLastError();
+}
+
+// Groups of a set in the seed-major passes (and entries of dh_part per set).
+template <typename T>
+int unroll_seed_groups(int P, const UGeom& g, int per_set) {
+  const int64_t seeds = (int64_t)g.B * g.m;
+  int ph = 1;
+  if (g.DP <= 4) ph = team_phases<T, 4>(P, seeds, g.sms);
+  else if (g.DP <= 8) ph = team_phases<T, 8>(P, seeds, g.sms);
+  else if (g.DP <= 16) ph = team_phases<T, 16>(P, seeds, g.sms);
+  return ph == 1 ? per_set : (g.m + 32 / ph - 1) / (32 / ph);
+}
+template int unroll_seed_groups<float>(int, const UGeom&, int);
+template int unroll_seed_groups<double>(int, const UGeom&, int);
 
 template <typename T>
 cudaError_t unroll_backward_segment(const T* X, const View<T>& cv, const USegment<T>& sg,
