@@ -632,7 +632,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           at<int32_t>(ws, Lo.off_start), at<float>(ws, Lo.off_ctr), at<int32_t>(ws, Lo.off_npiv),
           at<float>(ws, Lo.off_rad), at<int2>(ws, Lo.off_table), s_);
       if (e != cudaSuccess || !cv.ext) return e;
-      return cells::launch_extents(rows, DP, P, cv.start, cv.ctr, at<float2>(ws, Lo.off_ext), s_);
+      return cells::launch_extents(rows, DP, P, at<int32_t>(ws, Lo.off_npiv), cv.start, cv.ctr, at<float2>(ws, Lo.off_ext), s_);
     };
     auto seeds_launch = [&](const RoundCtl* rcp, int N_, int max_N, int target_,
                             cudaStream_t s_) -> cudaError_t {
@@ -754,7 +754,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           e = launch_seed_init(Xs, n, DP, o.rng_seed, nullptr, 0, 0, N0, seed_idx, y, it, conv,
                                state, status, cs, init_state);
         if (e == cudaSuccess) e = launch_round_begin(rctl_round, N0, o.gamma, cs);
-        slot->kernels_pre = 3 + (P > 0 ? 4 : 0) + (cv.ext ? 1 : 0);
+        slot->kernels_pre = 3 + (P > 0 ? 5 : 0) + (cv.ext ? 1 : 0);
         // the rounds
         cudaGraph_t body = nullptr;
         if (e == cudaSuccess) e = add_conditional(cs, h_loop, cudaGraphCondTypeWhile, &body);
@@ -884,7 +884,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                     cosine ? 1 : 0, pcopy));
       if (tensor) FMS_LAUNCH(launch_tc_pack(Xs, n, d, DP, img, st));
       if (P > 0) {
-        n_launches += cv.ext ? 4 : 3;   // (and the one counted below)
+        n_launches += cv.ext ? 5 : 4;   // (and the one counted below)
         FMS_LAUNCH(sort_points(st));
       }
       N = N0;
@@ -1455,7 +1455,7 @@ cudaError_t group_step(const float* points, int64_t n, int32_t d, float scale, c
                                   at<int32_t>(ws, L.off_xperm), at<int32_t>(ws, L.off_start), ctr,
                                   npiv, at<float>(ws, L.off_rad), nullptr, st);
   if (e == cudaSuccess && d > 8)
-    e = cells::launch_extents(Xs, L.DP, L.P, at<int32_t>(ws, L.off_start), ctr,
+    e = cells::launch_extents(Xs, L.DP, L.P, npiv, at<int32_t>(ws, L.off_start), ctr,
                               at<float2>(ws, L.off_ext), st);
   if (e == cudaSuccess)
     e = cells::launch_sort<float>(Yp, 1, m, L.DP, false, L.P, at<void>(ws, L.off_sort), Ys,

@@ -236,8 +236,8 @@ cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points,
 
 // The extents of the P cells of one sorted set towards each other's centres
 // (View::ext), for d > 8.
-cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* start,
-                           const float* ctr, float2* ext, cudaStream_t st);
+cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* npiv,
+                           const int32_t* start, const float* ctr, float2* ext, cudaStream_t st);
 
 }  // namespace cells
 

@@ -36,20 +36,23 @@ __device__ __forceinline__ void load_pivots(const T* __restrict__ set, int64_t n
     pv[e] = set[pivot_row(e / DP, P, n) * DP + e % DP];
 }
 
-// Nearest of the pivots [p0, p1) in shared memory for two rows at a time
-// (ties: the lower pivot); b0, b1, i0, i1 carry the best so far.  Bound by FP32
-// issue: 2 DP operations per (row, pivot) pair plus the pivot's broadcast loads.
+// Nearest of the pivots [p0, p1) in shared memory for two rows at a time (ties: the
+// lower pivot); b0, b1, i0, i1 carry the best so far.  Half the squared distance
+// less the row's own part, |c|^2 / 2 - x.c, decides (half[p] = |c_p|^2 / 2; any
+// choice is a valid cell), which is DP multiply-adds a pair against the 2 DP of the
+// differences.  Bound by FP32 issue and the pivots' broadcast loads.
 template <typename T, int DP>
-__device__ __forceinline__ void nearest(const T (&x0)[DP], const T (&x1)[DP], const T* pv, int p0,
-                                        int p1, T& b0, T& b1, int& i0, int& i1) {
+__device__ __forceinline__ void nearest(const T (&x0)[DP], const T (&x1)[DP], const T* pv,
+                                        const T* half, int p0, int p1, T& b0, T& b1, int& i0,
+                                        int& i1) {
+#pragma unroll 2
   for (int p = p0; p < p1; ++p) {
-    T d0 = T(0), d1 = T(0);
+    T d0 = half[p], d1 = d0;
 #pragma unroll
     for (int k = 0; k < DP; ++k) {
       const T q = pv[p * DP + k];
-      const T e0 = x0[k] - q, e1 = x1[k] - q;
-      d0 += e0 * e0;
-      d1 += e1 * e1;
+      d0 -= x0[k] * q;
+      d1 -= x1[k] * q;
     }
     if (p == 0 || d0 < b0) {
       b0 = d0;
@@ -60,6 +63,25 @@ __device__ __forceinline__ void nearest(const T (&x0)[DP], const T (&x1)[DP], co
       i1 = p;
     }
   }
+}
+
+// Moves the n pivots to the first one as origin (kept in org: products of coordinates
+// far from zero would cancel) and sets half[p] = |c_p|^2 / 2.  Ends with a barrier.
+template <typename T, int DP>
+__device__ __forceinline__ void center_pivots(T* pv, T* org, T* half, int n) {
+  for (int k = threadIdx.x; k < DP; k += blockDim.x) org[k] = pv[k];
+  __syncthreads();
+  for (int p = threadIdx.x; p < n; p += blockDim.x) {
+    T s = T(0);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      const T v = pv[p * DP + k] - org[k];
+      pv[p * DP + k] = v;
+      s += v * v;
+    }
+    half[p] = T(0.5) * s;
+  }
+  __syncthreads();
 }
 
 template <typename T, int DP>
@@ -75,29 +97,52 @@ __device__ __forceinline__ void row_values(const T* p, T (&x)[DP]) {
 
 // First pass over the points: the nearest of the P0 strided pivots, and each
 // pivot's farthest row as (squared distance bits, row).
+// two rows a thread at a time (wide rows: fewer threads, for their registers)
+template <typename T, int DP>
+constexpr int assign_threads() {
+  return DP * sizeof(T) > 128 ? kChunkRows / 4 : kChunkRows / 2;
+}
+
+constexpr int kPivotRows = 512;   // (smaller blocks: 200,000 rows over 152 SMs leave less idle)
+
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
     pivot_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int P0,
                  int per, unsigned char* __restrict__ id, unsigned long long* __restrict__ far_) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
+  __shared__ T org[DP];
   T* pv = reinterpret_cast<T*>(cell_smem);                                        // [P0][DP]
-  unsigned long long* fs = reinterpret_cast<unsigned long long*>(pv + P0 * DP);   // [P0]
+  T* half = pv + P0 * DP;                                                         // [P0]
+  unsigned long long* fs = reinterpret_cast<unsigned long long*>(half + P0);      // [P0]
   const int b = blockIdx.x / per, blk = blockIdx.x % per;
   int nrows;
   const int64_t row0 = set_rows(offs, b, each, &nrows);
-  if ((int64_t)blk * kChunkRows >= nrows) return;
+  if ((int64_t)blk * kPivotRows >= nrows) return;
   const T* set = src + row0 * DP;
   load_pivots<T, DP>(set, nrows, P0, pv);
   for (int p = threadIdx.x; p < P0; p += blockDim.x) fs[p] = 0ull;
   __syncthreads();
-  const int r_end = min((int64_t)nrows, ((int64_t)blk + 1) * kChunkRows);
-  for (int r0 = blk * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
+  center_pivots<T, DP>(pv, org, half, P0);
+  const int r_end = min((int64_t)nrows, ((int64_t)blk + 1) * kPivotRows);
+  for (int r0 = blk * kPivotRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
     const int r1 = r0 + (int)blockDim.x < r_end ? r0 + (int)blockDim.x : r0;
     T x0[DP], x1[DP], b0 = T(0), b1 = T(0);
     row_values<T, DP>(set + (int64_t)r0 * DP, x0);
     row_values<T, DP>(set + (int64_t)r1 * DP, x1);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      x0[k] -= org[k];
+      x1[k] -= org[k];
+    }
     int i0 = 0, i1 = 0;
-    nearest<T, DP>(x0, x1, pv, 0, P0, b0, b1, i0, i1);
+    nearest<T, DP>(x0, x1, pv, half, 0, P0, b0, b1, i0, i1);
+    b0 = b1 = T(0);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      const T e0 = x0[k] - pv[i0 * DP + k], e1 = x1[k] - pv[i1 * DP + k];
+      b0 += e0 * e0;
+      b1 += e1 * e1;
+    }
     id[row0 + r0] = (unsigned char)i0;
     id[row0 + r1] = (unsigned char)i1;
     auto key = [](T v, int r) {
@@ -112,26 +157,32 @@ __global__ void __launch_bounds__(256)
     if (fs[p]) atomicMax(&far_[(int64_t)b * P0 + p], fs[p]);
 }
 
-// The pivots of a set: the P0 strided ones, then the farthest row of every cell
-// whose radius is over twice the lowest eighth's (a cluster that no strided pivot
-// hit hangs on to cells of other ones and would make their balls span both; in
-// many dimensions a few such clusters reach most cells, hence not the median).  Fills pv,
-// returns their number; sel: P0 ints, red: 64 ints of shared memory.
+// The pivots of a set (one block): the P0 strided ones, then the farthest row of
+// every cell whose radius is over twice the lowest eighth's (a cluster that no
+// strided pivot hit hangs on to cells of other ones and would make their balls span
+// both; in many dimensions a few such clusters reach most cells, hence not the
+// median).  Writes them to ctr and their number to npiv.
 template <typename T, int DP>
-__device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
-                          const unsigned long long* __restrict__ far_, T* pv, int* sel, int* red) {
+__global__ void __launch_bounds__(kMaxCells)
+    select_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int P,
+                  const unsigned long long* __restrict__ far_, T* __restrict__ ctr,
+                  int32_t* __restrict__ npiv) {
+  __shared__ float r2s[kMaxCells / 2];
   __shared__ float small;
-  load_pivots<T, DP>(set, nrows, P0, pv);
-  float* r2s = reinterpret_cast<float*>(sel);
-  const int p = threadIdx.x;
+  __shared__ int sel[kMaxCells], red[64];
+  const int b = blockIdx.x, P0 = P / 2, p = threadIdx.x;
+  int nrows;
+  const T* set = src + set_rows(offs, b, each, &nrows) * DP;
   unsigned long long k = 0;
+  float r2 = 0.0f;
   if (p < P0) {
-    k = far_[p];
-    r2s[p] = __uint_as_float((unsigned)(k >> 32));
+    k = far_[(int64_t)b * P0 + p];
+    r2 = __uint_as_float((unsigned)(k >> 32));
+    r2s[p] = r2;
+    sel[p] = (int)pivot_row(p, P0, nrows);
   }
   if (p == 0) small = INFINITY;
   __syncthreads();
-  const float r2 = p < P0 ? r2s[p] : 0.0f;
   if (p < P0) {
     int rank = 0;
     for (int q = 0; q < P0; ++q) rank += (r2s[q] < r2 || (r2s[q] == r2 && q < p)) ? 1 : 0;
@@ -141,66 +192,63 @@ __device__ int all_pivots(const T* __restrict__ set, int nrows, int P0,
   const int take = p < P0 && r2 > 4.0f * small ? 1 : 0;
   int K = 0;
   const int at = block_exclusive_scan(take, &K, red);
-  if (take) sel[at] = (int)(unsigned)k;
+  if (take) sel[P0 + at] = (int)(unsigned)k;
   __syncthreads();
-  for (int e = threadIdx.x; e < K * DP; e += blockDim.x)
-    pv[P0 * DP + e] = set[(int64_t)sel[e / DP] * DP + e % DP];
-  __syncthreads();
-  return P0 + K;
+  T* out = ctr + (int64_t)b * P * DP;
+  for (int e = threadIdx.x; e < P * DP; e += blockDim.x)   // (the rest: empty cells)
+    out[e] = e < (P0 + K) * DP ? set[(int64_t)sel[e / DP] * DP + e % DP] : T(0);
+  if (p == 0) npiv[b] = P0 + K;
 }
 
-// Second pass (EXTEND: over the points; else over the seeds, against the points'
-// finished pivots): the cell of every row, the rows of every (block, cell) in
-// counts [B][blocks][P], and for the points the pivots (in ctr).
+// The cell of every row, and the rows of every (block, cell) in counts [chunks][P].
+// EXTEND (the points): id holds the nearest strided pivot and only the added ones are
+// tried; else (the seeds) all of them.
 template <typename T, int DP, bool EXTEND>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(assign_threads<T, DP>())
     assign_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int per,
                   int P, unsigned char* __restrict__ id,
-                  const unsigned long long* __restrict__ far_, int32_t* __restrict__ counts,
-                  T* __restrict__ ctr, int32_t* __restrict__ npiv) {
+                  int32_t* __restrict__ counts, const T* __restrict__ ctr,
+                  const int32_t* __restrict__ npiv) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
-  __shared__ int red[64];
-  __shared__ int sel[kMaxCells];
+  __shared__ T org[DP];
   T* pv = reinterpret_cast<T*>(cell_smem);                 // [P][DP]
-  int* hist = reinterpret_cast<int*>(pv + (size_t)P * DP);   // [P]
+  T* half = pv + (size_t)P * DP;                           // [P]
+  int* hist = reinterpret_cast<int*>(half + P);            // [P]
   const int b = blockIdx.x / per, blk = blockIdx.x % per, P0 = P / 2;
   int nrows;
   const int64_t row0 = set_rows(offs, b, each, &nrows);
   if ((int64_t)blk * kChunkRows >= nrows) return;
   const T* set = src + row0 * DP;
   for (int p = threadIdx.x; p < P; p += blockDim.x) hist[p] = 0;
-  int np;
-  if (EXTEND) {
-    np = all_pivots<T, DP>(set, nrows, P0, far_ + (int64_t)b * P0, pv, sel, red);
-    if (blk == 0) {
-      for (int e = threadIdx.x; e < P * DP; e += blockDim.x)
-        ctr[(int64_t)b * P * DP + e] = e < np * DP ? pv[e] : T(0);   // (the rest: empty cells)
-      if (threadIdx.x == 0) npiv[b] = np;
-    }
-  } else {
-    np = npiv[b];
-    for (int e = threadIdx.x; e < np * DP; e += blockDim.x) pv[e] = ctr[(int64_t)b * P * DP + e];
-    __syncthreads();
-  }
+  const int np = npiv[b];
+  for (int e = threadIdx.x; e < np * DP; e += blockDim.x) pv[e] = ctr[(int64_t)b * P * DP + e];
+  __syncthreads();
+  center_pivots<T, DP>(pv, org, half, np);
   const int r_end = min((int64_t)nrows, ((int64_t)blk + 1) * kChunkRows);
   for (int r0 = blk * kChunkRows + threadIdx.x; r0 < r_end; r0 += 2 * blockDim.x) {
     const int r1 = r0 + (int)blockDim.x < r_end ? r0 + (int)blockDim.x : r0;
     T x0[DP], x1[DP], b0 = T(0), b1 = T(0);
     row_values<T, DP>(set + (int64_t)r0 * DP, x0);
     row_values<T, DP>(set + (int64_t)r1 * DP, x1);
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      x0[k] -= org[k];
+      x1[k] -= org[k];
+    }
     int i0 = 0, i1 = 0;
     if (EXTEND) {
       i0 = id[row0 + r0];
       i1 = id[row0 + r1];
+      b0 = half[i0];
+      b1 = half[i1];
 #pragma unroll
       for (int k = 0; k < DP; ++k) {
-        const T e0 = x0[k] - pv[i0 * DP + k], e1 = x1[k] - pv[i1 * DP + k];
-        b0 += e0 * e0;
-        b1 += e1 * e1;
+        b0 -= x0[k] * pv[i0 * DP + k];
+        b1 -= x1[k] * pv[i1 * DP + k];
       }
-      nearest<T, DP>(x0, x1, pv, P0, np, b0, b1, i0, i1);
+      nearest<T, DP>(x0, x1, pv, half, P0, np, b0, b1, i0, i1);
     } else {
-      nearest<T, DP>(x0, x1, pv, 0, np, b0, b1, i0, i1);
+      nearest<T, DP>(x0, x1, pv, half, 0, np, b0, b1, i0, i1);
     }
     id[row0 + r0] = (unsigned char)i0;
     atomicAdd(&hist[i0], 1);
@@ -215,12 +263,14 @@ __global__ void __launch_bounds__(256)
 }
 
 // Mean and radius of every cell (one block each): its rows are contiguous by now.
+constexpr int kBoundWarps = 8;
+
 template <typename T, int DP>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kBoundWarps)
     bound_kernel(const T* __restrict__ rows, const int64_t* __restrict__ offs, int each, int P,
                  const int32_t* __restrict__ start,
                  T* __restrict__ ctr, T* __restrict__ rad) {
-  __shared__ T red[4][DP];
+  __shared__ T red[kBoundWarps][DP];
   __shared__ T mean[DP];
   const int b = blockIdx.x / P, p = blockIdx.x % P, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int a = start[(int64_t)b * (P + 1) + p], e = start[(int64_t)b * (P + 1) + p + 1];
@@ -247,7 +297,9 @@ __global__ void __launch_bounds__(128)
   }
   __syncthreads();
   for (int k = threadIdx.x; k < DP; k += blockDim.x) {
-    const T v = (red[0][k] + red[1][k] + red[2][k] + red[3][k]) / T(e - a);
+    T v = red[0][k];
+    for (int u = 1; u < kBoundWarps; ++u) v += red[u][k];
+    v /= T(e - a);
     mean[k] = v;
     ctr[((int64_t)b * P + p) * DP + k] = v;
   }
@@ -267,7 +319,7 @@ __global__ void __launch_bounds__(128)
   if (lane == 0) red[w][0] = far_;
   __syncthreads();
   if (w == 0) {
-    far_ = warp_max(red[lane & 3][0]);
+    far_ = warp_max(red[lane % kBoundWarps][0]);
     if (lane == 0) rad[(int64_t)b * P + p] = csqrt(far_);
   }
 }
@@ -297,9 +349,9 @@ __global__ void __launch_bounds__(256)
   int tot = 0, before = 0;
   if ((int)threadIdx.x < P) {
     const int32_t* c = counts + chunk0(offs, b, per) * P + threadIdx.x;
-#pragma unroll 8
+#pragma unroll 16
     for (int q = 0; q < nblk; ++q) {
-      const int v = c[(int64_t)q * P];
+      const int v = __ldg(c + (int64_t)q * P);
       tot += v;
       if (q < blk) before += v;
     }
@@ -365,62 +417,97 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Thread q of a block keeps the unit vector from cell p's centre to cell q's, the
-// rows of p come by broadcast from shared memory.  DP multiply-adds a (row, q).
+// Thread q of a block keeps the unit vectors from cell p's centre to those of cells q
+// and q + P / 2, the rows of p come by broadcast from shared memory; DP multiply-adds
+// a (row, cell), and a row's loads serve two of them.  Only cells below *npiv have
+// rows, so the second half is often skipped.
 constexpr int kExtRows = 64;
 
-template <int DP>
-__global__ void __launch_bounds__(kMaxCells)
-    extent_kernel(const float* __restrict__ rows, int P, const int32_t* __restrict__ start,
-                  const float* __restrict__ ctr, float2* __restrict__ ext) {
-  __shared__ __align__(16) float tile[kExtRows * DP];
-  const int p = blockIdx.x, q = threadIdx.x;
-  const int a = start[p], e = start[p + 1];
-  float v[DP], d2 = 0.0f;
+template <int DP, int NU>
+__device__ __forceinline__ void extent_rows(const float* tile, int nr, const float (&v)[2][DP],
+                                            float (&far_)[2]) {
+#pragma unroll (DP <= 16 ? 4 : 2)
+  for (int r = 0; r < nr; ++r) {
+    float s[NU];
 #pragma unroll
-  for (int k = 0; k < DP; ++k) {
-    v[k] = ctr[q * DP + k] - ctr[p * DP + k];
-    d2 = fmaf(v[k], v[k], d2);
+    for (int u = 0; u < NU; ++u) s[u] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DP; k += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(tile + r * DP + k);
+#pragma unroll
+      for (int u = 0; u < NU; ++u) {
+        s[u] = fmaf(x.x, v[u][k], s[u]);
+        s[u] = fmaf(x.y, v[u][k + 1], s[u]);
+        s[u] = fmaf(x.z, v[u][k + 2], s[u]);
+        s[u] = fmaf(x.w, v[u][k + 3], s[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+      far_[u] = (s[u] > far_[u] || !(s[u] == s[u])) ? s[u] : far_[u];   // NaN wins
   }
-  const float dist = sqrtf(d2), inv = dist > 0.0f ? 1.0f / dist : 0.0f;
+}
+
+template <int DP>
+__global__ void __launch_bounds__(kMaxCells / 2)
+    extent_kernel(const float* __restrict__ rows, int P, const int32_t* __restrict__ npiv,
+                  const int32_t* __restrict__ start, const float* __restrict__ ctr,
+                  float2* __restrict__ ext) {
+  __shared__ __align__(16) float tile[kExtRows * DP];
+  const int p = blockIdx.x;
+  const int a = start[p], e = start[p + 1];
+  const bool both = *npiv > P / 2;
+  if (a + (int)blockIdx.y * kExtRows >= e && blockIdx.y > 0) return;
+  float v[2][DP], dist[2], far_[2] = {0.0f, 0.0f};
 #pragma unroll
-  for (int k = 0; k < DP; ++k) v[k] *= inv;
-  float far_ = 0.0f;
+  for (int u = 0; u < 2; ++u) {
+    const int q = threadIdx.x + u * (P / 2);
+    float d2 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DP; k += 4) {
+      const float4 c = __ldg(reinterpret_cast<const float4*>(ctr + q * DP + k));
+      const float4 o = __ldg(reinterpret_cast<const float4*>(ctr + p * DP + k));
+      v[u][k] = c.x - o.x;
+      v[u][k + 1] = c.y - o.y;
+      v[u][k + 2] = c.z - o.z;
+      v[u][k + 3] = c.w - o.w;
+    }
+#pragma unroll
+    for (int k = 0; k < DP; ++k) d2 = fmaf(v[u][k], v[u][k], d2);
+    dist[u] = sqrtf(d2);
+    const float inv = dist[u] > 0.0f ? 1.0f / dist[u] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < DP; ++k) v[u][k] *= inv;
+  }
   for (int r0 = a + blockIdx.y * kExtRows; r0 < e; r0 += gridDim.y * kExtRows) {
     const int nr = min(kExtRows, e - r0);
     __syncthreads();
     for (int i = threadIdx.x; i < nr * DP; i += blockDim.x)
-      tile[i] = rows[(int64_t)r0 * DP + i] - ctr[p * DP + i % DP];
+      tile[i] = rows[(int64_t)r0 * DP + i] - __ldg(ctr + p * DP + i % DP);
     __syncthreads();
-#pragma unroll 4
-    for (int r = 0; r < nr; ++r) {
-      float s = 0.0f;
-#pragma unroll
-      for (int k = 0; k < DP; k += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(tile + r * DP + k);
-        s = fmaf(x.x, v[k], s);
-        s = fmaf(x.y, v[k + 1], s);
-        s = fmaf(x.z, v[k + 2], s);
-        s = fmaf(x.w, v[k + 3], s);
-      }
-      far_ = (s > far_ || !(s == s)) ? s : far_;   // NaN wins
-    }
+    if (both) extent_rows<DP, 2>(tile, nr, v, far_);
+    else extent_rows<DP, 1>(tile, nr, v, far_);
   }
-  // (cleared to zero: not negative, so the bits order as integers do)
-  float* o = reinterpret_cast<float*>(ext + q * P + p);
-  atomicMax(reinterpret_cast<unsigned*>(o), __float_as_uint(far_) & 0x7fffffffu);
-  if (blockIdx.y == 0) o[1] = dist;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (u == 1 && !both) continue;   // (never looked up)
+    // (cleared to zero: not negative, so the bits order as integers do)
+    float* o = reinterpret_cast<float*>(ext + (threadIdx.x + u * (P / 2)) * P + p);
+    atomicMax(reinterpret_cast<unsigned*>(o), __float_as_uint(far_[u]) & 0x7fffffffu);
+    if (blockIdx.y == 0) o[1] = dist[u];
+  }
 }
 
-cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* start,
-                           const float* ctr, float2* ext, cudaStream_t st) {
+cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* npiv,
+                           const int32_t* start, const float* ctr, float2* ext, cudaStream_t st) {
   const cudaError_t e = cudaMemsetAsync(ext, 0, (size_t)P * P * 8, st);
   if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)P, 8);
+  // (cells differ in size by an order of magnitude: blocks past a cell's rows leave at once)
+  const dim3 grid((unsigned)P, 32);
   switch (DP) {
-    case 16: extent_kernel<16><<<grid, P, 0, st>>>(rows, P, start, ctr, ext); break;
-    case 32: extent_kernel<32><<<grid, P, 0, st>>>(rows, P, start, ctr, ext); break;
-    case 64: extent_kernel<64><<<grid, P, 0, st>>>(rows, P, start, ctr, ext); break;
+    case 16: extent_kernel<16><<<grid, P / 2, 0, st>>>(rows, P, npiv, start, ctr, ext); break;
+    case 32: extent_kernel<32><<<grid, P / 2, 0, st>>>(rows, P, npiv, start, ctr, ext); break;
+    case 64: extent_kernel<64><<<grid, P / 2, 0, st>>>(rows, P, npiv, start, ctr, ext); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -439,8 +526,8 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
   if (per64 * B > INT32_MAX || (int64_t)P * B > INT32_MAX) return cudaErrorInvalidValue;
   const int per = (int)per64;
   const unsigned grid = (unsigned)(per64 * B);
-  const size_t sm = (size_t)P * DP * sizeof(T) + (size_t)P * 4;
-  const size_t sm0 = (size_t)P / 2 * DP * sizeof(T) + (size_t)P / 2 * 8;
+  const size_t sm = (size_t)P * (DP + 1) * sizeof(T) + (size_t)P * 4;
+  const size_t sm0 = (size_t)P / 2 * (DP + 1) * sizeof(T) + (size_t)P / 2 * 8;
   cudaError_t e = cudaSuccess;
   if (sm > 40 * 1024) {   // (static arrays count against the default 48 KB)
     e = cudaFuncSetAttribute(assign_kernel<T, DP, true>,
@@ -453,17 +540,21 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
   if (points) {
     e = cudaMemsetAsync(far_, 0, (size_t)B * (P / 2) * 8, st);
     if (e != cudaSuccess) return e;
-    pivot_kernel<T, DP><<<grid, 256, sm0, st>>>(src, offs, (int)nrows, P / 2, per, id, far_);
-    assign_kernel<T, DP, true><<<grid, 256, sm, st>>>(src, offs, (int)nrows, per, P, id, far_, counts, ctr,
-                                                      npiv);
+    const int64_t pper = (nrows + kPivotRows - 1) / kPivotRows;
+    if (pper * B > INT32_MAX) return cudaErrorInvalidValue;
+    pivot_kernel<T, DP><<<(unsigned)(pper * B), 256, sm0, st>>>(src, offs, (int)nrows, P / 2,
+                                                               (int)pper, id, far_);
+    select_kernel<T, DP><<<B, kMaxCells, 0, st>>>(src, offs, (int)nrows, P, far_, ctr, npiv);
+    assign_kernel<T, DP, true><<<grid, assign_threads<T, DP>(), sm, st>>>(
+        src, offs, (int)nrows, per, P, id, counts, ctr, npiv);
   } else {
-    assign_kernel<T, DP, false><<<grid, 256, sm, st>>>(src, offs, (int)nrows, per, P, id, nullptr, counts,
-                                                       ctr, npiv);
+    assign_kernel<T, DP, false><<<grid, assign_threads<T, DP>(), sm, st>>>(
+        src, offs, (int)nrows, per, P, id, counts, ctr, npiv);
   }
   scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, (int)nrows, per, P, id, counts, dst, perm, start,
                                              table, group_cap(nrows, P, group), group, gcell);
   if (points)
-    bound_kernel<T, DP><<<(unsigned)(P * B), 128, 0, st>>>(dst, offs, (int)nrows, P, start,
+    bound_kernel<T, DP><<<(unsigned)(P * B), 32 * kBoundWarps, 0, st>>>(dst, offs, (int)nrows, P, start,
                                                                         ctr, rad);
   return cudaGetLastError();
 }
