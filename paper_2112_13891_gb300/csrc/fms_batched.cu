@@ -110,13 +110,14 @@ struct BLayout {
       mscore, modes_full, part, sc, task_off, part_off, list_off, totals, counters, pt_off, status,
       sorted, start, ctr, npiv, rad, sort, wlast, total;
   int DP, DA, R, TW, P;
+  bool queued;
   Tiling tl;
 };
 
-// d > 7: every seed is taken to convergence by one block (k_travel.cu).  For
-// d <= 7 a low-d warp task shares each point it loads among up to 8 seeds and an
-// update of all sets is one launch.
-bool by_queue(int d) { return d > 7; }
+// Every seed is taken to convergence by one block (k_travel.cu).  For d <= 7 and
+// sets too small to gain from their cells, a low-d warp task shares each point it
+// loads among up to 8 seeds and an update of all sets is one launch.
+bool by_queue(int d, int64_t total, int B) { return d > 7 || total / B >= 2048; }
 
 // Cells of every set (0: sets too small to gain from them): as for one set of the
 // mean size, half as many at most (4 to 40 clusters a set; the cost of finding the
@@ -127,7 +128,7 @@ int batch_cells(int64_t total, int B) {
   return P < 128 ? P : 128;
 }
 
-// Partial-sum capacity (d <= 7): per set C_b * cnt_b * DA with C_b from choose_chunks
+// Partial-sum capacity (not queued): per set C_b * cnt_b * DA with C_b from choose_chunks
 // (<= 4 * tl.target_warps / G_b + 1), so sum_b <= (4 * TWb * B + total_groups) * R * DA.
 BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw_mult,
                      int min_chunk) {
@@ -135,7 +136,8 @@ BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw
   L.DP = padded(d);
   L.DA = step_accumulators(d);
   L.R = step_seeds_per_warp(d);
-  L.P = by_queue(d) ? batch_cells(total, B) : 0;
+  L.queued = by_queue(d, total, B);
+  L.P = L.queued ? batch_cells(total, B) : 0;
   L.TW = (sms > 0 ? sms : 1) * step_resident_warps_per_sm(d);
   // every set gets a share of the GPU's warps for its chunking (all sets run
   // in the same launches)
@@ -172,7 +174,7 @@ BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw
   L.mdone = take((size_t)total * 4);
   L.mscore = take((size_t)total * 8);
   L.modes_full = take((size_t)total * d * 4);
-  L.part = take(by_queue(d) ? 0 : part_floats * 4);
+  L.part = take(L.queued ? 0 : part_floats * 4);
   L.sc = take((size_t)B * sizeof(SetCtl));
   L.task_off = take((size_t)(B + 1) * 8);
   L.part_off = take((size_t)(B + 1) * 8);
@@ -181,7 +183,7 @@ BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw
   L.counters = take(64);
   L.pt_off = take((size_t)(B + 1) * 8);
   L.status = take(64);
-  if (by_queue(d)) L.wlast = take((size_t)total * 4);
+  if (L.queued) L.wlast = take((size_t)total * 4);
   if (L.P > 0) {
     L.sorted = take((size_t)total * L.DP * 4);
     L.start = take((size_t)B * (L.P + 1) * 4);
@@ -355,7 +357,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
   int dev = 0;
   cudaGetDevice(&dev);
   const auto key = std::make_tuple(dev, (int)d, ilog2(total), ilog2(B));
-  bool tuned = by_queue(d);   // (the queue has no tiling)
+  bool tuned = by_queue(d, total, B);   // (the queue has no tiling)
   std::pair<int, int> cfg{kTwMults[0], d <= 7 ? kMinChunksLow[1] : kMinChunksWide[1]};
   if (!tuned) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -415,7 +417,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
     int32_t* counters = at<int32_t>(ws, Lo.counters);
     int64_t* pt_off = at<int64_t>(ws, Lo.pt_off);
     uint32_t* status = at<uint32_t>(ws, Lo.status);
-    const bool queued = by_queue(d);
+    const bool queued = Lo.queued;
     float* wlast = at<float>(ws, Lo.wlast);
     float* rows = Lo.P > 0 ? at<float>(ws, Lo.sorted) : Xs;
     cells::View<float> cv{};
@@ -717,7 +719,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       stats->n_discarded = seeds - kept_n;
       stats->n_modes = modes;
       stats->refine_iterations = refines;
-      // (d > 7: pack, the sort's five, seed init; per round seeds, travel, kept,
+      // (queued: pack, the sort's five, seed init; per round seeds, travel, kept,
       // (density,) prune, advance, seed init; setup, queue, refinement or density)
       stats->kernel_launches =
           queued ? 2 + (cv.P > 0 ? 5 : 0) + (o.gamma >= 1.f ? 7 : 6) * rounds + 3 + 3

@@ -133,7 +133,7 @@ struct SetCtl {
   int32_t rr;      // refinement clock
   int32_t rdone;
   int32_t Mr;      // modes after refinement and the second prune
-  int32_t total;   // (d > 7) seeds converged so far, in all rounds
+  int32_t total;   // (queued) seeds converged so far, in all rounds
   int64_t evals;
 };
 

@@ -7,7 +7,7 @@
 // control blocks (SetCtl) hold each set's clock, counts and chunking; a plan
 // (prefix sums over sets of warp tasks, partial-sum blocks and list entries)
 // lets one launch of the step / update kernels map a global task or list
-// index to (set, local index) by binary search.  For d > 7 one queue of all sets'
+// index to (set, local index) by binary search.  For d > 7, or large sets, one queue of all sets'
 // seeds takes each of them to convergence in one launch instead (k_travel.cu).  One CTA per set runs the
 // per-set bookkeeping (compaction under the Early Stopping clock rule, kept
 // list, prune, ordering); the last CTA to finish (atomic ticket, no waiting)
@@ -479,7 +479,7 @@ __global__ void batched_score(const float* __restrict__ part, const SetCtl* __re
 }
 
 // ---------------------------------------------------------------------------
-// d > 7: the queues of k_travel.cu
+// The queues of k_travel.cu
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int queue_count(const SetCtl& c, int kind) {
   if (kind == kPlanActive) return __ldcg(&c.s);
