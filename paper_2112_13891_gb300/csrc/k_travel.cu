@@ -213,14 +213,14 @@ __global__ void __launch_bounds__(512)
 // row (four coordinates each), so row-major rows are read as whole 128-byte
 // lines.  Bound by L2 bandwidth (4 DP bytes a row and seed).
 // ---------------------------------------------------------------------------
-constexpr int kSeedWarps = 8;    // one set: as many warps as the seeds leave idle
+constexpr int kSeedWarps = 16;   // one set: as many warps as the seeds leave idle
 constexpr int kQueueWarps = 4;   // many sets: more seeds in flight instead
 
 template <int DP, typename ST, int NW>
 struct SeedSmem {
   float y[DP];
   int2 list[cells::kMaxCells];
-  unsigned mask[cells::kMaxCells / 32], near[NW];
+  unsigned mask[cells::kMaxCells / 32 > NW ? cells::kMaxCells / 32 : NW], near[NW];
   ST red[NW][DP + 1];
   ST tot[DP + 1];
   float cut;
@@ -240,7 +240,7 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
     nl = 1;
     __syncthreads();
   } else {
-    constexpr int U = cells::kMaxCells / 32 / NW;   // cells of a thread
+    constexpr int U = (cells::kMaxCells / 32 + NW - 1) / NW;   // cells of a thread
     const float rc = sqrtf(sh.cut);
     float a[U], far_[U];   // distance of the cell's centre, reach of its rows from there
     int2 mine[U];
@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kQueueWarps * 32)
 }
 
 int seed_grid(int max_seeds, int sms) {
-  const int g = sms * 4;   // (resident blocks; each takes its seeds in turn)
+  const int g = sms * 2;   // (resident blocks; each takes its seeds in turn)
   return max_seeds < g ? (max_seeds > 0 ? max_seeds : 1) : g;
 }
 
