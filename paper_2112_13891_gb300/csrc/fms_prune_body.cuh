@@ -1,51 +1,76 @@
 // Device body of the sorted prune, shared by the single-set and batched kernels.
 #pragma once
 
+#include <type_traits>
+
 #include "fms_internal.cuh"
 
 namespace fms {
 
-// Same prune with the candidates in shared memory, in two parallel stages:
-// (1) the block sorts the candidates by (score descending, rank ascending):
-// up to 512 candidates by counting, for each, the candidates ordered before
-// it (FP32 scores as one packed 64-bit key comparison per pair), else with a
-// bitonic sort; (2) the sorted list is walked 32 candidates at a time, one
-// candidate per lane.  Register visit (d = DT known at compile time, the
-// candidates' coordinates preloaded into shared memory): every warp holds the
-// batch in registers, tests it against its share of the modes accepted so
-// far and computes one member's neighbour mask by shuffles; warp 0 accepts
-// the survivors lowest lane first with those masks.  Block visit
-// (any d): the batch is staged in a transposed, padded tile (conflict-free
-// per-lane reads; two tiles, warp 1 stages the next batch while the current
-// one is tested), every warp tests it against its share of the accepted
-// modes, warp v records which batch members lie within r of member v (a
-// 32-bit mask), and warp 0 resolves the survivors in order with those masks.
-// Both use the distance of the test against an accepted mode for every
-// suppression, so the accepted set and its order are those of the one-by-one
-// greedy visit.  With acc_in_smem the accepted modes' coordinates are kept in
-// shared memory, else read back from global memory (all lanes read the same
-// row).
-constexpr int kPruneTileStride = 33;   // padded row of the transposed batch tile
+// Same prune with the candidates in shared memory, in two stages: (1) the block
+// sorts the candidates by (score descending, rank ascending); (2) it takes batches
+// of up to 32 from the list of those still alive, resolves each batch in visit
+// order, tests the whole list against the modes accepted from it and compacts the
+// list in place.
+//
+// Candidates that converged to one mode have nearly the same score and stand in a
+// row, so a batch takes its members from as far down the list as it can: a
+// candidate within r of the one before it is passed over (it is expected to fall
+// to the mode its predecessor fell to).  The test of the list shows whether each
+// one passed over does lie within r of a mode accepted before its turn; at the
+// first that does not, the batch is cut: modes after it are put back, it heads the
+// next batch, and from then on batches pass over nothing.  Every suppression uses
+// the distance of the one-by-one greedy visit, so the accepted set and its order
+// are that visit's.
+//
+// What bounds it is the chain of barriers and dependent shared memory loads of
+// one block (a batch is nine barriers, 3 us at d = 2 and 5 at d = 32), hence few
+// batches: of 32 modes, not of 32 candidates.  2,000 candidates of 5 modes at d = 2
+// take 22 us (batches of 32 candidates, each tested against all modes so far: 50);
+// the three prunes of a 65,536 x 32 clustering of 64 modes 48 (135), its FP64 prune
+// 24 (72), the two of 200,000 x 16 directions 19 (34) and 10 (19).
+constexpr int kPruneTileStride = 36;   // row of the transposed batch tile (16-byte aligned)
 constexpr int kPruneMaxDim = 64;
+constexpr int kPruneThreads = 1024;    // block size of the sorted prune
+constexpr int kPruneModes = 4;         // modes x entries of one thread at a time: a broadcast
+constexpr int kPruneEntries = 4;       //   of 16 bytes takes the shared memory pipe 4 cycles
 
-// Bytes of the sort keys, indices and 96 scratch ints (batch flags, count,
-// the batch's neighbour masks).
-constexpr int kPruneScratchInts = 96;
-template <typename ST>
-__host__ __device__ inline size_t greedy_keys_bytes(int P) {
-  return (((size_t)P * (sizeof(ST) + 4) + kPruneScratchInts * 4 + 15) / 16) * 16;
+// Wider FP32 candidates are tested by their first coordinates, and the whole
+// distance is taken only of the pairs that these leave within r: of 64 modes and
+// 512 candidates at d = 32 that is a quarter of the arithmetic of one SM.
+constexpr int kPruneFirst = 8;
+
+// sort slots: a power of two
+__host__ __device__ inline int prune_slots(int K) {
+  int P = 32;
+  while (P < K) P <<= 1;
+  return P;
 }
 
-// preload: every candidate's coordinates are copied to shared memory once,
-// before the sort (P x d values, transposed), so that staging a batch reads
-// shared memory instead of two dependent global loads per batch.
-template <typename PT, typename ST>
-__host__ __device__ inline size_t greedy_sorted_smem(int K, int d, int P, bool acc_in_smem,
-                                                     bool preload = false) {
-  return greedy_keys_bytes<ST>(P) +
-         2 * (size_t)kPruneMaxDim * kPruneTileStride * sizeof(PT) +
-         (preload ? (size_t)P * d * sizeof(PT) : 0) +
-         (acc_in_smem ? (size_t)K * d * sizeof(PT) : 0);
+// row length of the coordinates: odd, so that neither storing columns nor reading
+// rows meets a bank twice
+__host__ __device__ inline int prune_row(int K) { return (K + 31) / 32 * 32 + 1; }
+
+// two buffers of rank words; masks, modes' norms and indices, members' places;
+// horizon and cut; masks of the groups
+constexpr int kPruneScratchInts = 64 + 4 * 32 + 32 + kPruneThreads;
+
+// Shared memory for up to K candidates of d coordinates: the batch's tile and
+// the modes accepted from it, scratch, sort keys (then the list), the visit order
+// and the first `pre` coordinates of every candidate in that order, transposed.
+// FP64 positions are held rounded to FP32 (see PruneTest).
+template <typename ST>
+__host__ __device__ inline size_t greedy_sorted_smem(int K, int d, int pre) {
+  return (size_t)((d + 3) & ~3) * (kPruneTileStride + 32) * 4 + kPruneScratchInts * 4 +
+         (size_t)prune_slots(K) * (sizeof(ST) + 4) + (size_t)prune_row(K) * pre * 4;
+}
+
+// The coordinates to preload: all, else those of the first test, else none.
+template <typename ST>
+__host__ __device__ inline int greedy_sorted_pre(int K, int d, size_t limit) {
+  if (greedy_sorted_smem<ST>(K, d, d) <= limit) return d;
+  if (d > kPruneFirst && greedy_sorted_smem<ST>(K, d, kPruneFirst) <= limit) return kPruneFirst;
+  return 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -191,277 +216,532 @@ __device__ void greedy_global_body(const int32_t* __restrict__ cand_row, const i
   if (threadIdx.x == 0) *M_out = M;
 }
 
-template <typename PT, typename ST, int DT = 0>
+// Sort key of a score: ascending order of the keys is the visit order.
+__device__ __forceinline__ unsigned visit_key(float f) {
+  if (!(f == f)) f = -INFINITY;   // a NaN score counts as -inf
+  if (f == 0.0f) f = 0.0f;        // -0 and +0 are equal scores
+  const unsigned u = __float_as_uint(f);
+  return (u & 0x80000000u) ? u : ~(u | 0x80000000u);
+}
+
+__device__ __forceinline__ unsigned long long visit_key(double f) {
+  if (!(f == f)) f = -INFINITY;
+  if (f == 0.0) f = 0.0;
+  const unsigned long long u = (unsigned long long)__double_as_longlong(f);
+  return (u >> 63) ? u : ~(u | (1ull << 63));
+}
+
+// Whether two candidates lie within r.  FP32 positions: the squared distance
+// itself.  FP64 positions: the distance of the positions rounded to FP32 decides
+// where it is surely right, else FP64 does (its rate is 1/64 of FP32's, and all
+// but the pairs within about 1e-6 of r are decided in FP32).  Rounding moves a
+// position by at most u|x|, u = 2^-24, and a difference by another u|e|; the sum
+// and the root are good to (d + 4) u.  So the FP32 distance differs from the
+// true one by less than (d + 8) u times itself plus u (|x| + |y|); the margins
+// here are twice that.
+template <typename PT>
+struct PruneTest {
+  const PT* pos;
+  const int32_t* cand_row;
+  int DP, d;
+  PT r2;
+  float lo, hi;   // FP64 positions: surely within r below lo, surely not above hi
+  __device__ PruneTest(const PT* pos_, const int32_t* rows, int DP_, int d_, PT r2_)
+      : pos(pos_), cand_row(rows), DP(DP_), d(d_), r2(r2_), lo(0.0f), hi(0.0f) {
+    if constexpr (sizeof(PT) == 8) {
+      const float r = sqrtf((float)r2), c = (float)(2 * d + 32) * 5.9604645e-8f;
+      const bool usable = r > 1e-10f && r < 1e10f;   // no under- or overflow of a square near r
+      lo = usable ? r - r * c : -INFINITY;
+      hi = usable ? r + r * c : INFINITY;
+    }
+  }
+  __device__ __forceinline__ int64_t row(int q) const {
+    return cand_row ? (int64_t)cand_row[q] : (int64_t)q;
+  }
+  // s, a, b: squared FP32 distance and squared norms of candidates p and q
+  __device__ __forceinline__ bool within(float s, float a, float b, int p, int q) const {
+    if constexpr (sizeof(PT) == 4) {
+      return s < r2;
+    } else {
+      const float D = sqrtf(s), m = (sqrtf(a) + sqrtf(b)) * 2.3841858e-7f + 1e-17f;
+      if (D + m < lo) return true;
+      if (D - m > hi && D < 1e15f) return false;
+      const PT *x = pos + row(p) * DP, *y = pos + row(q) * DP;
+      PT d2 = 0;
+      for (int k = 0; k < d; ++k) {
+        const PT e = x[k] - y[k];
+        d2 += e * e;
+      }
+      return d2 < r2;
+    }
+  }
+};
+
+// A candidate in the sort: key, then index.  FP32 scores: both in one integer.
+struct VisitF {
+  unsigned long long v;
+  __device__ __forceinline__ void set(unsigned key, int i) {
+    v = ((unsigned long long)key << 32) | (unsigned)i;
+  }
+  __device__ __forceinline__ void pad() { v = ~0ull; }
+  __device__ __forceinline__ int index() const { return (int)(unsigned)v; }
+  __device__ __forceinline__ bool before(const VisitF& o) const { return v < o.v; }
+  __device__ __forceinline__ VisitF shfl_xor(int m) const {
+    VisitF o;
+    o.v = __shfl_xor_sync(kFull, v, m);
+    return o;
+  }
+  __device__ __forceinline__ void put(unsigned char* buf, int, int i) const {
+    reinterpret_cast<unsigned long long*>(buf)[i] = v;
+  }
+  __device__ __forceinline__ void get(const unsigned char* buf, int, int i) {
+    v = reinterpret_cast<const unsigned long long*>(buf)[i];
+  }
+};
+
+struct VisitD {
+  unsigned long long k;
+  int at;
+  __device__ __forceinline__ void set(unsigned long long key, int i) {
+    k = key;
+    at = i;
+  }
+  __device__ __forceinline__ void pad() {
+    k = ~0ull;
+    at = INT32_MAX;
+  }
+  __device__ __forceinline__ int index() const { return at; }
+  __device__ __forceinline__ bool before(const VisitD& o) const {
+    return k < o.k || (k == o.k && at < o.at);
+  }
+  __device__ __forceinline__ VisitD shfl_xor(int m) const {
+    VisitD o;
+    o.k = __shfl_xor_sync(kFull, k, m);
+    o.at = __shfl_xor_sync(kFull, at, m);
+    return o;
+  }
+  __device__ __forceinline__ void put(unsigned char* buf, int P, int i) const {
+    reinterpret_cast<unsigned long long*>(buf)[i] = k;
+    reinterpret_cast<int*>(buf + (size_t)P * 8)[i] = at;
+  }
+  __device__ __forceinline__ void get(const unsigned char* buf, int P, int i) {
+    k = reinterpret_cast<const unsigned long long*>(buf)[i];
+    at = reinterpret_cast<const int*>(buf + (size_t)P * 8)[i];
+  }
+};
+
+// Bitonic sort of P slots in registers, E a thread of the first P / E: strides
+// below E within the thread, up to 16 E by shuffles, beyond through `buf`.  At P =
+// 2,048, E = 8, that is 30, 30 and 6 of the 66 steps.  What bounds it is some 15
+// instructions a slot and step (12 us at 2,048 slots, as with a slot a thread), and
+// beyond 8,192 slots it would be the barriers of a sort in shared memory (9,000
+// candidates: 195 us there, 112 so).
+template <typename V, typename ST, int E>
+__device__ __forceinline__ void sort_slots(const ST* __restrict__ score, int K, int P,
+                                           unsigned char* buf, int* order) {
+  V x[E];
+  const int tid = threadIdx.x, T = P / E;
+  const bool in = tid < T;   // (whole warps)
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = tid * E + e;
+    if (i < K) x[e].set(visit_key(score[i]), i);
+    else x[e].pad();
+  }
+  auto merge = [&](int e, const V& o, int k, int j) {
+    const int i = tid * E + e;
+    const bool low = ((i & j) == 0) == ((i & k) == 0);   // this slot takes the earlier one
+    if (o.before(x[e]) == low) x[e] = o;
+  };
+  for (int k = 2; k <= P; k <<= 1) {
+    for (int j = k >> 1; j >= 32 * E; j >>= 1) {
+      if (in)
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[e].put(buf, P, e * T + tid);
+      __syncthreads();
+      if (in)
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          V o;
+          o.get(buf, P, e * T + (tid ^ (j / E)));
+          merge(e, o, k, j);
+        }
+      __syncthreads();
+    }
+    if (!in) continue;
+    for (int j = min(k >> 1, 16 * E); j >= E; j >>= 1)
+#pragma unroll
+      for (int e = 0; e < E; ++e) merge(e, x[e].shfl_xor(j / E), k, j);
+#pragma unroll
+    for (int j = E / 2; j > 0; j >>= 1)
+      if (j < k)
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (!(e & j)) {
+            const V a = x[e], b = x[e | j];
+            merge(e, b, k, j);
+            merge(e | j, a, k, j);
+          }
+  }
+  if (in)
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (tid * E + e < K) order[tid * E + e] = x[e].index();
+}
+
+// order[i] = the i-th candidate in visit order.  buf: prune_slots(K) x (sizeof(ST)
+// + 4) bytes, the last four a slot of which are `order`.
+template <typename ST>
+__device__ void visit_order(const ST* __restrict__ score, int K, unsigned char* buf, int* order) {
+  using V = typename std::conditional<sizeof(ST) == 4, VisitF, VisitD>::type;
+  const int P = prune_slots(K);
+  if (P <= 256) {
+    // a candidate's place is the number of those before it: four candidates a
+    // thread, a group of 4,096 / P lanes (16 or 32, then several groups) to each four
+    constexpr int Q = 4;
+    const int G = min(32, Q * kPruneThreads / P), c = threadIdx.x / G * Q, at = threadIdx.x % G;
+    if ((int)threadIdx.x < P) {
+      V x;
+      if ((int)threadIdx.x < K) x.set(visit_key(score[threadIdx.x]), threadIdx.x);
+      else x.pad();
+      x.put(buf, P, threadIdx.x);
+    }
+    __syncthreads();
+    int r[Q] = {0, 0, 0, 0};
+    if (c < P) {   // (whole warps)
+      V x[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) x[q].get(buf, P, c + q);
+#pragma unroll 4
+      for (int j = at; j < P; j += G) {
+        V o;
+        o.get(buf, P, j);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) r[q] += o.before(x[q]) ? 1 : 0;
+      }
+      for (int o = G >> 1; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) r[q] += __shfl_xor_sync(kFull, r[q], o);
+    }
+    __syncthreads();
+    if (at == 0)
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (c + q < K) order[r[q]] = c + q;
+  } else if (P <= 512) {
+    sort_slots<V, ST, 2>(score, K, P, buf, order);
+  } else if (P <= 1024) {
+    sort_slots<V, ST, 4>(score, K, P, buf, order);
+  } else if (P <= 8 * kPruneThreads) {
+    sort_slots<V, ST, 8>(score, K, P, buf, order);
+  } else {   // at most 16,384 fit in shared memory
+    sort_slots<V, ST, 16>(score, K, P, buf, order);
+  }
+  __syncthreads();
+}
+
+// Number of true flags of the block's threads below this one, and in all (*total):
+// one barrier.  `words` is one of two buffers of 32, used in turn.
+__device__ __forceinline__ int block_rank(bool flag, int* total, unsigned* words) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned m = __ballot_sync(kFull, flag);
+  if (lane == 0) words[warp] = m;
+  __syncthreads();
+  const int n = lane < (int)(blockDim.x >> 5) ? __popc(words[lane]) : 0;
+  *total = __reduce_add_sync(kFull, n);
+  return __reduce_add_sync(kFull, lane < warp ? n : 0) + __popc(m & ((1u << lane) - 1u));
+}
+
+__device__ __forceinline__ void load_row4(const float* p, float x[4]) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+}
+
+__device__ __forceinline__ void load_row4(const double* p, float x[4]) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+  x[0] = (float)a.x, x[1] = (float)a.y, x[2] = (float)b.x, x[3] = (float)b.y;
+}
+
+// Two FP32 values in one register pair: x - m and s + e e for two modes at once,
+// each half rounded as the scalar operation is.
+__device__ __forceinline__ void add_square2(unsigned long long& s, unsigned long long x,
+                                            unsigned long long minus_m) {
+  unsigned long long e;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(e) : "l"(x), "l"(minus_m));
+  asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s) : "l"(e));
+}
+
+template <typename PT, typename ST>
 __device__ void greedy_sorted_body(const int32_t* __restrict__ cand_row, const int K,
                                    const ST* __restrict__ score, const PT* __restrict__ pos,
                                    int DP, int d, PT r2, int32_t* __restrict__ accepted,
-                                   int32_t* __restrict__ M_out, int P, unsigned char* smem,
-                                   bool acc_in_smem = true, bool preload = false) {
-  // layout: keys[P] (ST), idx[P] (int), scratch[96] (int), ctile[2][64 x 33] (PT),
-  // [cpre[d][P] (PT)], [apos[K*d] (PT)]
-  ST* keys = reinterpret_cast<ST*>(smem);
-  int* idx = reinterpret_cast<int*>(keys + P);
-  PT* ctile2 = reinterpret_cast<PT*>(smem + greedy_keys_bytes<ST>(P));
-  constexpr int kTile = kPruneMaxDim * kPruneTileStride;
-  PT* cpre = ctile2 + 2 * kTile;
-  PT* apos = cpre + (preload ? (size_t)P * d : 0);
-  auto row_of = [&](int q) -> int64_t { return cand_row ? (int64_t)cand_row[q] : (int64_t)q; };
-  if (preload)   // read by stage() after the sort's barriers
-    for (int t = threadIdx.x; t < K; t += blockDim.x) {
-      const PT* src = pos + row_of(t) * DP;
-      for (int k = 0; k < d; ++k) cpre[(size_t)k * P + t] = src[k];
-    }
-  // order: "a before b" iff a.key > b.key, or equal keys and a.idx < b.idx
-  if (sizeof(ST) == 4 && K <= 512 && K <= (int)blockDim.x) {
-    // FP32 scores: (score, index) packed into one 64-bit key whose unsigned
-    // order is the visit order (score bits mapped to an unsigned order, the
-    // complemented index below them), so the rank count is one comparison
-    // per pair; the keys occupy the keys + idx region until the ranks are known
-    unsigned long long* vk = reinterpret_cast<unsigned long long*>(smem);
-    const int t = threadIdx.x;
-    unsigned long long mv = 0;
-    if (t < K) {
-      float f = (float)score[t];
-      if (!(f == f)) f = -INFINITY;   // a NaN score counts as -inf
-      if (f == 0.0f) f = 0.0f;        // -0 and +0 are equal scores
-      unsigned u = __float_as_uint(f);
-      u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-      mv = ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)t);
-      vk[t] = mv;
-    }
-    __syncthreads();
-    int rank = 0;
-    if (t < K) {
-      int j = 0;
-      for (; j + 8 <= K; j += 8) {
-        unsigned long long kk[8];
+                                   int32_t* __restrict__ M_out, unsigned char* smem,
+                                   int pre) {
+  constexpr bool kWide = sizeof(PT) == 8;
+  const int P = prune_slots(K), XS = prune_row(K), d4 = (d + 3) & ~3;
+  float* tile = reinterpret_cast<float*>(smem);             // [d4][kPruneTileStride]
+  float* modes = tile + (size_t)d4 * kPruneTileStride;      // [d4][32], negated
+  unsigned* words = reinterpret_cast<unsigned*>(modes + (size_t)d4 * 32);   // two buffers
+  unsigned* near = words + 64;
+  float* mnorm = reinterpret_cast<float*>(near + 32);
+  int* mcand = reinterpret_cast<int*>(mnorm + 32);
+  int* member = mcand + 32;                                 // a batch member's place in the list
+  int* horizon = member + 32;                               // the batch's members lie before it
+  int* cut = horizon + 1;
+  unsigned* part = reinterpret_cast<unsigned*>(horizon + 32);
+  unsigned char* buf = reinterpret_cast<unsigned char*>(part + kPruneThreads);
+  // an entry: 2 x its place in the visit order + (it lies within r of the place before)
+  int* list = reinterpret_cast<int*>(buf);
+  int* order = reinterpret_cast<int*>(buf + (size_t)P * sizeof(ST));
+  float* xs = reinterpret_cast<float*>(order + P);          // [d][XS]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const PruneTest<PT> test(pos, cand_row, DP, d, r2);
+  visit_order<ST>(score, K, buf, order);
+  if (pre) {   // DP is a power of two: whole rows, read together, eight loads in flight
+    const int shift = 31 - __clz(DP);
+    for (int e0 = threadIdx.x; e0 < K << shift; e0 += 8 * blockDim.x) {
+      float v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) kk[u] = vk[j + u];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) rank += kk[u] > mv ? 1 : 0;
+      for (int u = 0; u < 8; ++u) {
+        const int e = e0 + u * blockDim.x, k = e & (DP - 1);
+        v[u] = e < K << shift && k < pre ? (float)pos[test.row(order[e >> shift]) * DP + k] : 0.0f;
       }
-      for (; j < K; ++j) rank += vk[j] > mv ? 1 : 0;
-    }
-    __syncthreads();
-    if (t < K) idx[rank] = t;
-    __syncthreads();   // the sorted order is read by other threads below
-  } else if (K <= 512 && K <= (int)blockDim.x) {
-    // rank of candidate t = number of candidates before it (a permutation:
-    // the order is total; a NaN score counts as -inf)
-    const int t = threadIdx.x;
-    ST mk = (ST)-INFINITY;
-    if (t < K) {
-      mk = score[t];
-      if (!(mk == mk)) mk = (ST)-INFINITY;
-      keys[t] = mk;
-    }
-    __syncthreads();
-    int rank = 0;
-    if (t < K) {
-      // eight independent (broadcast) loads in flight per step
-      int j = 0;
-      for (; j + 8 <= K; j += 8) {
-        ST kk[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) kk[u] = keys[j + u];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) rank += (kk[u] > mk || (kk[u] == mk && j + u < t)) ? 1 : 0;
-      }
-      for (; j < K; ++j) {
-        const ST kj = keys[j];
-        rank += (kj > mk || (kj == mk && j < t)) ? 1 : 0;
+      for (int u = 0; u < 8; ++u) {
+        const int e = e0 + u * blockDim.x, k = e & (DP - 1);
+        if (e < K << shift && k < pre) xs[k * XS + (e >> shift)] = v[u];
       }
     }
     __syncthreads();
-    if (t < K) {
-      keys[rank] = mk;
-      idx[rank] = t;
-    }
-    __syncthreads();   // the sorted order is read by other threads below
-  } else {
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {
-    keys[i] = i < K ? score[i] : (ST)-INFINITY;
-    idx[i] = i < K ? i : INT32_MAX;
   }
-  __syncthreads();
-  // bitonic sort
-  for (int k = 2; k <= P; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const int l = i ^ j;
-        if (l > i) {
-          const ST ka = keys[i], kb = keys[l];
-          const int ia = idx[i], ib = idx[l];
-          const bool a_first = (ka > kb) || (ka == kb && ia < ib);
-          const bool up = (i & k) == 0;
-          if (up != a_first) {
-            keys[i] = kb;
-            keys[l] = ka;
-            idx[i] = ib;
-            idx[l] = ia;
+  auto coord = [&](int i, int64_t row, int k) -> float {
+    return k < pre ? xs[k * XS + i] : (float)pos[row * DP + k];
+  };
+  const int first_d = kWide ? d : min(d, kPruneFirst);
+  const int near_d = pre ? pre : first_d;   // (a guess that the batches verify)
+  for (int i = threadIdx.x; i < K; i += blockDim.x) {
+    float s = i > 0 ? 0.0f : INFINITY;
+    if (i > 0) {
+      const int64_t r0 = test.row(order[i - 1]), r1 = test.row(order[i]);
+#pragma unroll 8
+      for (int k = 0; k < near_d; ++k) {
+        const float e = coord(i, r1, k) - coord(i - 1, r0, k);
+        s += e * e;
+      }
+    }
+    list[i] = 2 * i + (s < (float)r2 ? 1 : 0);
+  }
+  part[threadIdx.x] = 0;
+  int len = K, nacc = 0;
+  int turn = 0;
+  bool pass_over = true;
+  while (len > 0) {
+    if (threadIdx.x == 0) {
+      *horizon = min(len, (int)blockDim.x);
+      *cut = INT32_MAX;
+    }
+    __syncthreads();   // the list is written, the last batch's tile and modes are read
+    // the batch: the first 32 of the block's first entries that are not passed over
+    int before, nb;    // members before this thread's entry; members
+    {
+      const int i = threadIdx.x;
+      bool lead = i < len;
+      if (lead && i > 0 && pass_over) {
+        const int e = list[i];
+        lead = !(e & 1) || (list[i - 1] >> 1) != (e >> 1) - 1;
+      }
+      int tot;
+      before = block_rank(lead, &tot, words + 32 * (turn ^= 1));
+      if (lead && before < 32) member[before] = i;
+      if (lead && before == 32) *horizon = i;
+      nb = min(tot, 32);
+    }
+    __syncthreads();
+    const int end = *horizon;
+    const int slot = lane < nb ? member[lane] : INT32_MAX;   // lane's member, in every warp
+    const int place = lane < nb ? list[slot] >> 1 : -1;
+    const int mine = lane < nb ? order[place] : -1;
+    {
+      const int64_t row = mine >= 0 ? test.row(mine) : 0;
+      for (int k = warp; k < d4; k += nwarps)
+        tile[k * kPruneTileStride + lane] = mine >= 0 && k < d ? coord(place, row, k) : 0.0f;
+    }
+    __syncthreads();
+    float n2 = 0.0f;   // |member|^2, in the warps that need it
+    for (int v0 = warp * 4; v0 < 32; v0 += nwarps * 4) {
+      float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      n2 = 0.0f;
+#pragma unroll 4
+      for (int k = 0; k < d; ++k) {
+        const float x = tile[k * kPruneTileStride + lane];
+        const float4 m = *reinterpret_cast<const float4*>(&tile[k * kPruneTileStride + v0]);
+        const float e0 = x - m.x, e1 = x - m.y, e2 = x - m.z, e3 = x - m.w;
+        s[0] += e0 * e0;
+        s[1] += e1 * e1;
+        s[2] += e2 * e2;
+        s[3] += e3 * e3;
+        if (kWide) n2 += x * x;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float b = kWide ? __shfl_sync(kFull, n2, v0 + j) : 0.0f;
+        const int other = kWide ? __shfl_sync(kFull, mine, v0 + j) : 0;
+        const bool in = lane < nb && v0 + j < nb && test.within(s[j], n2, b, mine, other);
+        const unsigned m = __ballot_sync(kFull, in);
+        if (lane == 0) near[v0 + j] = m;
+      }
+    }
+    __syncthreads();
+    // every warp: the members accepted in visit order.  One with no earlier live
+    // neighbour is accepted, its neighbours go, until none is left.
+    const unsigned nm = near[lane];
+    unsigned alive = nb == 32 ? kFull : (1u << nb) - 1u, acc = 0;
+    while (alive) {
+      const bool live = (alive >> lane) & 1u;
+      const bool first = live && !(nm & alive & ((1u << lane) - 1u));
+      const unsigned F = __ballot_sync(kFull, first);
+      acc |= F;
+      alive = __ballot_sync(kFull, live && !first && !(nm & F));
+    }
+    const int nn = __popc(acc);
+    const bool taken = (acc >> lane) & 1u;
+    const int at = __popc(acc & ((1u << lane) - 1u));
+    if (len <= nb) {   // nothing but members
+      if (warp == 0 && taken) accepted[nacc + at] = mine;
+      nacc += nn;
+      break;
+    }
+    for (int k = warp; k < d4; k += nwarps)
+      if (taken) modes[k * 32 + at] = -tile[k * kPruneTileStride + lane];
+    if (warp == 0 && taken) {
+      mnorm[at] = n2;   // (warp 0 had members 0-3: n2 is set)
+      mcand[at] = mine;
+    }
+    __syncthreads();
+    // The list against the modes just accepted, a block of entries at a time,
+    // compacted in place (a step writes only below the end of what it read, and
+    // every read precedes the barriers).  A warp takes 128 entries and groups of
+    // warps share the modes.
+    int newlen = 0;
+    unsigned valid = 0;                                       // modes not put back
+    for (int b = 0; b < len; b += blockDim.x) {
+      const int wide = (min(len - b, (int)blockDim.x) + 32 * kPruneEntries - 1) / (32 * kPruneEntries);
+      const int groups = nwarps / wide, group = warp / wide;
+      const int first = (warp - group * wide) * 32 * kPruneEntries + lane;
+      for (int m0 = group * kPruneModes; m0 < nn && group < groups; m0 += groups * kPruneModes) {
+        int p[kPruneEntries];
+        unsigned long long s2[kPruneEntries][kPruneModes / 2];
+        float a[kPruneEntries];
+#pragma unroll
+        for (int q = 0; q < kPruneEntries; ++q) {
+          const int i = b + first + q * 32;
+          p[q] = i < len ? list[i] >> 1 : 0;   // (past the end: entry 0, unused)
+          a[q] = 0.0f;
+#pragma unroll
+          for (int j = 0; j < kPruneModes / 2; ++j) s2[q][j] = 0ull;
+        }
+        auto add = [&](int k, const float (&x)[kPruneEntries]) {
+          const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(&modes[k * 32 + m0]);
+#pragma unroll
+          for (int q = 0; q < kPruneEntries; ++q) {
+            unsigned long long xx;
+            asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x[q]));
+            add_square2(s2[q][0], xx, m.x);
+            add_square2(s2[q][1], xx, m.y);
+            if (kWide) a[q] += x[q] * x[q];
           }
+        };
+        if (first_d <= pre) {
+#pragma unroll 4
+          for (int k = 0; k < first_d; ++k) {
+            float x[kPruneEntries];
+#pragma unroll
+            for (int q = 0; q < kPruneEntries; ++q) x[q] = xs[k * XS + p[q]];
+            add(k, x);
+          }
+        } else {   // DP is a multiple of 4
+          for (int k0 = 0; k0 < first_d; k0 += 4) {
+            float x[kPruneEntries][4];
+#pragma unroll
+            for (int q = 0; q < kPruneEntries; ++q) load_row4(pos + test.row(order[p[q]]) * DP + k0, x[q]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (k0 + u < first_d) {
+                const float xu[kPruneEntries] = {x[0][u], x[1][u], x[2][u], x[3][u]};
+                add(k0 + u, xu);
+              }
+          }
+        }
+        // (FP32: the whole distance, or of the first coordinates, which is no larger)
+        const unsigned some = nn - m0 >= kPruneModes ? (1u << kPruneModes) - 1u : (1u << (nn - m0)) - 1u;
+#pragma unroll
+        for (int q = 0; q < kPruneEntries; ++q) {
+          unsigned mask = 0;
+#pragma unroll
+          for (int j = 0; j < kPruneModes; ++j) {
+            const unsigned long long h = s2[q][j / 2];
+            const float s = __uint_as_float((unsigned)(j % 2 ? h >> 32 : h));
+            if constexpr (kWide) {
+              if (m0 + j < nn && b + first + q * 32 < len &&
+                  test.within(s, a[q], mnorm[m0 + j], order[p[q]], mcand[m0 + j]))
+                mask |= 1u << j;
+            } else {
+              mask |= s < r2 ? 1u << j : 0u;
+            }
+          }
+          mask = b + first + q * 32 < len ? (mask & some) << m0 : 0u;
+          if (mask) atomicOr(&part[first + q * 32], mask);
         }
       }
       __syncthreads();
-    }
-  }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  // coordinates of accepted mode a (a candidate index in accepted[a])
-  auto acc_ptr = [&](int a) -> const PT* {
-    if (acc_in_smem) return apos + (size_t)a * d;
-    return pos + row_of(accepted[a]) * DP;
-  };
-  int* s_dead = idx + P;                             // scratch: batch suppression flags
-  int* s_nacc = s_dead + 32;                         // scratch: modes accepted so far
-  unsigned* s_near = reinterpret_cast<unsigned*>(s_dead + 64);   // scratch: batch masks
-  // warp w stages batch `base` (lane c: sorted candidate base + c; tile[k * 33 + c] is
-  // its coordinate k)
-  auto stage = [&](int base, PT* tile) {
-    const int i = base + lane;
-    if (i < K) {
-      const int c = idx[i];
-      if (preload) {
-        for (int k = 0; k < d; ++k) tile[k * kPruneTileStride + lane] = cpre[(size_t)k * P + c];
-      } else {
-        const PT* src = pos + row_of(c) * DP;
-        for (int k = 0; k < d; ++k) tile[k * kPruneTileStride + lane] = src[k];
+      const int i = b + threadIdx.x;
+      bool keep = i < len;
+      const int entry = keep ? list[i] : 0;
+      unsigned mask = part[threadIdx.x];   // the modes within r
+      part[threadIdx.x] = 0;
+      if (first_d < d && mask) {   // the whole distance to those that the first test left
+        const int64_t row = test.row(order[entry >> 1]);
+        unsigned left = mask;
+        mask = 0;
+        while (left) {
+          const int m = __ffs(left) - 1;
+          left &= left - 1;
+          float s = 0.0f;
+#pragma unroll 8
+          for (int k = 0; k < d; ++k) {
+            const float e = coord(entry >> 1, row, k) + modes[k * 32 + m];
+            s += e * e;
+          }
+          if (test.within(s, 0.0f, 0.0f, 0, 0)) mask |= 1u << m;
+        }
       }
-    }
-  };
-  if constexpr (DT > 0) {
-    if (preload && acc_in_smem) {
-      // Register visit (d = DT known at compile time): every warp holds the
-      // batch's coordinates in registers (lane c: sorted candidate base + c),
-      // tests them against its share of the modes accepted so far, and warp v
-      // records which members lie within r of member v (shuffles and a
-      // ballot); warp 0 then accepts the survivors lowest lane first, each
-      // removing its neighbours by mask, and the accepted lanes write their
-      // rows in parallel.  The distances are those of the test against an
-      // accepted mode, so the accepted set and its order are the greedy
-      // visit's.
-      if (threadIdx.x == 0) *s_nacc = 0;
-      if (warp == 0) s_dead[lane] = 0;
-      for (int base = 0; base < K; base += 32) {
-        const int i = base + lane;
-        const int c = i < K ? idx[i] : 0;
-        PT x[DT];
-#pragma unroll
-        for (int k = 0; k < DT; ++k) x[k] = i < K ? cpre[(size_t)k * P + c] : (PT)0;
-        __syncthreads();   // accepted rows, their count and cleared flags are visible
-        const int nacc = *s_nacc;
-        bool dead = false;
-        if (i < K)
-          for (int a = warp; a < nacc && !dead; a += nwarps) {
-            const PT* ap = apos + (size_t)a * DT;
-            PT d2 = 0;
-#pragma unroll
-            for (int k = 0; k < DT; ++k) {
-              const PT e = x[k] - ap[k];
-              d2 += e * e;
-            }
-            dead = d2 < r2;
-          }
-        if (dead) s_dead[lane] = 1;
-        // warp v: the batch members within r of member v (bit l of s_near[v])
-        for (int v = warp; v < 32; v += nwarps) {
-          PT d2 = 0;
-#pragma unroll
-          for (int k = 0; k < DT; ++k) {
-            const PT e = x[k] - __shfl_sync(kFull, x[k], v);
-            d2 += e * e;
-          }
-          const unsigned m = __ballot_sync(kFull, i < K && d2 < r2);
-          if (lane == 0) s_near[v] = m;
+      __syncwarp();
+      if (b == 0) {
+        const bool is_member = keep && before < nb && member[before] == i;
+        if (keep && !is_member && i < end) {
+          const unsigned earlier = before >= 32 ? acc : acc & ((1u << before) - 1u);
+          const int ne = __popc(earlier);
+          if (!(mask & (ne >= 32 ? kFull : (1u << ne) - 1u))) atomicMin(cut, i);
         }
         __syncthreads();
-        if (warp == 0) {
-          // survivors accepted lowest lane first, each removing its neighbours;
-          // then every accepted lane writes its own row
-          unsigned alive = __ballot_sync(kFull, i < K && !s_dead[lane]);
-          unsigned acc = 0;
-          while (alive) {
-            const int w = __ffs(alive) - 1;
-            acc |= 1u << w;
-            alive &= ~(s_near[w] | (1u << w));
-          }
-          if ((acc >> lane) & 1u) {
-            const int at = nacc + __popc(acc & ((1u << lane) - 1u));
-            accepted[at] = c;
-#pragma unroll
-            for (int k = 0; k < DT; ++k) apos[(size_t)at * DT + k] = x[k];
-          }
-          s_dead[lane] = 0;
-          if (lane == 0) *s_nacc = nacc + __popc(acc);
-        }
+        const int stop = *cut;
+        valid = __ballot_sync(kFull, taken && slot < stop);
+        const int nv = __popc(valid);
+        if (warp == 0 && taken && slot < stop) accepted[nacc + at] = mine;
+        nacc += nv;
+        valid = nv >= 32 ? kFull : (1u << nv) - 1u;   // as bits of `mask`
+        if (stop != INT32_MAX) pass_over = false;
+        if (is_member && i < stop) keep = false;
       }
-      __syncthreads();
-      if (threadIdx.x == 0) *M_out = *s_nacc;
-      return;
+      keep = keep && !(mask & valid);
+      int tot;
+      const int off = block_rank(keep, &tot, words + 32 * (turn ^= 1));
+      if (keep) list[newlen + off] = entry;
+      newlen += tot;
     }
+    len = newlen;
   }
-  if (threadIdx.x == 0) *s_nacc = 0;
-  if (warp == 0) {
-    stage(0, ctile2);
-    s_dead[lane] = 0;
-  }
-  for (int base = 0, b = 0; base < K; base += 32, ++b) {
-    const int i = base + lane;
-    PT* ctile = ctile2 + (b & 1) * kTile;
-    __syncthreads();   // this batch's tile and cleared flags are visible
-    const int nacc = *s_nacc;
-    // every warp tests the batch against its share of the modes accepted so far
-    if (i < K) {
-      bool dead = false;
-      for (int a = warp; a < nacc && !dead; a += nwarps) {
-        const PT* ap = acc_ptr(a);
-        PT d2 = 0;
-        for (int k = 0; k < d; ++k) {
-          const PT e = ctile[k * kPruneTileStride + lane] - ap[k];
-          d2 += e * e;
-        }
-        dead = d2 < r2;
-      }
-      if (dead) s_dead[lane] = 1;
-    }
-    // masks: bit l of s_near[v] <=> batch members l and v lie within r (the
-    // same FP arithmetic as the test against an accepted mode: the coordinate
-    // differences are exact negations of each other)
-    for (int v = warp; v < 32; v += nwarps) {
-      bool nb = false;
-      if (i < K && base + v < K) {
-        PT d2 = 0;
-        for (int k = 0; k < d; ++k) {
-          const PT e = ctile[k * kPruneTileStride + lane] - ctile[k * kPruneTileStride + v];
-          d2 += e * e;
-        }
-        nb = d2 < r2;
-      }
-      const unsigned m = __ballot_sync(kFull, nb);
-      if (lane == 0) s_near[v] = m;
-    }
-    // the next batch's tile (its last readers finished before this batch's barrier)
-    if (warp == (nwarps > 1 ? 1 : 0) && base + 32 < K) stage(base + 32, ctile2 + ((b + 1) & 1) * kTile);
-    __syncthreads();
-    if (warp == 0) {
-      // survivors of the batch, resolved in order by one warp
-      unsigned alive = __ballot_sync(kFull, i < K && !s_dead[lane]);
-      int na = nacc;
-      while (alive) {
-        const int w = __ffs(alive) - 1;
-        if (lane == w) accepted[na] = idx[i];
-        if (acc_in_smem)
-          for (int k = lane; k < d; k += 32)
-            apos[(size_t)na * d + k] = ctile[k * kPruneTileStride + w];
-        alive &= ~(s_near[w] | (1u << w));
-        ++na;
-      }
-      s_dead[lane] = 0;
-      if (lane == 0) *s_nacc = na;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *M_out = *s_nacc;
+  if (threadIdx.x == 0) *M_out = nacc;
 }
 
 }  // namespace fms

@@ -610,11 +610,11 @@ __global__ void __launch_bounds__(1024)
 }
 
 // Prune of each set (one CTA per set): the sorted visit while its sort keys
-// (and, when they fit too, the accepted modes' coordinates) fit in the launch's
+// (and, when they fit too, the candidates' coordinates) fit in the launch's
 // smem_bytes of shared memory, else the one-block global greedy over the set's
 // own region of `list`; both give the one-by-one greedy visit's result.
 template <typename PT, typename ST>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kPruneThreads)
     batched_prune(SetCtl* sc, const int32_t* __restrict__ kept, const ST* __restrict__ score,
                   const PT* __restrict__ pos, int DP, int d, PT r2, int32_t* __restrict__ accepted,
                   int32_t* __restrict__ list, int smem_bytes, int second) {
@@ -628,12 +628,9 @@ __global__ void __launch_bounds__(1024)
   const int32_t* rows = second ? nullptr : kept + p0;
   const PT* cpos = second ? pos + (int64_t)p0 * DP : pos;
   int32_t* M_out = second ? &c->Mr : &c->M;
-  int P = 1;
-  while (P < K) P <<= 1;
-  if (greedy_sorted_smem<PT, ST>(K, d, P, false) <= (size_t)smem_bytes) {
-    const bool acc_in_smem = greedy_sorted_smem<PT, ST>(K, d, P, true) <= (size_t)smem_bytes;
-    greedy_sorted_body<PT, ST>(rows, K, score + p0, cpos, DP, d, r2, accepted + p0, M_out, P, smem,
-                               acc_in_smem);
+  if (greedy_sorted_smem<ST>(K, d, 0) <= (size_t)smem_bytes) {
+    greedy_sorted_body<PT, ST>(rows, K, score + p0, cpos, DP, d, r2, accepted + p0, M_out, smem,
+                               greedy_sorted_pre<ST>(K, d, (size_t)smem_bytes));
   } else {
     greedy_global_body<PT, ST>(rows, K, score + p0, cpos, DP, d, r2, list + p0, accepted + p0,
                                M_out, smem);
@@ -956,14 +953,12 @@ cudaError_t launch_queue_modes(const SetCtl* sc, int B, int64_t* list_off, int64
 }
 
 // Shared memory of the per-set prune launch for sets of up to maxK candidates:
-// the sorted visit's keys, indices, tiles and accepted coordinates when they
-// fit in kBatchedPruneSmem, else kBatchedPruneSmem (sets whose keys do not fit
-// take the global greedy).
+// what the sorted visit takes with the coordinates preloaded when that fits in
+// kBatchedPruneSmem, else kBatchedPruneSmem (sets whose keys do not fit take the
+// global greedy).
 template <typename PT, typename ST>
 static size_t prune_launch_smem(int maxK, int d) {
-  int P = 1;
-  while (P < maxK) P <<= 1;
-  size_t sm = greedy_sorted_smem<PT, ST>(maxK, d, P, true);
+  size_t sm = greedy_sorted_smem<ST>(maxK, d, d);
   if (sm > kBatchedPruneSmem) sm = kBatchedPruneSmem;
   if (sm < greedy_global_smem<PT, ST>()) sm = greedy_global_smem<PT, ST>();
   return sm;
@@ -981,7 +976,7 @@ static cudaError_t launch_prune_t(SetCtl* sc, int B, const int32_t* kept, const 
     attr = true;
   }
   const size_t sm = prune_launch_smem<PT, ST>(maxK, d);
-  batched_prune<PT, ST><<<B, 1024, sm, st>>>(sc, kept, score, pos, DP, d, r2, accepted, list,
+  batched_prune<PT, ST><<<B, kPruneThreads, sm, st>>>(sc, kept, score, pos, DP, d, r2, accepted, list,
                                              (int)sm, second);
   return cudaGetLastError();
 }

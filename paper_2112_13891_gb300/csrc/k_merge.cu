@@ -298,43 +298,15 @@ static cudaError_t launch_greedy_grid(const int32_t* cand_row, const int32_t* K_
   }
 }
 
-// DT > 0: d = DT at compile time (candidates in registers during the visit)
-template <typename PT, typename ST, int DT>
-__global__ void __launch_bounds__(1024)
+template <typename PT, typename ST>
+__global__ void __launch_bounds__(kPruneThreads)
     greedy_sorted_kernel(const int32_t* __restrict__ cand_row, const int32_t* __restrict__ K_ptr,
                          const ST* __restrict__ score, const PT* __restrict__ pos, int DP, int d,
                          PT r2, int32_t* __restrict__ accepted, int32_t* __restrict__ M_out,
-                         int P, int acc_in_smem, int preload) {
+                         int pre) {
   extern __shared__ __align__(16) unsigned char smem[];
-  greedy_sorted_body<PT, ST, DT>(cand_row, *K_ptr, score, pos, DP, DT > 0 ? DT : d, r2, accepted,
-                                 M_out, P, smem, acc_in_smem != 0, preload != 0);
-}
-
-template <typename PT, typename ST, int DT>
-static cudaError_t launch_sorted_t(const int32_t* cand_row, const int32_t* K_ptr, const ST* score,
-                                   const PT* pos, int DP, int d, PT r2, int32_t* accepted,
-                                   int32_t* M_out, int P, int with_pos, int preload, size_t sm,
-                                   int smem_max, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(greedy_sorted_kernel<PT, ST, DT>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-    attr = true;
-  }
-  greedy_sorted_kernel<PT, ST, DT><<<1, 1024, sm, st>>>(cand_row, K_ptr, score, pos, DP, d, r2,
-                                                        accepted, M_out, P, with_pos, preload);
-  return cudaGetLastError();
-}
-
-// Shared memory of the sorted prune for up to K candidates: sort keys and
-// indices, the batch tiles, plus (preload) every candidate's coordinates and
-// (with_pos) the accepted modes' coordinates.
-template <typename PT, typename ST>
-size_t greedy_sorted_bytes(int K, int d, int* P_out, bool with_pos, bool preload) {
-  int P = 1;
-  while (P < K) P <<= 1;
-  *P_out = P;
-  return greedy_sorted_smem<PT, ST>(K, d, P, with_pos, preload);
+  greedy_sorted_body<PT, ST>(cand_row, *K_ptr, score, pos, DP, d, r2, accepted, M_out, smem,
+                             pre);
 }
 
 constexpr size_t kGreedySmemMax = 200 * 1024;
@@ -347,36 +319,18 @@ cudaError_t launch_greedy(const int32_t* cand_row, const int32_t* K_ptr, const S
                           const PT* pos, int DP, int d, PT r2, int32_t* alive,
                           int32_t* accepted, int32_t* M_out, int max_K, cudaStream_t st,
                           uint32_t* status = nullptr) {
-  // largest layout that fits: preloaded candidates and accepted modes in
-  // shared memory, then accepted modes only, then neither
-  int P = 1;
-  int with_pos = 1, preload = 1;
-  size_t sm = greedy_sorted_bytes<PT, ST>(max_K, d, &P, true, true);
-  if (sm > kGreedySmemMax) {
-    preload = 0;
-    sm = greedy_sorted_bytes<PT, ST>(max_K, d, &P, true, false);
-  }
-  if (sm > kGreedySmemMax) {
-    sm = greedy_sorted_bytes<PT, ST>(max_K, d, &P, false, false);
-    with_pos = 0;
-  }
+  const int pre = greedy_sorted_pre<ST>(max_K, d, kGreedySmemMax);
+  const size_t sm = greedy_sorted_smem<ST>(max_K, d, pre);
   if (sm <= kGreedySmemMax && d <= kPruneMaxDim) {
-    const int mx = (int)kGreedySmemMax;
-#define FMS_SORTED(DT_)                                                                      \
-  return launch_sorted_t<PT, ST, DT_>(cand_row, K_ptr, score, pos, DP, d, r2, accepted, M_out, \
-                                      P, with_pos, preload, sm, mx, st)
-    if (preload && with_pos) switch (d) {
-        case 1: FMS_SORTED(1);
-        case 2: FMS_SORTED(2);
-        case 3: FMS_SORTED(3);
-        case 4: FMS_SORTED(4);
-        case 5: FMS_SORTED(5);
-        case 6: FMS_SORTED(6);
-        case 7: FMS_SORTED(7);
-        case 8: FMS_SORTED(8);
-      }
-    FMS_SORTED(0);
-#undef FMS_SORTED
+    static bool attr = false;
+    if (!attr) {
+      cudaFuncSetAttribute(greedy_sorted_kernel<PT, ST>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGreedySmemMax);
+      attr = true;
+    }
+    greedy_sorted_kernel<PT, ST><<<1, kPruneThreads, sm, st>>>(
+        cand_row, K_ptr, score, pos, DP, d, r2, accepted, M_out, pre);
+    return cudaGetLastError();
   }
   if constexpr (sizeof(ST) == 4 && sizeof(PT) == 4) {
     // FP32 scores: the visit on the whole GPU when its shares fit

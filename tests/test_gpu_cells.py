@@ -136,3 +136,48 @@ def test_coarse_step_by_cells(n, m, d, box, h):
     assert np.all(np.abs(out[pick] - ref).max(axis=1) <= bnd)
     assert np.all(np.abs(W[pick] - refW) <= 1.5 * eps * refW)
     assert W[3] == 0.0 and np.isnan(out[3]).all()
+
+
+def _greedy(X, score, r2):
+    """Greedy radius suppression in order of (score descending, index ascending);
+    exact for integer points."""
+    alive = np.ones(len(X), bool)
+    out = []
+    for i in np.lexsort((np.arange(len(X)), -score)):
+        if alive[i]:
+            out.append(i)
+            alive &= ~(((X - X[i]) ** 2).sum(axis=1) < r2)
+    return X[out]
+
+
+# Integer points far apart next to h stay where they are, with their multiplicity for a
+# density, so the merge alone decides: every comparison of distances is between an
+# integer and r^2 = 4.5.  Neighbours lie in chains, so that passing over a candidate is
+# often wrong.  Sizes at the edges of the sort (256 counted, 512, 1,024, 2,048, 8,192
+# slots) and of a batch; at d = 32 and 64 not all coordinates fit in shared memory.
+# d <= 7: densities are exact, many of them tied (lowest index first).  Above, the
+# densities are good to |s x|^2 2^-23 (s = 0.85 / h, 45 a coordinate, d = 64: 1 %), so no two
+# points have multiplicities closer than 1 in 64 and their order is certain.
+@pytest.mark.parametrize("refine", [False, True])
+@pytest.mark.parametrize("n,d", [(31, 3), (33, 3), (256, 2), (257, 7), (1025, 5), (2049, 4),
+                                 (8200, 3), (22, 9), (23, 16), (32, 16), (54, 32), (63, 32),
+                                 (45, 64), (64, 64)])
+def test_merge_of_points_that_stay(n, d, refine):
+    rng = np.random.default_rng(n + d)
+    k = max(n // (12 if d <= 7 else 4), 1)
+    side = max(int(np.ceil(k ** (1.0 / d))), 1)
+    centre = 3 * rng.integers(0, side + 1, (k, d))
+    X = centre[rng.integers(0, k, n)]
+    for _ in range(3):
+        X[np.arange(n), rng.integers(0, d, n)] += rng.integers(-1, 2, n)
+    X, times = np.unique(X, axis=0, return_counts=True)
+    at = rng.permutation(len(X))
+    X, times = X[at], times[at] if d <= 7 else 1 + np.arange(len(X))
+    rows = np.repeat(X, times, axis=0).astype(np.float32)
+    r = fms.cluster(torch.from_numpy(rows).cuda(), 0.05 if d <= 7 else 0.15, 1e-3, 20,
+                    all_seeds=True, gamma=1.0, merge_radius=float(np.sqrt(4.5)),
+                    skip_refine=not refine, precision="fp32")
+    got = np.rint(r.modes.cpu().numpy()).astype(int)
+    want = _greedy(X, times, 4.5)
+    assert len(got) == len(want)
+    assert {tuple(p) for p in got} == {tuple(p) for p in want}
