@@ -926,7 +926,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           const cells::Groups gr{P > 0 ? at<int2>(ws, Lo.off_table) : nullptr,
                                  P > 0 ? cells::group_cap(n, P) : (int)((n + 31) / 32)};
           FMS_LAUNCH(launch_travel_groups(
-              rows, cv, (int)n, DP, gr, perm, kf, max_iter, tol2_s, sphere_r, y, it, conv, state,
+              rows, cv, (int)n, d, DP, gr, perm, kf, max_iter, tol2_s, sphere_r, y, it, conv, state,
               wlast, hist, reinterpret_cast<unsigned long long*>(&ctl->evals),
               reinterpret_cast<unsigned long long*>(&mctl->evals), dv.sms, st));
         } else if (use_grid) {

@@ -260,7 +260,7 @@ cudaError_t launch_step_groups(const float* Xs, const cells::View<float>& cv, in
                                double inv_scale, float* out_seeds, float* out_wsum, int sms,
                                cudaStream_t st);
 // Every point a seed, DP = 4 or 8: states, hist and the densities at the last positions.
-cudaError_t launch_travel_groups(const float* Xs, const cells::View<float>& cv, int n, int DP,
+cudaError_t launch_travel_groups(const float* Xs, const cells::View<float>& cv, int n, int d, int DP,
                                  const cells::Groups& gr, const int32_t* perm, int kf,
                                  int max_iter, float tol2_s, float sphere_r, float* y, int32_t* it,
                                  int32_t* conv, int32_t* state, float* wlast, int32_t* hist,

@@ -13,12 +13,13 @@
 //                  take the next (set, seed) from a queue
 //
 // Measured on one GB300 against the kernels that took every pair, one launch an
-// update: 20,011 seeds x 65,537 points x 32 (one update) 4.92 -> 1.10 ms, of which
-// step_groups 0.70; 200,000 x 3, every point a seed, 90.0 -> 17.4 ms; 2,000 x 2 (not
-// sorted) 0.59 -> 0.29 ms; 65,536 x 32 with 128 to 512 seeds 2.96 -> 0.93 ms, of
-// which the three travel_seeds 0.24; 200,000 x 16 directions 1.49 -> 0.80 ms, of
-// which the two travel_seeds 0.14; 256 sets of 1,000 to 50,000 x 16 in one call
-// (travel_queue, 4 warps a seed) 29.0 -> 7.3 ms.
+// update: 20,011 seeds x 65,537 points x 32 (one update) 4.91 -> 0.90 ms, of which
+// step_groups 0.70; 200,000 x 3, every point a seed, 86 -> 12.8 ms (17.4 with the
+// padding column evaluated); 2,000 x 2 (not sorted) 0.56 -> 0.16 ms; 65,536 x 32 with
+// 128 to 512 seeds 2.96 -> 0.62 ms, of which the three travel_seeds 0.21 (0.25 with 8
+// warps a seed); 200,000 x 16 directions 1.45 -> 0.47 ms, of which the two
+// travel_seeds 0.12 (0.14); 256 sets of 1,000 to 50,000 x 16 in one call
+// (travel_queue, 4 warps a seed) 29.0 -> 5.4 ms.
 #include "fms_team.cuh"
 
 namespace fms {
@@ -34,12 +35,15 @@ __device__ __forceinline__ float first_cut() {
 
 // W and S of the group at y (acc[0], acc[1 + k]); `act` lanes decide the ball
 // and the cutoff, which comes in as a guess and leaves as the one their smallest
-// W asks for.  Returns the rows visited.
-template <int DP, int KF, int PH, int SUMS>
+// W asks for.  Returns the rows visited.  The first NX of the DP columns count (the
+// others are zero padding): the loop is bound by instruction issue, 11 of them at
+// three columns, 15 at four.
+template <int DP, int KF, int PH, int SUMS, int NA>
 __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const View<float>& cv, int n,
                                           const float (&y)[DP], bool act, float log2n, float& cut,
                                           const TeamSmem<float, DP, SUMS>& sm, int w, int W,
-                                          int lane, float (&acc)[DP + 1]) {
+                                          int lane, float (&acc)[NA]) {
+  constexpr int NX = NA - 1;
   int rows = 0;
   for (int pass = 0;; ++pass) {
     float reach;
@@ -49,28 +53,29 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
     else
       for (int i = lane; i < nl; i += 32) rows += sm.list[i].y;
 #pragma unroll
-    for (int k = 0; k <= DP; ++k) acc[k] = 0.0f;
+    for (int k = 0; k <= NX; ++k) acc[k] = 0.0f;
     sm.walk(Xs, n, nl, w, W, lane, [&](const float* tile, int nr) {
-      float ta[DP + 1];
+      float ta[NX + 1];
 #pragma unroll
-      for (int k = 0; k <= DP; ++k) ta[k] = 0.0f;
+      for (int k = 0; k <= NX; ++k) ta[k] = 0.0f;
       constexpr int UNROLL = DP <= 4 ? 8 : (DP <= 8 ? 4 : (DP <= 16 ? 2 : 1));
       tile_rows<DP, PH, UNROLL>(tile, nr, lane, [&](const float* row, bool in) {
         float x[DP];
         smem_row<DP>(row, x);
-        float t = 0.0f;
+        x[0] -= y[0];
+        float t = -x[0] * x[0];
 #pragma unroll
-        for (int k = 0; k < DP; ++k) {
+        for (int k = 1; k < NX; ++k) {
           x[k] -= y[k];
           t = fmaf(-x[k], x[k], t);
         }
         const float wt = in ? kweight<KF>(t) : 0.0f;
         ta[0] += wt;
 #pragma unroll
-        for (int k = 0; k < DP; ++k) ta[1 + k] = fmaf(wt, x[k], ta[1 + k]);
+        for (int k = 0; k < NX; ++k) ta[1 + k] = fmaf(wt, x[k], ta[1 + k]);
       });
 #pragma unroll
-      for (int k = 0; k <= DP; ++k) acc[k] += ta[k];
+      for (int k = 0; k <= NX; ++k) acc[k] += ta[k];
     });
     phase_sum<PH>(acc);
     team_sum<32 / PH>(acc, sm.sums, SUMS, w, W, lane);
@@ -88,7 +93,7 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
 }
 
 // out = seed + (S / W) / scale in the caller's order and units, as in step_finish.
-template <int DP>
+template <int DP, int NX>
 __global__ void __launch_bounds__(256)
     step_groups(const float* __restrict__ Xs, View<float> cv, int n, const float* __restrict__ Ys,
                 Groups gr, int m, const int32_t* __restrict__ perm, int d, const float* seeds,
@@ -99,7 +104,7 @@ __global__ void __launch_bounds__(256)
   int row0, cnt;
   if (!group_rows(gr, 0, blockIdx.x, m, &row0, &cnt)) return;
   const int e = row0 + min(lane, cnt - 1);
-  float y[DP], acc[DP + 1];
+  float y[DP], acc[NX + 1];
   load_row<DP>(Ys + (int64_t)e * DP, y);
   const float log2n = log2f((float)n);
   float cut = first_cut<kKernelGaussian>();
@@ -107,7 +112,7 @@ __global__ void __launch_bounds__(256)
   if (w != 0 || lane >= cnt) return;
   const int64_t i = perm[e];
 #pragma unroll
-  for (int k = 0; k < DP; ++k)
+  for (int k = 0; k < NX; ++k)
     if (k < d)
       out_seeds[i * d + k] =
           (float)((double)seeds[i * d + k] + (double)(acc[1 + k] / acc[0]) * inv_scale);
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(256)
 // Every point a seed, slot = the point's row in the caller's order (perm; null:
 // unsorted): updates until it converges, fails or has made max_iter of them, then
 // the density at its last position (wlast).  hist counts the convergence updates.
-template <int DP, int KF, int PH>
+template <int DP, int NX, int KF, int PH>
 __global__ void __launch_bounds__(512)
     travel_groups(const float* __restrict__ Xs, View<float> cv, int n, Groups gr,
                   const int32_t* __restrict__ perm, int max_iter, float tol2_s, float sphere_r,
@@ -132,7 +137,7 @@ __global__ void __launch_bounds__(512)
   if (!group_rows(gr, 0, blockIdx.x, n, &row0, &cnt, GS)) return;
   const TeamSmem<float, DP, DP + 1> sm(travel_smem, w, W, Xs, resident ? n : 0);
   const int e = row0 + min(lane % GS, cnt - 1);
-  float y[DP], acc[DP + 1];
+  float y[DP], acc[NX + 1];
   load_row<DP>(Xs + (int64_t)e * DP, y);
   const float log2n = log2f((float)n);
   float cut = first_cut<KF>(), wl = 0.0f;
@@ -148,9 +153,9 @@ __global__ void __launch_bounds__(512)
     wl = acc[0];
     ++it;
     bool ok = (wl > 0.0f) && isfinite(wl);
-    float dl[DP], step2 = 0.0f;
+    float dl[NX], step2 = 0.0f;
 #pragma unroll
-    for (int k = 0; k < DP; ++k) {
+    for (int k = 0; k < NX; ++k) {
       dl[k] = ok ? acc[1 + k] / wl : 0.0f;
       step2 = fmaf(dl[k], dl[k], step2);
     }
@@ -158,14 +163,14 @@ __global__ void __launch_bounds__(512)
     if (ok && sphere_r > 0.0f) {
       float nn = 0.0f;
 #pragma unroll
-      for (int k = 0; k < DP; ++k) {
+      for (int k = 0; k < NX; ++k) {
         dl[k] += y[k];
         nn = fmaf(dl[k], dl[k], nn);
       }
       const float f = sphere_r / sqrtf(nn);
       step2 = 0.0f;
 #pragma unroll
-      for (int k = 0; k < DP; ++k) {
+      for (int k = 0; k < NX; ++k) {
         dl[k] = dl[k] * f - y[k];
         step2 = fmaf(dl[k], dl[k], step2);
       }
@@ -173,7 +178,7 @@ __global__ void __launch_bounds__(512)
     }
     if (ok) {
 #pragma unroll
-      for (int k = 0; k < DP; ++k) y[k] += dl[k];
+      for (int k = 0; k < NX; ++k) y[k] += dl[k];
     }
     if (!ok) {
       stt = kFailed;
@@ -724,32 +729,45 @@ int seed_grid(int max_seeds, int sms) {
 
 }  // namespace
 
+// RUN(padded width, columns that count) for d <= 8.
+#define FMS_BY_COLUMNS(RUN)   \
+  switch (d) {                \
+    case 1:                   \
+    case 2: RUN(4, 2)         \
+    case 3: RUN(4, 3)         \
+    case 4: RUN(4, 4)         \
+    case 5:                   \
+    case 6: RUN(8, 6)         \
+    case 7:                   \
+    case 8: RUN(8, 8)         \
+  }
+
 cudaError_t launch_step_groups(const float* Xs, const View<float>& cv, int n, const float* Ys,
                                const Groups& gr, int m, const int32_t* perm, int d, int DP,
                                const float* seeds, double inv_scale, float* out_seeds,
                                float* out_wsum, int sms, cudaStream_t st) {
-#define FMS_STEP_GROUPS(DP_)                                                                     \
+#define FMS_STEP_GROUPS(DP_, NX_)                                                                \
   {                                                                                              \
     constexpr int ws = team_warp_smem<float, DP_, DP_ + 1>();                                    \
     const int W = team_warps(gr.per_set, sms, ws);                                               \
     const int smem = group_team_smem<float, DP_, DP_ + 1>(W);                                    \
-    const cudaError_t e = team_attr(step_groups<DP_>, smem);                                     \
+    const cudaError_t e = team_attr(step_groups<DP_, NX_>, smem);                                \
     if (e != cudaSuccess) return e;                                                              \
-    step_groups<DP_><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, Ys, gr, m, perm, d, seeds,   \
-                                                         inv_scale, out_seeds, out_wsum);        \
+    step_groups<DP_, NX_><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, Ys, gr, m, perm, d,       \
+                                                            seeds, inv_scale, out_seeds,         \
+                                                            out_wsum);                           \
     return cudaGetLastError();                                                                   \
   }
+  FMS_BY_COLUMNS(FMS_STEP_GROUPS)
   switch (DP) {
-    case 4: FMS_STEP_GROUPS(4)
-    case 8: FMS_STEP_GROUPS(8)
-    case 16: FMS_STEP_GROUPS(16)
-    case 32: FMS_STEP_GROUPS(32)
+    case 16: FMS_STEP_GROUPS(16, 16)
+    case 32: FMS_STEP_GROUPS(32, 32)
   }
 #undef FMS_STEP_GROUPS
   return cudaErrorInvalidValue;
 }
 
-template <int DP, int KF, int PH>
+template <int DP, int NX, int KF, int PH>
 static cudaError_t travel_groups_t(const float* Xs, const View<float>& cv, int n, Groups gr,
                                    const int32_t* perm, int max_iter, float tol2_s,
                                    float sphere_r, float* y, int32_t* it, int32_t* conv,
@@ -763,32 +781,30 @@ static cudaError_t travel_groups_t(const float* Xs, const View<float>& cv, int n
   const bool res = team_resident<float, DP>(cv.P, n);
   const int smem =
       res ? resident_team_smem<float, DP, DP + 1>(W, n) : group_team_smem<float, DP, DP + 1>(W);
-  const cudaError_t e = team_attr(travel_groups<DP, KF, PH>, smem);
+  const cudaError_t e = team_attr(travel_groups<DP, NX, KF, PH>, smem);
   if (e != cudaSuccess) return e;
-  travel_groups<DP, KF, PH><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, gr, perm, max_iter, tol2_s,
-                                                            sphere_r, y, it, conv, state, wlast,
-                                                            hist, evals, score_evals,
-                                                            res ? 1 : 0);
+  travel_groups<DP, NX, KF, PH><<<gr.per_set, 32 * W, smem, st>>>(
+      Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it, conv, state, wlast, hist, evals,
+      score_evals, res ? 1 : 0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_travel_groups(const float* Xs, const View<float>& cv, int n, int DP,
+cudaError_t launch_travel_groups(const float* Xs, const View<float>& cv, int n, int d, int DP,
                                  const Groups& gr, const int32_t* perm, int kf, int max_iter,
                                  float tol2_s, float sphere_r, float* y, int32_t* it,
                                  int32_t* conv, int32_t* state, float* wlast, int32_t* hist,
                                  unsigned long long* evals, unsigned long long* score_evals,
                                  int sms, cudaStream_t st) {
-#define FMS_TRAVEL_PH(DP_, KF_, PH_)                                                            \
-  travel_groups_t<DP_, KF_, PH_>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it, conv,  \
-                                 state, wlast, hist, evals, score_evals, sms, st)
-#define FMS_TRAVEL(DP_)                                                                        \
-  if (team_phases<float, DP_>(cv.P, n, sms) == 4)                                              \
-    return kf ? FMS_TRAVEL_PH(DP_, 1, 4) : FMS_TRAVEL_PH(DP_, 0, 4);                           \
-  return kf ? FMS_TRAVEL_PH(DP_, 1, 1) : FMS_TRAVEL_PH(DP_, 0, 1)
-  switch (DP) {
-    case 4: FMS_TRAVEL(4);
-    case 8: FMS_TRAVEL(8);
+#define FMS_TRAVEL_PH(DP_, NX_, KF_, PH_)                                                       \
+  travel_groups_t<DP_, NX_, KF_, PH_>(Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it,   \
+                                      conv, state, wlast, hist, evals, score_evals, sms, st)
+#define FMS_TRAVEL(DP_, NX_)                                                                   \
+  {                                                                                            \
+    if (team_phases<float, DP_>(cv.P, n, sms) == 4)                                            \
+      return kf ? FMS_TRAVEL_PH(DP_, NX_, 1, 4) : FMS_TRAVEL_PH(DP_, NX_, 0, 4);               \
+    return kf ? FMS_TRAVEL_PH(DP_, NX_, 1, 1) : FMS_TRAVEL_PH(DP_, NX_, 0, 1);                 \
   }
+  FMS_BY_COLUMNS(FMS_TRAVEL)
 #undef FMS_TRAVEL
 #undef FMS_TRAVEL_PH
   return cudaErrorInvalidValue;
