@@ -41,10 +41,11 @@
 //
 // Bound by FP32 issue (3 DP + 3, 5 DP + 6 and 6 DP + 6 operations per visible pair).
 // 8 sets x 16,384 points and seeds x 16, 32 blobs, T = 20, k = 5: each group sees
-// about 515 of the 16,384 points; forward and backward 390.4 -> 18.3 ms (forward
-// 3.8, recomputed positions 3.1, seed-major 5.2, point-major 6.0) against kernels
+// about 515 of the 16,384 points; forward and backward 390.4 -> 19 ms (forward
+// 3.9, recomputed positions 3.8, seed-major 5.2, point-major 6.0) against kernels
 // that took every pair.  3 sets x 1,500 points x 701 seeds x 3, T = 10 (nothing
-// sorted): 0.955 -> 0.561 ms from 94 launches going to 15.
+// sorted): 0.99 -> 0.40 ms, of which 0.43 came from 94 launches going to 15 and 0.13
+// from resident points and phases; the zero column of d <= 3 left out is the rest.
 #include "fms_team.cuh"
 
 namespace fms {
@@ -106,7 +107,7 @@ __device__ T rescue_seed(const T* __restrict__ Xb, int n, T c, const T (&y)[DP],
 // t the positions go to slot ceil(t / every) - slot0 of pos where t is a
 // multiple of `every` or the last one; W and the shift of update t to row t - 1
 // of Wout and Sh (nullable).
-template <typename T, int DP, int PH>
+template <typename T, int DP, int NX, int PH>
 __global__ void __launch_bounds__(32 * most_warps<T, DP>())
     unroll_travel(const T* __restrict__ X, View<T> cv, const T* __restrict__ Y0, Groups gr,
                   UGeom g, T c, int steps, int every, int slot0, T* __restrict__ pos,
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
           smem_row<DP>(row, x);
           T D2 = T(0);
 #pragma unroll
-          for (int k = 0; k < DP; ++k) {
+          for (int k = 0; k < NX; ++k) {
             x[k] -= y[k];
             D2 = ufma(x[k], x[k], D2);
           }
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
           ta[0] += wt;
           ta[DP + 1] = ufma(wt, D2, ta[DP + 1]);
 #pragma unroll
-          for (int k = 0; k < DP; ++k) ta[1 + k] = ufma(wt, x[k], ta[1 + k]);
+          for (int k = 0; k < NX; ++k) ta[1 + k] = ufma(wt, x[k], ta[1 + k]);
         });
 #pragma unroll
         for (int k = 0; k < DP + 2; ++k) acc[k] += ta[k];
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
 // ||y_i - x_j||^2 under p (kept by the forward) makes the terms smallest, and a
 // far seed's residual sum p a (FP32 rounding of a D2 of hundreds leaves ~1e-5
 // instead of 0) is not multiplied by D2.  DH is summed over tiles in FP64.
-template <typename T, int DP, int PH>
+template <typename T, int DP, int NX, int PH>
 __global__ void __launch_bounds__(32 * most_warps<T, DP>())
     unroll_bwd_seed(const T* __restrict__ X, View<T> cv, USegment<T> sg, Groups gr, UGeom g, T c,
                     T inv_h2, double inv_h3, const T* __restrict__ Gin, T* __restrict__ Gout,
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
         smem_row<DP>(row, x);
         T D2 = T(0), a = gd;
 #pragma unroll
-        for (int k = 0; k < DP; ++k) {
+        for (int k = 0; k < NX; ++k) {
           x[k] -= y[k];
           D2 = ufma(x[k], x[k], D2);
           a = ufma(gg[k], x[k], a);
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
         ta[0] = ufma(pa, D2 - s0, ta[0]);
         ta[1] += pa;
 #pragma unroll
-        for (int k = 0; k < DP; ++k) ta[2 + k] = ufma(pa, x[k], ta[2 + k]);
+        for (int k = 0; k < NX; ++k) ta[2 + k] = ufma(pa, x[k], ta[2 + k]);
       });
 #pragma unroll
       for (int k = 0; k <= DP; ++k) acc[k] += ta[1 + k];
@@ -342,7 +343,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
 // of 32 points adds
 //   DX_j = sum_i p_ij g_i - (1/h^2) sum_i p_ij a_ij (x_j - y_i)
 // to its rows of dX.
-template <typename T, int DP>
+template <typename T, int DP, int NX>
 __global__ void __launch_bounds__(32 * most_warps<T, DP>())
     unroll_bwd_point(const T* __restrict__ X, Groups gx, Groups gr, UGeom g, int len, T c,
                      T inv_h2, const T* __restrict__ SD, const T* __restrict__ bctr,
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
           smem_row<4>(sd + 2 * DP, tail);
           T D2 = T(0), a = tail[2];
 #pragma unroll
-          for (int k = 0; k < DP; ++k) {
+          for (int k = 0; k < NX; ++k) {
             dx[k] = x[k] - dx[k];
             D2 = ufma(dx[k], dx[k], D2);
             a = ufma(gv[k], dx[k], a);
@@ -414,7 +415,7 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
           const T p = uex2(ufma(-c, D2, tail[1])) * tail[0];
           const T q2 = p * a * inv_h2;
 #pragma unroll
-          for (int k = 0; k < DP; ++k) ta[k] = ufma(p, gv[k], ufma(-q2, dx[k], ta[k]));
+          for (int k = 0; k < NX; ++k) ta[k] = ufma(p, gv[k], ufma(-q2, dx[k], ta[k]));
         }
 #pragma unroll
         for (int k = 0; k < DP; ++k) acc[k] += ta[k];
@@ -484,7 +485,7 @@ static int blocks_for(int64_t work, int per = 256) {
   return (int)b;
 }
 
-template <typename T, int DP, int PH>
+template <typename T, int DP, int NX, int PH>
 static cudaError_t travel_p(const T* X, const View<T>& cv, const T* Y0, Groups gr, const UGeom& g,
                             T c, int steps, int every, int slot0, T* pos, T* Wout, T* Sh, T* M2,
                             cudaStream_t st) {
@@ -494,27 +495,28 @@ static cudaError_t travel_p(const T* X, const View<T>& cv, const T* Y0, Groups g
   const int W = team_warps(NG, g.sms, ws, most_warps<T, DP>());
   const bool res = team_resident<T, DP>(cv.P, g.n);
   const int smem = res ? resident_team_smem<T, DP, DP + 3>(W, g.n) : group_team_smem<T, DP, DP + 3>(W);
-  const cudaError_t e = team_attr(unroll_travel<T, DP, PH>, smem);
+  const cudaError_t e = team_attr(unroll_travel<T, DP, NX, PH>, smem);
   if (e != cudaSuccess) return e;
-  unroll_travel<T, DP, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
+  unroll_travel<T, DP, NX, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
       X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, res ? 1 : 0);
   return cudaGetLastError();
 }
 
-template <typename T, int DP>
+template <typename T, int DP, int NX = DP>
 static cudaError_t travel_t(const T* X, const View<T>& cv, const T* Y0, const Groups& gr,
                             const UGeom& g, T c, int steps, int every, int slot0, T* pos, T* Wout,
                             T* Sh, T* M2, cudaStream_t st) {
   if constexpr (sizeof(T) == 4 && DP <= 16)
     if (team_phases<T, DP>(cv.P, (int64_t)g.B * g.m, g.sms) == 4)
-      return travel_p<T, DP, 4>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
-  return travel_p<T, DP, 1>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
+      return travel_p<T, DP, NX, 4>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
+  return travel_p<T, DP, NX, 1>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
 }
 
 template <typename T>
 cudaError_t unroll_forward_steps(const T* X, const View<T>& cv, const T* Y0, const Groups& gr,
                                  const UGeom& g, T c, int steps, int every, int slot0, T* pos,
                                  T* Wout, T* Sh, T* M2, cudaStream_t st) {
+  if (g.d <= 3) return travel_t<T, 4, 3>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
   switch (g.DP) {
     case 4: return travel_t<T, 4>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
     case 8: return travel_t<T, 8>(X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, st);
@@ -525,7 +527,7 @@ cudaError_t unroll_forward_steps(const T* X, const View<T>& cv, const T* Y0, con
 }
 
 // the seed-major pass; *groups: its groups in all (the entries of dh_part)
-template <typename T, int DP, int PH>
+template <typename T, int DP, int NX, int PH>
 static cudaError_t bwd_seed_p(const T* X, const View<T>& cv, const USegment<T>& sg, Groups gr,
                               const UGeom& g, T c, T inv_h2, double inv_h3, const T* Gin, T* Gout,
                               T* SD, T* bctr, T* breach, double* dh_part, int first,
@@ -536,14 +538,14 @@ static cudaError_t bwd_seed_p(const T* X, const View<T>& cv, const USegment<T>& 
   const int W = team_warps(NG, g.sms, ws, most_warps<T, DP>());
   const bool res = team_resident<T, DP>(cv.P, g.n);
   const int smem = res ? resident_team_smem<T, DP, DP + 2>(W, g.n) : group_team_smem<T, DP, DP + 2>(W);
-  const cudaError_t e = team_attr(unroll_bwd_seed<T, DP, PH>, smem);
+  const cudaError_t e = team_attr(unroll_bwd_seed<T, DP, NX, PH>, smem);
   if (e != cudaSuccess) return e;
-  unroll_bwd_seed<T, DP, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
+  unroll_bwd_seed<T, DP, NX, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
       X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, first, res ? 1 : 0);
   return cudaGetLastError();
 }
 
-template <typename T, int DP>
+template <typename T, int DP, int NX = DP>
 static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, const Groups& gx,
                          const Groups& gr, const UGeom& g, T c, T inv_h2, double inv_h3,
                          const T* Gin, T* Gout, T* SD, T* bctr, T* breach, double* dh_part, T* dX,
@@ -552,21 +554,21 @@ static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, c
   bool done = false;
   if constexpr (sizeof(T) == 4 && DP <= 16)
     if (team_phases<T, DP>(cv.P, (int64_t)g.B * g.m, g.sms) == 4) {
-      e = bwd_seed_p<T, DP, 4>(X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach,
+      e = bwd_seed_p<T, DP, NX, 4>(X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach,
                                dh_part, first, st);
       done = true;
     }
   if (!done)
-    e = bwd_seed_p<T, DP, 1>(X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach,
+    e = bwd_seed_p<T, DP, NX, 1>(X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach,
                              dh_part, first, st);
   if (e != cudaSuccess) return e;
-  const int64_t NX = (int64_t)g.B * gx.per_set;
+  const int64_t PG = (int64_t)g.B * gx.per_set;
   constexpr int wp = team_warp_smem<T, 2 * DP + 4, DP>();
-  const int Wp = team_warps(NX, g.sms, wp, most_warps<T, DP>());
+  const int Wp = team_warps(PG, g.sms, wp, most_warps<T, DP>());
   const int smem_p = list_team_smem<T, 2 * DP + 4, DP>(Wp);
-  e = team_attr(unroll_bwd_point<T, DP>, smem_p);
+  e = team_attr(unroll_bwd_point<T, DP, NX>, smem_p);
   if (e != cudaSuccess) return e;
-  unroll_bwd_point<T, DP><<<(unsigned)NX, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
+  unroll_bwd_point<T, DP, NX><<<(unsigned)PG, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
                                                                  SD, bctr, breach, dX, first);
   return cudaGetLastError();
 }
@@ -590,6 +592,7 @@ cudaError_t unroll_backward_segment(const T* X, const View<T>& cv, const USegmen
                                     T inv_h2, double inv_h3, const T* Gin, T* Gout, T* SD, T* bctr,
                                     T* breach, double* dh_part, T* dX, int first,
                                     cudaStream_t st) {
+  if (g.d <= 3) return bwd_t<T, 4, 3>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
   switch (g.DP) {
     case 4: return bwd_t<T, 4>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
     case 8: return bwd_t<T, 8>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
