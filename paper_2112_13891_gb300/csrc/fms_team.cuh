@@ -318,17 +318,13 @@ inline int team_phases(int P, int64_t seeds, int sms) {
   return (seeds + 31) / 32 >= sms ? 1 : 4;
 }
 
-// Sums v over the team in warp order; every warp gets the result.  Lanes l and
+// Sums over the team in warp order; every warp gets the result.  Lanes l and
 // l + GS hold the same values; a thread adds one value's W parts (every warp adding
-// all of them would read W^2 rows of shared memory).
+// all of them would read W^2 rows of shared memory).  The values are already in the
+// warps' parts of `sums`:
 template <int GS, typename T, int N>
-__device__ __forceinline__ void team_sum(T (&v)[N], T* sums, int stride, int w, int W, int lane) {
-  if (W == 1) return;
+__device__ __forceinline__ void team_total(T (&v)[N], T* sums, int stride, int W, int lane) {
   T* total = sums + W * stride * 32;
-  if (lane < GS) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) sums[(w * stride + k) * 32 + lane] = v[k];
-  }
   __syncthreads();
   for (int i = threadIdx.x; i < N * GS; i += 32 * W) {
     const int at = i / GS * 32 + i % GS;
@@ -340,6 +336,17 @@ __device__ __forceinline__ void team_sum(T (&v)[N], T* sums, int stride, int w, 
   // (rewritten only after the next call's first barrier)
 #pragma unroll
   for (int k = 0; k < N; ++k) v[k] = total[k * 32 + lane % GS];
+}
+
+// ... or in v:
+template <int GS, typename T, int N>
+__device__ __forceinline__ void team_sum(T (&v)[N], T* sums, int stride, int w, int W, int lane) {
+  if (W == 1) return;
+  if (lane < GS) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) sums[(w * stride + k) * 32 + lane] = v[k];
+  }
+  team_total<GS>(v, sums, stride, W, lane);
 }
 
 __device__ __forceinline__ bool group_rows(const Groups& g, int b, int gi, int rows, int* row0,

@@ -13,8 +13,8 @@
 //                  take the next (set, seed) from a queue
 //
 // Measured on one GB300 against the kernels that took every pair, one launch an
-// update: 20,011 seeds x 65,537 points x 32 (one update) 4.91 -> 0.90 ms, of which
-// step_groups 0.70; 200,000 x 3, every point a seed, 86 -> 12.8 ms (17.4 with the
+// update: 20,011 seeds x 65,537 points x 32 (one update) 4.91 -> 0.86 ms, of which
+// step_groups 0.53 (0.67 with the sums in registers, one block an SM); 200,000 x 3, every point a seed, 86 -> 12.8 ms (17.4 with the
 // padding column evaluated); 2,000 x 2 (not sorted) 0.56 -> 0.16 ms; 65,536 x 32 with
 // 128 to 512 seeds 2.96 -> 0.62 ms, of which the three travel_seeds 0.21 (0.25 with 8
 // warps a seed); 200,000 x 16 directions 1.45 -> 0.47 ms, of which the two
@@ -44,6 +44,13 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
                                           const TeamSmem<float, DP, SUMS>& sm, int w, int W,
                                           int lane, float (&acc)[NA]) {
   constexpr int NX = NA - 1;
+  // The sums over tiles: 33 registers of wide rows, or, once a tile, the warp's part of
+  // the team's exchange, so that two blocks of 8 warps fit an SM (163 -> 128 registers).
+  constexpr bool kSmemSums = DP >= 32 && PH == 1;
+  auto add_to = [&](int k) -> float& {
+    if constexpr (kSmemSums) return sm.sums[(w * SUMS + k) * 32 + lane];
+    else return acc[k];
+  };
   int rows = 0;
   for (int pass = 0;; ++pass) {
     float reach;
@@ -53,7 +60,7 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
     else
       for (int i = lane; i < nl; i += 32) rows += sm.list[i].y;
 #pragma unroll
-    for (int k = 0; k <= NX; ++k) acc[k] = 0.0f;
+    for (int k = 0; k <= NX; ++k) add_to(k) = 0.0f;
     sm.walk(Xs, n, nl, w, W, lane, [&](const float* tile, int nr) {
       float ta[NX + 1];
 #pragma unroll
@@ -75,10 +82,14 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
         for (int k = 0; k < NX; ++k) ta[1 + k] = fmaf(wt, x[k], ta[1 + k]);
       });
 #pragma unroll
-      for (int k = 0; k <= NX; ++k) acc[k] += ta[k];
+      for (int k = 0; k <= NX; ++k) add_to(k) += ta[k];
     });
-    phase_sum<PH>(acc);
-    team_sum<32 / PH>(acc, sm.sums, SUMS, w, W, lane);
+    if constexpr (kSmemSums) {
+      team_total<32>(acc, sm.sums, SUMS, W, lane);
+    } else {
+      phase_sum<PH>(acc);
+      team_sum<32 / PH>(acc, sm.sums, SUMS, w, W, lane);
+    }
     if (KF == kKernelFlat || cv.P == 0) break;
     const float need = cells::cut_bits(cells::warp_min(act ? acc[0] : INFINITY), log2n);
     if (!(need > cut) || cut >= cells::zero_bits<float>()) {
@@ -94,7 +105,7 @@ __device__ __forceinline__ int group_pass(const float* __restrict__ Xs, const Vi
 
 // out = seed + (S / W) / scale in the caller's order and units, as in step_finish.
 template <int DP, int NX>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
     step_groups(const float* __restrict__ Xs, View<float> cv, int n, const float* __restrict__ Ys,
                 Groups gr, int m, const int32_t* __restrict__ perm, int d, const float* seeds,
                 double inv_scale, float* out_seeds, float* __restrict__ out_wsum) {
