@@ -1527,7 +1527,7 @@ fms_status fms_mean_shift_step(const float* points, int64_t n, int32_t d, float 
     FMS_CUDA(launch_ms_step(Xs, n, d, L.DP, Ys, active, &ctl->s, &ctl->C, &ctl->Lc, part,
                             L.grid_ctas * 8, st, nullptr, nullptr, kKernelGaussian, status));
     FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,
-                                (int)m, st));
+                                (int)m, L.C, st));
     }
     if (owns) {
       FMS_CUDA(cudaMemcpyAsync(&hstatus, status, 4, cudaMemcpyDeviceToHost, st));
@@ -1656,8 +1656,8 @@ cudaError_t coarse_cells(const CoarseLayout& L, void* ws, int64_t n, int d, int6
     e = launch_ms_step_tc(img, n, d, L.DP, L.DA, Yc, active, &ctl->s, &ctl->s, &ctl->C, &ctl->Lc,
                           part, status, st, nullptr, TcTiles{list, count, L.tiles});
   if (e == cudaSuccess)
-    e = launch_step_finish(part, ctl, seeds, d, L.DA, inv_scale, out_seeds, out_wsum, places, st,
-                           out_row);
+    e = launch_step_finish(part, ctl, seeds, d, L.DA, inv_scale, out_seeds, out_wsum, places,
+                           L.C, st, out_row);
   return e;
 }
 }  // namespace
@@ -1709,7 +1709,7 @@ fms_status fms_mean_shift_step_coarse(const float* points, int64_t n, int32_t d,
       FMS_CUDA(launch_ms_step_tc(img, n, d, L.DP, L.DA, Ys, active, &ctl->s, &ctl->s, &ctl->C,
                                  &ctl->Lc, part, status, st));
       FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,
-                                  (int)m, st));
+                                  (int)m, L.C, st));
     }
     if (owns) {
       FMS_CUDA(cudaMemcpyAsync(&hstatus, status, 4, cudaMemcpyDeviceToHost, st));

@@ -359,7 +359,7 @@ cudaError_t launch_step_small(const float* X, int64_t n, int d, float scale, con
 // out_row (nullable): the caller's row of each active position, -1 for none
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,
-                               int m, cudaStream_t st, const int32_t* out_row = nullptr);
+                               int m, int C, cudaStream_t st, const int32_t* out_row = nullptr);
 
 // k_round.cu
 cudaError_t launch_ms_round(const float* Xs, int64_t n, int d, float* y, int32_t* it,

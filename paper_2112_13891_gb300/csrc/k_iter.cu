@@ -10,23 +10,39 @@ namespace fms {
 // Xcopy (nullable) receives the rows unchanged, for later passes over the
 // original points (X may be host memory read over the CPU-GPU link).
 // ---------------------------------------------------------------------------
-__global__ void pack_points_kernel(const float* __restrict__ X, int64_t n, int d, int DP,
+// DP = 16, 32, 64: a thread takes four columns; VEC: rows of whole, aligned 16 bytes.
+// (A thread per column, its row by a 64-bit division: 9 us for 65,536 x 16; so 3.)
+template <bool VEC>
+__global__ void pack_points_kernel(const float* __restrict__ X, int64_t n, int d, int log_dp,
                                    float scale, float* __restrict__ Xs, uint32_t* status,
                                    float* __restrict__ Xcopy) {
-  const int64_t total = n * DP;
+  const int64_t total = n << (log_dp - 2);
   bool bad = false;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = e / DP;
-    const int k = (int)(e - j * DP);
-    float v = 0.0f;
-    if (k < d) {
-      v = X[j * d + k];
-      if (Xcopy) Xcopy[j * d + k] = v;
-      if (!isfinite(v)) bad = true;
-      v *= scale;
+    const int64_t j = e >> (log_dp - 2);
+    const int k = (int)(e & ((1 << (log_dp - 2)) - 1)) * 4;
+    const float* r = X + j * d + k;
+    float* o = Xcopy ? Xcopy + j * d + k : nullptr;
+    float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (VEC) {
+      if (k < d) {
+        const float4 t = *reinterpret_cast<const float4*>(r);
+        if (o) *reinterpret_cast<float4*>(o) = t;
+        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k + u < d) {
+          v[u] = r[u];
+          if (o) o[u] = v[u];
+        }
     }
-    Xs[e] = v;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) bad = bad || !isfinite(v[u]);
+    reinterpret_cast<float4*>(Xs)[e] =
+        make_float4(v[0] * scale, v[1] * scale, v[2] * scale, v[3] * scale);
   }
   if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(status, kStNonFinite);
 }
@@ -100,10 +116,14 @@ cudaError_t launch_pack_points(const float* X, int64_t n, int d, int DP, float s
       pack_rows_kernel<8><<<(int)blocks, 256, 0, st>>>(X, (int)n, d, scale, Xs, status, Xcopy);
     return cudaGetLastError();
   }
-  int64_t total = n * DP;
-  int64_t blocks = (total + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  pack_points_kernel<<<(int)blocks, 256, 0, st>>>(X, n, d, DP, scale, Xs, status, Xcopy);
+  int log_dp = 2;
+  while ((1 << log_dp) < DP) ++log_dp;
+  int64_t blocks = ((n << (log_dp - 2)) + 255) / 256;
+  if (blocks > 8192) blocks = 8192;
+  const bool vec = d % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0 &&
+                   (reinterpret_cast<uintptr_t>(Xcopy) & 15u) == 0;
+  auto kern = vec ? pack_points_kernel<true> : pack_points_kernel<false>;
+  kern<<<(int)blocks, 256, 0, st>>>(X, n, d, log_dp, scale, Xs, status, Xcopy);
   return cudaGetLastError();
 }
 
@@ -732,9 +752,44 @@ __global__ void step_finish_kernel(const float* __restrict__ part, const IterCtl
   }
 }
 
+// The same for few chunks, a thread per coordinate.  A warp per seed spends its time on
+// shuffles that add up to 32 chunks and on FP64 instructions of which d of 32 lanes
+// count: 65,536 seeds x 16 of one chunk take 15 us here, 56 there.
+constexpr int kFinishChunks = 4;
+__global__ void step_finish_few(const float* __restrict__ part, const IterCtl* __restrict__ ctl,
+                                const float* seeds, int d, int DA, double inv_scale,
+                                float* out_seeds, float* __restrict__ out_wsum,
+                                const int32_t* __restrict__ out_row) {
+  const int s = ctl->s, C = ctl->C;
+  const int64_t total = (int64_t)s * d;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int p = (int)(e / d), k = (int)(e - (int64_t)p * d);
+    const int64_t i = out_row ? out_row[p] : p;
+    if (i < 0) continue;
+    float W = 0.0f, S = 0.0f;
+    for (int c = 0; c < C; ++c) {
+      const float* q = part + ((int64_t)c * s + p) * DA;
+      W += q[0];
+      S += q[1 + k];
+    }
+    // (seeds may alias out_seeds: a thread reads the element that it writes)
+    out_seeds[i * d + k] = (float)((double)seeds[i * d + k] + (double)(S / W) * inv_scale);
+    if (k == 0 && out_wsum) out_wsum[i] = W;
+  }
+}
+
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,
-                               int m, cudaStream_t st, const int32_t* out_row) {
+                               int m, int C, cudaStream_t st, const int32_t* out_row) {
+  if (C <= kFinishChunks) {
+    int64_t blocks = ((int64_t)m * d + 255) / 256;
+    if (blocks < 1) blocks = 1;
+    if (blocks > 4096) blocks = 4096;
+    step_finish_few<<<(int)blocks, 256, 0, st>>>(part, ctl, seeds, d, DA, inv_scale, out_seeds,
+                                                 out_wsum, out_row);
+    return cudaGetLastError();
+  }
   int blocks = (m + 7) / 8;
   if (blocks < 1) blocks = 1;
   if (blocks > 4096) blocks = 4096;
