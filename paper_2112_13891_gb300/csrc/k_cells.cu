@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256)
 // Thread q of a block keeps the unit vectors from cell p's centre to those of cells q
 // and q + P / 2, the rows of p come by broadcast from shared memory; DP multiply-adds
 // a (row, cell), and a row's loads serve two of them.  Only cells below *npiv have
-// rows, so the second half is often skipped.
+// rows, so a warp whose second 32 lie beyond it skips them (200,000 x 16: 61 -> 52 us).
 constexpr int kExtRows = 64;
 
 template <int DP, int NU>
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kMaxCells / 2)
   __shared__ __align__(16) float tile[kExtRows * DP];
   const int p = blockIdx.x;
   const int a = start[p], e = start[p + 1];
-  const bool both = *npiv > P / 2;
+  const bool both = *npiv > P / 2 + (int)(threadIdx.x & ~31u);   // (the same for a warp)
   if (a + (int)blockIdx.y * kExtRows >= e && blockIdx.y > 0) return;
   float v[2][DP], dist[2], far_[2] = {0.0f, 0.0f};
 #pragma unroll
