@@ -77,9 +77,14 @@ typedef struct fms_options {
   int32_t profile;          /* 1: time every ms_step launch with CUDA events and
                                report it in fms_stats (adds event records)        */
   int32_t precision;        /* arithmetic of the seed updates (FMS_PRECISION_*):
-                               AUTO (0) = TENSOR for 9 <= d <= 32, else FP32.
+                               AUTO (0) = TENSOR for 9 <= d <= 32 where every
+                                  point is a seed or n_initial (or the seed list)
+                                  exceeds 4096, else FP32.
                                FP32 (1): every update evaluates the weights in
-                                  FP32 from exact differences.
+                                  FP32 from exact differences.  (Sorted points:
+                                  weights that cannot count, all together below
+                                  2^-32 of the sum of weights, are left out; the
+                                  bound is checked after the fact.)
                                TENSOR (2, 8 <= d <= 32; FP32 elsewhere): a
                                   seed's updates take the coarse tensor-core
                                   step (BF16 weights, FP32 sums; see
@@ -134,7 +139,8 @@ typedef struct fms_stats {
   int32_t refine_iterations;/* FP64-accumulated refinement updates                */
   int32_t t_star_last;      /* stop iteration of the last round                   */
   int32_t kernel_launches;  /* CUDA kernels this call launched                    */
-  int64_t evals;            /* seed-point kernel evaluations in mean-shift updates */
+  int64_t evals;            /* seed-point kernel evaluations in mean-shift updates
+                               (sorted points: of the cells that a seed sees)      */
   int64_t score_evals;      /* evaluations spent on prune scores and refinement   */
   uint64_t workspace_bytes; /* bytes of workspace the call used                   */
   /* filled when opt->profile = 1 (else zero): */
@@ -275,7 +281,9 @@ fms_status fms_cluster_host(const float* points, int64_t n, int32_t d, float h, 
  * The graph is built on the first call with a given (pointers, B, total,
  * largest set, d, h, tol, max_iter, max_modes, options) and reused by later
  * calls with the same values; the per-set sizes are copied in before every
- * launch.  The step kernel's tiling is chosen by a built-in autotuner the
+ * launch.  Sets of d > 7, or of 2,048 points and more on average, have their
+ * seeds carried to convergence one a block; for the others, whose updates are
+ * one launch each, the step kernel's tiling is chosen by a built-in autotuner the
  * first time a shape (d, size class of the total, size class of B) is seen
  * on a device: it times one update with each candidate tiling (synchronising
  * on each) and keeps the fastest.
