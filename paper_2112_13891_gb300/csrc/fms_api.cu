@@ -183,12 +183,15 @@ struct Route {
   bool tensor;   // updates start on the tensor-core step
 };
 
-// Seeds up to which a block per seed is the better split; more of them reuse a
-// row of points too little (each block reads its own rows from L2), and the
-// tensor-core or wide step takes them.
+// Seeds up to which a block per seed is the better split.  65,536 points of 32 blobs,
+// d = 16: 512 seeds 0.31 ms (the steps 0.70), 4,096 0.94 (1.61), 8,192 1.78 (2.80); but
+// over every pair 1.10 and 6.1 ms, since each block reads its rows from L2 for one seed,
+// so the line lies where data without clusters begins to lose much.
 constexpr int32_t kTravelMaxSeeds = 4096;
-// Points from which sorting them pays: ~30 us, against the dense passes of
-// 128 seeds, or of every point.
+// Points from which they are sorted.  On 8 blobs it pays a step later (128 seeds, d = 16:
+// 8,192 points 207 us sorted, 162 not; 16,384 214 and 208; 32,768 233 and 284.  Every
+// point a seed, d = 3: 4,096 points 459 and 340; 8,192 825 and 907); the more clusters,
+// the more a seed leaves out.
 constexpr int64_t kSortSeedsMin = 8192, kSortGroupsMin = 4096;
 
 Route choose_route(int64_t n, int d, const fms_options& o, int32_t max_iter) {
