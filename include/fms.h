@@ -197,10 +197,14 @@ size_t fms_workspace_size(int64_t n, int32_t d, const fms_options* opt);
  *                moves it by at most tol (in point units); 0 -> 1e-3*h.
  *   max_iter     cap on updates per seed (> 0).
  *   out_modes    [max_modes x d] float32, device: the modes, in canonical
- *                order: density descending (sum w of the mode's last
- *                refinement update, one step of at most 1e-5*h before the
- *                mode, so within O(1e-10) relative of the KDE value at the
- *                mode), ties by coordinates.
+ *                order: density descending, ties by coordinates.  The
+ *                density is sum w of the mode's last refinement update (one
+ *                step of at most 1e-5*h before the mode); Gaussian densities
+ *                that its FP32 weights cannot tell apart (4e-6, more far
+ *                from the origin) are taken from FP64 weights of the given
+ *                points at the refined position, within O(1e-10) relative
+ *                of the KDE value at the mode.  (skip_refine: the prune's
+ *                FP32 densities.)
  *   out_n_modes  host int32: M.  If M > max_modes, FMS_ERR_CAPACITY is
  *                returned, *out_n_modes = M and out_modes holds the first
  *                max_modes modes; labels are still written.

@@ -9,6 +9,7 @@
 
 #include "../../include/fms.h"
 #include "fms_cells.cuh"
+#include "fms_density.cuh"
 
 using namespace fms;
 
@@ -42,7 +43,7 @@ Dev device_info() {
 // Workspace carving.  All sizes in bytes, every region 256-byte aligned.
 struct Layout {
   size_t off_Xs, off_y, off_seed_idx, off_it, off_conv, off_state, off_active, off_kept,
-      off_alive, off_acc1, off_acc2, off_score, off_ym, off_mdone, off_mscore, off_modes_full,
+      off_alive, off_acc1, off_acc2, off_score, off_ym, off_mdone, off_mscore, off_dens, off_modes_full,
       off_part, off_part64, off_ctl, off_mctl, off_status, off_slog, off_yf, off_ract, off_rctl,
       off_hist, off_S, off_img, off_wlast, off_grid, off_sorted, off_perm, off_start, off_ctr,
       off_npiv, off_rad, off_table, off_ext, off_sort, total;
@@ -253,6 +254,7 @@ Layout make_layout(int64_t n, int d, int64_t Ncap, int sms, const Route& route) 
   L.off_ym = take((size_t)Ncap * L.DP * 8);
   L.off_mdone = take((size_t)Ncap * 4);
   L.off_mscore = take((size_t)Ncap * 8);
+  L.off_dens = take((size_t)Ncap * 8);
   L.off_modes_full = take((size_t)Ncap * d * 4);
   L.off_part = take(part_floats * 4);
   L.off_part64 = take(part64_doubles * 8);
@@ -498,6 +500,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     double* ym = at<double>(ws, Lo.off_ym);
     int32_t* mdone = at<int32_t>(ws, Lo.off_mdone);
     double* mscore = at<double>(ws, Lo.off_mscore);
+    double* dens = at<double>(ws, Lo.off_dens);
     float* modes_full = at<float>(ws, Lo.off_modes_full);
     float* part = at<float>(ws, Lo.off_part);
     IterCtl* ctl = at<IterCtl>(ws, Lo.off_ctl);
@@ -649,6 +652,16 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                  mscore, tol2, kRefineMaxIter, &rctl->steps,
                                  reinterpret_cast<unsigned long long*>(&rctl->evals), kf,
                                  sphere_rd, dv.sms, s_);
+    };
+
+    // the final order of the modes that the second prune left (refined: with their
+    // densities; flat windows hold whole numbers of points)
+    auto order_launch = [&](const int32_t* acc, bool refined, int max_M, cudaStream_t s_) {
+      DensityRows D{};
+      if (refined && kf == kKernelGaussian) D = {lpoints, n, scale, cosine ? 1 : 0};
+      n_launches += order_launches(D.X != nullptr, max_M) - 1;   // (and the one counted there)
+      return launch_canonical_order(D, ym, mscore, dens, acc, &mctl->Mr, d, DP, 1.0 / scale,
+                                    out_modes, max_modes, modes_full, &mctl->ticket, max_M, s_);
     };
 
     // --- Seed Selection (Alg. 2): initial seed count ---
@@ -814,10 +827,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           if (e2 == cudaSuccess)
             e2 = launch_greedy_merge_d(&mctl->M, mscore, ym, DP, d, r2_s, alive, acc2, &mctl->Mr,
                                        cap_modes, cs2);
-          if (e2 == cudaSuccess)
-            e2 = launch_canonical_order(ym, mscore, acc2, &mctl->Mr, d, DP, 1.0 / scale,
-                                        out_modes, max_modes, modes_full, nullptr, cap_modes,
-                                        cs2);
+          if (e2 == cudaSuccess) e2 = order_launch(acc2, true, cap_modes, cs2);
           if (e2 == cudaSuccess)
             e2 = launch_label(lpoints, n, d, modes_full, &mctl->Mr, 0, out_labels, out_margins,
                               cs2, cosine ? 1 : 0);
@@ -1021,8 +1031,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       FMS_LAUNCH(refine_launch(hm.M, rtol_s * rtol_s, st));
       FMS_LAUNCH(launch_greedy_merge_d(&mctl->M, mscore, ym, DP, d, r2_s, alive, acc2, &mctl->Mr,
                                        hm.M, st));
-      FMS_LAUNCH(launch_canonical_order(ym, mscore, acc2, &mctl->Mr, d, DP, 1.0 / scale,
-                                        out_modes, max_modes, modes_full, nullptr, hm.M, st));
+      FMS_LAUNCH(order_launch(acc2, true, hm.M, st));
     } else if (!o.skip_refine && hm.M > 0 && qmax > 0 && hm.M <= qmax * kModesPerCluster) {
       // cluster-persistent refinement (all updates, and each mode's density, in one launch)
       const double rtol_s = kRefineTolFactor * (double)h * scale;
@@ -1039,8 +1048,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                     sphere_rd));
       FMS_LAUNCH(launch_greedy_merge_d(&mctl->M, mscore, ym, DP, d, r2_s, alive, acc2, &mctl->Mr,
                                        hm.M, st));
-      FMS_LAUNCH(launch_canonical_order(ym, mscore, acc2, &mctl->Mr, d, DP, 1.0 / scale,
-                                        out_modes, max_modes, modes_full, nullptr, hm.M, st));
+      FMS_LAUNCH(order_launch(acc2, true, hm.M, st));
     } else if (!o.skip_refine && hm.M > 0) {
       // refinement with the ms_step kernel (many modes, or d > 7)
       const double rtol_s = kRefineTolFactor * (double)h * scale;
@@ -1060,13 +1068,11 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       // last refinement update, recorded by refine_update (as in ms_refine)
       FMS_LAUNCH(launch_greedy_merge_d(&mctl->M, mscore, ym, DP, d, r2_s, alive, acc2, &mctl->Mr,
                                        hm.M, st));
-      FMS_LAUNCH(launch_canonical_order(ym, mscore, acc2, &mctl->Mr, d, DP, 1.0 / scale,
-                                        out_modes, max_modes, modes_full, nullptr, hm.M, st));
+      FMS_LAUNCH(order_launch(acc2, true, hm.M, st));
     } else {
       FMS_LAUNCH(launch_unrefined_modes(y, kept, acc1, score, mctl, DP, ym, mscore, hm.M, st));
       FMS_CUDA(cudaMemcpyAsync(&mctl->Mr, &mctl->M, 4, cudaMemcpyDeviceToDevice, st));
-      FMS_LAUNCH(launch_canonical_order(ym, mscore, nullptr, &mctl->Mr, d, DP, 1.0 / scale,
-                                      out_modes, max_modes, modes_full, nullptr, hm.M, st));
+      FMS_LAUNCH(order_launch(nullptr, false, hm.M, st));
     }
     // --- labels (the labelling of Alg. 2) ---
     mark(3);

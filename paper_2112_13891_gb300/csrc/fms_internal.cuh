@@ -87,7 +87,7 @@ struct MergeCtl {
   int32_t Lcr;
   int32_t refine_active;  // modes still moving
   int32_t refine_iters;
-  int32_t pad0;
+  int32_t ticket;         // blocks done with the near ties of the final order
   int64_t evals;          // evaluations of prune scores and refinement
 };
 
@@ -134,6 +134,8 @@ struct SetCtl {
   int32_t rdone;
   int32_t Mr;      // modes after refinement and the second prune
   int32_t total;   // (queued) seeds converged so far, in all rounds
+  int32_t ticket;  // blocks done with the set's near ties
+  int32_t pad0;
   int64_t evals;
 };
 
@@ -565,10 +567,13 @@ cudaError_t launch_refine_update(const float* part, int32_t* active, IterCtl* rc
                                  double tol2_s, int max_iter, int64_t n, int32_t R,
                                  Tiling tl, int max_M, cudaStream_t st,
                                  double sphere_r = 0.0);
-cudaError_t launch_canonical_order(const double* ym, const double* mscore,
-                                   const int32_t* accepted, const int32_t* M_ptr, int d, int DP,
-                                   double inv_scale, float* out_modes, int32_t max_modes,
-                                   float* modes_full, float* out_scores, int max_M,
+// dens: scratch like mscore; ticket: 0 on entry and on return.  refined: D.X is set.
+struct DensityRows;
+int order_launches(bool refined, int max_M);
+cudaError_t launch_canonical_order(const DensityRows& D, const double* ym, const double* mscore,
+                                   double* dens, const int32_t* accepted, const int32_t* M_ptr,
+                                   int d, int DP, double inv_scale, float* out_modes,
+                                   int32_t max_modes, float* modes_full, int32_t* ticket, int max_M,
                                    cudaStream_t st);
 cudaError_t launch_unrefined_modes(const float* y, const int32_t* kept, const int32_t* accepted,
                                    const float* score, const MergeCtl* mctl, int DP, double* ym,

@@ -16,6 +16,7 @@
 // through conditional-node handles, whether another update, another seed round
 // or another refinement update follows.
 #include "fms_cells.cuh"
+#include "fms_density.cuh"
 #include "fms_label.cuh"
 #include "fms_prune_body.cuh"
 #include "fms_seedperm.cuh"
@@ -820,34 +821,52 @@ __global__ void __launch_bounds__(1024)
 // ---------------------------------------------------------------------------
 // canonical order and labels
 // ---------------------------------------------------------------------------
-__global__ void batched_canonical(const SetCtl* __restrict__ sc, const double* __restrict__ ym,
-                                  const double* __restrict__ mscore,
-                                  const int32_t* __restrict__ acc2, int d, int DP,
-                                  double inv_scale, float* __restrict__ out_modes, int max_modes,
-                                  float* __restrict__ modes_full, int32_t* __restrict__ out_n) {
-  const SetCtl& c = sc[blockIdx.x];
+// gridDim.y blocks to a set.  X non-null: the densities of near ties from FP64
+// (fms_density.cuh), shared by the set's blocks; the last to finish orders them.
+__global__ void __launch_bounds__(32 * kDensityWarps)
+    batched_canonical(SetCtl* sc, const float* __restrict__ X, const double* __restrict__ ym,
+                      const double* __restrict__ mscore, double* dens,
+                      const int32_t* __restrict__ acc2, int d, int DP, double scale,
+                      float* __restrict__ out_modes, int max_modes,
+                      float* __restrict__ modes_full, int32_t* __restrict__ out_n) {
+  __shared__ DensitySmem sm;
+  __shared__ int sh_last;
+  SetCtl& c = sc[blockIdx.x];
   const int M = c.Mr, p0 = c.p0;
+  const int32_t* acc = acc2 + p0;
+  const double* pos = ym + (int64_t)p0 * DP;
+  const double* score = mscore + p0;
+  if (X) {
+    const DensityRows D{X + (int64_t)p0 * d, c.n, scale, 0};
+    for (int i = blockIdx.y; i < M; i += gridDim.y) {
+      const int ai = acc[i];
+      int tie = 0;
+      for (int j = threadIdx.x; j < M && !tie; j += blockDim.x)
+        tie = j != i && near_tie(score[ai], pos + (int64_t)ai * DP, score[acc[j]],
+                                 pos + (int64_t)acc[j] * DP, d);
+      tie = __syncthreads_or(tie);
+      const double v = tie ? mode_density(D, d, pos + (int64_t)ai * DP, sm) : score[ai];
+      if (threadIdx.x == 0) dens[p0 + ai] = v;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) sh_last = atomicAdd(&c.ticket, 1) == (int)gridDim.y - 1;
+    __syncthreads();
+    if (!sh_last) return;
+    __threadfence();
+    score = dens + p0;
+  }
   if (threadIdx.x == 0 && out_n) out_n[blockIdx.x] = M;
+  const double inv_scale = 1.0 / scale;
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    const int64_t ai = (int64_t)p0 + acc2[p0 + i];
-    const double si = mscore[ai];
-    const double* pi = ym + ai * DP;
+    const int64_t ai = acc[i];
+    const double si = __ldcg(score + ai);
+    const double* pi = pos + ai * DP;
     int rank = 0;
     for (int j = 0; j < M; ++j) {
       if (j == i) continue;
-      const int64_t aj = (int64_t)p0 + acc2[p0 + j];
-      const double sj = mscore[aj];
-      bool less = false;
-      if (sj != si) less = sj > si;
-      else {
-        const double* pj = ym + aj * DP;
-        for (int k = 0; k < d; ++k)
-          if (pj[k] != pi[k]) {
-            less = pj[k] < pi[k];
-            break;
-          }
-      }
-      rank += less;
+      const int64_t aj = acc[j];
+      rank += mode_before(__ldcg(score + aj), pos + aj * DP, si, pi, d) ? 1 : 0;
     }
     for (int k = 0; k < d; ++k) {
       const float v = (float)(pi[k] * inv_scale);
@@ -1040,12 +1059,14 @@ cudaError_t launch_batched_refine_compact(SetCtl* sc, int B, const int32_t* mdon
   return cudaGetLastError();
 }
 
-cudaError_t launch_batched_canonical(const SetCtl* sc, int B, const double* ym,
-                                     const double* mscore, const int32_t* acc2, int d, int DP,
-                                     double inv_scale, float* out_modes, int max_modes,
+cudaError_t launch_batched_canonical(SetCtl* sc, int B, const float* X, const double* ym,
+                                     const double* mscore, double* dens, const int32_t* acc2,
+                                     int d, int DP, double scale, float* out_modes, int max_modes,
                                      float* modes_full, int32_t* out_n, cudaStream_t st) {
-  batched_canonical<<<B, 256, 0, st>>>(sc, ym, mscore, acc2, d, DP, inv_scale, out_modes,
-                                       max_modes, modes_full, out_n);
+  int per = X && B < 1216 ? 1216 / B : 1;
+  if (per > 64) per = 64;
+  batched_canonical<<<dim3((unsigned)B, (unsigned)per), 32 * kDensityWarps, 0, st>>>(
+      sc, X, ym, mscore, dens, acc2, d, DP, scale, out_modes, max_modes, modes_full, out_n);
   return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 // canonical ordering and nearest-mode labelling.
 #include <float.h>
 
+#include "fms_density.cuh"
 #include "fms_label.cuh"
 #include "fms_prune_body.cuh"
 
@@ -614,38 +615,98 @@ cudaError_t launch_refine_update(const float* part, int32_t* active, IterCtl* rc
 }
 
 // ---------------------------------------------------------------------------
-// Canonical order: score descending, ties by lexicographic coordinates.
-// rank_i = #{j : key_j < key_i}; modes are written in original units.
+// Canonical order: density descending, ties by lexicographic coordinates, the
+// densities of near ties from FP64 (fms_density.cuh).  rank_i = #{j : j before i};
+// modes are written in original units.
 // ---------------------------------------------------------------------------
-template <typename PT>
-__device__ __forceinline__ bool key_less(double sa, const PT* a, double sb, const PT* b, int d) {
-  if (sa != sb) return sa > sb;
-  for (int k = 0; k < d; ++k)
-    if (a[k] != b[k]) return a[k] < b[k];
-  return false;
+constexpr int kOrderStage = 1024;    // modes whose scores fit in shared memory
+constexpr int kOrderThreads = 32 * kDensityWarps;
+
+// FP64 densities of the near ties among modes i = blockIdx.x, + gridDim.x, .. into
+// dens (indexed as mscore), the others' scores as they are.
+__device__ __forceinline__ void tie_densities(const DensityRows& D, const double* __restrict__ ym,
+                                              const double* __restrict__ mscore,
+                                              const int32_t* __restrict__ accepted, int M, int d,
+                                              int DP, double* __restrict__ dens,
+                                              DensitySmem& sm) {
+  for (int i = blockIdx.x; i < M; i += gridDim.x) {
+    const int ai = accepted ? accepted[i] : i;
+    const double* pa = ym + (int64_t)ai * DP;
+    const double sa = mscore[ai];
+    int tie = 0;
+    for (int j = threadIdx.x; j < M && !tie; j += blockDim.x) {
+      const int aj = accepted ? accepted[j] : j;
+      tie = j != i && near_tie(sa, pa, mscore[aj], ym + (int64_t)aj * DP, d);
+    }
+    const double v = __syncthreads_or(tie) ? mode_density(D, d, pa, sm) : sa;
+    if (threadIdx.x == 0) dens[ai] = v;
+  }
 }
 
-__global__ void canonical_order_kernel(const double* __restrict__ ym,
-                                       const double* __restrict__ mscore,
-                                       const int32_t* __restrict__ accepted,
-                                       const int32_t* __restrict__ M_ptr, int d, int DP,
-                                       double inv_scale, float* __restrict__ out_modes,
-                                       int32_t max_modes, float* __restrict__ modes_full,
-                                       float* __restrict__ out_scores) {
+__global__ void __launch_bounds__(kOrderThreads)
+    tie_density_kernel(DensityRows D, const double* __restrict__ ym,
+                       const double* __restrict__ mscore, const int32_t* __restrict__ accepted,
+                       const int32_t* __restrict__ M_ptr, int d, int DP,
+                       double* __restrict__ dens) {
+  __shared__ DensitySmem sm;
+  tie_densities(D, ym, mscore, accepted, *M_ptr, d, DP, dens, sm);
+}
+
+// D.X null: mscore as it is.  Up to kOrderStage modes, every block looks for near
+// ties among all of them (a few hundred comparisons for tens of modes); where there
+// are none, each ranks its share at once, else the blocks share the FP64 densities
+// and the last to finish (*ticket counts them, no waiting) ranks them all.
+__global__ void __launch_bounds__(kOrderThreads)
+    canonical_order_kernel(DensityRows D, const double* __restrict__ ym,
+                           const double* __restrict__ mscore, double* dens,
+                           const int32_t* __restrict__ accepted,
+                           const int32_t* __restrict__ M_ptr, int d, int DP, double inv_scale,
+                           float* __restrict__ out_modes, int32_t max_modes,
+                           float* __restrict__ modes_full, int32_t* ticket) {
   // the modes' scores are staged in shared memory (one load each instead of a
   // dependent load per comparison); coordinates are read only on equal scores
-  constexpr int kStage = 1024;
-  __shared__ double s_sc[kStage];
+  __shared__ double s_sc[kOrderStage];
+  __shared__ DensitySmem sm;
+  __shared__ int sh_last;
   const int M = *M_ptr;
-  const bool staged = M <= kStage;
+  const bool staged = M <= kOrderStage;
   if (staged) {
     for (int j = threadIdx.x; j < M; j += blockDim.x) s_sc[j] = mscore[accepted ? accepted[j] : j];
     __syncthreads();
   }
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
+  int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  if (D.X && staged) {
+    int tie = 0;
+    for (int i = threadIdx.x; i < M && !tie; i += blockDim.x) {
+      const double si = s_sc[i];
+      for (int j = 0; j < M && !tie; ++j) {
+        if (j <= i || !(fabs(si - s_sc[j]) <= 0.05 * fmax(si, s_sc[j]))) continue;
+        const int64_t ai = accepted ? accepted[i] : i, aj = accepted ? accepted[j] : j;
+        tie = near_tie(si, ym + ai * DP, s_sc[j], ym + aj * DP, d);
+      }
+    }
+    if (__syncthreads_or(tie)) {
+      tie_densities(D, ym, mscore, accepted, M, d, DP, dens, sm);
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        sh_last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+        if (sh_last) *ticket = 0;
+      }
+      __syncthreads();
+      if (!sh_last) return;
+      __threadfence();
+      for (int j = threadIdx.x; j < M; j += blockDim.x)
+        s_sc[j] = __ldcg(dens + (accepted ? accepted[j] : j));
+      __syncthreads();
+      first = threadIdx.x;
+      step = blockDim.x;
+    }
+  }
+  for (int i = first; i < M; i += step) {
     const int ai = accepted ? accepted[i] : i;
     const double* pa = ym + (int64_t)ai * DP;
-    const double sa = mscore[ai];
+    const double sa = staged ? s_sc[i] : mscore[ai];
     int rank = 0;
     for (int j = 0; j < M; ++j) {
       if (j == i) continue;
@@ -654,7 +715,7 @@ __global__ void canonical_order_kernel(const double* __restrict__ ym,
         rank += sj > sa ? 1 : 0;
       } else {
         const int aj = accepted ? accepted[j] : j;
-        if (key_less(sj, ym + (int64_t)aj * DP, sa, pa, d)) ++rank;
+        if (mode_before(sj, ym + (int64_t)aj * DP, sa, pa, d)) ++rank;
       }
     }
     for (int k = 0; k < d; ++k) {
@@ -662,20 +723,32 @@ __global__ void canonical_order_kernel(const double* __restrict__ ym,
       modes_full[(int64_t)rank * d + k] = v;
       if (out_modes && rank < max_modes) out_modes[(int64_t)rank * d + k] = v;
     }
-    if (out_scores) out_scores[rank] = (float)sa;
   }
 }
 
-cudaError_t launch_canonical_order(const double* ym, const double* mscore,
-                                   const int32_t* accepted, const int32_t* M_ptr, int d, int DP,
-                                   double inv_scale, float* out_modes, int32_t max_modes,
-                                   float* modes_full, float* out_scores, int max_M,
+int order_launches(bool refined, int max_M) { return refined && max_M > kOrderStage ? 2 : 1; }
+
+cudaError_t launch_canonical_order(const DensityRows& D, const double* ym, const double* mscore,
+                                   double* dens, const int32_t* accepted, const int32_t* M_ptr,
+                                   int d, int DP, double inv_scale, float* out_modes,
+                                   int32_t max_modes, float* modes_full, int32_t* ticket, int max_M,
                                    cudaStream_t st) {
-  int blocks = (max_M + 127) / 128;
+  DensityRows rows = D;
+  if (D.X && max_M > kOrderStage) {   // (one block would rank them all)
+    tie_density_kernel<<<max_M < 1216 ? max_M : 1216, kOrderThreads, 0, st>>>(
+        D, ym, mscore, accepted, M_ptr, d, DP, dens);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    mscore = dens;
+    rows.X = nullptr;
+  }
+  int blocks = rows.X ? max_M : (max_M + kOrderThreads - 1) / kOrderThreads;
+  const int most = rows.X ? 152 : 1024;
   if (blocks < 1) blocks = 1;
-  if (blocks > 1024) blocks = 1024;
-  canonical_order_kernel<<<blocks, 128, 0, st>>>(ym, mscore, accepted, M_ptr, d, DP, inv_scale,
-                                                 out_modes, max_modes, modes_full, out_scores);
+  if (blocks > most) blocks = most;
+  canonical_order_kernel<<<blocks, kOrderThreads, 0, st>>>(rows, ym, mscore, dens, accepted, M_ptr,
+                                                           d, DP, inv_scale, out_modes, max_modes,
+                                                           modes_full, ticket);
   return cudaGetLastError();
 }
 

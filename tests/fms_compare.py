@@ -7,8 +7,8 @@ threshold -- their nearest mode is decided by rounding.  The mode ORDER is
 part of the output contract (canonical order: density score descending, ties
 by coordinates), so the matched GPU order must equal the oracle's, except that
 two modes whose oracle scores agree within a relative score tolerance may
-appear in either order (their GPU scores are FP32 sums at positions within
-the mode tolerance, so such a near-tie can be decided either way).
+appear in either order: near ties are decided by FP64 densities at the refined
+positions, which are within 1e-5 h of the maximum (1e-10 of the density).
 """
 import numpy as np
 from scipy.optimize import linear_sum_assignment
@@ -26,7 +26,7 @@ def match_modes(gpu_modes, ref_modes):
     return perm, float(D[gi, ri].max()) if len(gi) else 0.0
 
 
-def order_violations(perm, ref_scores, score_rtol=1e-4):
+def order_violations(perm, ref_scores, score_rtol=1e-8):
     """Pairs of GPU positions i < j whose matched oracle modes come in the
     opposite canonical order although their oracle scores differ by more than
     score_rtol (relative to the larger score)."""
@@ -39,7 +39,7 @@ def order_violations(perm, ref_scores, score_rtol=1e-4):
 
 
 def compare_clustering(gpu_modes, gpu_labels, ref, h, mode_tol=1e-3, margin_tol=1e-2,
-                       score_rtol=1e-4):
+                       score_rtol=1e-8):
     """Returns a dict of errors; raises on a mode-count mismatch.  mode_ok
     requires every matched mode within mode_tol*h and the canonical order."""
     perm, err = match_modes(gpu_modes, ref.modes)
