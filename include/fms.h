@@ -200,11 +200,11 @@ size_t fms_workspace_size(int64_t n, int32_t d, const fms_options* opt);
  *                order: density descending, ties by coordinates.  The
  *                density is sum w of the mode's last refinement update (one
  *                step of at most 1e-5*h before the mode); Gaussian densities
- *                that its FP32 weights cannot tell apart (4e-6, more far
- *                from the origin) are taken from FP64 weights of the given
- *                points at the refined position, within O(1e-10) relative
- *                of the KDE value at the mode.  (skip_refine: the prune's
- *                FP32 densities.)
+ *                that its FP32 weights cannot tell apart (some 1e-7, more
+ *                far from the origin) are taken from FP64 weights of the
+ *                given points at the refined position, within O(1e-10)
+ *                relative of the KDE value at the mode and rounded to 36
+ *                bits.  (skip_refine: the prune's FP32 densities.)
  *   out_n_modes  host int32: M.  If M > max_modes, FMS_ERR_CAPACITY is
  *                returned, *out_n_modes = M and out_modes holds the first
  *                max_modes modes; labels are still written.

@@ -43,8 +43,9 @@ Dev device_info() {
 // Workspace carving.  All sizes in bytes, every region 256-byte aligned.
 struct Layout {
   size_t off_Xs, off_y, off_seed_idx, off_it, off_conv, off_state, off_active, off_kept,
-      off_alive, off_acc1, off_acc2, off_score, off_ym, off_mdone, off_mscore, off_dens, off_modes_full,
-      off_part, off_part64, off_ctl, off_mctl, off_status, off_slog, off_yf, off_ract, off_rctl,
+      off_alive, off_acc1, off_acc2, off_score, off_ym, off_mdone, off_mscore, off_dens, off_ties,
+      off_modes_full, off_part, off_part64, off_ctl, off_mctl, off_status, off_slog, off_yf,
+      off_ract, off_rctl,
       off_hist, off_S, off_img, off_wlast, off_grid, off_sorted, off_perm, off_start, off_ctr,
       off_npiv, off_rad, off_table, off_ext, off_sort, total;
   int DP, DA, R, grid_ctas;
@@ -255,6 +256,7 @@ Layout make_layout(int64_t n, int d, int64_t Ncap, int sms, const Route& route) 
   L.off_mdone = take((size_t)Ncap * 4);
   L.off_mscore = take((size_t)Ncap * 8);
   L.off_dens = take((size_t)Ncap * 8);
+  L.off_ties = take(order_scratch_bytes(d));
   L.off_modes_full = take((size_t)Ncap * d * 4);
   L.off_part = take(part_floats * 4);
   L.off_part64 = take(part64_doubles * 8);
@@ -660,8 +662,9 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       DensityRows D{};
       if (refined && kf == kKernelGaussian) D = {lpoints, n, scale, cosine ? 1 : 0};
       n_launches += order_launches(D.X != nullptr, max_M) - 1;   // (and the one counted there)
-      return launch_canonical_order(D, ym, mscore, dens, acc, &mctl->Mr, d, DP, 1.0 / scale,
-                                    out_modes, max_modes, modes_full, &mctl->ticket, max_M, s_);
+      return launch_canonical_order(D, ym, mscore, dens, at<double>(ws, Lo.off_ties), acc,
+                                    &mctl->Mr, d, DP, 1.0 / scale, out_modes, max_modes,
+                                    modes_full, &mctl->ticket, max_M, s_);
     };
 
     // --- Seed Selection (Alg. 2): initial seed count ---

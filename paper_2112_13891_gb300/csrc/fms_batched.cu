@@ -77,10 +77,12 @@ cudaError_t launch_batched_refine_compact(SetCtl* sc, int B, const int32_t* mdon
                                           int64_t* task_off, int64_t* part_off, int64_t* list_off,
                                           int64_t* totals, int32_t* counters, BatchCond cond,
                                           const uint32_t* status, cudaStream_t st);
+size_t batched_order_scratch(int B, int d);
 cudaError_t launch_batched_canonical(SetCtl* sc, int B, const float* X, const double* ym,
-                                     const double* mscore, double* dens, const int32_t* acc2,
-                                     int d, int DP, double scale, float* out_modes, int max_modes,
-                                     float* modes_full, int32_t* out_n, cudaStream_t st);
+                                     const double* mscore, double* dens, double* scratch,
+                                     const int32_t* acc2, int d, int DP, double scale,
+                                     float* out_modes, int max_modes, float* modes_full,
+                                     int32_t* out_n, cudaStream_t st);
 cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int max_n, int d,
                                  const SetCtl* sc, const float* modes_full, int32_t* labels,
                                  float* margins, cudaStream_t st);
@@ -107,7 +109,7 @@ int sms_now() {
 
 struct BLayout {
   size_t Xs, y, it, conv, state, active, kept, acc1, acc2, plist, score, ym, yf, ract, mdone,
-      mscore, dens, modes_full, part, sc, task_off, part_off, list_off, totals, counters, pt_off, status,
+      mscore, dens, ties, modes_full, part, sc, task_off, part_off, list_off, totals, counters, pt_off, status,
       sorted, start, ctr, npiv, rad, sort, wlast, total;
   int DP, DA, R, TW, P;
   bool queued;
@@ -174,6 +176,7 @@ BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw
   L.mdone = take((size_t)total * 4);
   L.mscore = take((size_t)total * 8);
   L.dens = take((size_t)total * 8);
+  L.ties = take(batched_order_scratch(B, d));
   L.modes_full = take((size_t)total * d * 4);
   L.part = take(L.queued ? 0 : part_floats * 4);
   L.sc = take((size_t)B * sizeof(SetCtl));
@@ -662,8 +665,8 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         e = launch_batched_prune_d(sc, B, mscore, ym, DP, d, r2_s, acc2, plist, max_n, cs0);
       if (e == cudaSuccess)
         e = launch_batched_canonical(sc, B, o.skip_refine ? nullptr : points, ym, mscore, dens,
-                                     acc2, d, DP, scale, out_modes, max_modes, modes_full,
-                                     out_n_modes, cs0);
+                                     at<double>(ws, Lo.ties), acc2, d, DP, scale, out_modes,
+                                     max_modes, modes_full, out_n_modes, cs0);
       if (e == cudaSuccess)
         e = launch_batched_label(points, pt_off, B, max_n, d, sc, modes_full, out_labels,
                                  out_margins, cs0);

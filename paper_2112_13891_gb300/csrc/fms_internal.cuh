@@ -567,14 +567,16 @@ cudaError_t launch_refine_update(const float* part, int32_t* active, IterCtl* rc
                                  double tol2_s, int max_iter, int64_t n, int32_t R,
                                  Tiling tl, int max_M, cudaStream_t st,
                                  double sphere_r = 0.0);
-// dens: scratch like mscore; ticket: 0 on entry and on return.  refined: D.X is set.
+// dens: scratch like mscore; scratch: order_scratch_bytes(d); ticket: 0 on entry and on
+// return.  refined: D.X is set.
 struct DensityRows;
 int order_launches(bool refined, int max_M);
+size_t order_scratch_bytes(int d);
 cudaError_t launch_canonical_order(const DensityRows& D, const double* ym, const double* mscore,
-                                   double* dens, const int32_t* accepted, const int32_t* M_ptr,
-                                   int d, int DP, double inv_scale, float* out_modes,
-                                   int32_t max_modes, float* modes_full, int32_t* ticket, int max_M,
-                                   cudaStream_t st);
+                                   double* dens, double* scratch, const int32_t* accepted,
+                                   const int32_t* M_ptr, int d, int DP, double inv_scale,
+                                   float* out_modes, int32_t max_modes, float* modes_full,
+                                   int32_t* ticket, int max_M, cudaStream_t st);
 cudaError_t launch_unrefined_modes(const float* y, const int32_t* kept, const int32_t* accepted,
                                    const float* score, const MergeCtl* mctl, int DP, double* ym,
                                    double* mscore, int max_M, cudaStream_t st);

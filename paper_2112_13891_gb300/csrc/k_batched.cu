@@ -822,51 +822,68 @@ __global__ void __launch_bounds__(1024)
 // canonical order and labels
 // ---------------------------------------------------------------------------
 // gridDim.y blocks to a set.  X non-null: the densities of near ties from FP64
-// (fms_density.cuh), shared by the set's blocks; the last to finish orders them.
+// (fms_density.cuh), shared by the set's blocks.
 __global__ void __launch_bounds__(32 * kDensityWarps)
     batched_canonical(SetCtl* sc, const float* __restrict__ X, const double* __restrict__ ym,
-                      const double* __restrict__ mscore, double* dens,
+                      const double* __restrict__ mscore, double* dens, double* scratch,
                       const int32_t* __restrict__ acc2, int d, int DP, double scale,
                       float* __restrict__ out_modes, int max_modes,
                       float* __restrict__ modes_full, int32_t* __restrict__ out_n) {
-  __shared__ DensitySmem sm;
-  __shared__ int sh_last;
+  __shared__ OrderSmem sm;
   SetCtl& c = sc[blockIdx.x];
-  const int M = c.Mr, p0 = c.p0;
+  const int M = c.Mr, p0 = c.p0, bi = blockIdx.y, nb = gridDim.y;
   const int32_t* acc = acc2 + p0;
   const double* pos = ym + (int64_t)p0 * DP;
   const double* score = mscore + p0;
-  if (X) {
-    const DensityRows D{X + (int64_t)p0 * d, c.n, scale, 0};
-    for (int i = blockIdx.y; i < M; i += gridDim.y) {
+  DensityRows D{};
+  if (X) D = {X + (int64_t)p0 * d, c.n, scale, 0};
+  const bool staged = M <= kOrderStage;
+  if (staged) {
+    bool tied;
+    if (!order_densities(D, pos, score, dens + p0, acc, M, d, DP,
+                         scratch + (int64_t)blockIdx.x * nb * kTieCap * (d + 1), &c.ticket, bi,
+                         nb, sm, &tied) ||
+        (!tied && bi > 0))
+      return;
+  } else {
+    for (int i = bi; D.X && i < M; i += nb) {
       const int ai = acc[i];
-      int tie = 0;
-      for (int j = threadIdx.x; j < M && !tie; j += blockDim.x)
-        tie = j != i && near_tie(score[ai], pos + (int64_t)ai * DP, score[acc[j]],
-                                 pos + (int64_t)acc[j] * DP, d);
-      tie = __syncthreads_or(tie);
-      const double v = tie ? mode_density(D, d, pos + (int64_t)ai * DP, sm) : score[ai];
+      const double* pa = pos + (int64_t)ai * DP;
+      const float ea = density_error(score[ai], mode_norm(pa, d));
+      bool tie = false;
+      for (int j = threadIdx.x; j < M && !tie; j += blockDim.x) {
+        const double sj = score[acc[j]];
+        tie = j != i && near_tie((float)score[ai], 0.03f, (float)sj, 0.03f) &&
+              near_tie((float)score[ai], ea, (float)sj,
+                       density_error(sj, mode_norm(pos + (int64_t)acc[j] * DP, d)));
+      }
+      double v = score[ai];
+      if (__syncthreads_or(tie)) {
+        density_sums(D, 0, D.n, d, pa, density_bits(v, D.n), sm);
+        v = mode_density(sm.red[0], d, scale);
+      }
       if (threadIdx.x == 0) dens[p0 + ai] = v;
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) sh_last = atomicAdd(&c.ticket, 1) == (int)gridDim.y - 1;
+    if (threadIdx.x == 0) sm.last = atomicAdd(&c.ticket, 1) == nb - 1;
     __syncthreads();
-    if (!sh_last) return;
+    if (!sm.last) return;
     __threadfence();
-    score = dens + p0;
+    if (D.X) score = dens + p0;
   }
   if (threadIdx.x == 0 && out_n) out_n[blockIdx.x] = M;
   const double inv_scale = 1.0 / scale;
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
     const int64_t ai = acc[i];
-    const double si = __ldcg(score + ai);
+    const double si = staged ? sm.score[i] : __ldcg(score + ai);
     const double* pi = pos + ai * DP;
     int rank = 0;
     for (int j = 0; j < M; ++j) {
       if (j == i) continue;
       const int64_t aj = acc[j];
-      rank += mode_before(__ldcg(score + aj), pos + aj * DP, si, pi, d) ? 1 : 0;
+      const double sj = staged ? sm.score[j] : __ldcg(score + aj);
+      rank += mode_before(sj, pos + aj * DP, si, pi, d) ? 1 : 0;
     }
     for (int k = 0; k < d; ++k) {
       const float v = (float)(pi[k] * inv_scale);
@@ -1059,14 +1076,22 @@ cudaError_t launch_batched_refine_compact(SetCtl* sc, int B, const int32_t* mdon
   return cudaGetLastError();
 }
 
+// Blocks that share a set's near ties, and their scratch in all.
+static int order_share(int B) { return B < 1216 ? (1216 / B < 64 ? 1216 / B : 64) : 1; }
+size_t batched_order_scratch(int B, int d) {
+  const int per = order_share(B);
+  return per > 1 ? tie_scratch_bytes(B * per, d) : 0;
+}
+
 cudaError_t launch_batched_canonical(SetCtl* sc, int B, const float* X, const double* ym,
-                                     const double* mscore, double* dens, const int32_t* acc2,
-                                     int d, int DP, double scale, float* out_modes, int max_modes,
-                                     float* modes_full, int32_t* out_n, cudaStream_t st) {
-  int per = X && B < 1216 ? 1216 / B : 1;
-  if (per > 64) per = 64;
+                                     const double* mscore, double* dens, double* scratch,
+                                     const int32_t* acc2, int d, int DP, double scale,
+                                     float* out_modes, int max_modes, float* modes_full,
+                                     int32_t* out_n, cudaStream_t st) {
+  const int per = X ? order_share(B) : 1;
   batched_canonical<<<dim3((unsigned)B, (unsigned)per), 32 * kDensityWarps, 0, st>>>(
-      sc, X, ym, mscore, dens, acc2, d, DP, scale, out_modes, max_modes, modes_full, out_n);
+      sc, X, ym, mscore, dens, scratch, acc2, d, DP, scale, out_modes, max_modes, modes_full,
+      out_n);
   return cudaGetLastError();
 }
 

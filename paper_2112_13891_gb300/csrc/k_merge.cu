@@ -619,120 +619,105 @@ cudaError_t launch_refine_update(const float* part, int32_t* active, IterCtl* rc
 // densities of near ties from FP64 (fms_density.cuh).  rank_i = #{j : j before i};
 // modes are written in original units.
 // ---------------------------------------------------------------------------
-constexpr int kOrderStage = 1024;    // modes whose scores fit in shared memory
 constexpr int kOrderThreads = 32 * kDensityWarps;
+constexpr int kOrderBlocks = 152;    // blocks that share near ties (sums in block order)
 
-// FP64 densities of the near ties among modes i = blockIdx.x, + gridDim.x, .. into
-// dens (indexed as mscore), the others' scores as they are.
-__device__ __forceinline__ void tie_densities(const DensityRows& D, const double* __restrict__ ym,
-                                              const double* __restrict__ mscore,
-                                              const int32_t* __restrict__ accepted, int M, int d,
-                                              int DP, double* __restrict__ dens,
-                                              DensitySmem& sm) {
-  for (int i = blockIdx.x; i < M; i += gridDim.x) {
-    const int ai = accepted ? accepted[i] : i;
-    const double* pa = ym + (int64_t)ai * DP;
-    const double sa = mscore[ai];
-    int tie = 0;
-    for (int j = threadIdx.x; j < M && !tie; j += blockDim.x) {
-      const int aj = accepted ? accepted[j] : j;
-      tie = j != i && near_tie(sa, pa, mscore[aj], ym + (int64_t)aj * DP, d);
-    }
-    const double v = __syncthreads_or(tie) ? mode_density(D, d, pa, sm) : sa;
-    if (threadIdx.x == 0) dens[ai] = v;
-  }
-}
-
+// More than kOrderStage modes: their densities into dens, a block per mode.
 __global__ void __launch_bounds__(kOrderThreads)
     tie_density_kernel(DensityRows D, const double* __restrict__ ym,
                        const double* __restrict__ mscore, const int32_t* __restrict__ accepted,
                        const int32_t* __restrict__ M_ptr, int d, int DP,
                        double* __restrict__ dens) {
-  __shared__ DensitySmem sm;
-  tie_densities(D, ym, mscore, accepted, *M_ptr, d, DP, dens, sm);
+  __shared__ OrderSmem sm;
+  const int M = *M_ptr;
+  for (int i = blockIdx.x; i < M; i += gridDim.x) {
+    const int ai = accepted ? accepted[i] : i;
+    const double* pa = ym + (int64_t)ai * DP;
+    const double sa = mscore[ai];
+    const float ea = density_error(sa, mode_norm(pa, d));
+    bool tie = false;
+    for (int j = threadIdx.x; j < M && !tie; j += blockDim.x) {
+      const int aj = accepted ? accepted[j] : j;
+      const double sj = mscore[aj];
+      // (the position is not read where nothing could make them near)
+      tie = j != i && near_tie((float)sa, 0.03f, (float)sj, 0.03f) &&
+            near_tie((float)sa, ea, (float)sj,
+                     density_error(sj, mode_norm(ym + (int64_t)aj * DP, d)));
+    }
+    double v = sa;
+    if (__syncthreads_or(tie)) {
+      density_sums(D, 0, D.n, d, pa, density_bits(sa, D.n), sm);
+      v = mode_density(sm.red[0], d, D.scale);
+    }
+    if (threadIdx.x == 0) dens[ai] = v;
+  }
 }
 
-// D.X null: mscore as it is.  Up to kOrderStage modes, every block looks for near
-// ties among all of them (a few hundred comparisons for tens of modes); where there
-// are none, each ranks its share at once, else the blocks share the FP64 densities
-// and the last to finish (*ticket counts them, no waiting) ranks them all.
 __global__ void __launch_bounds__(kOrderThreads)
     canonical_order_kernel(DensityRows D, const double* __restrict__ ym,
-                           const double* __restrict__ mscore, double* dens,
+                           const double* __restrict__ mscore, double* dens, double* scratch,
                            const int32_t* __restrict__ accepted,
                            const int32_t* __restrict__ M_ptr, int d, int DP, double inv_scale,
                            float* __restrict__ out_modes, int32_t max_modes,
                            float* __restrict__ modes_full, int32_t* ticket) {
-  // the modes' scores are staged in shared memory (one load each instead of a
-  // dependent load per comparison); coordinates are read only on equal scores
-  __shared__ double s_sc[kOrderStage];
-  __shared__ DensitySmem sm;
-  __shared__ int sh_last;
+  // up to kOrderStage scores in shared memory (one load each instead of a dependent
+  // load per comparison); coordinates are read only on equal scores
+  __shared__ OrderSmem sm;
   const int M = *M_ptr;
   const bool staged = M <= kOrderStage;
+  int first = blockIdx.x * blockDim.x, step = gridDim.x * blockDim.x;
   if (staged) {
-    for (int j = threadIdx.x; j < M; j += blockDim.x) s_sc[j] = mscore[accepted ? accepted[j] : j];
-    __syncthreads();
-  }
-  int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
-  if (D.X && staged) {
-    int tie = 0;
-    for (int i = threadIdx.x; i < M && !tie; i += blockDim.x) {
-      const double si = s_sc[i];
-      for (int j = 0; j < M && !tie; ++j) {
-        if (j <= i || !(fabs(si - s_sc[j]) <= 0.05 * fmax(si, s_sc[j]))) continue;
-        const int64_t ai = accepted ? accepted[i] : i, aj = accepted ? accepted[j] : j;
-        tie = near_tie(si, ym + ai * DP, s_sc[j], ym + aj * DP, d);
-      }
-    }
-    if (__syncthreads_or(tie)) {
-      tie_densities(D, ym, mscore, accepted, M, d, DP, dens, sm);
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        sh_last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
-        if (sh_last) *ticket = 0;
-      }
-      __syncthreads();
-      if (!sh_last) return;
-      __threadfence();
-      for (int j = threadIdx.x; j < M; j += blockDim.x)
-        s_sc[j] = __ldcg(dens + (accepted ? accepted[j] : j));
-      __syncthreads();
-      first = threadIdx.x;
+    bool tied;
+    if (!order_densities(D, ym, mscore, dens, accepted, M, d, DP, scratch, ticket, blockIdx.x,
+                         gridDim.x, sm, &tied))
+      return;
+    if (tied) {   // this block ranks all
+      first = 0;
       step = blockDim.x;
     }
   }
-  for (int i = first; i < M; i += step) {
-    const int ai = accepted ? accepted[i] : i;
-    const double* pa = ym + (int64_t)ai * DP;
-    const double sa = staged ? s_sc[i] : mscore[ai];
-    int rank = 0;
-    for (int j = 0; j < M; ++j) {
-      if (j == i) continue;
-      const double sj = staged ? s_sc[j] : mscore[accepted ? accepted[j] : j];
-      if (sj != sa) {
-        rank += sj > sa ? 1 : 0;
-      } else {
-        const int aj = accepted ? accepted[j] : j;
-        if (mode_before(sj, ym + (int64_t)aj * DP, sa, pa, d)) ++rank;
+  // a thread finds a mode's rank, then the block writes the modes' coordinates
+  __shared__ int rank_of[kOrderThreads];
+  for (int i0 = first; i0 < M; i0 += step) {
+    const int i = i0 + (int)threadIdx.x;
+    if (i < M) {
+      const int ai = accepted ? accepted[i] : i;
+      const double* pa = ym + (int64_t)ai * DP;
+      const double sa = staged ? sm.score[i] : mscore[ai];
+      int rank = 0;
+      for (int j = 0; j < M; ++j) {
+        if (j == i) continue;
+        const double sj = staged ? sm.score[j] : mscore[accepted ? accepted[j] : j];
+        if (sj != sa) {
+          rank += sj > sa ? 1 : 0;
+        } else {
+          const int aj = accepted ? accepted[j] : j;
+          if (mode_before(sj, ym + (int64_t)aj * DP, sa, pa, d)) ++rank;
+        }
       }
+      rank_of[threadIdx.x] = rank;
     }
-    for (int k = 0; k < d; ++k) {
-      const float v = (float)(pa[k] * inv_scale);
+    __syncthreads();
+    const int cnt = min((int)blockDim.x, M - i0) * d;
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+      const int q = e / d, k = e - q * d, rank = rank_of[q];
+      const int ai = accepted ? accepted[i0 + q] : i0 + q;
+      const float v = (float)(ym[(int64_t)ai * DP + k] * inv_scale);
       modes_full[(int64_t)rank * d + k] = v;
       if (out_modes && rank < max_modes) out_modes[(int64_t)rank * d + k] = v;
     }
+    __syncthreads();
   }
 }
 
 int order_launches(bool refined, int max_M) { return refined && max_M > kOrderStage ? 2 : 1; }
+size_t order_scratch_bytes(int d) { return tie_scratch_bytes(kOrderBlocks, d); }
 
 cudaError_t launch_canonical_order(const DensityRows& D, const double* ym, const double* mscore,
-                                   double* dens, const int32_t* accepted, const int32_t* M_ptr,
-                                   int d, int DP, double inv_scale, float* out_modes,
-                                   int32_t max_modes, float* modes_full, int32_t* ticket, int max_M,
-                                   cudaStream_t st) {
+                                   double* dens, double* scratch, const int32_t* accepted,
+                                   const int32_t* M_ptr, int d, int DP, double inv_scale,
+                                   float* out_modes, int32_t max_modes, float* modes_full,
+                                   int32_t* ticket, int max_M, cudaStream_t st) {
   DensityRows rows = D;
   if (D.X && max_M > kOrderStage) {   // (one block would rank them all)
     tie_density_kernel<<<max_M < 1216 ? max_M : 1216, kOrderThreads, 0, st>>>(
@@ -742,13 +727,13 @@ cudaError_t launch_canonical_order(const DensityRows& D, const double* ym, const
     mscore = dens;
     rows.X = nullptr;
   }
-  int blocks = rows.X ? max_M : (max_M + kOrderThreads - 1) / kOrderThreads;
-  const int most = rows.X ? 152 : 1024;
+  int blocks = (max_M + kOrderThreads - 1) / kOrderThreads;
   if (blocks < 1) blocks = 1;
-  if (blocks > most) blocks = most;
-  canonical_order_kernel<<<blocks, kOrderThreads, 0, st>>>(rows, ym, mscore, dens, accepted, M_ptr,
-                                                           d, DP, inv_scale, out_modes, max_modes,
-                                                           modes_full, ticket);
+  if (blocks > 1024) blocks = 1024;
+  if (rows.X) blocks = kOrderBlocks;
+  canonical_order_kernel<<<blocks, kOrderThreads, 0, st>>>(
+      rows, ym, mscore, dens, scratch, accepted, M_ptr, d, DP, inv_scale, out_modes, max_modes,
+      modes_full, ticket);
   return cudaGetLastError();
 }
 
