@@ -371,22 +371,16 @@ inline int team_warps(int64_t groups, int sms, int warp_smem, int most = 8) {
   return W;
 }
 
-// Lets a kernel use all the dynamic shared memory that the device leaves beside its
-// static arrays: one limit for every launch of the kernel, whatever its size, since
-// the attribute belongs to the kernel (another thread's launch may come in between)
-// and the default of 48 KB counts the static arrays as well.
+// Lets a kernel use the device's 227 KB of shared memory a block, less kTeamStatic for
+// its static arrays: one limit for every launch of the kernel, whatever its size, since
+// the attribute belongs to the kernel (another thread's launch may come in between).
+// The default of 48 KB counts the static arrays as well.
+constexpr int kTeamStatic = 256;
 template <typename K>
-inline cudaError_t team_attr(K kernel) {
-  int dev = 0, most = 0;
-  cudaFuncAttributes at;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess)
-    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
-  if (e != cudaSuccess) return e;
-  const int limit = most - (int)at.sharedSizeBytes;
-  if (at.maxDynamicSharedSizeBytes == limit) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+inline cudaError_t team_attr(K kernel, int bytes) {
+  if (bytes + kTeamStatic <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              227 * 1024 - kTeamStatic);
 }
 
 }  // namespace fms

@@ -762,7 +762,7 @@ cudaError_t launch_step_groups(const float* Xs, const View<float>& cv, int n, co
     constexpr int ws = team_warp_smem<float, DP_, DP_ + 1>();                                    \
     const int W = team_warps(gr.per_set, sms, ws);                                               \
     const int smem = group_team_smem<float, DP_, DP_ + 1>(W);                                    \
-    const cudaError_t e = team_attr(step_groups<DP_, NX_>);                                \
+    const cudaError_t e = team_attr(step_groups<DP_, NX_>, smem);                                \
     if (e != cudaSuccess) return e;                                                              \
     step_groups<DP_, NX_><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, Ys, gr, m, perm, d,       \
                                                             seeds, inv_scale, out_seeds,         \
@@ -792,7 +792,7 @@ static cudaError_t travel_groups_t(const float* Xs, const View<float>& cv, int n
   const bool res = team_resident<float, DP>(cv.P, n);
   const int smem =
       res ? resident_team_smem<float, DP, DP + 1>(W, n) : group_team_smem<float, DP, DP + 1>(W);
-  const cudaError_t e = team_attr(travel_groups<DP, NX, KF, PH>);
+  const cudaError_t e = team_attr(travel_groups<DP, NX, KF, PH>, smem);
   if (e != cudaSuccess) return e;
   travel_groups<DP, NX, KF, PH><<<gr.per_set, 32 * W, smem, st>>>(
       Xs, cv, n, gr, perm, max_iter, tol2_s, sphere_r, y, it, conv, state, wlast, hist, evals,

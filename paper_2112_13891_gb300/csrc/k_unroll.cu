@@ -495,7 +495,7 @@ static cudaError_t travel_p(const T* X, const View<T>& cv, const T* Y0, Groups g
   const int W = team_warps(NG, g.sms, ws, most_warps<T, DP>());
   const bool res = team_resident<T, DP>(cv.P, g.n);
   const int smem = res ? resident_team_smem<T, DP, DP + 3>(W, g.n) : group_team_smem<T, DP, DP + 3>(W);
-  const cudaError_t e = team_attr(unroll_travel<T, DP, NX, PH>);
+  const cudaError_t e = team_attr(unroll_travel<T, DP, NX, PH>, smem);
   if (e != cudaSuccess) return e;
   unroll_travel<T, DP, NX, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
       X, cv, Y0, gr, g, c, steps, every, slot0, pos, Wout, Sh, M2, res ? 1 : 0);
@@ -538,7 +538,7 @@ static cudaError_t bwd_seed_p(const T* X, const View<T>& cv, const USegment<T>& 
   const int W = team_warps(NG, g.sms, ws, most_warps<T, DP>());
   const bool res = team_resident<T, DP>(cv.P, g.n);
   const int smem = res ? resident_team_smem<T, DP, DP + 2>(W, g.n) : group_team_smem<T, DP, DP + 2>(W);
-  const cudaError_t e = team_attr(unroll_bwd_seed<T, DP, NX, PH>);
+  const cudaError_t e = team_attr(unroll_bwd_seed<T, DP, NX, PH>, smem);
   if (e != cudaSuccess) return e;
   unroll_bwd_seed<T, DP, NX, PH><<<(unsigned)NG, 32 * W, smem, st>>>(
       X, cv, sg, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, first, res ? 1 : 0);
@@ -566,7 +566,7 @@ static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, c
   constexpr int wp = team_warp_smem<T, 2 * DP + 4, DP>();
   const int Wp = team_warps(PG, g.sms, wp, most_warps<T, DP>());
   const int smem_p = list_team_smem<T, 2 * DP + 4, DP>(Wp);
-  e = team_attr(unroll_bwd_point<T, DP, NX>);
+  e = team_attr(unroll_bwd_point<T, DP, NX>, smem_p);
   if (e != cudaSuccess) return e;
   unroll_bwd_point<T, DP, NX><<<(unsigned)PG, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
                                                                  SD, bctr, breach, dX, first);
