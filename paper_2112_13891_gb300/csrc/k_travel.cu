@@ -239,6 +239,7 @@ struct SeedSmem {
   unsigned mask[cells::kMaxCells / 32 > NW ? cells::kMaxCells / 32 : NW], near[NW];
   ST red[NW][DP + 1];
   ST tot[DP + 1];
+  ST part[NW][5][32];   // a lane's sums
   float cut;
   int flag;
 };
@@ -321,9 +322,13 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
   }
   const int part = lane % LP, pl = lane / LP;
   const float4 y4 = reinterpret_cast<const float4*>(sh.y)[part];
+  // FP32 sums of at most kFlush steps (64 or 128 rows of a lane), then added to totals of
+  // type ST in shared memory: one chain over all of a lane's rows would round a sum of
+  // 10^5 terms in FP32.  (Totals in registers cost 256 sets of 16-D 2.8 -> 3.1 ms.)
+  constexpr int kFlush = 16;
   float aw = 0.0f;
   float4 as = make_float4(0.f, 0.f, 0.f, 0.f);
-  int rows = 0, t = w;
+  int rows = 0, t = w, steps = 0;
   const float4* X4 = reinterpret_cast<const float4*>(Xs);
   for (int v = 0; v < nl; ++v) {
     const int2 c = sh.list[v];
@@ -357,10 +362,24 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
         as.z = fmaf(wt, x[u].z, as.z);
         as.w = fmaf(wt, x[u].w, as.w);
       }
+      if (++steps % kFlush == 0) {
+        const float a[5] = {aw, as.x, as.y, as.z, as.w};
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          ST& q = sh.part[w][k][lane];
+          q = (steps > kFlush ? q : ST(0)) + (ST)a[k];
+        }
+        aw = 0.0f;
+        as = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
     }
     t -= nt;
   }
   ST s[5] = {(ST)aw, (ST)as.x, (ST)as.y, (ST)as.z, (ST)as.w};
+  if (steps >= kFlush) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) s[k] += sh.part[w][k][lane];
+  }
 #pragma unroll
   for (int k = 0; k < 5; ++k)
 #pragma unroll

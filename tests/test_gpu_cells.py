@@ -181,3 +181,18 @@ def test_merge_of_points_that_stay(n, d, refine):
     want = _greedy(X, times, 4.5)
     assert len(got) == len(want)
     assert {tuple(p) for p in got} == {tuple(p) for p in want}
+
+
+def test_block_per_seed_long_sums():
+    """A window that holds every point: the mode is their mean, and its error that of the
+    sums of x - y.  Rounding the differences to FP32 leaves 2.6e-9 whatever n is (y's last
+    bits, the same for all rows); sums of 128 terms at a time add 7e-10 at random, one
+    chain of n / 32 terms (whose terms have one sign for long runs: the rows of a cell lie
+    on one side) 4e-9 at n = 10^6."""
+    n, d = 1_000_000, 64
+    X = 0.3 * torch.randn((n, d), generator=torch.Generator(device="cuda").manual_seed(3),
+                          device="cuda")
+    r = fms.cluster(X, 8.0, 8e-3, 50, kernel="flat")
+    assert len(r.modes) == 1
+    err = r.modes[0].double() - X.double().mean(0)
+    assert err.pow(2).mean().sqrt().item() <= 3.6e-9 and err.abs().max().item() <= 9e-9
