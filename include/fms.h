@@ -140,7 +140,10 @@ typedef struct fms_stats {
   int32_t t_star_last;      /* stop iteration of the last round                   */
   int32_t kernel_launches;  /* CUDA kernels this call launched                    */
   int64_t evals;            /* seed-point kernel evaluations in mean-shift updates
-                               (sorted points: of the cells that a seed sees)      */
+                               (sorted points: of the cells that a seed sees; where
+                               a block takes a seed to convergence, those of the
+                               updates that it made before it noticed a round's
+                               stop too, some more or fewer from call to call)     */
   int64_t score_evals;      /* evaluations spent on prune scores and refinement   */
   uint64_t workspace_bytes; /* bytes of workspace the call used                   */
   /* filled when opt->profile = 1 (else zero): */

@@ -432,8 +432,12 @@ __device__ int travel_seed(const float* __restrict__ Xs, const View<float>& cv, 
   const float log2n = log2f((float)n);
   __syncthreads();   // the previous seed's values are no longer read
   for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[s * DP + k];
-  if (threadIdx.x == 0) sh.cut = first_cut<KF>();
   int done = it[s], rows = 0;
+  // A seed that an earlier round's stop left goes on with the cutoff that it had: when it
+  // noticed the stop depends on timing, and its later updates must not.
+  if (threadIdx.x == 0)
+    sh.cut = done > 0 && KF != kKernelFlat ? cells::widen(cells::cut_bits(wlast[s], log2n))
+                                           : first_cut<KF>();
   __syncthreads();
   for (;;) {
     int seen = 0;   // (read ahead of the pass that hides it)

@@ -196,3 +196,34 @@ def test_block_per_seed_long_sums():
     assert len(r.modes) == 1
     err = r.modes[0].double() - X.double().mean(0)
     assert err.pow(2).mean().sqrt().item() <= 3.6e-9 and err.abs().max().item() <= 9e-9
+
+
+@pytest.mark.parametrize("d,B", [(16, 0), (32, 0), (16, 3), (3, 3)])
+def test_rounds_repeat_to_the_bit(d, B):
+    """Several rounds of doubled seeds (70 clusters: 128 seeds become 1,024): the seeds that
+    a round's stop leaves (half of them, at gamma = 0.5) are taken up again, and when a seed
+    notices a stop depends on timing, which other work on the GPU varies here.  The modes
+    (unrefined: positions of seeds), margins and labels must not."""
+    sets = [fi.separated_blobs(seed=d + b, k=70, d=d, per=240 + 10 * b, sigma=0.9, h=2.0)
+            for b in range(max(B, 1))]
+    Xs = [torch.from_numpy(w.X).cuda() for w in sets]
+    big = torch.randn((2048, 2048), device="cuda")
+    side = torch.cuda.Stream()
+    kw = dict(gamma=0.5, skip_refine=True, n_initial=48)
+    first = None
+    for i in range(24):
+        if i % 3:
+            with torch.cuda.stream(side):
+                for _ in range(i):
+                    big = (big @ big).clamp_(-1, 1)
+        if B:
+            r = fms.cluster_batched(Xs, 2.0, 2e-3, 300, rng_seed=1, max_modes=128, **kw)
+            modes = torch.cat(r.modes)
+            assert r.stats["rounds"] > 2
+        else:
+            r = fms.cluster(Xs[0], 2.0, 2e-3, 300, rng_seed=1, **kw)
+            modes = r.modes
+            assert r.stats["rounds"] > 2 and len(modes) == 70
+        now = (modes, r.labels, r.margins)
+        first = first or [t.clone() for t in now]
+        assert all(torch.equal(a, b) for a, b in zip(first, now)), i
