@@ -402,9 +402,9 @@ __device__ int seed_pass(const float* __restrict__ Xs, const View<float>& cv, in
 
 // Passes until the cutoff covers the W that came out (see fms_cells.cuh).
 template <int DP, int KF, typename ST, int NW>
-__device__ int seed_sums(const float* __restrict__ Xs, const View<float>& cv, int n, float log2n,
-                         SeedSmem<DP, ST, NW>& sh) {
-  int rows = 0;
+__device__ long long seed_sums(const float* __restrict__ Xs, const View<float>& cv, int n,
+                               float log2n, SeedSmem<DP, ST, NW>& sh) {
+  long long rows = 0;
   for (int pass = 0;; ++pass) {
     rows += seed_pass<DP, KF, ST, NW>(Xs, cv, n, sh);
     if (KF == kKernelFlat || cv.P == 0) return rows;
@@ -423,16 +423,19 @@ __device__ int seed_sums(const float* __restrict__ Xs, const View<float>& cv, in
 // seen(): seeds converged so far; stop(t): whether the convergence counts say that
 // the round ends at or before update t (warp 0 calls; the counts only grow, so a
 // stop can come late, never early); converged(t): counts this one.
+// Returns the rows visited (10 million points and some hundred updates pass 2^31).
 template <int DP, int KF, int NW, typename Seen, typename Stop, typename Conv>
-__device__ int travel_seed(const float* __restrict__ Xs, const View<float>& cv, int n, int d,
-                           int64_t s, float* y, int32_t* it, int32_t* conv, int32_t* state,
-                           float* wlast, int target, int max_iter, float tol2_s, float sphere_r,
-                           SeedSmem<DP, float, NW>& sh, Seen&& seen_, Stop&& stop_, Conv&& conv_) {
+__device__ long long travel_seed(const float* __restrict__ Xs, const View<float>& cv, int n, int d,
+                                 int64_t s, float* y, int32_t* it, int32_t* conv, int32_t* state,
+                                 float* wlast, int target, int max_iter, float tol2_s,
+                                 float sphere_r, SeedSmem<DP, float, NW>& sh, Seen&& seen_,
+                                 Stop&& stop_, Conv&& conv_) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const float log2n = log2f((float)n);
   __syncthreads();   // the previous seed's values are no longer read
   for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[s * DP + k];
-  int done = it[s], rows = 0;
+  int done = it[s];
+  long long rows = 0;
   // A seed that an earlier round's stop left goes on with the cutoff that it had: when it
   // noticed the stop depends on timing, and its later updates must not.
   if (threadIdx.x == 0)
@@ -592,7 +595,7 @@ __global__ void __launch_bounds__(kQueueWarps * 32)
   while (next_entry(q, &b, &at)) {
     SetCtl* c = q.sc + b;
     const int p0 = c->p0, N = c->N, target = c->target;
-    const int rows = travel_seed<DP, kKernelGaussian, kQueueWarps>(
+    const long long rows = travel_seed<DP, kKernelGaussian, kQueueWarps>(
         Xs + (int64_t)p0 * DP, set_view<DP>(cv, b), c->n, d, q.list[p0 + at], y, it, conv, state,
         wlast, target, max_iter, tol2_s, 0.0f, sh,
         [&] { return *(volatile int32_t*)&c->total; },
@@ -626,7 +629,7 @@ __global__ void __launch_bounds__(kQueueWarps * 32)
     for (int k = threadIdx.x; k < DP; k += blockDim.x) sh.y[k] = y[s * DP + k];
     if (threadIdx.x == 0) sh.cut = first_cut<kKernelGaussian>();
     __syncthreads();
-    const int rows = seed_sums<DP, kKernelGaussian, double, kQueueWarps>(
+    const long long rows = seed_sums<DP, kKernelGaussian, double, kQueueWarps>(
         Xs + (int64_t)c->p0 * DP, set_view<DP>(cv, b), c->n, log2f((float)c->n), sh);
     if (threadIdx.x == 0) {
       if (score) score[c->p0 + at] = (float)sh.tot[0];

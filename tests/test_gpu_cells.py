@@ -227,3 +227,14 @@ def test_rounds_repeat_to_the_bit(d, B):
         now = (modes, r.labels, r.margins)
         first = first or [t.clone() for t in now]
         assert all(torch.equal(a, b) for a, b in zip(first, now)), i
+
+
+def test_evaluations_beyond_32_bits():
+    """One seed over 18 million points that it all sees, 130 updates: 2.3e9 evaluations
+    (a pass with too small a cutoff more)."""
+    n, d, updates = 18_000_000, 9, 130
+    X = torch.randn((n, d), generator=torch.Generator(device="cuda").manual_seed(1),
+                    device="cuda")
+    r = fms.cluster(X, 5.0, 1e-14, updates, n_initial=1, L=0.01, gamma=1.0, skip_refine=True)
+    assert r.stats["iterations"] == updates
+    assert n * updates <= r.stats["evals"] <= n * (updates + 2)
