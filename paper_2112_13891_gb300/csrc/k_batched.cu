@@ -1077,7 +1077,7 @@ cudaError_t launch_batched_refine_compact(SetCtl* sc, int B, const int32_t* mdon
 }
 
 // Blocks that share a set's near ties, and their scratch in all.
-static int order_share(int B) { return B < 1216 ? (1216 / B < 64 ? 1216 / B : 64) : 1; }
+static int order_share(int B) { return B < 2432 ? (2432 / B < 64 ? 2432 / B : 64) : 1; }
 size_t batched_order_scratch(int B, int d) {
   const int per = order_share(B);
   return per > 1 ? tie_scratch_bytes(B * per, d) : 0;

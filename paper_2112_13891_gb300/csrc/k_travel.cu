@@ -585,7 +585,7 @@ __device__ __forceinline__ bool next_entry(const SeedQueue& q, int* set, int* at
 }
 
 template <int DP>
-__global__ void __launch_bounds__(kQueueWarps * 32)
+__global__ void __launch_bounds__(kQueueWarps * 32, 5)   // (121 registers: 4 blocks an SM)
     travel_queue(const float* __restrict__ Xs, View<float> cv, int d, SeedQueue q, float* y,
                  int32_t* it, int32_t* conv, int32_t* state, float* wlast, int max_iter,
                  float tol2_s) {
