@@ -773,7 +773,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           e = launch_seed_init(Xs, n, DP, o.rng_seed, nullptr, 0, 0, N0, seed_idx, y, it, conv,
                                state, status, cs, init_state);
         if (e == cudaSuccess) e = launch_round_begin(rctl_round, N0, o.gamma, cs);
-        slot->kernels_pre = 3 + (P > 0 ? 5 : 0) + (cv.ext ? 1 : 0);
+        slot->kernels_pre = 3 + (P > 0 ? cells::sort_launches(n) : 0) + (cv.ext ? 1 : 0);
         // the rounds
         cudaGraph_t body = nullptr;
         if (e == cudaSuccess) e = add_conditional(cs, h_loop, cudaGraphCondTypeWhile, &body);
@@ -900,7 +900,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                     cosine ? 1 : 0, pcopy));
       if (tensor) FMS_LAUNCH(launch_tc_pack(Xs, n, d, DP, img, st));
       if (P > 0) {
-        n_launches += cv.ext ? 5 : 4;   // (and the one counted below)
+        n_launches += cells::sort_launches(n) - (cv.ext ? 0 : 1);   // (and the one counted below)
         FMS_LAUNCH(sort_points(st));
       }
       N = N0;

@@ -728,7 +728,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       // (queued: pack, the sort's five, seed init; per round seeds, travel, kept,
       // (density,) prune, advance, seed init; setup, queue, refinement or density)
       stats->kernel_launches =
-          queued ? 2 + (cv.P > 0 ? 5 : 0) + (o.gamma >= 1.f ? 7 : 6) * rounds + 3 + 3
+          queued ? 2 + (cv.P > 0 ? cells::sort_launches(max_n) : 0) + (o.gamma >= 1.f ? 7 : 6) * rounds + 3 + 3
                  : 2 + 7 * rounds + 3 * updates + (o.skip_refine ? 0 : 2 + 3 * refines) + 4 + 3;
       stats->evals = ev;
       stats->workspace_bytes = need;

@@ -200,13 +200,17 @@ inline int choose_cells(int64_t n, int64_t m) {
 }
 
 inline int64_t sort_blocks(int64_t rows) { return (rows + kChunkRows - 1) / kChunkRows; }
+constexpr int kScanChunks = 256;   // chunks of a set from which their counters are scanned
+// Kernels of one sort of points (the largest set: `rows`).
+inline int sort_launches(int64_t rows) { return sort_blocks(rows) > kScanChunks ? 6 : 5; }
 inline int group_cap(int64_t rows, int P, int size = 32) {
   return (int)((rows + size - 1) / size) + P;
 }
 
-// Scratch of one sort of B sets of `rows` rows: cell ids, block counts, farthest rows.
+// Scratch of one sort of B sets of `rows` rows: cell ids, block counts, farthest rows,
+// the cells' numbers of rows.
 struct SortScratch {
-  size_t id, counts, far_, total;
+  size_t id, counts, far_, cell_rows, total;
 };
 // (rows: of the largest set; total: of all sets, 0: B rows)
 inline SortScratch sort_scratch(int64_t B, int64_t rows, int P, int64_t total = 0) {
@@ -214,7 +218,8 @@ inline SortScratch sort_scratch(int64_t B, int64_t rows, int P, int64_t total = 
   s.counts = align256((size_t)(total > 0 ? total : B * rows));
   const size_t chunks = total > 0 ? (size_t)(total / kChunkRows + B) + 1 : (size_t)(B * sort_blocks(rows));
   s.far_ = s.counts + align256(chunks * P * 4);
-  s.total = s.far_ + align256((size_t)B * (P / 2) * 8);
+  s.cell_rows = s.far_ + align256((size_t)B * (P / 2) * 8);
+  s.total = s.cell_rows + align256((size_t)B * P * 4);
   return s;
 }
 

@@ -324,16 +324,51 @@ __global__ void __launch_bounds__(32 * kBoundWarps)
   }
 }
 
-// Each block finds where its rows of every cell go (rows of earlier cells,
-// then of the same cell in earlier blocks), ranks its rows in order warp by
-// warp, and copies them.  Latency bound; blocks x P counters are read by every
-// block from L2.
+// From kScanChunks chunks a set on, one pass turns the counters of a set's chunks into
+// those of the chunks before, and keeps the cells' totals: 32 cells a block, a lane each,
+// every warp a run of chunks.  (Every block of the scatter adding up all of them grows
+// with the square of n: 10^7 rows of d = 9 took 7.5 ms more.)
+__global__ void __launch_bounds__(1024)
+    scan_kernel(const int64_t* __restrict__ offs, int each, int per, int P,
+                int32_t* __restrict__ counts, int32_t* __restrict__ cell_rows) {
+  __shared__ int part[32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int b = blockIdx.x / (P / 32), p = blockIdx.x % (P / 32) * 32 + lane;
+  int nrows;
+  set_rows(offs, b, each, &nrows);
+  const int nblk = (int)(((int64_t)nrows + kChunkRows - 1) / kChunkRows);
+  const int run = (nblk + 31) / 32, q0 = min(nblk, w * run), q1 = min(nblk, q0 + run);
+  int32_t* c = counts + chunk0(offs, b, per) * P + p;
+  int s = 0;
+#pragma unroll 8
+  for (int q = q0; q < q1; ++q) s += c[(int64_t)q * P];
+  part[w][lane] = s;
+  __syncthreads();
+  int at = 0, all = 0;
+  for (int u = 0; u < 32; ++u) {
+    const int v = part[u][lane];
+    if (u < w) at += v;
+    all += v;
+  }
+  if (w == 0) cell_rows[(int64_t)b * P + p] = all;
+#pragma unroll 8
+  for (int q = q0; q < q1; ++q) {
+    const int v = c[(int64_t)q * P];
+    c[(int64_t)q * P] = at;
+    at += v;
+  }
+}
+
+// Each block finds where its rows of every cell go (rows of earlier cells, then of the
+// same cell in earlier blocks), ranks its rows in order warp by warp, and copies them.
+// Latency bound; without the scan (cell_rows null) every block reads blocks x P counters
+// from L2.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
     scatter_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int per,
                    int P,
                    const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
-                   T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
+                   const int32_t* __restrict__ cell_rows, T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
                    int2* __restrict__ table, int cap, int gsz, int32_t* __restrict__ gcell) {
   constexpr int WARPS = 8, ITER = kChunkRows / (WARPS * 32);
   __shared__ int wcnt[WARPS][kMaxCells];
@@ -349,11 +384,16 @@ __global__ void __launch_bounds__(256)
   int tot = 0, before = 0;
   if ((int)threadIdx.x < P) {
     const int32_t* c = counts + chunk0(offs, b, per) * P + threadIdx.x;
+    if (cell_rows) {
+      tot = __ldg(cell_rows + (int64_t)b * P + threadIdx.x);
+      before = __ldg(c + (int64_t)blk * P);
+    } else {
 #pragma unroll 16
-    for (int q = 0; q < nblk; ++q) {
-      const int v = __ldg(c + (int64_t)q * P);
-      tot += v;
-      if (q < blk) before += v;
+      for (int q = 0; q < nblk; ++q) {
+        const int v = __ldg(c + (int64_t)q * P);
+        tot += v;
+        if (q < blk) before += v;
+      }
     }
   }
   int all = 0;
@@ -551,8 +591,15 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
     assign_kernel<T, DP, false><<<grid, assign_threads<T, DP>(), sm, st>>>(
         src, offs, (int)nrows, per, P, id, counts, ctr, npiv);
   }
-  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, (int)nrows, per, P, id, counts, dst, perm, start,
-                                             table, group_cap(nrows, P, group), group, gcell);
+  int32_t* cell_rows = nullptr;
+  if (per > kScanChunks) {
+    cell_rows = reinterpret_cast<int32_t*>(base + sc.cell_rows);
+    scan_kernel<<<(unsigned)(P / 32 * B), 1024, 0, st>>>(offs, (int)nrows, per, P, counts,
+                                                         cell_rows);
+  }
+  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, (int)nrows, per, P, id, counts, cell_rows,
+                                              dst, perm, start, table,
+                                              group_cap(nrows, P, group), group, gcell);
   if (points)
     bound_kernel<T, DP><<<(unsigned)(P * B), 32 * kBoundWarps, 0, st>>>(dst, offs, (int)nrows, P, start,
                                                                         ctr, rad);

@@ -28,6 +28,9 @@ def _blobs(seed, n, d, k, box, sigma):
 # just above the rule's line; a last sort block of one row; fewer seeds than points
 @pytest.mark.parametrize("n,m,d,box,h", [(20_620, 20_623, 3, 200.0, 5.0), (14_580, 14_579, 6, 60.0, 4.0),
                                          (10_241, 10_400, 9, 50.0, 2.5), (51_201, 2_080, 16, 50.0, 2.5),
+                                         # 256, 257 chunks of the sort and many: a scan of its counters
+                                         (262_144, 2_048, 3, 200.0, 5.0), (262_145, 2_049, 5, 60.0, 4.0),
+                                         (1_500_000, 2_050, 9, 50.0, 2.5),
                                          (7_300, 7_291, 32, 12.0, 1.5)])
 def test_step_by_groups(n, m, d, box, h):
     X = _blobs(n, n, d, 12, box, 1.0)
