@@ -83,9 +83,9 @@ cudaError_t launch_batched_canonical(SetCtl* sc, int B, const float* X, const do
                                      const int32_t* acc2, int d, int DP, double scale,
                                      float* out_modes, int max_modes, float* modes_full,
                                      int32_t* out_n, cudaStream_t st);
-cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int max_n, int d,
-                                 const SetCtl* sc, const float* modes_full, int32_t* labels,
-                                 float* margins, cudaStream_t st);
+cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int64_t total,
+                                 int d, const SetCtl* sc, const float* modes_full,
+                                 int32_t* labels, float* margins, cudaStream_t st);
 }  // namespace fms
 
 using namespace fms;
@@ -668,7 +668,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
                                      at<double>(ws, Lo.ties), acc2, d, DP, scale, out_modes,
                                      max_modes, modes_full, out_n_modes, cs0);
       if (e == cudaSuccess)
-        e = launch_batched_label(points, pt_off, B, max_n, d, sc, modes_full, out_labels,
+        e = launch_batched_label(points, pt_off, B, total, d, sc, modes_full, out_labels,
                                  out_margins, cs0);
       if (capturing) {
         cudaGraph_t gout = g;

@@ -223,6 +223,27 @@ inline SortScratch sort_scratch(int64_t B, int64_t rows, int P, int64_t total = 
   return s;
 }
 
+// Sets of different sizes share one grid: run g of R rows belongs to the last set b whose
+// first run, offs[b] / R + b, is not beyond g.  That leaves a set the runs it needs and at
+// most one more, so total / R + B blocks serve them all however the sizes are spread
+// (B times the largest set's runs would be mostly empty).  Returns the set, *run its run.
+template <int R>
+__device__ __forceinline__ int set_of_run(const int64_t* __restrict__ offs, int B, int64_t g,
+                                          int* run) {
+  int lo = 0, hi = B - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(offs + mid) / R + mid <= g) lo = mid;
+    else hi = mid - 1;
+  }
+  *run = (int)(g - (__ldg(offs + lo) / R + lo));
+  return lo;
+}
+template <int R>
+inline int64_t runs_of_sets(int64_t total, int B) {
+  return total / R + B;
+}
+
 // Sorts B sets of nrows rows of DP values (set b at src + b nrows DP) into P
 // cells each.  points: the rows make the pivots, and the cells' means ctr
 // [B][P][DP], their number npiv [B] and radii rad [B][P] are written; else (seeds)

@@ -894,18 +894,19 @@ __global__ void __launch_bounds__(32 * kDensityWarps)
   }
 }
 
-// Blocks run over (set, run of kLabelRun points), `per` runs to a set.
+// Blocks run over (set, run of kLabelRun points).
 constexpr int kLabelRun = 1024;
 
 template <int DP>
 __global__ void __launch_bounds__(256)
-    batched_label(const float* __restrict__ X, const int64_t* __restrict__ pt_off, int per, int d,
+    batched_label(const float* __restrict__ X, const int64_t* __restrict__ pt_off, int B, int d,
                   const SetCtl* __restrict__ sc, const float* __restrict__ modes_full,
                   int32_t* __restrict__ labels, float* __restrict__ margins) {
   __shared__ __align__(16) float sm[kLabelFloats];
-  const int b = blockIdx.x / per;
+  int run;
+  const int b = cells::set_of_run<kLabelRun>(pt_off, B, blockIdx.x, &run);
   const int64_t p0 = pt_off[b], p1 = pt_off[b + 1];
-  const int64_t j0 = p0 + (int64_t)(blockIdx.x % per) * kLabelRun, j1 = min(p1, j0 + kLabelRun);
+  const int64_t j0 = p0 + (int64_t)run * kLabelRun, j1 = min(p1, j0 + kLabelRun);
   if (j0 < j1)
     label_block<DP, false>(X, j0, j1, d, modes_full + p0 * d, sc[b].Mr, labels, margins, sm);
 }
@@ -1095,14 +1096,12 @@ cudaError_t launch_batched_canonical(SetCtl* sc, int B, const float* X, const do
   return cudaGetLastError();
 }
 
-cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int max_n, int d,
-                                 const SetCtl* sc, const float* modes_full, int32_t* labels,
-                                 float* margins, cudaStream_t st) {
-  const int64_t per = ((int64_t)max_n + kLabelRun - 1) / kLabelRun;
-  if (per * B > INT32_MAX) return cudaErrorInvalidValue;
-  const unsigned g = (unsigned)(per * B);
-#define FMS_LABEL(DP_)                                                                        \
-  batched_label<DP_><<<g, 256, 0, st>>>(X, pt_off, (int)per, d, sc, modes_full, labels, margins); \
+cudaError_t launch_batched_label(const float* X, const int64_t* pt_off, int B, int64_t total,
+                                 int d, const SetCtl* sc, const float* modes_full,
+                                 int32_t* labels, float* margins, cudaStream_t st) {
+  const unsigned g = (unsigned)cells::runs_of_sets<kLabelRun>(total, B);
+#define FMS_LABEL(DP_)                                                                          \
+  batched_label<DP_><<<g, 256, 0, st>>>(X, pt_off, B, d, sc, modes_full, labels, margins);      \
   break
   switch (padded_dim(d)) {
     case 4: FMS_LABEL(4);

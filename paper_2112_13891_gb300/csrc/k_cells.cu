@@ -18,8 +18,17 @@ __device__ __forceinline__ int64_t set_rows(const int64_t* __restrict__ offs, in
   return o;
 }
 
-// Blocks run over (set, chunk of kChunkRows rows), `per` chunks to a set; the
-// counters of set b's first chunk are row chunk0 of counts [chunks][P].
+// Blocks run over (set, run of R rows): `per` runs to a set of `each` rows, or set_of_run.
+template <int R>
+__device__ __forceinline__ int block_set(const int64_t* __restrict__ offs, int B, int per,
+                                         int* run) {
+  if (offs) return set_of_run<R>(offs, B, blockIdx.x, run);
+  *run = blockIdx.x % per;
+  return blockIdx.x / per;
+}
+
+// The counters of set b's first chunk of kChunkRows rows are row chunk0 of counts
+// [chunks][P].
 __device__ __forceinline__ int64_t chunk0(const int64_t* __restrict__ offs, int b, int per) {
   return offs ? offs[b] / kChunkRows + b : (int64_t)b * per;
 }
@@ -107,15 +116,15 @@ constexpr int kPivotRows = 512;   // (smaller blocks: 200,000 rows over 152 SMs 
 
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
-    pivot_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int P0,
-                 int per, unsigned char* __restrict__ id, unsigned long long* __restrict__ far_) {
+    pivot_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
+                 int P0, int per, unsigned char* __restrict__ id, unsigned long long* __restrict__ far_) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
   __shared__ T org[DP];
   T* pv = reinterpret_cast<T*>(cell_smem);                                        // [P0][DP]
   T* half = pv + P0 * DP;                                                         // [P0]
   unsigned long long* fs = reinterpret_cast<unsigned long long*>(half + P0);      // [P0]
-  const int b = blockIdx.x / per, blk = blockIdx.x % per;
-  int nrows;
+  int blk, nrows;
+  const int b = block_set<kPivotRows>(offs, B, per, &blk);
   const int64_t row0 = set_rows(offs, b, each, &nrows);
   if ((int64_t)blk * kPivotRows >= nrows) return;
   const T* set = src + row0 * DP;
@@ -205,8 +214,8 @@ __global__ void __launch_bounds__(kMaxCells)
 // tried; else (the seeds) all of them.
 template <typename T, int DP, bool EXTEND>
 __global__ void __launch_bounds__(assign_threads<T, DP>())
-    assign_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int per,
-                  int P, unsigned char* __restrict__ id,
+    assign_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
+                  int per, int P, unsigned char* __restrict__ id,
                   int32_t* __restrict__ counts, const T* __restrict__ ctr,
                   const int32_t* __restrict__ npiv) {
   extern __shared__ __align__(16) unsigned char cell_smem[];
@@ -214,8 +223,9 @@ __global__ void __launch_bounds__(assign_threads<T, DP>())
   T* pv = reinterpret_cast<T*>(cell_smem);                 // [P][DP]
   T* half = pv + (size_t)P * DP;                           // [P]
   int* hist = reinterpret_cast<int*>(half + P);            // [P]
-  const int b = blockIdx.x / per, blk = blockIdx.x % per, P0 = P / 2;
-  int nrows;
+  const int P0 = P / 2;
+  int blk, nrows;
+  const int b = block_set<kChunkRows>(offs, B, per, &blk);
   const int64_t row0 = set_rows(offs, b, each, &nrows);
   if ((int64_t)blk * kChunkRows >= nrows) return;
   const T* set = src + row0 * DP;
@@ -365,17 +375,16 @@ __global__ void __launch_bounds__(1024)
 // from L2.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
-    scatter_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int per,
-                   int P,
-                   const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
+    scatter_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
+                   int per, int P, const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
                    const int32_t* __restrict__ cell_rows, T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
                    int2* __restrict__ table, int cap, int gsz, int32_t* __restrict__ gcell) {
   constexpr int WARPS = 8, ITER = kChunkRows / (WARPS * 32);
   __shared__ int wcnt[WARPS][kMaxCells];
   __shared__ int base[kMaxCells];
   __shared__ int scan[64];
-  const int b = blockIdx.x / per, blk = blockIdx.x % per;
-  int nrows;
+  int blk, nrows;
+  const int b = block_set<kChunkRows>(offs, B, per, &blk);
   const int64_t row0 = set_rows(offs, b, each, &nrows);
   const int nblk = (int)(((int64_t)nrows + kChunkRows - 1) / kChunkRows);
   if (blk >= nblk) return;
@@ -554,18 +563,21 @@ cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* npiv
 }
 
 template <typename T, int DP>
-static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrows, bool points, int P,
-                          int64_t total, void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr, int32_t* npiv, T* rad,
-                          int2* table, int group, int32_t* gcell, cudaStream_t st) {
+static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrows, bool points,
+                          int P, int64_t total, void* scratch, T* dst, int32_t* perm,
+                          int32_t* start, T* ctr, int32_t* npiv, T* rad, int2* table, int group,
+                          int32_t* gcell, cudaStream_t st) {
   const SortScratch sc = sort_scratch(B, nrows, P, total);
   unsigned char* base = static_cast<unsigned char*>(scratch);
   unsigned char* id = base + sc.id;
   int32_t* counts = reinterpret_cast<int32_t*>(base + sc.counts);
   unsigned long long* far_ = reinterpret_cast<unsigned long long*>(base + sc.far_);
-  const int64_t per64 = sort_blocks(nrows);
-  if (per64 * B > INT32_MAX || (int64_t)P * B > INT32_MAX) return cudaErrorInvalidValue;
-  const int per = (int)per64;
-  const unsigned grid = (unsigned)(per64 * B);
+  const int64_t per64 = sort_blocks(nrows), pper = (nrows + kPivotRows - 1) / kPivotRows;
+  const int64_t grid64 = offs ? runs_of_sets<kChunkRows>(total, B) : per64 * B;
+  const int64_t pgrid64 = offs ? runs_of_sets<kPivotRows>(total, B) : pper * B;
+  if (pgrid64 > INT32_MAX || (int64_t)P * B > INT32_MAX) return cudaErrorInvalidValue;
+  const int per = (int)per64, n32 = (int)nrows;
+  const unsigned grid = (unsigned)grid64;
   const size_t sm = (size_t)P * (DP + 1) * sizeof(T) + (size_t)P * 4;
   const size_t sm0 = (size_t)P / 2 * (DP + 1) * sizeof(T) + (size_t)P / 2 * 8;
   cudaError_t e = cudaSuccess;
@@ -580,28 +592,25 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
   if (points) {
     e = cudaMemsetAsync(far_, 0, (size_t)B * (P / 2) * 8, st);
     if (e != cudaSuccess) return e;
-    const int64_t pper = (nrows + kPivotRows - 1) / kPivotRows;
-    if (pper * B > INT32_MAX) return cudaErrorInvalidValue;
-    pivot_kernel<T, DP><<<(unsigned)(pper * B), 256, sm0, st>>>(src, offs, (int)nrows, P / 2,
-                                                               (int)pper, id, far_);
-    select_kernel<T, DP><<<B, kMaxCells, 0, st>>>(src, offs, (int)nrows, P, far_, ctr, npiv);
+    pivot_kernel<T, DP><<<(unsigned)pgrid64, 256, sm0, st>>>(src, offs, B, n32, P / 2, (int)pper,
+                                                             id, far_);
+    select_kernel<T, DP><<<B, kMaxCells, 0, st>>>(src, offs, n32, P, far_, ctr, npiv);
     assign_kernel<T, DP, true><<<grid, assign_threads<T, DP>(), sm, st>>>(
-        src, offs, (int)nrows, per, P, id, counts, ctr, npiv);
+        src, offs, B, n32, per, P, id, counts, ctr, npiv);
   } else {
     assign_kernel<T, DP, false><<<grid, assign_threads<T, DP>(), sm, st>>>(
-        src, offs, (int)nrows, per, P, id, counts, ctr, npiv);
+        src, offs, B, n32, per, P, id, counts, ctr, npiv);
   }
   int32_t* cell_rows = nullptr;
   if (per > kScanChunks) {
     cell_rows = reinterpret_cast<int32_t*>(base + sc.cell_rows);
-    scan_kernel<<<(unsigned)(P / 32 * B), 1024, 0, st>>>(offs, (int)nrows, per, P, counts,
-                                                         cell_rows);
+    scan_kernel<<<(unsigned)(P / 32 * B), 1024, 0, st>>>(offs, n32, per, P, counts, cell_rows);
   }
-  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, (int)nrows, per, P, id, counts, cell_rows,
+  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, B, n32, per, P, id, counts, cell_rows,
                                               dst, perm, start, table,
                                               group_cap(nrows, P, group), group, gcell);
   if (points)
-    bound_kernel<T, DP><<<(unsigned)(P * B), 32 * kBoundWarps, 0, st>>>(dst, offs, (int)nrows, P, start,
+    bound_kernel<T, DP><<<(unsigned)(P * B), 32 * kBoundWarps, 0, st>>>(dst, offs, n32, P, start,
                                                                         ctr, rad);
   return cudaGetLastError();
 }
@@ -613,15 +622,18 @@ cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points,
                         int64_t total, int group, int32_t* gcell) {
   if (total == 0) total = (int64_t)B * nrows;
   if (P < 32 || P > kMaxCells || (P & 31) || B < 1) return cudaErrorInvalidValue;
+#define FMS_SORT(DP_)                                                                           \
+  return sort_t<T, DP_>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, \
+                        npiv, rad, table, group, gcell, st)
   switch (DP) {
-    case 4: return sort_t<T, 4>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
-    case 8: return sort_t<T, 8>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
-    case 16: return sort_t<T, 16>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
-    case 32: return sort_t<T, 32>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
+    case 4: FMS_SORT(4);
+    case 8: FMS_SORT(8);
+    case 16: FMS_SORT(16);
+    case 32: FMS_SORT(32);
     case 64:
-      if constexpr (sizeof(T) == 4)
-        return sort_t<T, 64>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, npiv, rad, table, group, gcell, st);
+      if constexpr (sizeof(T) == 4) FMS_SORT(64);
   }
+#undef FMS_SORT
   return cudaErrorInvalidValue;
 }
 

@@ -209,3 +209,32 @@ def test_batched_single_set_equals_single_call():
     assert one.modes.shape == res.modes[0].shape
     assert torch.allclose(one.modes, res.modes[0], atol=1e-3 * h, rtol=0)
     assert torch.equal(one.labels, res.labels)
+
+
+@pytest.mark.parametrize("d", [3, 9, 16])
+def test_batched_uneven_sets(d):
+    # runs of 512 and 1,024 rows that no set or only part of one fills: sets of one and two
+    # points between larger ones (mean size above the line from which sets are sorted)
+    h = 2.0
+    per = [900, 1, 341, 2, 1366, 1, 1, 3, 57]
+    sets = [fi.separated_blobs(seed=60 + b, k=3 if p > 3 else 1, d=d, per=p, sigma=0.8, h=h)
+            for b, p in enumerate(per)]
+    X = [torch.from_numpy(w.X).cuda() for w in sets]
+    res = fms.cluster_batched(X, h, 1e-3 * h, 300, gamma=0.95, rng_seed=0, max_modes=64)
+    off = np.concatenate([[0], np.cumsum([w.X.shape[0] for w in sets])])
+    for b, w in enumerate(sets):
+        _check_set(w, res.modes[b], res.labels[off[b]:off[b + 1]])
+
+
+def test_batched_one_large_set_among_many():
+    # 65,600 sets, one of 33.5 million points: blocks are counted by points, not by the
+    # sets times the largest one's (2^31 of them, beyond a launch)
+    B, big = 65_600, 33_550_000
+    g = torch.Generator(device="cuda").manual_seed(4)
+    small = torch.randn((B - 1, 2), generator=g, device="cuda")
+    X = torch.cat([small, torch.randn((big, 2), generator=g, device="cuda")])
+    offs = np.concatenate([np.arange(B), [B - 1 + big]]).astype(np.int64)
+    r = fms.cluster_batched(X, 2.0, 2e-3, 300, offsets=offs, max_modes=2)
+    assert (r.n_modes == 1).all() and (r.labels == 0).all()
+    assert torch.allclose(torch.cat(r.modes[:-1]), small, rtol=1e-6, atol=1e-6)
+    assert r.modes[-1].abs().max() < 2e-3       # the mean of 3.4e7 normal points: 2e-4
