@@ -567,7 +567,7 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
                           int P, int64_t total, void* scratch, T* dst, int32_t* perm,
                           int32_t* start, T* ctr, int32_t* npiv, T* rad, int2* table, int group,
                           int32_t* gcell, cudaStream_t st) {
-  const SortScratch sc = sort_scratch(B, nrows, P, total);
+  const SortScratch sc = sort_scratch(B, nrows, P, offs ? total : 0);   // (as it was sized)
   unsigned char* base = static_cast<unsigned char*>(scratch);
   unsigned char* id = base + sc.id;
   int32_t* counts = reinterpret_cast<int32_t*>(base + sc.counts);
