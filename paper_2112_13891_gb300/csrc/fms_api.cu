@@ -1393,18 +1393,44 @@ fms_status fms_select_seeds(int64_t n, uint64_t rng_seed, int64_t start, int64_t
 
 
 namespace {
-// Scratch of one update whose points and seeds are sorted into cells.
+// Scratch of one update whose points and seeds may be sorted into cells (off_dense: that
+// of the update over every pair).
 struct GroupStepLayout {
   size_t off_Xp, off_Yp, off_Xs, off_Ys, off_xperm, off_yperm, off_start, off_ystart, off_ctr,
-      off_npiv, off_rad, off_table, off_ext, off_sort, off_status, total;
+      off_npiv, off_rad, off_table, off_ext, off_sort, off_status, off_dense, total;
   int DP, P;
+  StepLayout dense;
 };
 
-// The sorted form pays from ~200 us of dense evaluations on (sorting both sides
-// costs ~60 us): about 1.7e9 padded coordinates of pairs at every width.
+// The status block of an update: the status word, then the probe's answer.
+constexpr size_t kStepShareOff = 16, kStepWalkOff = 32;
+
+// Whether the cells of these packed points leave enough out for these seeds: *walk.
+cudaError_t probe_step(const float* Xp, int64_t n, const float* Yp, int64_t m, int d, int DP,
+                       int kind, void* status, cudaStream_t st, const int32_t** walk) {
+  ProbeArgs a{};
+  a.set[0] = {Xp, Yp, n, m};
+  a.sets = 1;
+  a.d = d;
+  a.ld = DP;
+  a.scale = 1.0;
+  a.kind = kind;
+  a.share = at<float>(status, kStepShareOff);
+  a.walk = at<int32_t>(status, kStepWalkOff);
+  *walk = a.walk;
+  return launch_probe<float>(a, st);
+}
+
+// Sizes from which the sorted form can pay: ~300 us of dense evaluations, about 2.5e9
+// padded coordinates of pairs at every width (sorting both sides costs ~60 us).  Whether it
+// does is for the probe to say (fms_route.cuh); both forms are launched, and the kernels
+// of the one not taken leave at once: 14 us, 4 % of the dense update at this size.  One
+// update where every point is in reach, dense / by cells / as it is: 40,000 x 20,000 x 3
+// 353 / 1,027 / 367 us, 40,000 x 10,000 x 16 760 / 2,462 / 790, 65,537 x 20,011 x 32 4,906 /
+// 11,875 / 4,937.
 bool step_by_groups(int64_t n, int d, int64_t m) {
   return d <= 32 && n >= 2048 && m >= 2048 &&
-         (double)n * (double)m * (double)padded_dim(d) >= 1.7e9;
+         (double)n * (double)m * (double)padded_dim(d) >= 2.5e9;
 }
 
 // One launch where it takes no longer than the five of the general path: a thread
@@ -1415,7 +1441,7 @@ bool step_small(int64_t n, int d, int64_t m) {
   return d <= 32 && coords <= 262144.0 && coords * (double)m <= 134217728.0;
 }
 
-GroupStepLayout group_step_layout(int64_t n, int d, int64_t m) {
+GroupStepLayout group_step_layout(int64_t n, int d, int64_t m, int sms) {
   GroupStepLayout L{};
   L.DP = padded_dim(d);
   L.P = cells::choose_cells(n, m);
@@ -1442,12 +1468,14 @@ GroupStepLayout group_step_layout(int64_t n, int d, int64_t m) {
   const size_t a = cells::sort_scratch(1, n, L.P).total, b = cells::sort_scratch(1, m, L.P).total;
   L.off_sort = take(a > b ? a : b);
   L.off_status = take(64);
+  L.dense = step_layout(n, d, m, sms);
+  L.off_dense = take(L.dense.total);
   L.total = o;
   return L;
 }
 
-// One update with the points and the seeds in cells: each group of 32 seeds
-// visits the cells within its cutoff.
+// One update: with the points and the seeds in cells, each group of 32 seeds visiting the
+// cells within its cutoff, or over every pair.
 cudaError_t group_step(const float* points, int64_t n, int32_t d, float scale, const float* seeds,
                        int64_t m, double inv_scale, float* out_seeds, float* out_wsum, void* ws,
                        const GroupStepLayout& L, int sms, cudaStream_t st) {
@@ -1459,20 +1487,39 @@ cudaError_t group_step(const float* points, int64_t n, int32_t d, float scale, c
   float* ctr = at<float>(ws, L.off_ctr);
   int32_t* npiv = at<int32_t>(ws, L.off_npiv);
   uint32_t* status = at<uint32_t>(ws, L.off_status);
+  void* wd = at<void>(ws, L.off_dense);
+  const StepLayout& D = L.dense;
+  const int32_t* walk = nullptr;
   cudaError_t e = cudaMemsetAsync(status, 0, 64, st);
   if (e == cudaSuccess) e = launch_pack_points(points, n, d, L.DP, scale, Xp, status, st);
   if (e == cudaSuccess) e = launch_pack_points(seeds, m, d, L.DP, scale, Yp, status, st);
   if (e == cudaSuccess)
+    e = probe_step(Xp, n, Yp, m, d, L.DP, d > 8 ? kProbeExtent : kProbeBall, status, st, &walk);
+  const Gate cells_gate{walk, 1, 0}, dense_gate{walk, 1, 1};
+  // over every pair
+  IterCtl* ctl = at<IterCtl>(wd, D.off_ctl);
+  int32_t* active = at<int32_t>(wd, D.off_active);
+  float* part = at<float>(wd, D.off_part);
+  if (e == cudaSuccess) e = launch_step_setup(active, (int)m, ctl, D.C, D.Lc, dense_gate, st);
+  if (e == cudaSuccess)
+    e = launch_ms_step(Xp, n, d, D.DP, Yp, active, &ctl->s, &ctl->C, &ctl->Lc, part,
+                       D.grid_ctas * 8, st, nullptr, nullptr, kKernelGaussian, status);
+  if (e == cudaSuccess)
+    e = launch_step_finish(part, ctl, seeds, d, D.DA, inv_scale, out_seeds, out_wsum, (int)m, D.C,
+                           st);
+  // over the cells
+  if (e == cudaSuccess)
     e = cells::launch_sort<float>(Xp, 1, n, L.DP, true, L.P, at<void>(ws, L.off_sort), Xs,
                                   at<int32_t>(ws, L.off_xperm), at<int32_t>(ws, L.off_start), ctr,
-                                  npiv, at<float>(ws, L.off_rad), nullptr, st);
+                                  npiv, at<float>(ws, L.off_rad), nullptr, st, nullptr, 0, 32,
+                                  nullptr, cells_gate);
   if (e == cudaSuccess && d > 8)
     e = cells::launch_extents(Xs, L.DP, L.P, npiv, at<int32_t>(ws, L.off_start), ctr,
-                              at<float2>(ws, L.off_ext), st);
+                              at<float2>(ws, L.off_ext), st, cells_gate);
   if (e == cudaSuccess)
     e = cells::launch_sort<float>(Yp, 1, m, L.DP, false, L.P, at<void>(ws, L.off_sort), Ys,
                                   at<int32_t>(ws, L.off_yperm), at<int32_t>(ws, L.off_ystart), ctr,
-                                  npiv, nullptr, table, st);
+                                  npiv, nullptr, table, st, nullptr, 0, 32, nullptr, cells_gate);
   if (e != cudaSuccess) return e;
   cells::View<float> cv{};
   cv.P = L.P;
@@ -1482,13 +1529,13 @@ cudaError_t group_step(const float* points, int64_t n, int32_t d, float scale, c
   if (d > 8) cv.ext = at<float2>(ws, L.off_ext);
   const cells::Groups gr{table, cells::group_cap(m, L.P)};
   return launch_step_groups(Xs, cv, (int)n, Ys, gr, (int)m, at<int32_t>(ws, L.off_yperm), d, L.DP,
-                            seeds, inv_scale, out_seeds, out_wsum, sms, st);
+                            seeds, inv_scale, out_seeds, out_wsum, sms, st, cells_gate);
 }
 }  // namespace
 
 size_t fms_step_workspace_size(int64_t n, int32_t d, int64_t m) {
   if (n < 1 || n > INT32_MAX || d < 1 || d > FMS_MAX_DIM || m < 1 || m > INT32_MAX) return 0;
-  if (step_by_groups(n, d, m)) return group_step_layout(n, d, m).total;
+  if (step_by_groups(n, d, m)) return group_step_layout(n, d, m, device_info().sms).total;
   return step_layout(n, d, m, device_info().sms).total;
 }
 
@@ -1503,7 +1550,7 @@ fms_status fms_mean_shift_step(const float* points, int64_t n, int32_t d, float 
   if (dv.sms <= 0) return FMS_ERR_CUDA;
   const bool groups = step_by_groups(n, d, m);
   const StepLayout L = groups ? StepLayout{} : step_layout(n, d, m, dv.sms);
-  const GroupStepLayout LG = groups ? group_step_layout(n, d, m) : GroupStepLayout{};
+  const GroupStepLayout LG = groups ? group_step_layout(n, d, m, dv.sms) : GroupStepLayout{};
   const size_t need = groups ? LG.total : L.total;
   fms_status rc = FMS_OK;
   bool owns = false;
@@ -1535,7 +1582,7 @@ fms_status fms_mean_shift_step(const float* points, int64_t n, int32_t d, float 
     FMS_CUDA(cudaMemsetAsync(status, 0, 64, st));
     FMS_CUDA(launch_pack_points(points, n, d, L.DP, (float)scale, Xs, status, st));
     FMS_CUDA(launch_pack_points(seeds, m, d, L.DP, (float)scale, Ys, status, st));
-    FMS_CUDA(launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, st));
+    FMS_CUDA(launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, Gate{}, st));
     FMS_CUDA(launch_ms_step(Xs, n, d, L.DP, Ys, active, &ctl->s, &ctl->C, &ctl->Lc, part,
                             L.grid_ctas * 8, st, nullptr, nullptr, kKernelGaussian, status));
     FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,
@@ -1557,14 +1604,19 @@ namespace {
 struct CoarseLayout {
   size_t off_Xs, off_img, off_Ys, off_active, off_part, off_ctl, off_status, total;
   int DP, DA, C, Lc, grid;
-  // P > 0: points and seeds in cells, tiles of up to 128 rows of one cell
-  int P, tiles, seed_tiles;
+  // P > 0: points and seeds may go into cells, tiles of up to 128 rows of one cell (C and
+  // Lc are then the dense form's, Cc chunks a tile of seeds the cells')
+  int P, tiles, seed_tiles, Cc;
   size_t off_Xc, off_Yc, off_xperm, off_yperm, off_start, off_ystart, off_ctr, off_npiv, off_rad,
       off_xtable, off_xcell, off_ytable, off_list, off_count, off_outrow, off_sort;
 };
 
-// Sorting takes ~120 us; the dense step takes that from about 3e8 pairs on.
-// (The list of visible tiles takes 4 bytes a pair of tiles: up to 1 GB.)
+// Sizes from which cells can pay: sorting takes ~120 us; the dense step takes that from
+// about 3e8 pairs on.  (The list of visible tiles takes 4 bytes a pair of tiles: up to 1
+// GB.)  With every tile in reach, the tiles' padding alone more than doubles the work
+// (64 centres on a sphere, 65,536 x 16: 1.74 ms dense, 2.39 by cells; 50,001 points and
+// 15,003 seeds 0.35 and 0.82), so the probe decides between the two (1.73 and 0.37; 32
+// blobs apart from each other, 65,536 x 16, 1.74 dense, 0.27 by cells and with the probe).
 bool coarse_by_cells(int64_t n, int64_t m) {
   const double pairs = (double)n * (double)m;
   return n >= 4096 && m >= 512 && pairs >= 6e8 && pairs <= 4e12;
@@ -1588,16 +1640,20 @@ CoarseLayout coarse_layout(int64_t n, int d, int64_t m) {
     L.seed_tiles = cells::group_cap(m, L.P, kTcTile);
     places = (int64_t)L.seed_tiles * kTcTile;
     // about 4 tasks to a CTA
-    L.C = (4 * L.grid + L.seed_tiles - 1) / L.seed_tiles;
-    L.Lc = kTcTile;
-  } else {
-    tc_choose_chunks(n, (int32_t)m, L.grid, &L.C, &L.Lc);
+    L.Cc = (4 * L.grid + L.seed_tiles - 1) / L.seed_tiles;
+  }
+  tc_choose_chunks(n, (int32_t)m, L.grid, &L.C, &L.Lc);
+  size_t img = tc_image_bytes(n, d), parts = (size_t)L.C * (size_t)m * L.DA * 4;
+  if (L.P > 0) {
+    const size_t ic = tc_tile_images(L.tiles, d), pc = (size_t)L.Cc * (size_t)places * L.DA * 4;
+    if (ic > img) img = ic;
+    if (pc > parts) parts = pc;
   }
   L.off_Xs = take((size_t)n * L.DP * 4);
-  L.off_img = take(L.P > 0 ? tc_tile_images(L.tiles, d) : tc_image_bytes(n, d));
+  L.off_img = take(img);
   L.off_Ys = take((size_t)m * L.DP * 4);
-  L.off_active = take((size_t)places * 4);
-  L.off_part = take((size_t)L.C * (size_t)places * L.DA * 4);
+  L.off_active = take((size_t)(places > m ? places : m) * 4);
+  L.off_part = take(parts);
   L.off_ctl = take(sizeof(IterCtl));
   L.off_status = take(64);
   if (L.P > 0) {
@@ -1623,10 +1679,13 @@ CoarseLayout coarse_layout(int64_t n, int d, int64_t m) {
   return L;
 }
 
-// The coarse step over cells: only the tile pairs that can have a nonzero weight.
+// The coarse step over cells, only the tile pairs that can have a nonzero weight, or over
+// all tiles in order, as the probe says.
 cudaError_t coarse_cells(const CoarseLayout& L, void* ws, int64_t n, int d, int64_t m,
                          const float* seeds, double inv_scale, float* out_seeds, float* out_wsum,
                          cudaStream_t st) {
+  float* Xs = at<float>(ws, L.off_Xs);
+  float* Ys = at<float>(ws, L.off_Ys);
   float* Xc = at<float>(ws, L.off_Xc);
   float* Yc = at<float>(ws, L.off_Yc);
   unsigned char* img = at<unsigned char>(ws, L.off_img);
@@ -1645,31 +1704,37 @@ cudaError_t coarse_cells(const CoarseLayout& L, void* ws, int64_t n, int d, int6
   uint32_t* status = at<uint32_t>(ws, L.off_status);
   void* scratch = at<void>(ws, L.off_sort);
   const int places = L.seed_tiles * kTcTile;
+  const int32_t* walk = nullptr;
   cells::View<float> cv{};
   cv.P = L.P;
   cv.start = at<int32_t>(ws, L.off_start);
   cv.ctr = ctr;
   cv.rad = at<float>(ws, L.off_rad);
-  cudaError_t e = cells::launch_sort<float>(
-      at<float>(ws, L.off_Xs), 1, n, L.DP, true, L.P, scratch, Xc, at<int32_t>(ws, L.off_xperm),
-      at<int32_t>(ws, L.off_start), ctr, npiv, at<float>(ws, L.off_rad), xtable, st, nullptr, 0,
-      kTcTile, xcell);
+  cudaError_t e = probe_step(Xs, n, Ys, m, d, L.DP, kProbeTile, status, st, &walk);
+  const Gate gate{walk, 1, 0};
   if (e == cudaSuccess)
-    e = cells::launch_sort<float>(at<float>(ws, L.off_Ys), 1, m, L.DP, false, L.P, scratch, Yc,
-                                  yperm, at<int32_t>(ws, L.off_ystart), ctr, npiv, nullptr, ytable,
-                                  st, nullptr, 0, kTcTile);
+    e = cells::launch_sort<float>(Xs, 1, n, L.DP, true, L.P, scratch, Xc,
+                                  at<int32_t>(ws, L.off_xperm), at<int32_t>(ws, L.off_start), ctr,
+                                  npiv, at<float>(ws, L.off_rad), xtable, st, nullptr, 0, kTcTile,
+                                  xcell, gate);
   if (e == cudaSuccess)
-    e = launch_tc_pack_table(Xc, n, d, L.DP, xtable, L.tiles, img, st);
-  if (e == cudaSuccess) e = launch_step_setup(active, places, ctl, L.C, L.Lc, st);
+    e = cells::launch_sort<float>(Ys, 1, m, L.DP, false, L.P, scratch, Yc, yperm,
+                                  at<int32_t>(ws, L.off_ystart), ctr, npiv, nullptr, ytable, st,
+                                  nullptr, 0, kTcTile, nullptr, gate);
+  if (e == cudaSuccess)
+    e = launch_tc_pack_table(Xc, Xs, n, d, L.DP, xtable, L.tiles, img, gate, st);
+  if (e == cudaSuccess)
+    e = launch_coarse_setup(active, (int)m, ctl, L.C, L.Lc, places, L.Cc, gate, st);
   if (e == cudaSuccess)
     e = launch_tc_visible(Yc, L.DP, ytable, L.seed_tiles, yperm, cv, xtable, xcell, L.tiles, list,
-                          count, active, out_row, st);
+                          count, active, out_row, st, gate);
   if (e == cudaSuccess)
-    e = launch_ms_step_tc(img, n, d, L.DP, L.DA, Yc, active, &ctl->s, &ctl->s, &ctl->C, &ctl->Lc,
-                          part, status, st, nullptr, TcTiles{list, count, L.tiles});
+    e = launch_ms_step_tc(img, n, d, L.DP, L.DA, Ys, active, &ctl->s, &ctl->s, &ctl->C, &ctl->Lc,
+                          part, status, st, nullptr, TcTiles{list, count, L.tiles, Yc, gate});
   if (e == cudaSuccess)
-    e = launch_step_finish(part, ctl, seeds, d, L.DA, inv_scale, out_seeds, out_wsum, places,
-                           L.C, st, out_row);
+    e = launch_step_finish(part, ctl, seeds, d, L.DA, inv_scale, out_seeds, out_wsum,
+                           places > m ? places : (int)m, L.C > L.Cc ? L.C : L.Cc, st, out_row,
+                           gate);
   return e;
 }
 }  // namespace
@@ -1717,7 +1782,7 @@ fms_status fms_mean_shift_step_coarse(const float* points, int64_t n, int32_t d,
       FMS_CUDA(coarse_cells(L, ws, n, d, m, seeds, 1.0 / scale, out_seeds, out_wsum, st));
     } else {
       FMS_CUDA(launch_tc_pack(Xs, n, d, L.DP, img, st));
-      FMS_CUDA(launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, st));
+      FMS_CUDA(launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, Gate{}, st));
       FMS_CUDA(launch_ms_step_tc(img, n, d, L.DP, L.DA, Ys, active, &ctl->s, &ctl->s, &ctl->C,
                                  &ctl->Lc, part, status, st));
       FMS_CUDA(launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum,

@@ -15,6 +15,7 @@
 #pragma once
 
 #include "fms_internal.cuh"
+#include "fms_route.cuh"
 
 namespace fms {
 namespace cells {
@@ -252,30 +253,37 @@ inline int64_t runs_of_sets(int64_t total, int B) {
 // of the set) and the table of groups [B][group_cap(nrows, P)].  Sets of different
 // sizes: set b has the rows [offs[b], offs[b + 1]) of `total` (offs on the device),
 // nrows is the largest, and there is no table.  The groups of the table hold up to
-// `group` rows, group_cell (nullable) is the cell of each.
+// `group` rows, group_cell (nullable) is the cell of each.  Nothing is done where the gate
+// is closed.
 template <typename T>
 cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
                         int32_t* npiv, T* rad, int2* table, cudaStream_t st,
                         const int64_t* offs = nullptr, int64_t total = 0, int group = 32,
-                        int32_t* group_cell = nullptr);
+                        int32_t* group_cell = nullptr, Gate gate = Gate{});
 
 // The extents of the P cells of one sorted set towards each other's centres
 // (View::ext), for d > 8.
 cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* npiv,
-                           const int32_t* start, const float* ctr, float2* ext, cudaStream_t st);
+                           const int32_t* start, const float* ctr, float2* ext, cudaStream_t st,
+                           Gate gate = Gate{});
 
 }  // namespace cells
 
 // ---- k_step_tc.cu: tiles of one cell each (up to 128 rows)
 size_t tc_tile_images(int64_t tiles, int d);
-cudaError_t launch_tc_pack_table(const float* Xs, int64_t n, int d, int DP, const int2* table,
-                                 int tiles, unsigned char* img, cudaStream_t st);
+// gate closed: tiles of the unsorted rows Xu, as launch_tc_pack.
+cudaError_t launch_tc_pack_table(const float* Xs, const float* Xu, int64_t n, int d, int DP,
+                                 const int2* table, int tiles, unsigned char* img, Gate gate,
+                                 cudaStream_t st);
+// ctl and, gate closed, the list of all m seeds: (places, Cc chunks of one tile) or (m, C, Lc).
+cudaError_t launch_coarse_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t C, int32_t Lc,
+                                int32_t places, int32_t Cc, Gate gate, cudaStream_t st);
 cudaError_t launch_tc_visible(const float* Ys, int DP, const int2* seed_table, int seed_tiles,
                               const int32_t* yperm, const cells::View<float>& cv,
                               const int2* tile_table, const int32_t* tile_cell, int tiles,
                               int32_t* list, int32_t* count, int32_t* active, int32_t* out_row,
-                              cudaStream_t st);
+                              cudaStream_t st, Gate gate = Gate{});
 
 // ---- k_travel.cu: whole trajectories in one launch (rows of DP floats, scaled)
 
@@ -284,7 +292,7 @@ cudaError_t launch_step_groups(const float* Xs, const cells::View<float>& cv, in
                                const float* Ys, const cells::Groups& gr, int m,
                                const int32_t* perm, int d, int DP, const float* seeds,
                                double inv_scale, float* out_seeds, float* out_wsum, int sms,
-                               cudaStream_t st);
+                               cudaStream_t st, Gate gate = Gate{});
 // Every point a seed, DP = 4 or 8: states, hist and the densities at the last positions.
 cudaError_t launch_travel_groups(const float* Xs, const cells::View<float>& cv, int n, int d, int DP,
                                  const cells::Groups& gr, const int32_t* perm, int kf,

@@ -139,6 +139,20 @@ struct SetCtl {
   int64_t evals;
 };
 
+// By which a kernel that was launched for one of two routes learns whether it was taken
+// (fms_route.cuh): open where every sampled set says so; null flags: always open.
+struct Gate {
+  const int32_t* walk;
+  int sets;
+  int closed_if;   // the answer to which the gate is closed
+  __device__ __forceinline__ bool open() const {
+    if (!walk) return true;
+    int w = 1;
+    for (int i = 0; i < sets; ++i) w &= __ldg(walk + i);
+    return w != closed_if;
+  }
+};
+
 // Batched call: a graph condition that a kernel sets when it finishes (on = 0:
 // the kernel runs outside the graph and sets nothing), and the slots of the
 // call's device counters.
@@ -352,16 +366,18 @@ cudaError_t launch_update(const float* part, int32_t* active, IterCtl* ctl, floa
                           float sphere_r = 0.0f,    // > 0: project onto that sphere
                           float* wlast = nullptr);  // sum w of each seed's last update
 cudaError_t launch_step_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t C, int32_t Lc,
-                              cudaStream_t st);
+                              const Gate& gate, cudaStream_t st);
 // One update of m seeds in one launch, for small problems (d <= 32); non-finite
 // inputs set kStNonFinite in *status.
 cudaError_t launch_step_small(const float* X, int64_t n, int d, float scale, const float* seeds,
                               int64_t m, double inv_scale, float* out_seeds, float* out_wsum,
                               uint32_t* status, cudaStream_t st);
-// out_row (nullable): the caller's row of each active position, -1 for none
+// out_row (nullable; not used where the gate is closed): the caller's row of each active
+// position, -1 for none
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,
-                               int m, int C, cudaStream_t st, const int32_t* out_row = nullptr);
+                               int m, int C, cudaStream_t st, const int32_t* out_row = nullptr,
+                               Gate rows_gate = Gate{});
 
 // k_round.cu
 cudaError_t launch_ms_round(const float* Xs, int64_t n, int d, float* y, int32_t* it,
@@ -522,12 +538,14 @@ inline StepLayout step_layout(int64_t n, int d, int64_t m, int sms) {
 // handles active positions [0, *count_ptr) of a list whose partials have the
 // stride *s_total_ptr, with chunks of *Lc_ptr (a multiple of 128) points.
 constexpr int kTcMaxDim = 32;
-// Point tiles that each tile of 128 active positions visits (count null: all of
-// them, in order): count[s] of list[s stride ..].
+// Point tiles that each tile of 128 active positions visits (count null, or the gate
+// closed: all of them, in order): count[s] of list[s stride ..], positions from y where set.
 struct TcTiles {
   const int32_t* list;
   const int32_t* count;
   int stride;
+  const float* y;
+  Gate gate;
 };
 size_t tc_image_bytes(int64_t n, int d);
 cudaError_t launch_tc_pack(const float* Xs, int64_t n, int d, int DP, unsigned char* img,

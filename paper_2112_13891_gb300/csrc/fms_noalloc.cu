@@ -19,6 +19,7 @@
 
 #include "../../include/fms.h"
 #include "fms_internal.cuh"
+#include "fms_route.cuh"
 
 using namespace fms;
 
@@ -72,7 +73,7 @@ extern "C" fms_status fms_mean_shift_step_noalloc(const float* points, int64_t n
   if (cudaMemsetAsync(status, 0, 4, st) != cudaSuccess) return FMS_ERR_CUDA;
   if (launch_pack_points(points, n, d, L.DP, (float)scale, Xs, status, st) != cudaSuccess ||
       launch_pack_points(seeds, m, d, L.DP, (float)scale, Ys, status, st) != cudaSuccess ||
-      launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, st) != cudaSuccess ||
+      launch_step_setup(active, (int32_t)m, ctl, L.C, L.Lc, Gate{}, st) != cudaSuccess ||
       launch_ms_step(Xs, n, d, L.DP, Ys, active, &ctl->s, &ctl->C, &ctl->Lc, part,
                      L.grid_ctas * 8, st, nullptr, nullptr, kKernelGaussian, status) != cudaSuccess ||
       launch_step_finish(part, ctl, seeds, d, L.DA, 1.0 / scale, out_seeds, out_wsum, (int)m,

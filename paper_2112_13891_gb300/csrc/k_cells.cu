@@ -117,7 +117,10 @@ constexpr int kPivotRows = 512;   // (smaller blocks: 200,000 rows over 152 SMs 
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
     pivot_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
-                 int P0, int per, unsigned char* __restrict__ id, unsigned long long* __restrict__ far_) {
+                 int P0, int per, unsigned char* __restrict__ id,
+                 unsigned long long* __restrict__ far_, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   extern __shared__ __align__(16) unsigned char cell_smem[];
   __shared__ T org[DP];
   T* pv = reinterpret_cast<T*>(cell_smem);                                        // [P0][DP]
@@ -175,7 +178,9 @@ template <typename T, int DP>
 __global__ void __launch_bounds__(kMaxCells)
     select_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int each, int P,
                   const unsigned long long* __restrict__ far_, T* __restrict__ ctr,
-                  int32_t* __restrict__ npiv) {
+                  int32_t* __restrict__ npiv, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   __shared__ float r2s[kMaxCells / 2];
   __shared__ float small;
   __shared__ int sel[kMaxCells], red[64];
@@ -217,7 +222,9 @@ __global__ void __launch_bounds__(assign_threads<T, DP>())
     assign_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
                   int per, int P, unsigned char* __restrict__ id,
                   int32_t* __restrict__ counts, const T* __restrict__ ctr,
-                  const int32_t* __restrict__ npiv) {
+                  const int32_t* __restrict__ npiv, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   extern __shared__ __align__(16) unsigned char cell_smem[];
   __shared__ T org[DP];
   T* pv = reinterpret_cast<T*>(cell_smem);                 // [P][DP]
@@ -278,8 +285,10 @@ constexpr int kBoundWarps = 8;
 template <typename T, int DP>
 __global__ void __launch_bounds__(32 * kBoundWarps)
     bound_kernel(const T* __restrict__ rows, const int64_t* __restrict__ offs, int each, int P,
-                 const int32_t* __restrict__ start,
-                 T* __restrict__ ctr, T* __restrict__ rad) {
+                 const int32_t* __restrict__ start, T* __restrict__ ctr, T* __restrict__ rad,
+                 Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   __shared__ T red[kBoundWarps][DP];
   __shared__ T mean[DP];
   const int b = blockIdx.x / P, p = blockIdx.x % P, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -340,7 +349,9 @@ __global__ void __launch_bounds__(32 * kBoundWarps)
 // with the square of n: 10^7 rows of d = 9 took 7.5 ms more.)
 __global__ void __launch_bounds__(1024)
     scan_kernel(const int64_t* __restrict__ offs, int each, int per, int P,
-                int32_t* __restrict__ counts, int32_t* __restrict__ cell_rows) {
+                int32_t* __restrict__ counts, int32_t* __restrict__ cell_rows, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   __shared__ int part[32][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int b = blockIdx.x / (P / 32), p = blockIdx.x % (P / 32) * 32 + lane;
@@ -378,7 +389,10 @@ __global__ void __launch_bounds__(256)
     scatter_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
                    int per, int P, const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
                    const int32_t* __restrict__ cell_rows, T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
-                   int2* __restrict__ table, int cap, int gsz, int32_t* __restrict__ gcell) {
+                   int2* __restrict__ table, int cap, int gsz, int32_t* __restrict__ gcell,
+                   Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   constexpr int WARPS = 8, ITER = kChunkRows / (WARPS * 32);
   __shared__ int wcnt[WARPS][kMaxCells];
   __shared__ int base[kMaxCells];
@@ -501,7 +515,9 @@ template <int DP>
 __global__ void __launch_bounds__(kMaxCells / 2)
     extent_kernel(const float* __restrict__ rows, int P, const int32_t* __restrict__ npiv,
                   const int32_t* __restrict__ start, const float* __restrict__ ctr,
-                  float2* __restrict__ ext) {
+                  float2* __restrict__ ext, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   __shared__ __align__(16) float tile[kExtRows * DP];
   const int p = blockIdx.x;
   const int a = start[p], e = start[p + 1];
@@ -548,25 +564,28 @@ __global__ void __launch_bounds__(kMaxCells / 2)
 }
 
 cudaError_t launch_extents(const float* rows, int DP, int P, const int32_t* npiv,
-                           const int32_t* start, const float* ctr, float2* ext, cudaStream_t st) {
+                           const int32_t* start, const float* ctr, float2* ext, cudaStream_t st,
+                           Gate gate) {
   const cudaError_t e = cudaMemsetAsync(ext, 0, (size_t)P * P * 8, st);
   if (e != cudaSuccess) return e;
   // (cells differ in size by an order of magnitude: blocks past a cell's rows leave at once)
-  const dim3 grid((unsigned)P, 32);
+  const dim3 grid((unsigned)P, gate.walk ? 16 : 32);   // (fewer where they may all be in vain)
+#define FMS_EXTENT(DP_) \
+  return launch_gated(gate, extent_kernel<DP_>, grid, P / 2, 0, st, rows, P, npiv, start, ctr, ext, gate)
   switch (DP) {
-    case 16: extent_kernel<16><<<grid, P / 2, 0, st>>>(rows, P, npiv, start, ctr, ext); break;
-    case 32: extent_kernel<32><<<grid, P / 2, 0, st>>>(rows, P, npiv, start, ctr, ext); break;
-    case 64: extent_kernel<64><<<grid, P / 2, 0, st>>>(rows, P, npiv, start, ctr, ext); break;
-    default: return cudaErrorInvalidValue;
+    case 16: FMS_EXTENT(16);
+    case 32: FMS_EXTENT(32);
+    case 64: FMS_EXTENT(64);
   }
-  return cudaGetLastError();
+#undef FMS_EXTENT
+  return cudaErrorInvalidValue;
 }
 
 template <typename T, int DP>
 static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrows, bool points,
                           int P, int64_t total, void* scratch, T* dst, int32_t* perm,
                           int32_t* start, T* ctr, int32_t* npiv, T* rad, int2* table, int group,
-                          int32_t* gcell, cudaStream_t st) {
+                          int32_t* gcell, Gate gate, cudaStream_t st) {
   const SortScratch sc = sort_scratch(B, nrows, P, offs ? total : 0);   // (as it was sized)
   unsigned char* base = static_cast<unsigned char*>(scratch);
   unsigned char* id = base + sc.id;
@@ -592,39 +611,42 @@ static cudaError_t sort_t(const T* src, const int64_t* offs, int B, int64_t nrow
   if (points) {
     e = cudaMemsetAsync(far_, 0, (size_t)B * (P / 2) * 8, st);
     if (e != cudaSuccess) return e;
-    pivot_kernel<T, DP><<<(unsigned)pgrid64, 256, sm0, st>>>(src, offs, B, n32, P / 2, (int)pper,
-                                                             id, far_);
-    select_kernel<T, DP><<<B, kMaxCells, 0, st>>>(src, offs, n32, P, far_, ctr, npiv);
-    assign_kernel<T, DP, true><<<grid, assign_threads<T, DP>(), sm, st>>>(
-        src, offs, B, n32, per, P, id, counts, ctr, npiv);
-  } else {
-    assign_kernel<T, DP, false><<<grid, assign_threads<T, DP>(), sm, st>>>(
-        src, offs, B, n32, per, P, id, counts, ctr, npiv);
+    e = launch_gated(gate, pivot_kernel<T, DP>, (unsigned)pgrid64, 256, sm0, st, src, offs, B, n32,
+                     P / 2, (int)pper, id, far_, gate);
+    if (e == cudaSuccess)
+      e = launch_gated(gate, select_kernel<T, DP>, B, kMaxCells, 0, st, src, offs, n32, P, far_, ctr,
+                       npiv, gate);
   }
+  auto assign = points ? assign_kernel<T, DP, true> : assign_kernel<T, DP, false>;
+  if (e == cudaSuccess)
+    e = launch_gated(gate, assign, grid, assign_threads<T, DP>(), sm, st, src, offs, B, n32, per, P,
+                     id, counts, ctr, npiv, gate);
   int32_t* cell_rows = nullptr;
-  if (per > kScanChunks) {
+  if (e == cudaSuccess && per > kScanChunks) {
     cell_rows = reinterpret_cast<int32_t*>(base + sc.cell_rows);
-    scan_kernel<<<(unsigned)(P / 32 * B), 1024, 0, st>>>(offs, n32, per, P, counts, cell_rows);
+    e = launch_gated(gate, scan_kernel, (unsigned)(P / 32 * B), 1024, 0, st, offs, n32, per, P,
+                     counts, cell_rows, gate);
   }
-  scatter_kernel<T, DP><<<grid, 256, 0, st>>>(src, offs, B, n32, per, P, id, counts, cell_rows,
-                                              dst, perm, start, table,
-                                              group_cap(nrows, P, group), group, gcell);
-  if (points)
-    bound_kernel<T, DP><<<(unsigned)(P * B), 32 * kBoundWarps, 0, st>>>(dst, offs, n32, P, start,
-                                                                        ctr, rad);
-  return cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_gated(gate, scatter_kernel<T, DP>, grid, 256, 0, st, src, offs, B, n32, per, P, id,
+                     counts, cell_rows, dst, perm, start, table, group_cap(nrows, P, group), group,
+                     gcell, gate);
+  if (e == cudaSuccess && points)
+    e = launch_gated(gate, bound_kernel<T, DP>, (unsigned)(P * B), 32 * kBoundWarps, 0, st, dst,
+                     offs, n32, P, start, ctr, rad, gate);
+  return e;
 }
 
 template <typename T>
 cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points, int P,
                         void* scratch, T* dst, int32_t* perm, int32_t* start, T* ctr,
                         int32_t* npiv, T* rad, int2* table, cudaStream_t st, const int64_t* offs,
-                        int64_t total, int group, int32_t* gcell) {
+                        int64_t total, int group, int32_t* gcell, Gate gate) {
   if (total == 0) total = (int64_t)B * nrows;
   if (P < 32 || P > kMaxCells || (P & 31) || B < 1) return cudaErrorInvalidValue;
 #define FMS_SORT(DP_)                                                                           \
   return sort_t<T, DP_>(src, offs, B, nrows, points, P, total, scratch, dst, perm, start, ctr, \
-                        npiv, rad, table, group, gcell, st)
+                        npiv, rad, table, group, gcell, gate, st)
   switch (DP) {
     case 4: FMS_SORT(4);
     case 8: FMS_SORT(8);
@@ -639,10 +661,10 @@ cudaError_t launch_sort(const T* src, int B, int64_t nrows, int DP, bool points,
 
 template cudaError_t launch_sort<float>(const float*, int, int64_t, int, bool, int, void*, float*,
                                         int32_t*, int32_t*, float*, int32_t*, float*, int2*,
-                                        cudaStream_t, const int64_t*, int64_t, int, int32_t*);
+                                        cudaStream_t, const int64_t*, int64_t, int, int32_t*, Gate);
 template cudaError_t launch_sort<double>(const double*, int, int64_t, int, bool, int, void*,
                                          double*, int32_t*, int32_t*, double*, int32_t*, double*,
-                                         int2*, cudaStream_t, const int64_t*, int64_t, int, int32_t*);
+                                         int2*, cudaStream_t, const int64_t*, int64_t, int, int32_t*, Gate);
 
 }  // namespace cells
 }  // namespace fms

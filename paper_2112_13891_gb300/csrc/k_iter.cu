@@ -1,5 +1,6 @@
 // Point packing, Seed Selection, the per-update seed update and the
 // Early-Stopping bookkeeping that compacts the active set.
+#include "fms_cells.cuh"
 #include "fms_label.cuh"
 #include "fms_seedperm.cuh"
 
@@ -700,8 +701,13 @@ cudaError_t launch_step_small(const float* X, int64_t n, int d, float scale, con
 // ---------------------------------------------------------------------------
 // Stand-alone single update (fms_mean_shift_step): every seed is active.
 // ---------------------------------------------------------------------------
+// (gate closed: no seeds, so the update's other kernels have nothing to do)
 __global__ void step_setup_kernel(int32_t* __restrict__ active, int32_t m, IterCtl* ctl, int32_t C,
-                                  int32_t Lc) {
+                                  int32_t Lc, Gate gate) {
+  if (!gate.open()) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->s = ctl->C = 0;
+    return;
+  }
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
     active[i] = i;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -711,12 +717,33 @@ __global__ void step_setup_kernel(int32_t* __restrict__ active, int32_t m, IterC
   }
 }
 
+__global__ void coarse_setup_kernel(int32_t* __restrict__ active, int32_t m, IterCtl* ctl,
+                                    int32_t C, int32_t Lc, int32_t places, int32_t Cc, Gate gate) {
+  const bool cells = gate.open();
+  if (!cells)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
+      active[i] = i;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ctl->s = cells ? places : m;
+    ctl->C = cells ? Cc : C;
+    ctl->Lc = cells ? kTcTile : Lc;
+  }
+}
+
+cudaError_t launch_coarse_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t C, int32_t Lc,
+                                int32_t places, int32_t Cc, Gate gate, cudaStream_t st) {
+  int blocks = (m + 255) / 256;
+  if (blocks > 1024) blocks = 1024;
+  coarse_setup_kernel<<<blocks, 256, 0, st>>>(active, m, ctl, C, Lc, places, Cc, gate);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_step_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t C, int32_t Lc,
-                              cudaStream_t st) {
+                              const Gate& gate, cudaStream_t st) {
   int blocks = (m + 255) / 256;
   if (blocks < 1) blocks = 1;
   if (blocks > 1024) blocks = 1024;
-  step_setup_kernel<<<blocks, 256, 0, st>>>(active, m, ctl, C, Lc);
+  step_setup_kernel<<<blocks, 256, 0, st>>>(active, m, ctl, C, Lc, gate);
   return cudaGetLastError();
 }
 
@@ -724,8 +751,9 @@ cudaError_t launch_step_setup(int32_t* active, int32_t m, IterCtl* ctl, int32_t 
 __global__ void step_finish_kernel(const float* __restrict__ part, const IterCtl* __restrict__ ctl,
                                    const float* __restrict__ seeds, int d, int DA, double inv_scale,
                                    float* __restrict__ out_seeds, float* __restrict__ out_wsum,
-                                   const int32_t* __restrict__ out_row) {
+                                   const int32_t* __restrict__ out_row, Gate rows_gate) {
   const int s = ctl->s, C = ctl->C;
+  if (out_row && !rows_gate.open()) out_row = nullptr;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
   for (int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < s; p += nw) {
@@ -759,8 +787,9 @@ constexpr int kFinishChunks = 4;
 __global__ void step_finish_few(const float* __restrict__ part, const IterCtl* __restrict__ ctl,
                                 const float* seeds, int d, int DA, double inv_scale,
                                 float* out_seeds, float* __restrict__ out_wsum,
-                                const int32_t* __restrict__ out_row) {
+                                const int32_t* __restrict__ out_row, Gate rows_gate) {
   const int s = ctl->s, C = ctl->C;
+  if (out_row && !rows_gate.open()) out_row = nullptr;
   const int64_t total = (int64_t)s * d;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -781,20 +810,21 @@ __global__ void step_finish_few(const float* __restrict__ part, const IterCtl* _
 
 cudaError_t launch_step_finish(const float* part, const IterCtl* ctl, const float* seeds, int d,
                                int DA, double inv_scale, float* out_seeds, float* out_wsum,
-                               int m, int C, cudaStream_t st, const int32_t* out_row) {
+                               int m, int C, cudaStream_t st, const int32_t* out_row,
+                               Gate rows_gate) {
   if (C <= kFinishChunks) {
     int64_t blocks = ((int64_t)m * d + 255) / 256;
     if (blocks < 1) blocks = 1;
     if (blocks > 4096) blocks = 4096;
     step_finish_few<<<(int)blocks, 256, 0, st>>>(part, ctl, seeds, d, DA, inv_scale, out_seeds,
-                                                 out_wsum, out_row);
+                                                 out_wsum, out_row, rows_gate);
     return cudaGetLastError();
   }
   int blocks = (m + 7) / 8;
   if (blocks < 1) blocks = 1;
   if (blocks > 4096) blocks = 4096;
   step_finish_kernel<<<blocks, 256, 0, st>>>(part, ctl, seeds, d, DA, inv_scale, out_seeds,
-                                             out_wsum, out_row);
+                                             out_wsum, out_row, rows_gate);
   return cudaGetLastError();
 }
 

@@ -1,151 +1,130 @@
-// The probe of fms_route.cuh: one cluster of eight blocks a sampled set.
+// The probe of fms_route.cuh: one block a sampled set.
 //
 // A cell's radius is about the distance M from a sampled point to the nearest other one
-// (the cells have as many pivots as the sample has points); a cell whose centre lies at
+// (half of the cells start from as many strided points); a cell whose centre lies at
 // distance a from a seed is seen within the cutoff and the cell's reach.  From a sampled
 // point x of the cell, a^2 = |x - y|^2 - M^2 / 2 (x is M / sqrt 2 from the centre, at right
 // angles to y - centre where there are many dimensions).  The cutoff follows from the
 // sample's weights, as the walk takes it from W.  A set of more clusters than points in the
 // sample has a large M and comes out as one without clusters.
 //
-// Bound by latency: 3 us at d = 3, 6 at d = 32.
-#include <cooperative_groups.h>
-
+// One SM, bound by its shared memory (five 16-byte loads for 16 squared differences) and
+// latency.  (Eight blocks in a cluster took 14 to 21 us, barriers and remote writes.)
 #include "fms_cells.cuh"
 #include "fms_route.cuh"
 
 namespace fms {
 namespace {
 
-constexpr int kBlocks = 8;
-constexpr int kNear = kProbePoints / kBlocks, kSeedsPer = kProbeSeeds / kBlocks;
-constexpr int kRowsPer = kNear + kSeedsPer;   // rows a block compares with all points
+constexpr int kNear = 32;                           // points whose nearest other one is found
+constexpr int kLoaded = kProbePoints + kProbeSeeds;
+constexpr int kRows = kNear + kProbeSeeds;          // compared with all points
+constexpr int kSplit = 1024 / kProbePoints;         // threads of a point
+constexpr int kMine = kRows / kSplit;               // rows of a thread
+constexpr int kWarps = kProbePoints / 32;           // warps of a part
+static_assert(kRows % (4 * kSplit) == 0, "rows of a thread");
 
 __device__ __forceinline__ int64_t strided(int i, int of, int64_t n) {
   return ((2 * (int64_t)i + 1) * n) / (2 * (int64_t)of);
 }
 
 template <typename T>
-__global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kProbePoints)
-    probe_kernel(ProbeArgs a) {
-  namespace cg = cooperative_groups;
+__global__ void __launch_bounds__(1024) probe_kernel(ProbeArgs a) {
   extern __shared__ __align__(16) float probe_smem[];
-  const int d4 = (a.d + 3) & ~3, ld = d4 + 4;   // (rows 16 bytes apart modulo 128: no conflicts)
-  float* pts = probe_smem;                      // [kProbePoints][ld]
-  float* seeds = pts + kProbePoints * ld;       // [kSeedsPer][ld]
-  __shared__ __align__(16) float near[kProbePoints];          // of the first block: all points'
-  __shared__ float red[kRowsPer][kProbePoints / 32];
+  const int d4 = (a.d + 3) & ~3, ld = d4 + 4;   // (16 bytes between rows: few conflicts)
+  float* rows = probe_smem;                     // [kLoaded][ld]: the points, then the seeds
+  __shared__ float red[kRows][kWarps];          // a row's parts: least distance or weights
   __shared__ float median;
-  __shared__ int seen[kBlocks], sum[32];
-  cg::cluster_group cl = cg::this_cluster();
-  const int b = blockIdx.x / kBlocks, rank = blockIdx.x % kBlocks, t = threadIdx.x;
-  const int lane = t & 31, w = t >> 5;
-  const ProbeSet s = a.set[b];
+  __shared__ int sum[32];
+  const ProbeSet s = a.set[blockIdx.x];
   const T *X = static_cast<const T*>(s.X), *Y = static_cast<const T*>(s.Y);
-  const float scale = (float)a.scale;
-  // a thread loads its point (eight values in flight) and an element or two of the seeds
-  const float in = a.unit ? 1.0f : scale;
-  const T* x = X + strided(t, kProbePoints, s.n) * a.ld;
-  float sv[2];
+  const int lane = threadIdx.x & 31;
+  const float in = a.unit ? 1.0f : (float)a.scale;
+  // rows over groups of 8 threads, four values of a thread in flight
+  for (int r = threadIdx.x / 8; r < kLoaded; r += 128) {
+    const T* x = r < kProbePoints ? X + strided(r, kProbePoints, s.n) * a.ld
+                                  : Y + strided(r - kProbePoints, kProbeSeeds, s.m) * a.ld;
+    for (int k0 = threadIdx.x % 8; k0 < d4; k0 += 32) {
+      float v[4];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int e = t + u * kProbePoints, r = e / d4, k = e - r * d4;
-    sv[u] = r < kSeedsPer && k < a.d
-                ? (float)Y[strided(rank * kSeedsPer + r, kProbeSeeds, s.m) * a.ld + k]
-                : 0.0f;
+      for (int u = 0; u < 4; ++u) v[u] = k0 + 8 * u < a.d ? (float)x[k0 + 8 * u] : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + 8 * u < d4) rows[r * ld + k0 + 8 * u] = v[u] * in;
+    }
   }
-  for (int k0 = 0; k0 < d4; k0 += 8) {
-    float v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = k0 + u < a.d ? (float)x[k0 + u] : 0.0f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (k0 + u < d4) pts[t * ld + k0 + u] = v[u] * in;
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int e = t + u * kProbePoints, r = e / d4, k = e - r * d4;
-    if (r < kSeedsPer) seeds[r * ld + k] = sv[u] * in;
-  }
+  if (threadIdx.x == 0) median = INFINITY;   // (rows that are not finite have none)
   __syncthreads();
   if (a.unit) {
-    for (int r = t; r < kProbePoints + kSeedsPer; r += blockDim.x) {
+    for (int r = threadIdx.x; r < kLoaded; r += blockDim.x) {
       float nn = 0.0f;
-      for (int k = 0; k < a.d; ++k) nn += pts[r * ld + k] * pts[r * ld + k];
-      const float f = scale / sqrtf(nn);
-      for (int k = 0; k < a.d; ++k) pts[r * ld + k] *= f;
+      for (int k = 0; k < a.d; ++k) nn += rows[r * ld + k] * rows[r * ld + k];
+      const float f = (float)a.scale / sqrtf(nn);
+      for (int k = 0; k < a.d; ++k) rows[r * ld + k] *= f;
     }
     __syncthreads();
   }
-  if (t == 0) median = INFINITY;   // (rows that are not finite have none)
-  // squared distances of the block's rows (its share of the points, then its seeds) to
-  // point t, four rows at a time
-  float e2[kSeedsPer];
+  // squared distances from point t to the thread's rows (every fourth point, then the
+  // seeds), four at a time
+  constexpr int kEvery = kProbePoints / kNear;
+  const int t = threadIdx.x % kProbePoints, part = threadIdx.x / kProbePoints, w = t >> 5;
+  float q[kMine];
 #pragma unroll
-  for (int g = 0; g < kRowsPer; g += 4) {
-    const float* row = g < kNear ? pts + (rank * kNear + g) * ld : seeds + (g - kNear) * ld;
-    float q[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  for (int g = 0; g < kMine; g += 4) {
+    const int r0 = part * kMine + g, stride = r0 < kNear ? kEvery * ld : ld;
+    const float* row = rows + (r0 < kNear ? r0 * kEvery : kProbePoints + r0 - kNear) * ld;
+    float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
     for (int k = 0; k < d4; k += 4) {
-      const float4 x = *reinterpret_cast<const float4*>(pts + t * ld + k);
+      const float4 x = *reinterpret_cast<const float4*>(rows + t * ld + k);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const float4 y = *reinterpret_cast<const float4*>(row + u * ld + k);
+        const float4 y = *reinterpret_cast<const float4*>(row + u * stride + k);
         float e = x.x - y.x;
-        q[u] = fmaf(e, e, q[u]);
+        c[u] = fmaf(e, e, c[u]);
         e = x.y - y.y;
-        q[u] = fmaf(e, e, q[u]);
+        c[u] = fmaf(e, e, c[u]);
         e = x.z - y.z;
-        q[u] = fmaf(e, e, q[u]);
+        c[u] = fmaf(e, e, c[u]);
         e = x.w - y.w;
-        q[u] = fmaf(e, e, q[u]);
+        c[u] = fmaf(e, e, c[u]);
       }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      float v = q[u];
-      if (g < kNear) {
-        if (t == rank * kNear + g + u) v = INFINITY;
+      const int r = part * kMine + g + u;
+      q[g + u] = c[u];
+      float v = r < kNear ? (r * kEvery == t ? INFINITY : c[u]) : ex2_ftz(-c[u]);
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v = fminf(v, __shfl_xor_sync(kFull, v, o));
-      } else {
-        e2[g - kNear + u] = v;
-        v = ex2_ftz(-v);
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+      for (int o = 16; o >= 1; o >>= 1) {
+        const float z = __shfl_xor_sync(kFull, v, o);
+        v = r < kNear ? fminf(v, z) : v + z;
       }
-      if (lane == 0) red[g + u][w] = v;
+      if (lane == 0) red[r][w] = v;
     }
   }
   __syncthreads();
-  if (t < kNear) {
-    float v = red[t][0];
-    for (int u = 1; u < kProbePoints / 32; ++u) v = fminf(v, red[t][u]);
-    *cl.map_shared_rank(&near[rank * kNear + t], 0) = v;
-  }
-  cl.sync();
-  if (rank == 0) {   // the median of the distances to the nearest other point
-    const float v = near[t];
+  if (threadIdx.x < kNear) {   // (one warp) the median of the distances to the nearest point
+    float v = red[lane][0];
+    for (int u = 1; u < kWarps; ++u) v = fminf(v, red[lane][u]);
     int below = 0;
-#pragma unroll 4
-    for (int u = 0; u < kProbePoints; u += 4) {
-      const float4 o = *reinterpret_cast<const float4*>(near + u);
-      below += (o.x < v || (o.x == v && u < t) ? 1 : 0) + (o.y < v || (o.y == v && u + 1 < t) ? 1 : 0) +
-               (o.z < v || (o.z == v && u + 2 < t) ? 1 : 0) + (o.w < v || (o.w == v && u + 3 < t) ? 1 : 0);
+    for (int u = 0; u < kNear; ++u) {
+      const float o = __shfl_sync(kFull, v, u);
+      below += o < v || (o == v && u < lane) ? 1 : 0;
     }
-    if (below == kProbePoints / 2) {
-      for (int c = 0; c < kBlocks; ++c) *cl.map_shared_rank(&median, c) = v;
-    }
+    if (below == kNear / 2) median = v;
   }
-  cl.sync();
-  const float M = sqrtf(median);
-  const float log2n = log2f((float)s.n);
+  __syncthreads();
+  const float M = sqrtf(median), log2n = log2f((float)s.n);
   int vis = 0;
 #pragma unroll
-  for (int q = 0; q < kSeedsPer; ++q) {
+  for (int g = 0; g < kMine; ++g) {
+    const int r = part * kMine + g;
+    if (r < kNear) continue;
     float W = 0.0f;
-    for (int u = 0; u < kProbePoints / 32; ++u) W += red[kNear + q][u];
+    for (int u = 0; u < kWarps; ++u) W += red[r][u];
     W = fmaxf(W * ((float)s.n / kProbePoints), 1.0f);
-    const float at = sqrtf(fmaxf(e2[q] - 0.5f * M * M, 0.0f));
+    const float at = sqrtf(fmaxf(q[g] - 0.5f * M * M, 0.0f));
     float lim;
     if (a.kind == kProbeTile) {
       lim = sqrtf(cells::zero_bits<float>()) + 2.0f * M;
@@ -158,14 +137,10 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kProbePoints)
     vis += at <= lim ? 1 : 0;
   }
   vis = block_sum(vis, sum);
-  if (t == 0) *cl.map_shared_rank(&seen[rank], 0) = vis;
-  cl.sync();
-  if (rank == 0 && t == 0) {
-    int v = 0;
-    for (int c = 0; c < kBlocks; ++c) v += seen[c];
-    const float share = (float)v / (kProbePoints * kProbeSeeds);
-    a.share[b] = share;
-    if (a.walk) a.walk[b] = share <= kWalkShare ? 1 : 0;
+  if (threadIdx.x == 0) {
+    const float share = (float)vis / (kProbePoints * kProbeSeeds);
+    a.share[blockIdx.x] = share;
+    if (a.walk) a.walk[blockIdx.x] = share <= kWalkShare ? 1 : 0;
   }
 }
 
@@ -174,13 +149,8 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kProbePoints)
 template <typename T>
 cudaError_t launch_probe(const ProbeArgs& a, cudaStream_t st) {
   if (a.sets < 1 || a.sets > kProbeSets || a.d > 64) return cudaErrorInvalidValue;
-  const int bytes = (kProbePoints + kSeedsPer) * (((a.d + 3) & ~3) + 4) * 4;   // 72 KB at d = 64
-  if (bytes > 40 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        probe_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
-    if (e != cudaSuccess) return e;
-  }
-  probe_kernel<T><<<kBlocks * a.sets, kProbePoints, bytes, st>>>(a);
+  const int bytes = kLoaded * (((a.d + 3) & ~3) + 4) * 4;   // 43.5 KB at d = 64
+  probe_kernel<T><<<a.sets, 1024, bytes, st>>>(a);
   return cudaGetLastError();
 }
 template cudaError_t launch_probe<float>(const ProbeArgs&, cudaStream_t);

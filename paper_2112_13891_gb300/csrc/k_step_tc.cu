@@ -64,13 +64,17 @@ struct Geo {
 };
 }  // namespace tc
 
-// Tile images of the scaled points Xs [n][DP] (DP >= d, zero padded); with a
-// table, tile t holds the rows table[t] = (first, count <= 128).
+// Tile images of the scaled points Xu [n][DP] (DP >= d, zero padded); with a table (and
+// the gate open), tile t holds the rows table[t] = (first, count <= 128) of Xs.
 template <int DPAD>
-__global__ void tc_pack_tiles(const float* __restrict__ Xs, int n, int DP,
-                              unsigned char* __restrict__ img, const int2* __restrict__ table) {
+__global__ void tc_pack_tiles(const float* __restrict__ Xs, const float* __restrict__ Xu, int n,
+                              int DP, unsigned char* __restrict__ img,
+                              const int2* __restrict__ table, int tiles, Gate gate) {
   using G = tc::Geo<DPAD>;
   const int t = blockIdx.x;
+  if (table && !gate.open()) table = nullptr;
+  if (!table) Xs = Xu;
+  else if (t >= tiles) return;
   const int first = table ? table[t].x : t * tc::kP;
   const int rows = table ? table[t].y : min(tc::kP, n - first);
   if (rows <= 0) return;
@@ -155,6 +159,10 @@ __global__ void __launch_bounds__(tc::kThreads, 1)
   unsigned char* sP = sYext + G::kYextBytes;             // P[0], P[1]
   unsigned char* sRing = sP + 2 * G::kPBytes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tl.count) {
+    if (!tl.gate.open()) tl.count = nullptr;
+    else if (tl.y) y = tl.y;
+  }
   const int s_total = *s_total_ptr;
   const int count = *count_ptr;  // coarse seeds: positions [0, count)
   const int C = *C_ptr, Lc = *Lc_ptr;
@@ -494,21 +502,23 @@ size_t tc_image_bytes(int64_t n, int d) {
 cudaError_t launch_tc_pack(const float* Xs, int64_t n, int d, int DP, unsigned char* img,
                            cudaStream_t st) {
   const int tiles = (int)((n + tc::kP - 1) / tc::kP);
-  if (d <= 16) tc_pack_tiles<16><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, nullptr);
-  else tc_pack_tiles<32><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, nullptr);
+  return launch_tc_pack_table(Xs, Xs, n, d, DP, nullptr, tiles, img, Gate{}, st);
+}
+
+cudaError_t launch_tc_pack_table(const float* Xs, const float* Xu, int64_t n, int d, int DP,
+                                 const int2* table, int tiles, unsigned char* img, Gate gate,
+                                 cudaStream_t st) {
+  const int all = (int)((n + tc::kP - 1) / tc::kP), grid = tiles > all ? tiles : all;
+  if (d <= 16)
+    tc_pack_tiles<16><<<grid, 256, 0, st>>>(Xs, Xu, (int)n, DP, img, table, tiles, gate);
+  else
+    tc_pack_tiles<32><<<grid, 256, 0, st>>>(Xs, Xu, (int)n, DP, img, table, tiles, gate);
   return cudaGetLastError();
 }
 
 // Bytes of `tiles` tile images.
 size_t tc_tile_images(int64_t tiles, int d) {
   return (size_t)tiles * (d <= 16 ? tc::Geo<16>::kTileBytes : tc::Geo<32>::kTileBytes);
-}
-
-cudaError_t launch_tc_pack_table(const float* Xs, int64_t n, int d, int DP, const int2* table,
-                                 int tiles, unsigned char* img, cudaStream_t st) {
-  if (d <= 16) tc_pack_tiles<16><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, table);
-  else tc_pack_tiles<32><<<tiles, 256, 0, st>>>(Xs, (int)n, DP, img, table);
-  return cudaGetLastError();
 }
 
 // The point tiles that a tile of up to 128 seeds (one block) can see: those of
@@ -521,7 +531,9 @@ __global__ void __launch_bounds__(128)
                const int32_t* __restrict__ yperm, cells::View<float> cv,
                const int2* __restrict__ tile_table, const int32_t* __restrict__ tile_cell,
                int tiles, int32_t* __restrict__ list, int32_t* __restrict__ count,
-               int32_t* __restrict__ active, int32_t* __restrict__ out_row) {
+               int32_t* __restrict__ active, int32_t* __restrict__ out_row, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   __shared__ float red[4][DP + 1];
   __shared__ float ball[DP + 1];
   __shared__ unsigned char sees[cells::kMaxCells];
@@ -599,19 +611,18 @@ cudaError_t launch_tc_visible(const float* Ys, int DP, const int2* seed_table, i
                               const int32_t* yperm, const cells::View<float>& cv,
                               const int2* tile_table, const int32_t* tile_cell, int tiles,
                               int32_t* list, int32_t* count, int32_t* active, int32_t* out_row,
-                              cudaStream_t st) {
+                              cudaStream_t st, Gate gate) {
 #define FMS_VIS(DP_)                                                                             \
-  tc_visible<DP_><<<seed_tiles, 128, 0, st>>>(Ys, seed_table, yperm, cv, tile_table, tile_cell, \
-                                              tiles, list, count, active, out_row)
+  return launch_gated(gate, tc_visible<DP_>, seed_tiles, 128, 0, st, Ys, seed_table, yperm, cv,  \
+                      tile_table, tile_cell, tiles, list, count, active, out_row, gate)
   switch (DP) {
-    case 4: FMS_VIS(4); break;
-    case 8: FMS_VIS(8); break;
-    case 16: FMS_VIS(16); break;
-    case 32: FMS_VIS(32); break;
-    default: return cudaErrorInvalidValue;
+    case 4: FMS_VIS(4);
+    case 8: FMS_VIS(8);
+    case 16: FMS_VIS(16);
+    case 32: FMS_VIS(32);
   }
 #undef FMS_VIS
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 // One persistent CTA per SM: each holds all 512 TMEM columns.

@@ -108,7 +108,9 @@ template <int DP, int NX>
 __global__ void __launch_bounds__(256, 2)
     step_groups(const float* __restrict__ Xs, View<float> cv, int n, const float* __restrict__ Ys,
                 Groups gr, int m, const int32_t* __restrict__ perm, int d, const float* seeds,
-                double inv_scale, float* out_seeds, float* __restrict__ out_wsum) {
+                double inv_scale, float* out_seeds, float* __restrict__ out_wsum, Gate gate) {
+  wait_for_previous();
+  if (!gate.open()) return;
   extern __shared__ __align__(16) unsigned char travel_smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
   const TeamSmem<float, DP, DP + 1> sm(travel_smem, w, W);
@@ -782,7 +784,7 @@ int seed_grid(int max_seeds, int sms) {
 cudaError_t launch_step_groups(const float* Xs, const View<float>& cv, int n, const float* Ys,
                                const Groups& gr, int m, const int32_t* perm, int d, int DP,
                                const float* seeds, double inv_scale, float* out_seeds,
-                               float* out_wsum, int sms, cudaStream_t st) {
+                               float* out_wsum, int sms, cudaStream_t st, Gate gate) {
 #define FMS_STEP_GROUPS(DP_, NX_)                                                                \
   {                                                                                              \
     constexpr int ws = team_warp_smem<float, DP_, DP_ + 1>();                                    \
@@ -790,10 +792,8 @@ cudaError_t launch_step_groups(const float* Xs, const View<float>& cv, int n, co
     const int smem = group_team_smem<float, DP_, DP_ + 1>(W);                                    \
     const cudaError_t e = team_attr(step_groups<DP_, NX_>, smem);                                \
     if (e != cudaSuccess) return e;                                                              \
-    step_groups<DP_, NX_><<<gr.per_set, 32 * W, smem, st>>>(Xs, cv, n, Ys, gr, m, perm, d,       \
-                                                            seeds, inv_scale, out_seeds,         \
-                                                            out_wsum);                           \
-    return cudaGetLastError();                                                                   \
+    return launch_gated(gate, step_groups<DP_, NX_>, gr.per_set, 32 * W, smem, st, Xs, cv, n,   \
+                        Ys, gr, m, perm, d, seeds, inv_scale, out_seeds, out_wsum, gate);       \
   }
   FMS_BY_COLUMNS(FMS_STEP_GROUPS)
   switch (DP) {

@@ -1,5 +1,5 @@
 """Sorted cells and whole trajectories in one launch, at the sizes where their
-rules begin: one update by groups (n m times the padded width >= 1.7e9), a block
+rules begin: one update by groups (n m times the padded width >= 2.5e9), a block
 per seed (d > 7; points sorted from n = 8,192 on) and every point a seed by groups
 (d <= 7; sorted from n = 4,096 on), against the FP64 oracle.
 
@@ -28,8 +28,11 @@ def _blobs(seed, n, d, k, box, sigma):
 # just above the rule's line; a last sort block of one row; fewer seeds than points
 @pytest.mark.parametrize("n,m,d,box,h", [(20_620, 20_623, 3, 200.0, 5.0), (14_580, 14_579, 6, 60.0, 4.0),
                                          (10_241, 10_400, 9, 50.0, 2.5), (51_201, 2_080, 16, 50.0, 2.5),
+                                         (25_000, 25_003, 3, 200.0, 5.0), (17_680, 17_679, 6, 60.0, 4.0),
+                                         (12_289, 12_800, 9, 50.0, 2.5), (76_801, 2_049, 16, 50.0, 2.5),
+                                         (8_900, 8_891, 32, 12.0, 1.5),
                                          # 256, 257 chunks of the sort and many: a scan of its counters
-                                         (262_144, 2_048, 3, 200.0, 5.0), (262_145, 2_049, 5, 60.0, 4.0),
+                                         (262_144, 2_400, 3, 200.0, 5.0), (262_145, 2_049, 5, 60.0, 4.0),
                                          (1_500_000, 2_050, 9, 50.0, 2.5),
                                          (7_300, 7_291, 32, 12.0, 1.5)])
 def test_step_by_groups(n, m, d, box, h):
@@ -52,8 +55,9 @@ def test_step_by_groups(n, m, d, box, h):
     assert W[m - 1] == 0.0 and np.isnan(out[m - 1]).all()   # 0 / 0, as without cells
 
 
-def test_step_by_groups_keeps_nonfinite():
-    n = m = 7_300
+@pytest.mark.parametrize("n", [7_300, 8_900])
+def test_step_by_groups_keeps_nonfinite(n):
+    m = n
     X = torch.randn((n, 32), device="cuda")
     X[5, 3] = float("inf")
     out = fms.mean_shift_step(X, torch.randn((m, 32), device="cuda"), 1.0)
@@ -241,3 +245,33 @@ def test_evaluations_beyond_32_bits():
     r = fms.cluster(X, 5.0, 1e-14, updates, n_initial=1, L=0.01, gamma=1.0, skip_refine=True)
     assert r.stats["iterations"] == updates
     assert n * updates <= r.stats["evals"] <= n * (updates + 2)
+
+
+# The updates where cells would leave nothing out (one blob of half a bandwidth, blobs next
+# to each other, centres of a sphere in reach of the coarse step's tiles) are made over
+# every pair; both sides of the decision at the smallest sizes where it is made.
+@pytest.mark.parametrize("n,m,d,k,box", [(25_000, 25_003, 3, 1, 0.0), (262_144, 2_400, 3, 6, 3.0),
+                                         (17_680, 17_679, 7, 1, 0.0), (17_680, 17_700, 8, 3, 2.0),
+                                         (76_801, 2_049, 16, 1, 0.0), (8_900, 8_891, 32, 4, 1.0),
+                                         (25_000, 25_003, 3, 30, 100.0), (12_500, 12_600, 16, 90, 60.0)])
+@pytest.mark.parametrize("coarse", [False, True])
+def test_step_where_cells_may_leave_nothing_out(n, m, d, k, box, coarse):
+    from test_gpu_coarse_step import _bound
+    h = 1.0
+    X = _blobs(n + k, n, d, k, box, 0.5)
+    rng = np.random.default_rng(3)
+    Y = (X[rng.integers(0, n, m)] + 0.1 * rng.standard_normal((m, d))).astype(np.float32)
+    Y[5] = X.max(axis=0) + 100.0                    # every weight zero
+    fn = fms.mean_shift_step_coarse if coarse else fms.mean_shift_step
+    out, W = fn(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), h, with_wsum=True)
+    out, W = out.cpu().numpy().astype(np.float64), W.cpu().numpy().astype(np.float64)
+    pick = np.unique(np.r_[0, m - 1, rng.integers(6, m, 60)])
+    ref, refW = orc.step(X, Y[pick], h), orc.kde(X, Y[pick], h)
+    if coarse:
+        bnd, eps = _bound(X, Y[pick], h, ref)
+        assert np.all(np.abs(out[pick] - ref).max(axis=1) <= bnd)
+        assert np.all(np.abs(W[pick] - refW) <= 1.5 * eps * refW)
+    else:
+        assert np.abs(W[pick] / refW - 1).max() <= 1e-4
+        assert np.abs(out[pick] - ref).max() <= 2e-4 * h + 2.0 ** -20 * np.abs(ref).max()
+    assert W[5] == 0.0 and np.isnan(out[5]).all()

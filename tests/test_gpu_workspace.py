@@ -41,7 +41,7 @@ def test_cluster(n, d, kw):
     ws.check()
 
 
-@pytest.mark.parametrize("n,m", [(262_144, 2_048), (65_536, 20_480), (50_000, 20_001)])
+@pytest.mark.parametrize("n,m", [(262_144, 2_400), (65_536, 20_480), (50_000, 20_001)])
 @pytest.mark.parametrize("d", [3, 9, 32])
 def test_steps(n, m, d):
     X = _blobs(n + d, n, d)
