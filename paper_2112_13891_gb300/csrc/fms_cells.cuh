@@ -45,6 +45,7 @@ struct View {
   const float2* ext;     // [P][P] (one set, FP32; nullable): at [q][p], how far cell p's
                          // rows reach from its centre towards cell q's, and the
                          // distance of the two centres
+  Gate gate;             // closed: the kernel takes every row, as without cells
 };
 
 // How far cell p's rows reach towards a seed y at distance a from its centre: the

@@ -132,9 +132,9 @@ BwdLayout bwd_layout(const UGeom& g, int P, int32_t k, size_t es) {
 // DP values, seeds in sorted order), then W_t, the weight shift and the mean
 // squared distance of every update t < T (one value per seed each), so the
 // backward recomputes only the positions between checkpoints; with cells, the
-// seeds' order and groups.
+// seeds' order and groups and the probe's answer.
 struct CkptLayout {
-  size_t pos, W, Sh, M2, perm, table, total;
+  size_t pos, W, Sh, M2, perm, table, walk, share, total;
 };
 CkptLayout ckpt_layout(const UGeom& g, int P, int32_t T, int32_t k, size_t es) {
   CkptLayout C{};
@@ -145,13 +145,35 @@ CkptLayout ckpt_layout(const UGeom& g, int P, int32_t T, int32_t k, size_t es) {
   C.M2 = C.Sh + (size_t)T * rowsY * es;
   C.perm = a256(C.M2 + (size_t)T * rowsY * es);
   C.table = C.perm + (P > 0 ? a256(rowsY * 4) : 0);
-  C.total = C.table + (P > 0 ? (size_t)g.B * cells::group_cap(g.m, P) * 8 : 0);
+  C.walk = C.table + (P > 0 ? a256((size_t)g.B * cells::group_cap(g.m, P) * 8) : 0);
+  C.share = C.walk + (P > 0 ? kProbeSets * 4 : 0);
+  C.total = C.share + (P > 0 ? kProbeSets * 4 : 0);
   return C;
 }
 
 template <typename T>
 T* at(void* base, size_t off) {
   return reinterpret_cast<T*>(static_cast<char*>(base) + off);
+}
+
+// Whether the cells leave enough out, asked of up to kProbeSets of the sets.
+int probed_sets(int B) { return B < kProbeSets ? B : kProbeSets; }
+
+template <typename E>
+cudaError_t probe_sets(const E* points, const E* seeds0, const UGeom& g, double c, void* ckpt,
+                       const CkptLayout& CL, cudaStream_t st) {
+  ProbeArgs a{};
+  a.sets = probed_sets(g.B);
+  for (int i = 0; i < a.sets; ++i) {
+    const int64_t b = ((2 * i + 1) * (int64_t)g.B) / (2 * a.sets);
+    a.set[i] = {points + b * g.n * g.d, seeds0 + b * g.m * g.d, g.n, g.m};
+  }
+  a.d = a.ld = g.d;
+  a.scale = sqrt(c);
+  a.kind = kProbeBall;
+  a.share = at<float>(ckpt, CL.share);
+  a.walk = at<int32_t>(ckpt, CL.walk);
+  return launch_probe<E>(a, st);
 }
 
 // Padded (and, with cells, sorted) copy of the points.
@@ -202,6 +224,9 @@ fms_status forward_impl(const E* points, const E* seeds0, int32_t B, int64_t n, 
   if (sort_points<E>(points, g, P, L.s, ws, &cv, st) != cudaSuccess) return FMS_ERR_CUDA;
   cells::Groups gr{nullptr, groups_for(m, P)};
   if (P > 0) {
+    if (probe_sets<E>(points, seeds0, g, (double)c, ckpt, CL, st) != cudaSuccess)
+      return FMS_ERR_CUDA;
+    cv.gate = Gate{at<int32_t>(ckpt, CL.walk), probed_sets(B), 0};
     const E* src = seeds0;
     if (d != g.DP || (reinterpret_cast<uintptr_t>(seeds0) & 15u)) {
       E* Yp = at<E>(ws, L.Yp);
@@ -264,6 +289,7 @@ fms_status backward_impl(const E* points, int32_t B, int64_t n, int64_t m, int32
   if (sort_points<E>(points, g, P, L.s, ws, &cv, st) != cudaSuccess ||
       unroll_pack_rows<E>(grad_out, rowsY, (int)m, d, g.DP, yperm, G, st) != cudaSuccess)
     return FMS_ERR_CUDA;
+  if (P > 0) cv.gate = Gate{at<int32_t>(ck, CL.walk), probed_sets(B), 0};
   int first = 1;
   for (int s = n_ckpt(T, k) - 1; s >= 0; --s) {
     const int t0 = s * k;

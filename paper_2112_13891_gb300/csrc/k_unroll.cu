@@ -14,7 +14,9 @@
 // segment of k updates from its checkpoint, then walks it in reverse.
 //
 // Points and seeds are kept sorted into cells (fms_cells.cuh), and a group of 32
-// seeds of one cell walks only the point cells within its cutoff radius.  Seeds
+// seeds of one cell walks only the point cells within its cutoff radius (where a
+// sample says that cells leave too little out, 32 seeds in a row walk every point,
+// in one pass an update).  Seeds
 // do not depend on each other, so one launch takes a group through all T updates
 // (or, in the adjoint, through a whole segment).  Kernels (FP32, or FP64 for
 // checking gradients; exact differences, fixed-order sums; rows padded to DP =
@@ -115,6 +117,10 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
   extern __shared__ __align__(16) unsigned char unroll_smem[];
   constexpr int SUMS = DP + 3, GS = 32 / PH;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  if (!cv.gate.open()) {
+    cv.P = 0;
+    gr.table = nullptr;
+  }
   const int b = blockIdx.x / gr.per_set;
   int row0, cnt;
   if (!group_rows(gr, b, blockIdx.x % gr.per_set, g.m, &row0, &cnt, GS)) return;
@@ -220,6 +226,10 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
   extern __shared__ __align__(16) unsigned char unroll_smem[];
   constexpr int SUMS = DP + 2, SDW = 2 * DP + 4, GS = 32 / PH;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  if (!cv.gate.open()) {
+    cv.P = 0;
+    gr.table = nullptr;
+  }
   __shared__ double dhs[16];
   const int b = blockIdx.x / gr.per_set, gi = blockIdx.x % gr.per_set;
   const int64_t NG = (int64_t)g.B * gr.per_set;
@@ -345,12 +355,13 @@ __global__ void __launch_bounds__(32 * most_warps<T, DP>())
 // to its rows of dX.
 template <typename T, int DP, int NX>
 __global__ void __launch_bounds__(32 * most_warps<T, DP>())
-    unroll_bwd_point(const T* __restrict__ X, Groups gx, Groups gr, UGeom g, int len, T c,
-                     T inv_h2, const T* __restrict__ SD, const T* __restrict__ bctr,
+    unroll_bwd_point(const T* __restrict__ X, Gate gate, Groups gx, Groups gr, UGeom g, int len,
+                     T c, T inv_h2, const T* __restrict__ SD, const T* __restrict__ bctr,
                      const T* __restrict__ breach, T* __restrict__ dX, int first) {
   extern __shared__ __align__(16) unsigned char unroll_smem[];
   constexpr int SUMS = DP, SDW = 2 * DP + 4;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  if (!gate.open()) gx.table = gr.table = nullptr;
   const TeamSmem<T, SDW, SUMS, false> sm(unroll_smem, w, W);
   const int b = blockIdx.x / gx.per_set;
   int row0, cnt;
@@ -568,7 +579,7 @@ static cudaError_t bwd_t(const T* X, const View<T>& cv, const USegment<T>& sg, c
   const int smem_p = list_team_smem<T, 2 * DP + 4, DP>(Wp);
   e = team_attr(unroll_bwd_point<T, DP, NX>, smem_p);
   if (e != cudaSuccess) return e;
-  unroll_bwd_point<T, DP, NX><<<(unsigned)PG, 32 * Wp, smem_p, st>>>(X, gx, gr, g, sg.len, c, inv_h2,
+  unroll_bwd_point<T, DP, NX><<<(unsigned)PG, 32 * Wp, smem_p, st>>>(X, cv.gate, gx, gr, g, sg.len, c, inv_h2,
                                                                  SD, bctr, breach, dX, first);
   return cudaGetLastError();
 }

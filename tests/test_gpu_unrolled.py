@@ -277,3 +277,32 @@ def test_threads_with_different_sizes():
     for t in ts:
         t.join()
     assert not failed, failed
+
+
+# One blob, or blobs in reach of each other: every point counts for every seed, and the
+# sorted form takes them all (the sizes as above; FP64 alike).
+@pytest.mark.parametrize("B,n,m,d,k,box,T,kk,dt", [
+    (1, 2049, 2049, 3, 1, 1.0, 5, 2, np.float32), (1, 4200, 1001, 16, 3, 2.0, 4, 3, np.float32),
+    (5, 1000, 900, 2, 4, 4.0, 3, 9, np.float32), (1, 2050, 2048, 32, 1, 1.0, 3, 1, np.float32),
+    (2, 1500, 1450, 7, 2, 2.0, 4, 3, np.float64)])
+def test_sorted_cells_that_leave_nothing_out(B, n, m, d, k, box, T, kk, dt):
+    h = 2.0
+    X = _wide_sets(d * 7 + n, B, n, d, k, box).astype(dt)
+    rng = np.random.default_rng(5)
+    Y0 = (X[:, :m] + 0.3 * rng.standard_normal((B, m, d))).astype(dt)
+    if d == 3:
+        Y0[0, 5] = X[0].max(axis=0) + 60.0       # every weight zero in FP32
+    G = rng.standard_normal(Y0.shape).astype(dt)
+    YT, ck = fms.unrolled_forward(torch.from_numpy(X).cuda(), torch.from_numpy(Y0).cuda(), h, T, kk)
+    dX, dY, dh = fms.unrolled_backward(torch.from_numpy(X).cuda(), ck, m, h, T, kk,
+                                       torch.from_numpy(G).cuda())
+    torch.cuda.synchronize()
+    tol = 2e-4 if dt == np.float32 else 1e-9
+    for b in range(B):
+        ref = orc.unrolled_forward(X[b], Y0[b], h, T)[-1]
+        assert np.abs(YT[b].cpu().numpy() - ref).max() <= tol * (1 + np.abs(ref).max())
+        rdX, rdY, rdh = orc.unrolled_backward(X[b], Y0[b], h, T, G[b])
+        for got, want in ((dX[b], rdX), (dY[b], rdY)):
+            got = got.cpu().numpy().astype(np.float64)
+            assert np.abs(got - want).max() <= tol * (1 + np.abs(want).max())
+        assert abs(dh[b].item() - rdh) <= tol * (1 + abs(rdh))
