@@ -77,9 +77,11 @@ typedef struct fms_options {
   int32_t profile;          /* 1: time every ms_step launch with CUDA events and
                                report it in fms_stats (adds event records)        */
   int32_t precision;        /* arithmetic of the seed updates (FMS_PRECISION_*):
-                               AUTO (0) = TENSOR for 9 <= d <= 32 where every
-                                  point is a seed or n_initial (or the seed list)
-                                  exceeds 4096, else FP32.
+                               AUTO (0) = FP32 where that takes less time (a
+                                  block per seed: few seeds, or data of which
+                                  each seed sees little, by the sizes and a
+                                  sample of the points), else TENSOR for
+                                  9 <= d <= 32, FP32 elsewhere.
                                FP32 (1): every update evaluates the weights in
                                   FP32 from exact differences.  (Sorted points:
                                   weights that cannot count, all together below

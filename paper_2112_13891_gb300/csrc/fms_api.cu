@@ -67,13 +67,14 @@ static_assert(sizeof(IterCtl) <= kCtlMergeOff && sizeof(MergeCtl) <= 256 &&
 
 // Pinned staging of the control region (one per host thread, kept for the
 // life of the thread): pageable destinations would make every readback a
-// staged, host-blocking copy.
+// staged, host-blocking copy.  Behind it, the word that the probe answers in.
 unsigned char* pinned_ctl() {
   thread_local unsigned char* buf = nullptr;
-  if (!buf && cudaMallocHost(&buf, kCtlBlockBytes) != cudaSuccess) buf = nullptr;
+  if (!buf && cudaMallocHost(&buf, kCtlBlockBytes + 64) != cudaSuccess) buf = nullptr;
   return buf;
 }
 
+constexpr size_t kCtlShareOff = 832, kCtlWalkOff = 836;   // a probe's answer
 constexpr size_t kCtlRoundOff = 896;   // RoundCtl of the device-driven rounds
 static_assert(kCtlRoundOff + sizeof(RoundCtl) <= kCtlBlockBytes, "control region");
 
@@ -97,6 +98,7 @@ struct GraphKey {
   size_t ws_bytes;
   int64_t n;
   int32_t d, max_iter, max_modes, dev;
+  int32_t travel, P, cap_seeds, cap_modes;   // the route that the data decided
   float h, tol;
   unsigned char opts[sizeof(fms_options)];
 };
@@ -134,12 +136,23 @@ GraphCache& graph_cache() {
 // Private capture streams (per device and purpose), kept for the thread's life.
 cudaStream_t capture_stream(int dev, int which) {
   constexpr int kMaxDevices = 64;
-  thread_local cudaStream_t s[kMaxDevices][2] = {};
+  thread_local cudaStream_t s[kMaxDevices][3] = {};
   if (dev < 0 || dev >= kMaxDevices) return nullptr;
   if (!s[dev][which] &&
       cudaStreamCreateWithFlags(&s[dev][which], cudaStreamNonBlocking) != cudaSuccess)
     s[dev][which] = nullptr;
   return s[dev][which];
+}
+
+// The event behind a call's probe (per device, kept for the thread's life).
+cudaEvent_t route_event() {
+  constexpr int kMaxDevices = 64;
+  thread_local cudaEvent_t ev[kMaxDevices] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  if (!ev[dev] && cudaEventCreateWithFlags(&ev[dev], cudaEventDisableTiming) != cudaSuccess)
+    ev[dev] = nullptr;
+  return ev[dev];
 }
 
 // During capture on `cs`: add a conditional node after the captured work and
@@ -179,38 +192,97 @@ enum Travel : int {
   kTravelSeeds = 1,    // travel_seeds: a block takes a seed to convergence
   kTravelGroups = 2,   // travel_groups: every point a seed, 32 to a group
 };
+// What a call's sizes and options allow; its data decide the rest (decide_route).
 struct Route {
   int travel;
-  int P;         // cells the points are sorted into (0: none)
-  bool tensor;   // updates start on the tensor-core step
+  int P;         // cells the points may be sorted into (0: none)
+  bool tensor;   // steps start on the tensor-core step
 };
 
-// Seeds up to which a block per seed is the better split.  65,536 points of 32 blobs,
-// d = 16: 512 seeds 0.31 ms (the steps 0.70), 4,096 0.94 (1.61), 8,192 1.78 (2.80); but
-// over every pair 1.10 and 6.1 ms, since each block reads its rows from L2 for one seed,
-// so the line lies where data without clusters begins to lose much.
-constexpr int32_t kTravelMaxSeeds = 4096;
-// Points from which they are sorted.  On 8 blobs it pays a step later (128 seeds, d = 16:
-// 8,192 points 207 us sorted, 162 not; 16,384 214 and 208; 32,768 233 and 284.  Every
-// point a seed, d = 3: 4,096 points 459 and 340; 8,192 825 and 907); the more clusters,
-// the more a seed leaves out.
-constexpr int64_t kSortSeedsMin = 8192, kSortGroupsMin = 4096;
+// Points from which they may be sorted.  8 blobs, sorted / not: 128 seeds, d = 16, 8,192
+// points 207 / 162 us, 16,384 214 / 208, 32,768 233 / 284; every point a seed, d = 3, 4,096
+// points 459 / 340, 8,192 825 / 907; the more clusters, the more a seed leaves out.
+constexpr int64_t kSortSeedsMin = 16384, kSortGroupsMin = 8192;
 
 Route choose_route(int64_t n, int d, const fms_options& o, int32_t max_iter) {
   Route r{};
   const bool plain = o.kernel == FMS_KERNEL_GAUSSIAN && o.metric != FMS_METRIC_COSINE;
-  const int64_t N0 = o.seed_indices ? o.n_seed_indices : o.n_initial;
   if (max_iter <= kHistCap && n <= INT32_MAX) {
     if (o.all_seeds) {
       if (d <= 7) r.travel = kTravelGroups;
-    } else if (d > 7 && N0 <= kTravelMaxSeeds && o.precision != FMS_PRECISION_TENSOR) {
+    } else if (d > 7 && o.precision != FMS_PRECISION_TENSOR) {
       r.travel = kTravelSeeds;
     }
   }
   if (r.travel == kTravelSeeds && n >= kSortSeedsMin) r.P = cells::choose_cells(n, n);
   if (r.travel == kTravelGroups && n >= kSortGroupsMin) r.P = cells::choose_cells(n, n);
-  r.tensor = r.travel == kTravelSteps && plain && use_tensor_step(d, o.precision);
+  r.tensor = r.travel != kTravelGroups && plain && use_tensor_step(d, o.precision);
   return r;
+}
+
+// Microseconds of one update of N seeds over n points, d > 7, as measured.
+// A block per seed reads 4 DP bytes a row from L2: 10 TB/s in all, 0.13 a block.  65,536 x
+// 16, 128 seeds, every row: 8 passes 489 us; 200,000 x 16 6 passes 995; 200,000 x 32 2,098.
+double travel_us(double n, double N, int DP, double share) {
+  const double rate = 1e7 < 1.3e5 * N ? 1e7 : 1.3e5 * N;
+  return 8.0 + 4.0 * DP * n * N * share / rate;
+}
+// Steps: two or three launches and an eighth of a read-back, then 3 ps a pair (4.5 for
+// d > 32) up to the pairs that fill the GPU, beyond 0.5 on the tensor cores, 0.12 DP in FP32.
+// The same calls 617, 784 and 901 us; 512 seeds at 65,536 x 16 158 an update, 128 at 10^7 x
+// 9 750.
+double steps_us(double n, double N, int DP, bool tensor) {
+  const double few = DP > 32 ? 4.5e-6 : 3e-6, many = tensor ? 0.5e-6 : 1.2e-7 * DP;
+  const double p = n * N, fill = 3.3e7;
+  return 55.0 + few * (p < fill ? p : fill) +
+         (p > fill ? (many < few ? many : few) * (p - fill) : 0.0);
+}
+// Sorting, and the extents (from HBM beyond the L2's size).
+double sort_us(double n, int DP) { return 40.0 + (n * DP < 2e7 ? 3.5e-5 : 5e-5) * n * DP; }
+// Updates of a call (their number drops out but for sorting); what the first pass of each
+// trajectory, which is made twice, adds to a walk.
+constexpr double kCallUpdates = 8.0, kWalkExtra = 1.2;
+// Every point a seed and no cells that leave enough out: up to here all rows in one launch
+// (blobs in reach of each other, d = 2 to 6: 8,192 points 2.1 to 2.7 ms, by steps 2.6 to
+// 5.0; 16,384 6.4 to 11.0, 5.5 to 10.0), beyond the steps, which leave converged seeds out
+// (50,000 points, d = 3: 68 and 25 ms).
+constexpr int64_t kPlainGroupsMax = 10240;
+
+// The share of the points in the cells that a seed sees up to which sorting pays.
+float share_limit(const Route& r, int64_t n, int DP, int64_t N0) {
+  if (r.P == 0) return -1.0f;
+  if (r.travel == kTravelGroups) return kWalkShare;
+  const double U = kCallUpdates, all = travel_us((double)n, (double)N0, DP, 1.0);
+  const double steps = steps_us((double)n, (double)N0, DP, r.tensor);
+  const double none = travel_us((double)n, (double)N0, DP, 0.0);   // (a walk of no rows)
+  const double s = ((steps < all ? steps : all) - sort_us((double)n, DP) / U - none) /
+                   (kWalkExtra * (all - none));
+  return (float)(s < 0.5 ? s : 0.5);
+}
+
+// How the seeds travel, and the most seeds for which that is the faster (a block per seed),
+// over sorted points of which a seed's cells hold `share`, or unsorted ones.
+void decide_route(const Route& r, int64_t n, int DP, int64_t N0, bool sorted, double share,
+                  int* travel, int64_t* most) {
+  *travel = r.travel;
+  *most = n;
+  if (r.travel == kTravelGroups) {
+    if (r.P > 0 && !sorted && n > kPlainGroupsMax) *travel = kTravelSteps;
+    return;
+  }
+  if (r.travel != kTravelSeeds) return;
+  const double sh = sorted ? kWalkExtra * share : 1.0;
+  auto by_seed = [&](int64_t N) {
+    return travel_us((double)n, (double)N, DP, sh) <=
+           steps_us((double)n, (double)N, DP, r.tensor);
+  };
+  if (!sorted && !by_seed(N0)) {
+    *travel = kTravelSteps;
+    return;
+  }
+  *most = N0;
+  while (*most < n && by_seed(2 * *most)) *most *= 2;
+  if (*most > n) *most = n;
 }
 
 Layout make_layout(int64_t n, int d, int64_t Ncap, int sms, const Route& route) {
@@ -461,7 +533,6 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
   if (dv.sms <= 0) return FMS_ERR_CUDA;
   const int64_t Ncap = seed_capacity(n, o);
   const Route route = choose_route(n, d, o, max_iter);
-  const bool tensor = route.tensor;
   const Layout Lo = make_layout(n, d, Ncap, dv.sms, route);
   const int DP = Lo.DP, DA = Lo.DA, R = Lo.R;
   bool owns_ws = false;
@@ -549,9 +620,6 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       return cudaSuccess;
     };
     int32_t* tclog = slog + kSlogCap;
-    Tiling tl_iter = Lo.tl;   // the seed-update loop (tensor-core chunking when on)
-    tl_iter.tc_ctas = Lo.tc_ctas;
-    const int32_t init_state = tensor ? kCoarse : kRunning;
     const int qmax = d <= 7 ? round_max_clusters(d) : 0;
     // persistent grid rounds (one CTA per SM) for d <= 7 when they fit
     const GridPlan gp = d <= 7 ? cached_grid_plan(n, d, dv.sms, max_iter) : GridPlan{};
@@ -568,6 +636,113 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     const double r_merge = o.merge_radius > 0.0f ? (double)o.merge_radius : (double)h;
     const double r2_s = (r_merge * scale) * (r_merge * scale);
     const bool allow_doubling = !o.all_seeds && !o.seed_indices;
+    // --- Seed Selection (Alg. 2): initial seed count ---
+    int32_t N0;
+    if (o.all_seeds) N0 = (int32_t)n;
+    else if (o.seed_indices) N0 = o.n_seed_indices;
+    else N0 = (int32_t)(o.n_initial < n ? o.n_initial : n);
+
+    // --- the route: by a sample of the points where they may be sorted ---
+    int travel = 0, P = 0, cap_seeds = 0, cap_modes = 0;
+    bool sorted = false, by_seed = false, tensor = false;
+    int64_t travel_max = 0;
+    float* rows = Xs;   // the rows that the trajectories read
+    int32_t* perm = nullptr;
+    cells::View<float> cv{};
+    Tiling tl_iter = Lo.tl;   // the seed-update loop (tensor-core chunking when on)
+    int32_t init_state = kRunning;
+    auto set_route = [&](bool sorted_, double share) {
+      sorted = sorted_;
+      decide_route(route, n, DP, N0, sorted, share, &travel, &travel_max);
+      by_seed = travel == kTravelSeeds;
+      tensor = route.tensor && travel == kTravelSteps;
+      tl_iter.tc_ctas = tensor ? Lo.tc_ctas : 0;
+      init_state = tensor ? kCoarse : kRunning;
+      P = sorted ? route.P : 0;
+      rows = P > 0 ? at<float>(ws, Lo.off_sorted) : Xs;
+      perm = P > 0 ? at<int32_t>(ws, Lo.off_perm) : nullptr;
+      cv = cells::View<float>{};
+      if (P > 0) {
+        cv.P = P;
+        cv.start = at<int32_t>(ws, Lo.off_start);
+        cv.ctr = at<float>(ws, Lo.off_ctr);
+        cv.rad = at<float>(ws, Lo.off_rad);
+        if (d > 8) cv.ext = at<float2>(ws, Lo.off_ext);
+      }
+      auto at_most = [&](int v) { return travel_max < v ? (int)travel_max : v; };
+      cap_seeds = by_seed ? at_most(kGridMaxSeeds)
+                          : (gp.ok ? gp.seeds : qmax * kSeedsPerCluster);
+      cap_modes = by_seed ? at_most(15 * kModesPerCluster) : qmax * kModesPerCluster;
+    };
+    auto clear_ctl = [&](cudaStream_t s_) -> cudaError_t {   // ctl, mctl, rctl, status, round
+      const cudaError_t e = cudaMemsetAsync(ctl, 0, kCtlBlockBytes, s_);
+      return e != cudaSuccess ? e : cudaMemsetAsync(hist, 0, (size_t)(kHistCap + 2) * 4, s_);
+    };
+    auto pack = [&](cudaStream_t s_) -> cudaError_t {
+      return launch_pack_points(points, n, d, DP, (float)scale, Xs, status, s_, cosine ? 1 : 0,
+                                pcopy);
+    };
+    auto sort_points = [&](const Gate& gate, cudaStream_t s_) -> cudaError_t {
+      float* to = at<float>(ws, Lo.off_sorted);
+      int32_t* start = at<int32_t>(ws, Lo.off_start);
+      float* ctr = at<float>(ws, Lo.off_ctr);
+      int32_t* npiv = at<int32_t>(ws, Lo.off_npiv);
+      const cudaError_t e = cells::launch_sort<float>(
+          Xs, 1, n, DP, true, route.P, at<void>(ws, Lo.off_sort), to, at<int32_t>(ws, Lo.off_perm),
+          start, ctr, npiv, at<float>(ws, Lo.off_rad), at<int2>(ws, Lo.off_table), s_, nullptr, 0,
+          32, nullptr, gate);
+      if (e != cudaSuccess || d <= 8) return e;
+      return cells::launch_extents(to, DP, route.P, npiv, start, ctr, at<float2>(ws, Lo.off_ext),
+                                   s_, gate);
+    };
+    // Where the points may be sorted, a probe says whether they are (the gate) and the host
+    // decides the rest.  A graph that starts sorted and by seed asks beside the packing and
+    // hands back if the answer is no; else the host reads the answer while the points are
+    // sorted (a read-back before a graph: 20 to 40 us of a call).
+    const float limit = share_limit(route, n, DP, N0);
+    int32_t* walk = at<int32_t>(ws, Lo.off_ctl + kCtlWalkOff);
+    auto probe = [&](const float* X, int ld, double scale_, int unit, float* share,
+                     cudaStream_t s_) -> cudaError_t {
+      ProbeArgs a{};
+      a.set[0] = {X, X, n, n};
+      a.sets = 1;
+      a.d = d;
+      a.ld = ld;
+      a.scale = scale_;
+      a.unit = unit;
+      a.kind = d > 8 ? kProbeExtent : kProbeBall;
+      a.limit = limit;
+      a.share = share;
+      a.walk = walk;
+      return launch_probe<float>(a, s_);
+    };
+    bool packed = false;   // the control region is clear and the points are packed
+    auto ask = [&]() -> cudaError_t {
+      const cudaEvent_t answered = route_event();
+      if (!answered) return cudaErrorUnknown;
+      float answer = 0.0f;
+      float* share = hbuf ? reinterpret_cast<float*>(hbuf + kCtlBlockBytes)
+                          : at<float>(ws, Lo.off_ctl + kCtlShareOff);
+      cudaError_t e = clear_ctl(st);
+      if (e == cudaSuccess) e = pack(st);
+      if (e == cudaSuccess) e = probe(Xs, DP, 1.0, 0, share, st);
+      if (e == cudaSuccess && !hbuf)
+        e = cudaMemcpyAsync(&answer, share, 4, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaEventRecord(answered, st);
+      if (e == cudaSuccess) e = sort_points(Gate{walk, 1, 0, 1}, st);
+      if (e == cudaSuccess) e = cudaEventSynchronize(answered);
+      if (e != cudaSuccess) return e;
+      n_launches += 2 + cells::sort_launches(n) + (d > 8 ? 1 : 0);
+      packed = true;
+      if (hbuf) answer = *reinterpret_cast<volatile float*>(share);
+      set_route(answer <= limit, answer);
+      return cudaSuccess;
+    };
+    // (as the data of a graph that asks would have it; a share that is not too large)
+    set_route(limit >= 0.0f, limit < 0.125f ? limit : 0.125);
+    const bool graph_asks = route.P > 0 && by_seed && sorted;
+    bool asked = route.P == 0;
+
     // one block per seed (many chunks) or one warp per seed: enough blocks for
     // either, at most 8 per SM
     auto update_grid = [&](int64_t m) -> int {
@@ -619,29 +794,6 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       return e;
     };
 
-    // --- the points in cells (trajectories in one launch) ---
-    const int P = route.P;
-    cells::View<float> cv{};
-    float* rows = Xs;   // the rows that the trajectories read
-    int32_t* perm = nullptr;
-    if (P > 0) {
-      rows = at<float>(ws, Lo.off_sorted);
-      perm = at<int32_t>(ws, Lo.off_perm);
-      cv.P = P;
-      cv.start = at<int32_t>(ws, Lo.off_start);
-      cv.ctr = at<float>(ws, Lo.off_ctr);
-      cv.rad = at<float>(ws, Lo.off_rad);
-      if (d > 8) cv.ext = at<float2>(ws, Lo.off_ext);
-    }
-    auto sort_points = [&](cudaStream_t s_) -> cudaError_t {
-      if (P == 0) return cudaSuccess;
-      const cudaError_t e = cells::launch_sort<float>(
-          Xs, 1, n, DP, true, P, at<void>(ws, Lo.off_sort), rows, perm,
-          at<int32_t>(ws, Lo.off_start), at<float>(ws, Lo.off_ctr), at<int32_t>(ws, Lo.off_npiv),
-          at<float>(ws, Lo.off_rad), at<int2>(ws, Lo.off_table), s_);
-      if (e != cudaSuccess || !cv.ext) return e;
-      return cells::launch_extents(rows, DP, P, at<int32_t>(ws, Lo.off_npiv), cv.start, cv.ctr, at<float2>(ws, Lo.off_ext), s_);
-    };
     auto seeds_launch = [&](const RoundCtl* rcp, int N_, int max_N, int target_,
                             cudaStream_t s_) -> cudaError_t {
       return launch_travel_seeds(rows, cv, (int)n, d, DP, y, it, conv, state, wlast, hist,
@@ -667,16 +819,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                     modes_full, &mctl->ticket, max_M, s_);
     };
 
-    // --- Seed Selection (Alg. 2): initial seed count ---
-    int32_t N0;
-    if (o.all_seeds) N0 = (int32_t)n;
-    else if (o.seed_indices) N0 = o.n_seed_indices;
-    else N0 = (int32_t)(o.n_initial < n ? o.n_initial : n);
     RoundCtl* rctl_round = at<RoundCtl>(ws, Lo.off_ctl + kCtlRoundOff);
-    const bool by_seed = route.travel == kTravelSeeds;
-    const int cap_seeds = gp.ok || by_seed ? (by_seed ? kGridMaxSeeds : gp.seeds)
-                                           : qmax * kSeedsPerCluster;
-    const int cap_modes = by_seed ? 15 * kModesPerCluster : qmax * kModesPerCluster;
     // one grid round over the RUNNING seeds of [0, N) (N and target from rcp
     // when non-null)
     auto grid_launch = [&](const RoundCtl* rcp, int N_, int target_, cudaStream_t s_) {
@@ -706,7 +849,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     // resume: 0 host path from the start, 1 host rounds from the graph's state,
     // 2 host refinement and labels, 3 the graph did everything
     int resume = 0;
-    const bool graph_ok = !graph_cache().disabled && !o.profile && !owns_ws && hbuf &&
+    const bool graph_ok = (asked || graph_asks) && !graph_cache().disabled && !o.profile && !owns_ws && hbuf &&
                           (qmax > 0 || by_seed) && !tensor &&
                           !o.all_seeds && !keep_exhausted && !o.seed_indices &&
                           !o.skip_refine && max_iter <= kHistCap && N0 <= cap_seeds;
@@ -724,6 +867,10 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       key.d = d;
       key.max_iter = max_iter;
       key.max_modes = max_modes;
+      key.travel = travel;
+      key.P = P;
+      key.cap_seeds = cap_seeds;
+      key.cap_modes = cap_modes;
       cudaGetDevice(&key.dev);
       key.h = h;
       key.tol = tol;
@@ -749,10 +896,15 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
         if (gc.used < GraphCache::kEntries) ++gc.used;
         *slot = GraphEntry();
         slot->key = key;
-        cudaStream_t cs = capture_stream(key.dev, 0), cs2 = capture_stream(key.dev, 1);
+        cudaStream_t cs = capture_stream(key.dev, 0), cs2 = capture_stream(key.dev, 1),
+                     cs3 = capture_stream(key.dev, 2);
         cudaGraph_t g = nullptr;
+        cudaEvent_t ev[2] = {nullptr, nullptr};
         bool capturing = false;
-        cudaError_t e = (cs && cs2) ? cudaGraphCreate(&g, 0) : cudaErrorNotSupported;
+        cudaError_t e = (cs && cs2 && cs3) ? cudaGraphCreate(&g, 0) : cudaErrorNotSupported;
+        for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+          e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+        const Gate gate = graph_asks ? Gate{walk, 1, 0, 0} : Gate{};
         cudaGraphConditionalHandle h_loop = 0, h_post = 0;
         if (e == cudaSuccess)
           e = cudaGraphConditionalHandleCreate(&h_loop, g, 1, cudaGraphCondAssignDefault);
@@ -763,17 +915,27 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
                                             cudaStreamCaptureModeThreadLocal);
         capturing = e == cudaSuccess;
         // before the rounds
-        if (e == cudaSuccess) e = cudaMemsetAsync(ctl, 0, kCtlBlockBytes, cs);
-        if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, (size_t)(kHistCap + 2) * 4, cs);
-        if (e == cudaSuccess)
-          e = launch_pack_points(points, n, d, DP, (float)scale, Xs, status, cs, cosine ? 1 : 0,
-                                 pcopy);
-        if (e == cudaSuccess) e = sort_points(cs);
+        if (e == cudaSuccess) e = clear_ctl(cs);
+        if (e == cudaSuccess && graph_asks) {
+          e = cudaEventRecord(ev[0], cs);
+          if (e == cudaSuccess) e = cudaStreamWaitEvent(cs3, ev[0], 0);
+          if (e == cudaSuccess)
+            e = probe(points, d, scale, cosine ? 1 : 0, at<float>(ws, Lo.off_ctl + kCtlShareOff),
+                      cs3);
+          if (e == cudaSuccess) e = cudaEventRecord(ev[1], cs3);
+        }
+        if (e == cudaSuccess) e = pack(cs);
+        if (e == cudaSuccess && graph_asks) {
+          e = cudaStreamWaitEvent(cs, ev[1], 0);
+          if (e == cudaSuccess) e = sort_points(gate, cs);
+        }
         if (e == cudaSuccess)
           e = launch_seed_init(Xs, n, DP, o.rng_seed, nullptr, 0, 0, N0, seed_idx, y, it, conv,
                                state, status, cs, init_state);
-        if (e == cudaSuccess) e = launch_round_begin(rctl_round, N0, o.gamma, cs);
-        slot->kernels_pre = 3 + (P > 0 ? cells::sort_launches(n) : 0) + (cv.ext ? 1 : 0);
+        if (e == cudaSuccess)
+          e = launch_round_begin(rctl_round, N0, o.gamma, gate, h_loop, cs);
+        slot->kernels_pre =
+            3 + (graph_asks ? 1 + cells::sort_launches(n) + (d > 8 ? 1 : 0) : 0);
         // the rounds
         cudaGraph_t body = nullptr;
         if (e == cudaSuccess) e = add_conditional(cs, h_loop, cudaGraphCondTypeWhile, &body);
@@ -846,6 +1008,8 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&slot->exec, g, 0);
         if (g) cudaGraphDestroy(g);
+        for (cudaEvent_t v : ev)
+          if (v) cudaEventDestroy(v);
         if (e != cudaSuccess) {
           if (slot->exec) cudaGraphExecDestroy(slot->exec);
           slot->exec = nullptr;
@@ -864,20 +1028,25 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
         rounds = rcv.rounds;
         N = rcv.N;
         K_last = rcv.K_last;
-        n_launches = ge->kernels_pre + ge->kernels_round * rcv.rounds +
-                     (rcv.leave == 0 ? ge->kernels_post : 0);
+        n_launches += ge->kernels_pre + ge->kernels_round * rcv.rounds +
+                      (rcv.leave == 0 ? ge->kernels_post : 0);
         if (hstatus & (kStNonFinite | kStBadArg)) goto device_error;
         if (hstatus & kStTimeout) {
           rc = FMS_ERR_TIMEOUT;
           goto done;
         }
-        resume = rcv.leave == 0 ? 3 : (rcv.leave == 1 ? 1 : 2);
+        if (graph_asks) {
+          float share;
+          memcpy(&share, hbuf + kCtlShareOff, 4);
+          asked = true;
+          set_route(share <= limit, share);
+        }
+        if (rcv.leave < 3) resume = rcv.leave == 0 ? 3 : (rcv.leave == 1 ? 1 : 2);
+        else packed = true;   // (and nothing else)
       }
     }
-    if (resume == 0) {
-      FMS_CUDA(cudaMemsetAsync(ctl, 0, kCtlBlockBytes, st));   // ctl, mctl, rctl, status, round
-      FMS_CUDA(cudaMemsetAsync(hist, 0, (size_t)(kHistCap + 2) * 4, st));
-    }
+    if (!asked) FMS_CUDA(ask());
+    if (resume == 0 && !packed) FMS_CUDA(clear_ctl(st));
     if (o.profile)
       for (int i = 0; i < 5; ++i)
         if (cudaEventCreate(&phase_ev[i]) != cudaSuccess) {
@@ -896,16 +1065,11 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     };
     if (resume == 0) {
       mark(0);
-      FMS_LAUNCH(launch_pack_points(points, n, d, DP, (float)scale, Xs, status, st,
-                                    cosine ? 1 : 0, pcopy));
+      if (!packed) FMS_LAUNCH(pack(st));
       if (tensor) FMS_LAUNCH(launch_tc_pack(Xs, n, d, DP, img, st));
-      if (P > 0) {
-        n_launches += cells::sort_launches(n) - (cv.ext ? 0 : 1);   // (and the one counted below)
-        FMS_LAUNCH(sort_points(st));
-      }
       N = N0;
       // (travel_groups starts from the points themselves)
-      if (route.travel != kTravelGroups)
+      if (travel != kTravelGroups)
         FMS_LAUNCH(launch_seed_init(Xs, n, DP, o.rng_seed, o.seed_indices, 0, 0, N, seed_idx, y,
                                     it, conv, state, status, st, init_state));
     }
@@ -916,14 +1080,14 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       if (target < 1) target = 1;
       if (target > N) target = N;
       // --- mean-shift iterations under Early Stopping (Sec. II-C) ---
-      const bool use_travel = route.travel != kTravelSteps;
+      const bool use_travel = travel != kTravelSteps && !(by_seed && N > travel_max);
       const bool use_grid = !use_travel && gp.ok && N <= gp.seeds;
       const bool use_clusters =
           use_grid || use_travel ||
           (qmax > 0 && N <= qmax * kSeedsPerCluster && max_iter <= kHistCap);
       // with gamma = 1 kept seeds need not have converged: their densities come from a
       // pass at their last positions (travel_groups makes that pass itself)
-      const bool score_pass = keep_exhausted && route.travel != kTravelGroups;
+      const bool score_pass = keep_exhausted && travel != kTravelGroups;
       if (use_clusters) {
         // persistent round (grid of one CTA per SM, or thread-block clusters
         // when the grid plan does not fit): no host round trips
@@ -936,7 +1100,7 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
           round_evs.push_back(ra);
           round_evs.push_back(rb);
         }
-        if (by_seed) {
+        if (use_travel && by_seed) {
           FMS_LAUNCH(seeds_launch(nullptr, N, N, target, st));
         } else if (use_travel) {
           const cells::Groups gr{P > 0 ? at<int2>(ws, Lo.off_table) : nullptr,
@@ -1016,6 +1180,13 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
       K_last = hm.K;
       if (hm.next_N > N) {
         mark(0);
+        if (by_seed && hm.next_N > travel_max && route.tensor && !tensor) {
+          // so many seeds are taken by steps from here on, the new ones' coarse first
+          FMS_LAUNCH(launch_tc_pack(Xs, n, d, DP, img, st));
+          tensor = true;
+          tl_iter.tc_ctas = Lo.tc_ctas;
+          init_state = kCoarse;
+        }
         FMS_LAUNCH(launch_seed_init(Xs, n, DP, o.rng_seed, nullptr, N, N, hm.next_N - N, seed_idx,
                                   y, it, conv, state, status, st, init_state));
         N = hm.next_N;
@@ -1028,8 +1199,9 @@ static fms_status cluster_impl(const float* points, int64_t n, int32_t d, float 
     if (resume <= 2) {
     mark(2);
     // --- refinement and second prune ---
-    if (!o.skip_refine && hm.M > 0 && (by_seed || (route.travel == kTravelGroups && P > 0 &&
-                                                   hm.M > grid_refine_capacity()))) {
+    if (!o.skip_refine && hm.M > 0 &&
+        ((by_seed && hm.M <= travel_max) ||
+         (travel == kTravelGroups && P > 0 && hm.M > grid_refine_capacity()))) {
       // a block per mode, all updates in one launch
       FMS_LAUNCH(refine_launch(hm.M, rtol_s * rtol_s, st));
       FMS_LAUNCH(launch_greedy_merge_d(&mctl->M, mscore, ym, DP, d, r2_s, alive, acc2, &mctl->Mr,
@@ -1415,6 +1587,7 @@ cudaError_t probe_step(const float* Xp, int64_t n, const float* Yp, int64_t m, i
   a.ld = DP;
   a.scale = 1.0;
   a.kind = kind;
+  a.limit = kWalkShare;
   a.share = at<float>(status, kStepShareOff);
   a.walk = at<int32_t>(status, kStepWalkOff);
   *walk = a.walk;
@@ -1495,7 +1668,7 @@ cudaError_t group_step(const float* points, int64_t n, int32_t d, float scale, c
   if (e == cudaSuccess) e = launch_pack_points(seeds, m, d, L.DP, scale, Yp, status, st);
   if (e == cudaSuccess)
     e = probe_step(Xp, n, Yp, m, d, L.DP, d > 8 ? kProbeExtent : kProbeBall, status, st, &walk);
-  const Gate cells_gate{walk, 1, 0}, dense_gate{walk, 1, 1};
+  const Gate cells_gate{walk, 1, 0, 1}, dense_gate{walk, 1, 1, 0};
   // over every pair
   IterCtl* ctl = at<IterCtl>(wd, D.off_ctl);
   int32_t* active = at<int32_t>(wd, D.off_active);
@@ -1711,7 +1884,7 @@ cudaError_t coarse_cells(const CoarseLayout& L, void* ws, int64_t n, int d, int6
   cv.ctr = ctr;
   cv.rad = at<float>(ws, L.off_rad);
   cudaError_t e = probe_step(Xs, n, Ys, m, d, L.DP, kProbeTile, status, st, &walk);
-  const Gate gate{walk, 1, 0};
+  const Gate gate{walk, 1, 0, 1};
   if (e == cudaSuccess)
     e = cells::launch_sort<float>(Xs, 1, n, L.DP, true, L.P, scratch, Xc,
                                   at<int32_t>(ws, L.off_xperm), at<int32_t>(ws, L.off_start), ctr,

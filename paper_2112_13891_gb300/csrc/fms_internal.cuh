@@ -61,7 +61,7 @@ struct RoundCtl {
   int32_t N;        // seeds in play
   int32_t target;   // ceil(gamma * N), clamped to [1, N]
   int32_t rounds;   // rounds completed
-  int32_t leave;    // != 0: the host continues (1: next round, 2: refinement)
+  int32_t leave;    // != 0: the host continues (1: next round, 2: refinement, 3: another route)
   int32_t K_last;   // prune candidates of the last round
   int32_t pad[3];
 };
@@ -145,6 +145,7 @@ struct Gate {
   const int32_t* walk;
   int sets;
   int closed_if;   // the answer to which the gate is closed
+  int chain;       // 1: launched while the kernel before still runs (launch_gated)
   __device__ __forceinline__ bool open() const {
     if (!walk) return true;
     int w = 1;
@@ -349,7 +350,8 @@ cudaError_t launch_seed_init(const float* Xs, int64_t n, int DP, uint64_t rng_se
                              int32_t init_state = kRunning);
 cudaError_t launch_select_seeds(int64_t n, uint64_t rng_seed, int64_t start, int64_t count,
                                 int32_t* out, cudaStream_t st);
-cudaError_t launch_round_begin(RoundCtl* rc, int32_t N, float gamma, cudaStream_t st);
+cudaError_t launch_round_begin(RoundCtl* rc, int32_t N, float gamma, Gate gate,
+                               cudaGraphConditionalHandle h_loop, cudaStream_t st);
 cudaError_t launch_round_advance(RoundCtl* rc, MergeCtl* mctl, int64_t n, float L, int allow,
                                  float gamma, int cap_seeds, int cap_modes, uint64_t rng_seed,
                                  const float* Xs, int DP, int32_t* seed_idx, float* y,

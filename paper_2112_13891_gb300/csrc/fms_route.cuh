@@ -20,11 +20,11 @@ constexpr float kWalkShare = 0.35f;
 
 constexpr int kProbeSets = 4;      // sets of a call that are sampled
 constexpr int kProbePoints = 128;  // points and seeds of a sample
-constexpr int kProbeSeeds = 32;
+constexpr int kProbeSeeds = 16;
 
-// Gated kernels follow each other in a chain of small launches.  They are launched while the
-// one before still runs and wait for its end (and all that ended before it) themselves,
-// which takes 1 us off each launch, empty or not.
+// Gated kernels follow each other in a chain of small launches.  On a stream they are
+// launched while the one before still runs and wait for its end (and all that ended before
+// it) themselves, which takes 1 us off each launch, empty or not.
 __device__ __forceinline__ void wait_for_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -40,7 +40,7 @@ inline cudaError_t launch_gated(const Gate& gate, void (*kernel)(P...), dim3 gri
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = gate.walk ? 1 : 0;
+  cfg.numAttrs = gate.chain ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
@@ -55,8 +55,9 @@ struct ProbeArgs {
   double scale;
   int unit;          // 1: directions of the rows (cosine metric)
   int kind;
+  float limit;       // share up to which *walk is 1
   float* share;      // [sets], device or mapped host memory
-  int32_t* walk;     // [sets] or null: 1 where the share is at most kWalkShare
+  int32_t* walk;     // [sets] or null
 };
 template <typename T>
 cudaError_t launch_probe(const ProbeArgs& a, cudaStream_t st);

@@ -171,6 +171,7 @@ cudaError_t probe_sets(const E* points, const E* seeds0, const UGeom& g, double 
   a.d = a.ld = g.d;
   a.scale = sqrt(c);
   a.kind = kProbeBall;
+  a.limit = kWalkShare;
   a.share = at<float>(ckpt, CL.share);
   a.walk = at<int32_t>(ckpt, CL.walk);
   return launch_probe<E>(a, st);
@@ -226,7 +227,7 @@ fms_status forward_impl(const E* points, const E* seeds0, int32_t B, int64_t n, 
   if (P > 0) {
     if (probe_sets<E>(points, seeds0, g, (double)c, ckpt, CL, st) != cudaSuccess)
       return FMS_ERR_CUDA;
-    cv.gate = Gate{at<int32_t>(ckpt, CL.walk), probed_sets(B), 0};
+    cv.gate = Gate{at<int32_t>(ckpt, CL.walk), probed_sets(B), 0, 0};
     const E* src = seeds0;
     if (d != g.DP || (reinterpret_cast<uintptr_t>(seeds0) & 15u)) {
       E* Yp = at<E>(ws, L.Yp);
@@ -289,7 +290,7 @@ fms_status backward_impl(const E* points, int32_t B, int64_t n, int64_t m, int32
   if (sort_points<E>(points, g, P, L.s, ws, &cv, st) != cudaSuccess ||
       unroll_pack_rows<E>(grad_out, rowsY, (int)m, d, g.DP, yperm, G, st) != cudaSuccess)
     return FMS_ERR_CUDA;
-  if (P > 0) cv.gate = Gate{at<int32_t>(ck, CL.walk), probed_sets(B), 0};
+  if (P > 0) cv.gate = Gate{at<int32_t>(ck, CL.walk), probed_sets(B), 0, 0};
   int first = 1;
   for (int s = n_ckpt(T, k) - 1; s >= 0; --s) {
     const int t0 = s * k;

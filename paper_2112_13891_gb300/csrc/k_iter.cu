@@ -195,16 +195,21 @@ __global__ void seed_init_kernel(const float* __restrict__ Xs, int64_t n, int DP
 // labels), and leaves the rest to the host (leave != 0) when the next round
 // or the refinement would not fit the cluster kernels.
 // ---------------------------------------------------------------------------
-__global__ void round_begin_kernel(RoundCtl* rc, int32_t N, float gamma) {
+// (gate closed: no rounds, the host takes another route)
+__global__ void round_begin_kernel(RoundCtl* rc, int32_t N, float gamma, Gate gate,
+                                   cudaGraphConditionalHandle h_loop) {
+  const bool open = gate.open();
   rc->N = N;
   rc->target = stop_target(gamma, N);
   rc->rounds = 0;
-  rc->leave = 0;
+  rc->leave = open ? 0 : 3;
   rc->K_last = 0;
+  if (!open) cudaGraphSetConditional(h_loop, 0u);
 }
 
-cudaError_t launch_round_begin(RoundCtl* rc, int32_t N, float gamma, cudaStream_t st) {
-  round_begin_kernel<<<1, 1, 0, st>>>(rc, N, gamma);
+cudaError_t launch_round_begin(RoundCtl* rc, int32_t N, float gamma, Gate gate,
+                               cudaGraphConditionalHandle h_loop, cudaStream_t st) {
+  round_begin_kernel<<<1, 1, 0, st>>>(rc, N, gamma, gate, h_loop);
   return cudaGetLastError();
 }
 

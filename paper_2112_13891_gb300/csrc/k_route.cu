@@ -16,7 +16,7 @@
 namespace fms {
 namespace {
 
-constexpr int kNear = 32;                           // points whose nearest other one is found
+constexpr int kNear = 16;                           // points whose nearest other one is found
 constexpr int kLoaded = kProbePoints + kProbeSeeds;
 constexpr int kRows = kNear + kProbeSeeds;          // compared with all points
 constexpr int kSplit = 1024 / kProbePoints;         // threads of a point
@@ -104,15 +104,15 @@ __global__ void __launch_bounds__(1024) probe_kernel(ProbeArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x < kNear) {   // (one warp) the median of the distances to the nearest point
-    float v = red[lane][0];
-    for (int u = 1; u < kWarps; ++u) v = fminf(v, red[lane][u]);
+  if (threadIdx.x < 32) {   // the median of the distances to the nearest point
+    float v = red[lane % kNear][0];
+    for (int u = 1; u < kWarps; ++u) v = fminf(v, red[lane % kNear][u]);
     int below = 0;
     for (int u = 0; u < kNear; ++u) {
       const float o = __shfl_sync(kFull, v, u);
       below += o < v || (o == v && u < lane) ? 1 : 0;
     }
-    if (below == kNear / 2) median = v;
+    if (lane < kNear && below == kNear / 2) median = v;
   }
   __syncthreads();
   const float M = sqrtf(median), log2n = log2f((float)s.n);
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(1024) probe_kernel(ProbeArgs a) {
   if (threadIdx.x == 0) {
     const float share = (float)vis / (kProbePoints * kProbeSeeds);
     a.share[blockIdx.x] = share;
-    if (a.walk) a.walk[blockIdx.x] = share <= kWalkShare ? 1 : 0;
+    if (a.walk) a.walk[blockIdx.x] = share <= a.limit ? 1 : 0;
   }
 }
 

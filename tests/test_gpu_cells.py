@@ -1,7 +1,7 @@
 """Sorted cells and whole trajectories in one launch, at the sizes where their
 rules begin: one update by groups (n m times the padded width >= 2.5e9), a block
-per seed (d > 7; points sorted from n = 8,192 on) and every point a seed by groups
-(d <= 7; sorted from n = 4,096 on), against the FP64 oracle.
+per seed (d > 7; points sorted from n = 16,384 on) and every point a seed by groups
+(d <= 7; sorted from n = 8,192 on), against the FP64 oracle.
 
 Tolerances: one update as in test_gpu_step_parity (FP32 weights, sums of n terms);
 clusterings by the cluster parity bar (modes within 1e-3 h, identical labels away
@@ -77,9 +77,11 @@ def _cluster(w, **kw):
 
 @pytest.mark.parametrize("d,per,sigma,kw", [
     (8, 1366, 1.0, {}), (9, 1366, 1.0, {}), (16, 1366, 1.0, {}), (16, 1365, 1.0, {}),
-    (33, 1400, 0.5, {}), (64, 1366, 0.4, {}), (16, 1400, 0.6, dict(kernel="flat"))])
+    (33, 1400, 0.5, {}), (64, 1366, 0.4, {}), (16, 1400, 0.6, dict(kernel="flat")),
+    (8, 2731, 1.0, {}), (9, 2730, 1.0, {}), (16, 2731, 1.0, {}), (33, 2740, 0.5, {}), (64, 2731, 0.4, {}),
+    (16, 2750, 0.6, dict(kernel="flat"))])
 def test_block_per_seed(d, per, sigma, kw):
-    # 6 blobs: 8,196 points sorted, 8,190 not
+    # 6 blobs: 16,386 points sorted, 16,380 not
     w = fi.separated_blobs(seed=d + per, k=6, d=d, per=per, sigma=sigma,
                            h=2.0 if not kw else 8.0)
     res, ref = _cluster(w, rng_seed=2, **kw)
@@ -87,13 +89,16 @@ def test_block_per_seed(d, per, sigma, kw):
 
 
 def test_block_per_seed_cosine():
-    _cluster(fi.directional_blobs(seed=3, k=12, d=16, per=700, spread=0.05, h=0.15),
-             metric="cosine", rng_seed=1)
+    for per in (700, 1400):
+        _cluster(fi.directional_blobs(seed=3, k=12, d=16, per=per, spread=0.05, h=0.15),
+                 metric="cosine", rng_seed=1)
 
 
 @pytest.mark.parametrize("d,n,kw", [(3, 4096, {}), (3, 4095, {}), (1, 4500, {}), (7, 4321, {}),
                                     (2, 63, {}), (3, 4100, dict(kernel="flat")),
-                                    (3, 4100, dict(metric="cosine"))])
+                                    (3, 4100, dict(metric="cosine")), (3, 8192, {}), (3, 8191, {}),
+                                    (1, 8500, {}), (7, 8321, {}), (3, 8200, dict(kernel="flat")),
+                                    (3, 8300, dict(metric="cosine"))])
 def test_every_point_a_seed(d, n, kw):
     if kw.get("metric") == "cosine":
         w = fi.directional_blobs(seed=5, k=5, d=d, per=n // 5, spread=0.05, h=0.15)
@@ -275,3 +280,26 @@ def test_step_where_cells_may_leave_nothing_out(n, m, d, k, box, coarse):
         assert np.abs(W[pick] / refW - 1).max() <= 1e-4
         assert np.abs(out[pick] - ref).max() <= 2e-4 * h + 2.0 ** -20 * np.abs(ref).max()
     assert W[5] == 0.0 and np.isnan(out[5]).all()
+
+
+# Clusters on the axes, 6.4 h apart: each reaches the others' rows, so nothing is sorted,
+# and all rows in one launch (few pairs) or the steps (many) take the updates; a limit L that
+# doubles the seeds across that line.  Every point a seed: all rows up to 10,240, then steps.
+@pytest.mark.parametrize("d,n,k,kw", [
+    (16, 20_000, 12, {}), (16, 20_000, 12, dict(n_initial=4096)), (48, 17_000, 14, dict(n_initial=512)),
+    (32, 40_000, 16, {}), (9, 20_000, 7, dict(n_initial=2048)),
+    (16, 20_000, 12, dict(L=128.0)), (40, 18_000, 9, dict(L=200.0)), (16, 17_000, 8, dict(gamma=1.0)),
+    (16, 20_000, 12, dict(metric="cosine", L=64.0)), (16, 17_000, 5, dict(kernel="flat", n_initial=3000)),
+    (7, 9_000, 6, dict(all_seeds=True)), (5, 12_000, 5, dict(all_seeds=True))])
+def test_clusters_in_reach_of_each_other(d, n, k, kw):
+    h = 1.0 if kw.get("metric") != "cosine" else 0.25
+    if kw.get("kernel") == "flat":
+        h = 3.0
+    rng = np.random.default_rng(d + n)
+    c = np.eye(d)[:k] * (4.5 if h >= 1.0 else 1.0)
+    X = (c[rng.integers(0, k, n)] + (0.4 if h >= 1.0 else 0.03) * rng.standard_normal((n, d)))
+    w = dict(X=X.astype(np.float32), h=h, tol=1e-3 * h, max_iter=300)
+    res, ref = _cluster(type("W", (), w), rng_seed=2, **kw)
+    assert len(ref.modes) == k
+    if not kw.get("all_seeds"):
+        assert res.stats["n_seeds_final"] == ref.n_seeds and res.stats["t_star_last"] == ref.t_star[-1]
