@@ -291,8 +291,9 @@ fms_status fms_cluster_host(const float* points, int64_t n, int32_t d, float h, 
  * largest set, d, h, tol, max_iter, max_modes, options) and reused by later
  * calls with the same values; the per-set sizes are copied in before every
  * launch.  Sets of d > 7, or of 2,048 points and more on average, have their
- * seeds carried to convergence one a block; for the others, whose updates are
- * one launch each, the step kernel's tiling is chosen by a built-in autotuner the
+ * seeds carried to convergence one a block where a sample of the points says
+ * that each sees little of its set; for the others, whose updates are one
+ * launch each, the step kernel's tiling is chosen by a built-in autotuner the
  * first time a shape (d, size class of the total, size class of B) is seen
  * on a device: it times one update with each candidate tiling (synchronising
  * on each) and keeps the fastest.

@@ -6,6 +6,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -27,7 +28,7 @@ cudaError_t launch_batched_step(const float* Xs, int d, int DP, const float* y,
                                 const int32_t* list, const SetCtl* sc, int B, int kind,
                                 const int64_t* task_off, const int64_t* part_off,
                                 const int64_t* totals, float* part, int target_warps,
-                                cudaStream_t st);
+                                uint32_t* status, cudaStream_t st);
 cudaError_t launch_queue_seeds(SetCtl* sc, int B, const int32_t* state, int32_t* list,
                                int64_t* list_off, int64_t* totals, int32_t* counters,
                                const uint32_t* status, cudaStream_t st);
@@ -112,14 +113,22 @@ struct BLayout {
       mscore, dens, ties, modes_full, part, sc, task_off, part_off, list_off, totals, counters, pt_off, status,
       sorted, start, ctr, npiv, rad, sort, wlast, total;
   int DP, DA, R, TW, P;
-  bool queued;
+  bool queued, steps;   // the routes that the call has the scratch for
   Tiling tl;
 };
 
-// Every seed is taken to convergence by one block (k_travel.cu).  For d <= 7 and
-// sets too small to gain from their cells, a low-d warp task shares each point it
-// loads among up to 8 seeds and an update of all sets is one launch.
-bool by_queue(int d, int64_t total, int B) { return d > 7 || total / B >= 2048; }
+// Whether every seed may be taken to convergence by one block (k_travel.cu), for the cells
+// it sees.  For d <= 7 and sets too small to gain from their cells, a low-d warp task
+// shares each point it loads among up to 8 seeds and an update of all sets is one launch.
+bool may_queue(int d, int64_t total, int B) { return d > 7 || total / B >= 2048; }
+
+// Partial sums of the steps up to which a call can take them instead (4 times 32 warps of
+// every set have one: 1,000 sets of d = 16 need 0.7 GB).
+constexpr size_t kMaxPartBytes = (size_t)1 << 30;
+
+// For d <= 7 the queue pays from this many seeds on (20 blobs of 400,000 x 3 in one set, 128
+// seeds, 4.5 ms, the steps 1.4; in two 2.9 and 1.8; in eight 1.5 and 1.9).
+constexpr int64_t kQueueSeedsLow = 1024;
 
 // Cells of every set (0: sets too small to gain from them): as for one set of the
 // mean size, half as many at most (4 to 40 clusters a set; the cost of finding the
@@ -130,15 +139,15 @@ int batch_cells(int64_t total, int B) {
   return P < 128 ? P : 128;
 }
 
-// Partial-sum capacity (not queued): per set C_b * cnt_b * DA with C_b from choose_chunks
+// Partial-sum capacity (the steps): per set C_b * cnt_b * DA with C_b from choose_chunks
 // (<= 4 * tl.target_warps / G_b + 1), so sum_b <= (4 * TWb * B + total_groups) * R * DA.
 BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw_mult,
                      int min_chunk) {
   BLayout L{};
   L.DP = padded(d);
   L.DA = step_accumulators(d);
-  L.R = step_seeds_per_warp(d);
-  L.queued = by_queue(d, total, B);
+  L.R = batched_seeds_per_warp(d);
+  L.queued = may_queue(d, total, B);
   L.P = L.queued ? batch_cells(total, B) : 0;
   L.TW = (sms > 0 ? sms : 1) * step_resident_warps_per_sm(d);
   // every set gets a share of the GPU's warps for its chunking (all sets run
@@ -178,7 +187,8 @@ BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw
   L.dens = take((size_t)total * 8);
   L.ties = take(batched_order_scratch(B, d));
   L.modes_full = take((size_t)total * d * 4);
-  L.part = take(L.queued ? 0 : part_floats * 4);
+  L.steps = !L.queued || part_floats * 4 <= kMaxPartBytes;
+  L.part = take(L.steps ? part_floats * 4 : 0);
   L.sc = take((size_t)B * sizeof(SetCtl));
   L.task_off = take((size_t)(B + 1) * 8);
   L.part_off = take((size_t)(B + 1) * 8);
@@ -198,6 +208,13 @@ BLayout make_blayout(int64_t total, int64_t max_n, int B, int d, int sms, int tw
   }
   L.total = o;
   return L;
+}
+
+// Page-locked memory that the probe answers in (one per host thread, kept).
+float* pinned_shares() {
+  thread_local float* buf = nullptr;
+  if (!buf && cudaMallocHost(&buf, kProbeSets * sizeof(float)) != cudaSuccess) buf = nullptr;
+  return buf;
 }
 
 int64_t largest_set(const int64_t* offsets, int32_t B) {
@@ -239,7 +256,7 @@ struct BGraphKey {
   const void* margins;
   const void* ws;
   int64_t total;
-  int32_t B, d, max_iter, max_modes, max_n, dev, tw_mult, min_chunk;
+  int32_t B, d, max_iter, max_modes, max_n, dev, tw_mult, min_chunk, queued;
   float h, tol;
   unsigned char opts[sizeof(fms_options)];
 };
@@ -357,20 +374,10 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
   const int sms = sms_now();
   if (sms <= 0) return FMS_ERR_CUDA;
 
-  // tuned tiling for this shape (or the first candidate until tuned)
   int dev = 0;
   cudaGetDevice(&dev);
-  const auto key = std::make_tuple(dev, (int)d, ilog2(total), ilog2(B));
-  bool tuned = by_queue(d, total, B);   // (the queue has no tiling)
+  // (the first candidate tiling until this shape is tuned)
   std::pair<int, int> cfg{kTwMults[0], d <= 7 ? kMinChunksLow[1] : kMinChunksWide[1]};
-  if (!tuned) {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto itc = g_tuned.find(key);
-    if (itc != g_tuned.end()) {
-      cfg = itc->second;
-      tuned = true;
-    }
-  }
   const int max_n = (int)largest_set(offsets, B);
   BLayout Lo = make_blayout(total, max_n, B, d, sms, cfg.first, cfg.second);
   const size_t need = Lo.total;  // identical for every candidate tiling
@@ -422,16 +429,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
     int32_t* counters = at<int32_t>(ws, Lo.counters);
     int64_t* pt_off = at<int64_t>(ws, Lo.pt_off);
     uint32_t* status = at<uint32_t>(ws, Lo.status);
-    const bool queued = Lo.queued;
     float* wlast = at<float>(ws, Lo.wlast);
-    float* rows = Lo.P > 0 ? at<float>(ws, Lo.sorted) : Xs;
-    cells::View<float> cv{};
-    if (Lo.P > 0) {
-      cv.P = Lo.P;
-      cv.start = at<int32_t>(ws, Lo.start);
-      cv.ctr = at<float>(ws, Lo.ctr);
-      cv.rad = at<float>(ws, Lo.rad);
-    }
     auto queue = [&](const int32_t* l) {
       return SeedQueue{l, list_off, totals, reinterpret_cast<unsigned long long*>(totals + 1), sc,
                        B};
@@ -444,6 +442,26 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
     const int grid_upd = sms * 8;
     const BatchCond no_cond{0, 0};
 
+    // the route: by a sample of the sets that hold points (2 i + 1) total / 8
+    const bool ask = Lo.queued && Lo.steps;
+    ProbeArgs pa{};
+    if (ask) {
+      pa.sets = B < kProbeSets ? B : kProbeSets;
+      for (int i = 0; i < pa.sets; ++i) {
+        const int64_t j = (2 * i + 1) * total / (2 * pa.sets);
+        const int b = (int)(std::upper_bound(offsets, offsets + B + 1, j) - offsets) - 1;
+        const float* X = points + offsets[b] * d;
+        pa.set[i] = {X, X, offsets[b + 1] - offsets[b], offsets[b + 1] - offsets[b]};
+      }
+      pa.d = pa.ld = d;
+      pa.scale = scale;
+      pa.kind = kProbeBall;
+      pa.limit = kWalkShare;
+      pa.share = pinned_shares();
+      if (!pa.share) pa.share = at<float>(ws, Lo.totals);
+      BC(launch_probe<float>(pa, st));
+    }
+    int64_t seeds0 = 0;
     for (int b = 0; b < B; ++b) {
       SetCtl& c = hsc[b];
       memset(&c, 0, sizeof(c));
@@ -451,13 +469,45 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       c.p0 = (int32_t)offsets[b];
       c.N = o.all_seeds ? c.n : (o.n_initial < c.n ? o.n_initial : c.n);
       c.prevN = 0;
+      seeds0 += c.N;
       const int t = (int)ceil((double)o.gamma * (double)c.N);
       c.target = t < 1 ? 1 : (t > c.N ? c.N : t);
     }
     BC(cudaMemcpyAsync(sc, hsc.data(), (size_t)B * sizeof(SetCtl), cudaMemcpyHostToDevice, st));
     BC(cudaMemcpyAsync(pt_off, offsets, (size_t)(B + 1) * 8, cudaMemcpyHostToDevice, st));
 
+    bool queued = Lo.queued;
+    if (ask) {
+      float share[kProbeSets] = {}, mean = 0.0f;
+      if (pa.share != pinned_shares())
+        BC(cudaMemcpyAsync(share, pa.share, pa.sets * 4, cudaMemcpyDeviceToHost, st));
+      BC(cudaStreamSynchronize(st));
+      if (pa.share == pinned_shares()) memcpy(share, pa.share, pa.sets * 4);
+      for (int i = 0; i < pa.sets; ++i) mean += share[i] / pa.sets;
+      queued = mean <= kWalkShare && (d > 7 || seeds0 >= kQueueSeedsLow);
+    }
+    const int P = queued ? Lo.P : 0;
+    float* rows = P > 0 ? at<float>(ws, Lo.sorted) : Xs;
+    cells::View<float> cv{};
+    if (P > 0) {
+      cv.P = P;
+      cv.start = at<int32_t>(ws, Lo.start);
+      cv.ctr = at<float>(ws, Lo.ctr);
+      cv.rad = at<float>(ws, Lo.rad);
+    }
+
     // --- autotune the step tiling once per shape: time one update per candidate ---
+    const auto key = std::make_tuple(dev, (int)d, ilog2(total), ilog2(B));
+    bool tuned = queued;   // (the queue has no tiling)
+    if (!tuned) {
+      std::lock_guard<std::mutex> lk(g_tune_mu);
+      auto itc = g_tuned.find(key);
+      if (itc != g_tuned.end()) {
+        cfg = itc->second;
+        tuned = true;
+        Lo = make_blayout(total, max_n, B, d, sms, cfg.first, cfg.second);
+      }
+    }
     if (!tuned) {
       BC(cudaMemsetAsync(counters, 0, 64, st));
       BC(cudaMemsetAsync(status, 0, 64, st));
@@ -478,7 +528,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
                                     status, st));
           BC(cudaEventRecord(e0, st));
           BC(launch_batched_step(Xs, d, DP, y, active, sc, B, kPlanActive, task_off, part_off,
-                                 totals, part, Lc.TW, st));
+                                 totals, part, Lc.TW, status, st));
           BC(cudaEventRecord(e1, st));
           BC(cudaEventSynchronize(e1));
           float ms = 0.f;
@@ -517,6 +567,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
     gk.dev = dev;
     gk.tw_mult = cfg.first;
     gk.min_chunk = cfg.second;
+    gk.queued = queued ? 1 : 0;
     gk.h = h;
     gk.tol = tol;
     memcpy(gk.opts, &o, sizeof(fms_options));
@@ -533,7 +584,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       bool capturing = false;
       if (e == cudaSuccess)
         e = cudaGraphConditionalHandleCreate(&h_round, g, 1, cudaGraphCondAssignDefault);
-      if (e == cudaSuccess && !queued)
+      if (e == cudaSuccess && !queued && !o.skip_refine)   // (a handle without a node is an error)
         e = cudaGraphConditionalHandleCreate(&h_ref, g, 0, cudaGraphCondAssignDefault);
       if (e == cudaSuccess)
         e = cudaStreamBeginCaptureToGraph(cs0, g, nullptr, nullptr, 0,
@@ -581,7 +632,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         if (e2 == cudaSuccess) e2 = begin_while(cs1, h_upd, cs2, &upd_body);
         if (e2 == cudaSuccess) {
           cudaError_t e3 = launch_batched_step(Xs, d, DP, y, active, sc, B, kPlanActive, task_off,
-                                               part_off, totals, part, Lo.TW, cs2);
+                                               part_off, totals, part, Lo.TW, status, cs2);
           if (e3 == cudaSuccess)
             e3 = launch_batched_update(part, active, sc, B, list_off, part_off, totals, y, it,
                                        conv, state, d, DP, DA, tol2_s, max_iter, grid_upd, cs2);
@@ -597,7 +648,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
                                    task_off, part_off, list_off, totals, counters, cs1);
         if (e2 == cudaSuccess)
           e2 = launch_batched_step(Xs, d, DP, y, kept, sc, B, kPlanKept, task_off, part_off,
-                                   totals, part, Lo.TW, cs1);
+                                   totals, part, Lo.TW, status, cs1);
         if (e2 == cudaSuccess)
           e2 = launch_batched_score(part, sc, B, list_off, part_off, totals, DA, score, grid_upd,
                                     cs1);
@@ -634,7 +685,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
         if (e == cudaSuccess) e = begin_while(cs0, h_ref, cs1, &ref_body);
         if (e == cudaSuccess) {
           cudaError_t e2 = launch_batched_step(Xs, d, DP, yf, ract, sc, B, kPlanModes, task_off,
-                                               part_off, totals, part, Lo.TW, cs1);
+                                               part_off, totals, part, Lo.TW, status, cs1);
           if (e2 == cudaSuccess)
             e2 = launch_batched_refine_update(part, ract, sc, B, list_off, part_off, totals, ym,
                                               yf, mdone, mscore, d, DP, DA, rtol_s * rtol_s, 0,
@@ -655,7 +706,7 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
                         status, cs0);
       if (e == cudaSuccess)
         e = launch_batched_step(Xs, d, DP, yf, ract, sc, B, kPlanModes, task_off, part_off,
-                                totals, part, Lo.TW, cs0);
+                                totals, part, Lo.TW, status, cs0);
       if (e == cudaSuccess)
         e = launch_batched_refine_update(part, ract, sc, B, list_off, part_off, totals, ym, yf,
                                          mdone, mscore, d, DP, DA, 0.0, 1, grid_upd, cs0);
@@ -728,8 +779,10 @@ fms_status fms_cluster_batched(const float* points, const int64_t* offsets, int3
       // (queued: pack, the sort's five, seed init; per round seeds, travel, kept,
       // (density,) prune, advance, seed init; setup, queue, refinement or density)
       stats->kernel_launches =
-          queued ? 2 + (cv.P > 0 ? cells::sort_launches(max_n) : 0) + (o.gamma >= 1.f ? 7 : 6) * rounds + 3 + 3
-                 : 2 + 7 * rounds + 3 * updates + (o.skip_refine ? 0 : 2 + 3 * refines) + 4 + 3;
+          (ask ? 1 : 0) +
+          (queued ? 2 + (P > 0 ? cells::sort_launches(max_n) : 0) +
+                        (o.gamma >= 1.f ? 7 : 6) * rounds + 3 + 3
+                  : 2 + 7 * rounds + 3 * updates + (o.skip_refine ? 0 : 2 + 3 * refines) + 4 + 3);
       stats->evals = ev;
       stats->workspace_bytes = need;
       stats->graph = 1;

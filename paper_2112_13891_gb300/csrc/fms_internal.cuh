@@ -482,6 +482,7 @@ cudaError_t launch_ms_step(const float* Xs, int64_t n, int d, int DP, const floa
                            const int32_t* p_lo_ptr = nullptr, int kf = kKernelGaussian,
                            uint32_t* status = nullptr);
 int step_seeds_per_warp(int d);
+int batched_seeds_per_warp(int d);   // the batched step's wide tasks (32 lanes x RG seeds)
 int step_resident_warps_per_sm(int d);
 // smallest chunk (points) of a warp task: the low-d kernel splits a chunk over
 // 32 lanes, the quad kernel (d = 8) over 4 point lanes, the wide kernel

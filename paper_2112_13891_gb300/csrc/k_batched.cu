@@ -7,8 +7,9 @@
 // control blocks (SetCtl) hold each set's clock, counts and chunking; a plan
 // (prefix sums over sets of warp tasks, partial-sum blocks and list entries)
 // lets one launch of the step / update kernels map a global task or list
-// index to (set, local index) by binary search.  For d > 7, or large sets, one queue of all sets'
-// seeds takes each of them to convergence in one launch instead (k_travel.cu).  One CTA per set runs the
+// index to (set, local index) by binary search.  Where cells leave enough out, one
+// queue of all sets' seeds takes each of them to convergence in one launch instead
+// (k_travel.cu).  One CTA per set runs the
 // per-set bookkeeping (compaction under the Early Stopping clock rule, kept
 // list, prune, ordering); the last CTA to finish (atomic ticket, no waiting)
 // rebuilds the plan for the next launch.  The whole call runs as one CUDA
@@ -302,12 +303,57 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+template <int DPAD, int RG>
+__global__ void __launch_bounds__(128)
+    batched_step_wide(const float* __restrict__ Xs, const float* __restrict__ y,
+                      const int32_t* __restrict__ list, const SetCtl* __restrict__ sc, int B,
+                      int kind, const int64_t* __restrict__ task_off,
+                      const int64_t* __restrict__ part_off, const int64_t* __restrict__ totals,
+                      float* __restrict__ part, uint32_t* __restrict__ status) {
+  extern __shared__ __align__(16) float wide_tiles[];
+  __shared__ __align__(8) uint64_t wide_bars[4][2];
+  constexpr int SPW = 32 * RG;
+  const int64_t T = totals[0];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t* bars = wide_bars[warp];
+  float* tiles = wide_tiles + warp * 2 * kWideTile * DPAD;
+  tc::ring_init(bars, lane);
+  uint32_t use0 = 0u, use1 = 0u;
+  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; t < T; t += nw) {
+    const int b = find_set(task_off, B, t);
+    const SetCtl& c = sc[b];
+    int cnt, C, Lc;
+    plan_counts(c, kind, &cnt, &C, &Lc);
+    const int64_t local = t - task_off[b];
+    const int G = (cnt + SPW - 1) / SPW;
+    const int g = (int)(local % G), ch = (int)(local / G);
+    const int j0 = ch * Lc, j1 = min(c.n, j0 + Lc);
+    if (!wide_task<DPAD, RG>(Xs + (int64_t)c.p0 * DPAD, j0, j1, y, list + c.p0, cnt, g, ch,
+                             part + part_off[b], lane, 0, tiles, bars, use0, use1, status))
+      break;
+  }
+}
+
+template <int DPAD, int RG>
+static void launch_bwide(int grid, const float* Xs, const float* y, const int32_t* list,
+                         const SetCtl* sc, int B, int kind, const int64_t* task_off,
+                         const int64_t* part_off, const int64_t* totals, float* part,
+                         uint32_t* status, cudaStream_t st) {
+  if (wide_smem_bytes<DPAD>() > 40 * 1024)   // (its barriers count against the default 48 KB)
+    cudaFuncSetAttribute(batched_step_wide<DPAD, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         wide_smem_bytes<DPAD>());
+  batched_step_wide<DPAD, RG><<<grid, 128, wide_smem_bytes<DPAD>(), st>>>(
+      Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status);
+}
+
 cudaError_t launch_batched_step(const float* Xs, int d, int DP, const float* y,
                                 const int32_t* list, const SetCtl* sc, int B, int kind,
                                 const int64_t* task_off, const int64_t* part_off,
                                 const int64_t* totals, float* part, int target_warps,
-                                cudaStream_t st) {
+                                uint32_t* status, cudaStream_t st) {
   const int g = (target_warps + 7) / 8;
+  if (d > 7 && DP != padded_dim(d)) return cudaErrorInvalidValue;   // rows of the compiled width
   switch (d) {
     case 1: batched_step_lowd<1, 4, 2><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
     case 2: batched_step_lowd<2, 4, 4><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
@@ -316,7 +362,15 @@ cudaError_t launch_batched_step(const float* Xs, int d, int DP, const float* y,
     case 5: batched_step_lowd<5, 8, 8><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
     case 6: batched_step_lowd<6, 8, 8><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
     case 7: batched_step_lowd<7, 8, 8><<<g, 256, 0, st>>>(Xs, y, list, sc, B, kind, task_off, part_off, totals, part); break;
-    default: return cudaErrorInvalidValue;   // (d > 7: the queue of k_travel.cu)
+    default:
+#define FMS_WIDE(DP_, RG_) \
+  launch_bwide<DP_, RG_>(2 * g, Xs, y, list, sc, B, kind, task_off, part_off, totals, part, status, st)
+      if (d <= 8) FMS_WIDE(8, 4);
+      else if (d <= 16) FMS_WIDE(16, 2);
+      else if (d <= 32) FMS_WIDE(32, 1);
+      else FMS_WIDE(64, 1);
+#undef FMS_WIDE
+      break;
   }
   return cudaGetLastError();
 }

@@ -145,6 +145,13 @@ int step_seeds_per_warp(int d) {
   return 32;                   // wide kernel: 32 lanes x 1 seed
 }
 
+int batched_seeds_per_warp(int d) {
+  if (d <= 7) return step_seeds_per_warp(d);
+  if (d <= 8) return 32 * 4;   // wide tasks: 32 lanes x RG seeds
+  if (d <= 16) return 32 * 2;
+  return 32;
+}
+
 int step_accumulators(int d) {
   if (d <= 1) return 2;
   if (d <= 3) return 4;

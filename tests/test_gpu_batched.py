@@ -238,3 +238,31 @@ def test_batched_one_large_set_among_many():
     assert (r.n_modes == 1).all() and (r.labels == 0).all()
     assert torch.allclose(torch.cat(r.modes[:-1]), small, rtol=1e-6, atol=1e-6)
     assert r.modes[-1].abs().max() < 2e-3       # the mean of 3.4e7 normal points: 2e-4
+
+
+@pytest.mark.parametrize("d", [3, 8, 9, 16, 30, 48])
+@pytest.mark.parametrize("kw", [{}, dict(gamma=1.0), dict(skip_refine=True)])
+def test_batched_clusters_in_reach_of_each_other(d, kw):
+    # clusters on the axes, 6.4 h apart: each seed sees all of its set, so the updates are
+    # steps of all sets (a ninth set of 20,000 points raises the mean above 2,048)
+    rng = np.random.default_rng(d)
+    h, sets = 1.0, []
+    for n in (900, 1500, 700, 2300, 1200, 40, 800, 1100, 20_000):
+        k = min(d, 3 + len(sets) % 3)
+        sets.append((4.5 * np.eye(d)[rng.integers(0, k, n)]
+                     + 0.4 * rng.standard_normal((n, d))).astype(np.float32))
+    X = [torch.from_numpy(s).cuda() for s in sets]
+    res = fms.cluster_batched(X, h, 1e-3 * h, 300, rng_seed=4, max_modes=64, **kw)
+    off = np.concatenate([[0], np.cumsum([len(s) for s in sets])])
+    okw = dict(kw)
+    if okw.pop("skip_refine", False):
+        okw["refine"] = False
+    for b, s in enumerate(sets):
+        ref = orc.cluster(s, h, 1e-3 * h, 300, rng_seed=4, **okw)
+        cmp = compare_clustering(res.modes[b].cpu().numpy(),
+                                 res.labels[off[b]:off[b + 1]].cpu().numpy(), ref, h,
+                                 # (unrefined: where some seed made a step of at most tol =
+                                 # 1e-3 h, 1 / (1 - contraction) of that from the mode)
+                                 **(dict(score_rtol=1e-4, mode_tol=1e-2) if "skip_refine" in kw
+                                    else {}))
+        assert cmp["mode_ok"] and cmp["label_mismatch"] == 0, (b, cmp)
