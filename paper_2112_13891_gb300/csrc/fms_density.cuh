@@ -185,37 +185,12 @@ __device__ __forceinline__ double mode_density(const double* sums, int d, double
   return ldexp(rint(ldexp(m, 36)), e - 36);
 }
 
-// The modes' densities for the final order, by blocks bi = 0 .. nb - 1 (32 kDensityWarps
-// threads each) of one set of modes acc[i] (null: i), M <= kOrderStage: sm.score[i], the
-// near ties' from FP64.  Every block looks for near ties among all modes; where there are
-// none, all return true at once (*tied = false).  Else the blocks share the rows of up to
-// kTieCap tied modes, or the tied modes, and only the last to finish returns true
-// (*ticket counts them; no waiting; 0 again afterwards).
-__device__ inline bool order_densities(const DensityRows& D, const double* __restrict__ pos,
-                                       const double* __restrict__ score, double* dens,
-                                       const int32_t* __restrict__ acc, int M, int d, int DP,
-                                       double* scratch, int32_t* ticket, int bi, int nb,
-                                       OrderSmem& sm, bool* tied) {
-  *tied = false;
-  for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    const int a = acc ? acc[j] : j;
-    sm.score[j] = score[a];
-    sm.rough[j] = (float)score[a];
-    if (D.X) sm.err[j] = density_error(score[a], mode_norm(pos + (int64_t)a * DP, d));
-  }
-  if (threadIdx.x == 0) sm.ntied = 0;
-  __syncthreads();
-  if (!D.X) return true;
-  int mine = 0;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    const float si = sm.rough[i], ei = sm.err[i];
-    bool t = false;
-    for (int j = 0; j < M; ++j) t = t || (j != i && near_tie(si, ei, sm.rough[j], sm.err[j]));
-    sm.flag[i] = t ? 1 : 0;
-    mine += t ? 1 : 0;
-  }
-  if (!__syncthreads_or(mine)) return true;
-  *tied = true;
+// The near ties' part of order_densities, for the modes that sm.flag marks (out of line:
+// without any, a call's time is that of fetching the rest).
+static __device__ __noinline__ bool share_ties(const DensityRows& D, const double* __restrict__ pos,
+                                        double* dens, const int32_t* __restrict__ acc, int M,
+                                        int d, int DP, double* scratch, int32_t* ticket, int bi,
+                                        int nb, OrderSmem& sm) {
   if (threadIdx.x < 32) {   // the tied modes, in order
     int n = 0;
     for (int i0 = 0; i0 < M; i0 += 32) {
@@ -275,6 +250,40 @@ __device__ inline bool order_densities(const DensityRows& D, const double* __res
   }
   __syncthreads();
   return true;
+}
+
+// The modes' densities for the final order, by blocks bi = 0 .. nb - 1 (32 kDensityWarps
+// threads each) of one set of modes acc[i] (null: i), M <= kOrderStage: sm.score[i], the
+// near ties' from FP64.  Every block looks for near ties among all modes; where there are
+// none, all return true at once (*tied = false).  Else the blocks share the rows of up to
+// kTieCap tied modes, or the tied modes, and only the last to finish returns true
+// (*ticket counts them; no waiting; 0 again afterwards).
+__device__ inline bool order_densities(const DensityRows& D, const double* __restrict__ pos,
+                                       const double* __restrict__ score, double* dens,
+                                       const int32_t* __restrict__ acc, int M, int d, int DP,
+                                       double* scratch, int32_t* ticket, int bi, int nb,
+                                       OrderSmem& sm, bool* tied) {
+  *tied = false;
+  for (int j = threadIdx.x; j < M; j += blockDim.x) {
+    const int a = acc ? acc[j] : j;
+    sm.score[j] = score[a];
+    sm.rough[j] = (float)score[a];
+    if (D.X) sm.err[j] = density_error(score[a], mode_norm(pos + (int64_t)a * DP, d));
+  }
+  if (threadIdx.x == 0) sm.ntied = 0;
+  __syncthreads();
+  if (!D.X) return true;
+  int mine = 0;
+  for (int i = threadIdx.x; i < M; i += blockDim.x) {
+    const float si = sm.rough[i], ei = sm.err[i];
+    bool t = false;
+    for (int j = 0; j < M; ++j) t = t || (j != i && near_tie(si, ei, sm.rough[j], sm.err[j]));
+    sm.flag[i] = t ? 1 : 0;
+    mine += t ? 1 : 0;
+  }
+  if (!__syncthreads_or(mine)) return true;
+  *tied = true;
+  return share_ties(D, pos, dens, acc, M, d, DP, scratch, ticket, bi, nb, sm);
 }
 
 // Order of two modes: density descending, ties by lexicographic coordinates.

@@ -266,14 +266,18 @@ struct PruneTest {
       const float D = sqrtf(s), m = (sqrtf(a) + sqrtf(b)) * 2.3841858e-7f + 1e-17f;
       if (D + m < lo) return true;
       if (D - m > hi && D < 1e15f) return false;
-      const PT *x = pos + row(p) * DP, *y = pos + row(q) * DP;
-      PT d2 = 0;
-      for (int k = 0; k < d; ++k) {
-        const PT e = x[k] - y[k];
-        d2 += e * e;
-      }
-      return d2 < r2;
+      return within_exactly(p, q);
     }
+  }
+  // (out of line: a small problem's time is that of fetching the code)
+  __device__ __noinline__ bool within_exactly(int p, int q) const {
+    const PT *x = pos + row(p) * DP, *y = pos + row(q) * DP;
+    PT d2 = 0;
+    for (int k = 0; k < d; ++k) {
+      const PT e = x[k] - y[k];
+      d2 += e * e;
+    }
+    return d2 < r2;
   }
 };
 
@@ -337,7 +341,7 @@ struct VisitD {
 // beyond 8,192 slots it would be the barriers of a sort in shared memory (9,000
 // candidates: 195 us there, 112 so).
 template <typename V, typename ST, int E>
-__device__ __forceinline__ void sort_slots(const ST* __restrict__ score, int K, int P,
+__device__ __noinline__ void sort_slots(const ST* __restrict__ score, int K, int P,
                                            unsigned char* buf, int* order) {
   V x[E];
   const int tid = threadIdx.x, T = P / E;

@@ -865,7 +865,6 @@ cudaError_t launch_travel_seeds(const float* Xs, const View<float>& cv, int n, i
                                                         tol2_s, sphere_r, evals);                \
   return cudaGetLastError();
   switch (DP) {
-    case 4: FMS_SEEDS(4)
     case 8: FMS_SEEDS(8)
     case 16: FMS_SEEDS(16)
     case 32: FMS_SEEDS(32)
