@@ -79,7 +79,7 @@ constexpr size_t kCtlRoundOff = 896;   // RoundCtl of the device-driven rounds
 static_assert(kCtlRoundOff + sizeof(RoundCtl) <= kCtlBlockBytes, "control region");
 
 // ---------------------------------------------------------------------------
-// CUDA-graph form of fms_cluster.  When every round fits the cluster kernels,
+// CUDA-graph form of fms_cluster.  When every round fits the grid or cluster kernels,
 // the whole call (packing, Seed Selection, the rounds with their prunes and
 // seed-count decisions, refinement, labels) is one graph: a conditional WHILE
 // node repeats the round body while round_advance asks for another round, and

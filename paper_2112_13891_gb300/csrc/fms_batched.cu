@@ -110,8 +110,8 @@ int sms_now() {
 
 struct BLayout {
   size_t Xs, y, it, conv, state, active, kept, acc1, acc2, plist, score, ym, yf, ract, mdone,
-      mscore, dens, ties, modes_full, part, sc, task_off, part_off, list_off, totals, counters, pt_off, status,
-      sorted, start, ctr, npiv, rad, sort, wlast, total;
+      mscore, dens, ties, modes_full, part, sc, task_off, part_off, list_off, totals, counters,
+      pt_off, status, sorted, start, ctr, npiv, rad, sort, wlast, total;
   int DP, DA, R, TW, P;
   bool queued, steps;   // the routes that the call has the scratch for
   Tiling tl;

@@ -6,9 +6,9 @@
 // 2^-(32 + log2 n) W changes W and S/W by less than 2^-32 of W, a 256th of one
 // FP32 rounding (guard_bits; more for FP64).  Points are therefore sorted into
 // cells (the nearest of up to P pivots; a stable counting sort, so the order and
-// every sum that follows is the same on each run), each with a bounding ball, and a group of seeds walks only the cells whose ball comes within the
-// cutoff radius of the group's own ball.  The bound is checked against the W that
-// came out: a group whose smallest W asks for a wider cutoff is evaluated again
+// every sum that follows is the same on each run), each with a bounding ball, and
+// a group of seeds walks only the cells whose ball comes within the cutoff radius
+// of the group's own ball.  The bound is checked against the W that came out: a group whose smallest W asks for a wider cutoff is evaluated again
 // with that one (up to the distance where exp2 itself gives zero), so no
 // assumption about the seeds enters.  A ball test that meets NaN or infinity
 // keeps the cell.
@@ -218,7 +218,8 @@ struct SortScratch {
 inline SortScratch sort_scratch(int64_t B, int64_t rows, int P, int64_t total = 0) {
   SortScratch s{};
   s.counts = align256((size_t)(total > 0 ? total : B * rows));
-  const size_t chunks = total > 0 ? (size_t)(total / kChunkRows + B) + 1 : (size_t)(B * sort_blocks(rows));
+  const size_t chunks =
+      total > 0 ? (size_t)(total / kChunkRows + B) + 1 : (size_t)(B * sort_blocks(rows));
   s.far_ = s.counts + align256(chunks * P * 4);
   s.cell_rows = s.far_ + align256((size_t)B * (P / 2) * 8);
   s.total = s.cell_rows + align256((size_t)B * P * 4);

@@ -92,7 +92,8 @@ constexpr int team_warp_smem() {
 }
 template <typename T, int DP, int SUMS>   // a team that walks cells
 constexpr int group_team_smem(int W) {
-  return W * team_warp_smem<T, DP, SUMS>() + SUMS * 32 * (int)sizeof(T) + kListCap * 8 + (int)sizeof(GroupSmem<T, DP>);
+  return W * team_warp_smem<T, DP, SUMS>() + SUMS * 32 * (int)sizeof(T) + kListCap * 8 +
+         (int)sizeof(GroupSmem<T, DP>);
 }
 // Few unsorted points are kept in shared memory by every team for all its updates,
 // in the place of the rings: an update of 1,500 points by 16 warps is three tiles a

@@ -9,13 +9,12 @@
 // lets one launch of the step / update kernels map a global task or list
 // index to (set, local index) by binary search.  Where cells leave enough out, one
 // queue of all sets' seeds takes each of them to convergence in one launch instead
-// (k_travel.cu).  One CTA per set runs the
-// per-set bookkeeping (compaction under the Early Stopping clock rule, kept
-// list, prune, ordering); the last CTA to finish (atomic ticket, no waiting)
-// rebuilds the plan for the next launch.  The whole call runs as one CUDA
-// graph: the compaction, advance and refinement kernels decide on the device,
-// through conditional-node handles, whether another update, another seed round
-// or another refinement update follows.
+// (k_travel.cu).  One CTA per set runs the per-set bookkeeping (compaction under
+// the Early Stopping clock rule, kept list, prune, ordering); the last CTA to
+// finish (atomic ticket, no waiting) rebuilds the plan for the next launch.  The
+// whole call runs as one CUDA graph: the compaction, advance and refinement
+// kernels decide on the device, through conditional-node handles, whether another
+// update, another seed round or another refinement update follows.
 #include "fms_cells.cuh"
 #include "fms_density.cuh"
 #include "fms_label.cuh"
@@ -607,8 +606,10 @@ __global__ void __launch_bounds__(1024)
 
 // ---------------------------------------------------------------------------
 // The round's stop t* (the first update by which the target of Early Stopping has
-// converged, max_iter if it never does) and the kept seeds of each set with the
-// densities of their last updates (keep_exhausted: a density pass over the queue of them follows).
+// converged, max_iter if it never does) and the kept seeds of each set with W of
+// their last updates, which the prune visits them by: the density one step of at most
+// tol before where they stand, lower by a share of the order of (step / h)^2, 1e-6 at the
+// default tol (keep_exhausted: a density pass over the queue of them follows instead).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024)
     queue_kept(SetCtl* sc, int B, const int32_t* __restrict__ state,

@@ -387,8 +387,9 @@ __global__ void __launch_bounds__(1024)
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
     scatter_kernel(const T* __restrict__ src, const int64_t* __restrict__ offs, int B, int each,
-                   int per, int P, const unsigned char* __restrict__ id, const int32_t* __restrict__ counts,
-                   const int32_t* __restrict__ cell_rows, T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
+                   int per, int P, const unsigned char* __restrict__ id,
+                   const int32_t* __restrict__ counts, const int32_t* __restrict__ cell_rows,
+                   T* __restrict__ dst, int32_t* __restrict__ perm, int32_t* __restrict__ start,
                    int2* __restrict__ table, int cap, int gsz, int32_t* __restrict__ gcell,
                    Gate gate) {
   wait_for_previous();

@@ -14,12 +14,13 @@
 //
 // Measured on one GB300 against the kernels that took every pair, one launch an
 // update: 20,011 seeds x 65,537 points x 32 (one update) 4.91 -> 0.77 ms, of which
-// step_groups 0.53 (0.67 with the sums in registers, one block an SM); 200,000 x 3, every point a seed, 86 -> 12.8 ms (17.4 with the
-// padding column evaluated); 2,000 x 2 (not sorted) 0.56 -> 0.16 ms; 65,536 x 32 with
-// 128 to 512 seeds 2.96 -> 0.62 ms, of which the three travel_seeds 0.21 (0.25 with 8
-// warps a seed); 200,000 x 16 directions 1.45 -> 0.47 ms, of which the two
-// travel_seeds 0.12 (0.14); 256 sets of 1,000 to 50,000 x 16 in one call
-// (travel_queue, 4 warps a seed) 29.0 -> 5.2 ms.
+// step_groups 0.53 (0.67 with the sums in registers, one block an SM); 200,000 x 3,
+// every point a seed, 86 -> 12.4 to 16.3 ms by the input (its slowest seeds hold their
+// groups; with the padding column evaluated 17.4 where it is 12.8); 2,000 x 2 (not
+// sorted) 0.56 -> 0.16 ms; 65,536 x 32 with 128 to 512 seeds 2.96 -> 0.63 ms, of which
+// the three travel_seeds 0.21 (0.25 with 8 warps a seed); 200,000 x 16 directions
+// 1.45 -> 0.49 ms, of which the two travel_seeds 0.12 (0.14); 256 sets of 1,000 to
+// 50,000 x 16 in one call (travel_queue, 4 warps a seed) 29.0 -> 5.2 ms.
 #include "fms_team.cuh"
 
 namespace fms {

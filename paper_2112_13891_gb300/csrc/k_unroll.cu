@@ -603,13 +603,17 @@ cudaError_t unroll_backward_segment(const T* X, const View<T>& cv, const USegmen
                                     T inv_h2, double inv_h3, const T* Gin, T* Gout, T* SD, T* bctr,
                                     T* breach, double* dh_part, T* dX, int first,
                                     cudaStream_t st) {
-  if (g.d <= 3) return bwd_t<T, 4, 3>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
+#define FMS_BWD(...)                                                                         \
+  return bwd_t<T, __VA_ARGS__>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, \
+                               breach, dh_part, dX, first, st)
+  if (g.d <= 3) FMS_BWD(4, 3);
   switch (g.DP) {
-    case 4: return bwd_t<T, 4>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
-    case 8: return bwd_t<T, 8>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
-    case 16: return bwd_t<T, 16>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
-    case 32: return bwd_t<T, 32>(X, cv, sg, gx, gr, g, c, inv_h2, inv_h3, Gin, Gout, SD, bctr, breach, dh_part, dX, first, st);
+    case 4: FMS_BWD(4);
+    case 8: FMS_BWD(8);
+    case 16: FMS_BWD(16);
+    case 32: FMS_BWD(32);
   }
+#undef FMS_BWD
   return cudaErrorInvalidValue;
 }
 
