@@ -15,7 +15,7 @@
 // Measured on one GB300 against the kernels that took every pair, one launch an
 // update: 20,011 seeds x 65,537 points x 32 (one update) 4.91 -> 0.77 ms, of which
 // step_groups 0.53 (0.67 with the sums in registers, one block an SM); 200,000 x 3,
-// every point a seed, 86 -> 12.4 to 16.3 ms by the input (its slowest seeds hold their
+// every point a seed, 86 -> 12.4 to 23.8 ms by the input (its slowest seeds hold their
 // groups; with the padding column evaluated 17.4 where it is 12.8); 2,000 x 2 (not
 // sorted) 0.56 -> 0.16 ms; 65,536 x 32 with 128 to 512 seeds 2.96 -> 0.63 ms, of which
 // the three travel_seeds 0.21 (0.25 with 8 warps a seed); 200,000 x 16 directions
